@@ -155,14 +155,18 @@ int sample_attempt(gelo_ctx* ctx, const Layout& L, int m, int kind, uint64_t see
     const int ldi = L.ldi;
     GELO_TRY(launch_gaussian(ctx, m, m, ldi, seed, GELO_STREAM_G0, attempt, 1.0f, nullptr, L.G, st, seed_dev));
     const int l3 = level3_kind(ctx, m, dtype, true);
-    if (l3 == 3) GELO_TRY(run_householder_qr_tf32(ctx, m, L.G, ldi, L.Qraw, L.qr, L.tc, st));
+    // the block route signs its columns itself; the others leave that to the copy (by the diagonal of R, in L.G)
+    const bool blocks = l3 == 3 && gaussian_qr_supports(m);
+    const float* sign = blocks ? nullptr : L.G;
+    if (blocks) GELO_TRY(run_gaussian_qr(ctx, m, L.G, ldi, L.Qraw, L.tc, st));
+    else if (l3 == 3) GELO_TRY(run_householder_qr_tf32(ctx, m, L.G, ldi, L.Qraw, L.qr, L.tc, st));
     else if (l3) GELO_TRY(run_householder_qr_tc(ctx, m, L.G, ldi, L.Qraw, L.qr, L.tc, st));
     else GELO_TRY(run_householder_qr(ctx, m, L.G, ldi, L.Qraw, L.qr, st));
     if (kind == GELO_ORTHOGONAL) {
         // tf32 updates: polish Q (A32 and X32 are free for this kind).  The non-orthogonal kind skips it: there Q0 only
         // has to keep A = Q0 + gamma G1 well conditioned, and A^-1 comes from the LU of the stored A.
         if (l3 == 3) GELO_TRY(polish_orthogonal_tf32(ctx, m, L.Qraw, ldi, L.X32, L.A32, st));
-        GELO_TRY(launch_finish_mixing(ctx, m, L.Qraw, ldi, L.G, ldi, dtype, A_out, Ainv_out, lda, st));
+        GELO_TRY(launch_finish_mixing(ctx, m, L.Qraw, ldi, sign, ldi, dtype, A_out, Ainv_out, lda, st));
         if (cond_dev) {
             set_scalar_kernel<<<1, 1, 0, st>>>(cond_dev, 1.0f);
             GELO_TRY(after_launch(ctx));
@@ -170,9 +174,9 @@ int sample_attempt(gelo_ctx* ctx, const Layout& L, int m, int kind, uint64_t see
         return GELO_OK;
     }
     // Q0 (signed, fp32) -> A = Q0 + gamma / sqrt(m) * G1 -> stored type -> inverse of the stored A
-    GELO_TRY(launch_finish_mixing(ctx, m, L.Qraw, ldi, L.G, ldi, GELO_F32, L.A32, nullptr, ldi, st));
+    if (sign) GELO_TRY(launch_finish_mixing(ctx, m, L.Qraw, ldi, sign, ldi, GELO_F32, L.A32, nullptr, ldi, st));
     const float s = ctx->gamma / sqrtf((float)m);
-    GELO_TRY(launch_gaussian(ctx, m, m, ldi, seed, GELO_STREAM_G1, attempt, s, L.A32, L.A32, st, seed_dev));
+    GELO_TRY(launch_gaussian(ctx, m, m, ldi, seed, GELO_STREAM_G1, attempt, s, sign ? L.A32 : L.Qraw, L.A32, st, seed_dev));
     // the inverse is that of the stored A: round, and carry on from the rounded values
     GELO_TRY(launch_narrow(ctx, m, L.A32, ldi, dtype, A_out, lda, st, dtype != GELO_F32 ? L.A32 : nullptr, ldi));
     // tensor-core updates serve the bf16 path; the fp32 path stays exact

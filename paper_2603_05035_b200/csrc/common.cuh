@@ -171,6 +171,9 @@ int launch_gemm_tc_split_k(gelo_ctx*, int M, int N, int K, const void* Ahi, cons
 int launch_gemm_tf32(gelo_ctx*, int M, int N, int K, const float* A, int lda, bool a_mn, const float* B, int ldb,
                      bool subtract, float* C, int ldc, bool round_out, float out_scale, int ksplit, size_t plane, int* used,
                      cudaStream_t, float diag_sub = 0.0f, float post_scale = 1.0f);
+// C (M x N) = out_scale * (A0^T B0 + A1^T B1) rounded to tf32; A0, A1: K x M, B0, B1: K x N, row-major
+int launch_gemm_tf32_dual(gelo_ctx*, int M, int N, int K, const float* A0, int lda0, const float* B0, int ldb0, const float* A1,
+                          int lda1, const float* B1, int ldb1, float* C, int ldc, float out_scale, cudaStream_t);
 // D (m x m bf16) = post_scale * (out_scale * Q^T Q - diag_sub I): tf32 product over the tiles on and above the diagonal only
 int launch_gram_sym_bf16(gelo_ctx*, int m, const float* Q, int ld, void* D, int ldd, float out_scale, float diag_sub,
                          float post_scale, cudaStream_t);
@@ -255,6 +258,8 @@ QrScratch carve_qr(Arena&, int m, int ld, char** idle = nullptr, size_t* idle_by
 // writes the orthogonal factor Q with G = Q R.  The caller flips column j of Q where
 // R_jj < 0 (launch_finish_mixing with sign_diag = R) to reach the unique factor.
 int run_householder_qr(gelo_ctx*, int m, float* R, int ld, float* Q, const QrScratch&, cudaStream_t);
+// The whole factorisation of an m x m matrix, m <= 128, in one launch: R (diagonal of either sign) overwrites G
+int launch_qr_small(gelo_ctx*, int m, float* G, int ld, float* Q, cudaStream_t);
 struct TcScratch;
 // Same factorisation with 128-column outer blocks whose updates run on the tensor cores in split precision.
 int run_householder_qr_tc(gelo_ctx*, int m, float* R, int ld, float* Q, const QrScratch&, const TcScratch&, cudaStream_t);
@@ -262,6 +267,11 @@ int run_householder_qr_tc(gelo_ctx*, int m, float* R, int ld, float* Q, const Qr
 // applied to the columns right of the group and, later, to Q, so the big matrices stream through the GPU once per
 // 512 columns instead of once per 128.
 int run_householder_qr_tf32(gelo_ctx*, int m, float* R, int ld, float* Q, const QrScratch&, const TcScratch&, cudaStream_t);
+// The orthogonal factor of a GAUSSIAN matrix on tf32 products, blocks factorised through their Gram matrices
+// (qr_block.cu; relies on the blocks being well conditioned).  G is overwritten with the reflectors; Q receives the
+// factor whose R has a positive diagonal.
+bool gaussian_qr_supports(int m);
+int run_gaussian_qr(gelo_ctx*, int m, float* G, int ld, float* Q, const TcScratch&, cudaStream_t);
 // One Newton-Schulz step Q <- Q - Q (Q^T Q - I) / 2 on the tensor cores in tf32: squares the orthogonality defect
 // that tf32 updates leave in Q.  D and Qold are m x ld scratch matrices.
 int polish_orthogonal_tf32(gelo_ctx*, int m, float* Q, int ld, float* D, float* Qold, cudaStream_t);

@@ -597,6 +597,8 @@ int launch_qr_small_rm(gelo_ctx* ctx, int m, float* G, int ld, float* Q, cudaStr
 
 constexpr int kSmallQrRows = 128;
 
+}  // namespace
+
 int launch_qr_small(gelo_ctx* ctx, int m, float* G, int ld, float* Q, cudaStream_t st)
 {
     if (m <= 32) return launch_qr_small_rm<32>(ctx, m, G, ld, Q, st);
@@ -604,9 +606,6 @@ int launch_qr_small(gelo_ctx* ctx, int m, float* G, int ld, float* Q, cudaStream
     if (m <= 96) return launch_qr_small_rm<96>(ctx, m, G, ld, Q, st);
     return launch_qr_small_rm<128>(ctx, m, G, ld, Q, st);
 }
-
-}  // namespace
-
 
 // Takes `bytes` from the idle region if it has that much left, else from the arena.
 void* take_idle(Arena& a, char** idle, size_t* idle_bytes, size_t bytes)

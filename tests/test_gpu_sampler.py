@@ -1,0 +1,43 @@
+"""The sampler's own factorisation routes on the GPU (block QR of a Gaussian) against the oracle's factor."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2603_05035_b200 import binding
+from gpu_util import f64, padded
+
+pytestmark = pytest.mark.gpu
+
+ORTHOGONAL, NONORTHOGONAL = binding.ORTHOGONAL, binding.NONORTHOGONAL
+TDT = {"f32": torch.float32, "bf16": torch.bfloat16, "f16": torch.float16}
+
+
+def _sample(m, kind, seed, dt):
+    c = binding.Context(0)
+    c.ensure_workspace(m, 0, 8, 24, dt)
+    ld = c.mixing_ld(m)
+    A = padded(m, ld, TDT[dt]); X = padded(m, ld, TDT[dt])
+    c.sample_mixing(m, kind, seed, dt, A, X, ld)
+    assert c.last_status() == binding.OK
+    c.close()
+    return f64(A[:, :m]), f64(X[:, :m])
+
+
+# 256: the first size of the route, one full block and a square of 128; 257: a block of four columns; 383 .. 385: the block
+# before the square is as wide as it gets, full, or four columns again; 513, 641: a second group of blocks begins
+@pytest.mark.parametrize("m", [256, 257, 383, 384, 385, 513, 641])
+def test_block_qr_of_a_gaussian(oracle, m):
+    a, x = _sample(m, ORTHOGONAL, 900 + m, "f16")
+    assert np.array_equal(x, a.T)
+    # rounding A to half: 2^-12 sqrt(2/3) per off-diagonal pair and twice that on the diagonal, 2.9e-4 in this norm, beside
+    # the 3.1e-4 of zero-mean tf32 noise that the polishing step leaves
+    d = a.T @ a - np.eye(m)
+    assert np.linalg.norm(d) / np.sqrt(m) <= 6e-4
+    assert abs(np.trace(d)) / m <= 1e-4
+    # the factor itself: tf32 products err by 2^-11 sqrt(2/3) = 4e-4 per block and the first half of the columns sees at
+    # most m / 256 of them; the last columns are conditioned like the Gaussian itself, so they are only aligned
+    G64 = oracle.gaussian(900 + m, 0, 0, m, m).astype(np.float32).astype(np.float64)
+    q_ref, _ = oracle.householder_qr(G64)
+    h = m // 2
+    assert np.linalg.norm(a[:, :h] - q_ref[:, :h]) / np.sqrt(h) <= 4e-4 * (2 + m / 256)
+    assert np.median(np.sum(a * q_ref, axis=0)) > 1 - 1e-4
