@@ -175,15 +175,27 @@ int sample_attempt(gelo_ctx* ctx, const Layout& L, int m, int kind, uint64_t see
     }
     // Q0 (signed, fp32) -> A = Q0 + gamma / sqrt(m) * G1 -> stored type -> inverse of the stored A
     if (sign) GELO_TRY(launch_finish_mixing(ctx, m, L.Qraw, ldi, sign, ldi, GELO_F32, L.A32, nullptr, ldi, st));
+    const float* Q0 = sign ? L.A32 : L.Qraw;
     const float s = ctx->gamma / sqrtf((float)m);
-    GELO_TRY(launch_gaussian(ctx, m, m, ldi, seed, GELO_STREAM_G1, attempt, s, sign ? L.A32 : L.Qraw, L.A32, st, seed_dev));
-    // the inverse is that of the stored A: round, and carry on from the rounded values
-    GELO_TRY(launch_narrow(ctx, m, L.A32, ldi, dtype, A_out, lda, st, dtype != GELO_F32 ? L.A32 : nullptr, ldi));
-    // tensor-core updates serve the bf16 path; the fp32 path stays exact
-    const int l3lu = level3_kind(ctx, m, dtype, false);
-    if (l3lu) GELO_TRY(run_lu_inverse_tc(ctx, m, L.A32, ldi, L.X32, L.lu, L.tc, l3lu == 3, st));
-    else GELO_TRY(run_lu_inverse(ctx, m, L.A32, ldi, L.X32, L.lu, st));
-    GELO_TRY(launch_narrow(ctx, m, L.X32, ldi, dtype, Ainv_out, lda, st));
+    if (ctx->level3 == 0 && newton_inverse_supports(m, dtype, ctx->gamma)) {
+        // X0 = Q0^T in the stored type; the fp32 matrices that are dead by now hold two 16-bit ones each
+        const size_t half = (size_t)m * ldi;
+        uint16_t* g16 = reinterpret_cast<uint16_t*>(L.G);
+        uint16_t* x16 = reinterpret_cast<uint16_t*>(L.X32);
+        GELO_TRY(launch_finish_mixing(ctx, m, Q0, ldi, nullptr, ldi, dtype, x16, g16, ldi, st));
+        GELO_TRY(launch_gaussian(ctx, m, m, ldi, seed, GELO_STREAM_G1, attempt, s, Q0, L.A32, st, seed_dev));
+        GELO_TRY(launch_narrow(ctx, m, L.A32, ldi, dtype, A_out, lda, st));
+        GELO_TRY(run_newton_inverse(ctx, m, dtype, A_out, lda, g16, g16 + half, x16, ldi, Ainv_out, lda, st));
+    } else {
+        GELO_TRY(launch_gaussian(ctx, m, m, ldi, seed, GELO_STREAM_G1, attempt, s, Q0, L.A32, st, seed_dev));
+        // the inverse is that of the stored A: round, and carry on from the rounded values
+        GELO_TRY(launch_narrow(ctx, m, L.A32, ldi, dtype, A_out, lda, st, dtype != GELO_F32 ? L.A32 : nullptr, ldi));
+        // tensor-core updates serve the 16-bit paths; the fp32 path stays exact
+        const int l3lu = level3_kind(ctx, m, dtype, false);
+        if (l3lu) GELO_TRY(run_lu_inverse_tc(ctx, m, L.A32, ldi, L.X32, L.lu, L.tc, l3lu == 3, st));
+        else GELO_TRY(run_lu_inverse(ctx, m, L.A32, ldi, L.X32, L.lu, st));
+        GELO_TRY(launch_narrow(ctx, m, L.X32, ldi, dtype, Ainv_out, lda, st));
+    }
     // the verified matrices are the stored ones: what mix and unmix will read
     return run_cond_estimate(ctx, m, A_out, Ainv_out, lda, dtype, ctx->cond_bound, cond_dev ? cond_dev : L.cond_val, L.cond,
                              st, deferred);

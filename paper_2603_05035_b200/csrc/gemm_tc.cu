@@ -43,7 +43,7 @@ constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr uint32_t kABytes = BM * BK * 2;            // 16 KiB
 constexpr uint32_t kTmemCols = 512;
 
-enum TcMode { TC_STORE_BF16 = 0, TC_STORE_F32 = 1, TC_SUB_F32 = 2, TC_EMIT_SPLIT = 3, TC_STORE_SYM16 = 4 };
+enum TcMode { TC_STORE_BF16 = 0, TC_STORE_F32 = 1, TC_SUB_F32 = 2, TC_EMIT_SPLIT = 3, TC_STORE_SYM16 = 4, TC_AFFINE16 = 5 };
 
 struct TcSegment { int a_sel, b_sel, a_k0, b_row0, kb; };
 
@@ -64,6 +64,7 @@ struct TcParams {
     int out_f16;                    // TC_STORE_BF16: operands and output are IEEE half instead of bfloat16
     const float* scale_a;           // TC_STORE_BF16 with 8-bit operands: the per-tensor scales (device scalars); the
     const float* scale_b;           //   accumulator is multiplied by their product before it is rounded
+    const void* add; int ldadd;     // TC_AFFINE16: out = out_scale * acc + diag_sub on the diagonal + the entry of `add` (optional)
     int tri, tri_tiles;             // TC_STORE_SYM16: the result is symmetric; only the tri_tiles tiles that reach the diagonal or lie
                                     // above it are computed, and what lies below them is filled in by mirroring
     uint32_t idesc;                 // instruction descriptor (filled in by the launcher)
@@ -163,6 +164,27 @@ __device__ __forceinline__ void epilogue_group(const TcParams& prm, int gm, int 
             pk.z = pack_bf16(v[4], v[5]); pk.w = pack_bf16(v[6], v[7]);
         }
         *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(base) + off) = pk;
+    } else if (prm.mode == TC_AFFINE16) {
+        float f[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            f[j] = fmaf(prm.out_scale, __uint_as_float(v[j]), (gm == gn + j) ? prm.diag_sub : 0.0f);
+        if (prm.add) {
+            const uint4 raw = *reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(prm.add) + (size_t)gm * prm.ldadd + gn);
+            const uint32_t w2[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 t = prm.out_f16 ? __half22float2(*reinterpret_cast<const __half2*>(&w2[j]))
+                                             : __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w2[j]));
+                f[2 * j] += t.x; f[2 * j + 1] += t.y;
+            }
+        }
+        uint32_t o[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            o[j] = prm.out_f16 ? pack_f16(__float_as_uint(f[2 * j]), __float_as_uint(f[2 * j + 1]))
+                               : pack_bf16(__float_as_uint(f[2 * j]), __float_as_uint(f[2 * j + 1]));
+        *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(prm.C0) + (size_t)gm * prm.ldc + gn) = make_uint4(o[0], o[1], o[2], o[3]);
     } else if (prm.mode == TC_STORE_F32) {
         const int chunk = gn / prm.csplit;                    // column block -> C0 / C1 / C2 (0 unless the output is split)
         float* base = static_cast<float*>(chunk == 0 ? prm.C0 : (chunk == 1 ? prm.C1 : prm.C2));
@@ -825,6 +847,35 @@ int launch_gemm_bf16_sub(gelo_ctx* ctx, int M, int N, int K, const void* A, int 
     p.mode = TC_SUB_F32;
     p.C0 = C; p.ldc = ldc;
     return launch_tiles<256, 3, true>(ctx, ma, ma, mb, mb, mc, p, 2.0 * M * (double)N * K, st);
+}
+
+// C (M x N, 16-bit type of the operands) = sign * A (M x K) B (K x N) + diag I + add (optional, M x N)
+int launch_gemm_affine16(gelo_ctx* ctx, int dtype, int M, int N, int K, const void* A, int lda, const void* B, int ldb, float sign,
+                         float diag, const void* add, int ldadd, void* C, int ldc, cudaStream_t st)
+{
+    if (M <= 0 || N <= 0 || K <= 0) return GELO_OK;
+    if (!ctx->tmap_encode) return GELO_ERR_CUDA;
+    if ((lda % 8) || (ldb % 8) || (ldc % 8) || (N % 8) || (ldadd % 8) || !aligned16(A) || !aligned16(B) || !aligned16(C) ||
+        !aligned16(add))
+        return GELO_ERR_INVALID;
+    CUtensorMap ma, mb;
+    bool b3d = false;
+    if (!make_map(ctx, &ma, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, BM) ||
+        !make_map_nmajor(ctx, &mb, B, 2, false, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, BK, 256, &b3d))
+        return GELO_ERR_CUDA;
+    TcParams p = {};
+    p.M = M; p.N = N;
+    p.nseg = 1;
+    p.seg[0] = TcSegment{0, 0, 0, 0, ceil_div(K, BK)};
+    p.ksplit = 1; p.kb_per_split = 1 << 30; p.plane = 0;
+    p.mode = TC_AFFINE16;
+    p.b3d = b3d ? 1 : 0;
+    p.out_f16 = dtype == GELO_F16 ? 1 : 0;
+    p.out_scale = sign; p.diag_sub = diag;
+    p.add = add; p.ldadd = ldadd;
+    p.C0 = C; p.ldc = ldc; p.csplit = N;
+    p.status = ctx->status_dev;
+    return launch_tiles<256, 4, false>(ctx, ma, ma, mb, mb, ma, p, 2.0 * M * (double)N * K, st);
 }
 
 // Y (M x N, bf16) = (sa sb) A8 (M x K, E4M3, row stride lda bytes) * B8 (K x N, E4M3, row stride ldb bytes): the offloaded

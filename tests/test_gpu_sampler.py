@@ -41,3 +41,24 @@ def test_block_qr_of_a_gaussian(oracle, m):
     h = m // 2
     assert np.linalg.norm(a[:, :h] - q_ref[:, :h]) / np.sqrt(h) <= 4e-4 * (2 + m / 256)
     assert np.median(np.sum(a * q_ref, axis=0)) > 1 - 1e-4
+
+
+# 256: the first size of the iteration, a single pair of tile rows; 257 and 300: ragged tiles; gamma 0.55 is the last it takes,
+# 0.6 goes to the LU
+@pytest.mark.parametrize("m,gamma,dt", [(256, 0.5, "f16"), (257, 0.5, "bf16"), (300, 0.55, "f16"), (700, 0.5, "f16"), (300, 0.6, "f16")])
+def test_inverse_of_the_nonorthogonal_sample(m, gamma, dt):
+    c = binding.Context(0)
+    c.ensure_workspace(m, 0, 8, 24, dt)
+    c.set_nonorthogonal(gamma)
+    ld = c.mixing_ld(m)
+    A = padded(m, ld, TDT[dt]); X = padded(m, ld, TDT[dt]); cond = torch.zeros(1, device="cuda")
+    c.sample_mixing(m, NONORTHOGONAL, 70 + m, dt, A, X, ld, cond)
+    assert c.last_status() == binding.OK
+    c.close()
+    a, x = f64(A[:, :m]), f64(X[:, :m])
+    ref = np.linalg.inv(a)
+    assert abs(cond.item() / np.linalg.cond(a) - 1) <= 0.12          # a lower estimate, see the estimator's own test
+    # what is left is one rounding of A^-1 to the storage type, half an ulp at most and 1/sqrt(3) of that in the mean over
+    # a binade: 2^-9 / sqrt(3) * 1.5 = 1.7e-3 (bf16), 2.1e-4 (half); the LU adds up to 1.3e-3
+    bound = {"bf16": 2.0e-3, "f16": 2.5e-4}[dt] + (1.3e-3 if gamma > 0.55 else 0.0)
+    assert np.linalg.norm(x - ref) / np.linalg.norm(ref) <= bound
