@@ -6,8 +6,14 @@
 // is the best estimate the Krylov space holds, the power iterate only its last vector.  A Ritz value never exceeds
 // lambda_max, so the estimate is a lower one.)
 // The operators are the matrices as stored (bf16 or fp32), i.e. exactly what the mixing and unmixing products
-// read.  All sums have a fixed order, so the estimate is bit-reproducible.  Every step streams both matrices once
-// from DRAM (the second touch of a row slab hits L2).
+// read.  All sums have a fixed order, so the estimate is bit-reproducible.
+//
+// A step is two launches: cond_step_kernel, bound by reading both operators (74 MB at 4300 rows in bf16, which stay in
+// L2 from step to step), and cond_reduce_kernel, whose last CTA also does the Lanczos recurrence.  What counts is
+// loads in flight: slabs of 16 rows (538 CTAs at 4300 rows) with two rows per warp and whole-vector loads of x, the
+// slab sums spread over sixteen threads per column, the eigenvalues searched by 32 lanes at a time.  Against 32-row
+// slabs with scalar loads of x, a thread per column in the sums, a launch of its own for the recurrence and bisection by
+// a single thread: 630 -> 250 us per estimate at 4300 rows (the pass over both operators 63 -> 23 us).
 #include "common.cuh"
 #include "philox.cuh"
 
@@ -15,8 +21,10 @@ namespace gelo {
 
 namespace {
 
-constexpr int kCondSlabsMax = 160;   // row slabs of one operator pass (one CTA each)
-constexpr int kCondChunkCols = 256;  // entries per CTA of the reduction over slabs
+constexpr int kCondRows = 16;        // rows of a slab (one CTA each), as long as that makes no more than ...
+constexpr int kCondSlabsMax = 512;   // ... this many slabs
+constexpr int kCondChunkCols = 64;   // entries per CTA of the reduction over slabs
+constexpr int kCondParts = 16;       // threads that share an entry's sum
 constexpr int kLanczosSteps = 6;     // the estimate is within about 6% of kappa_2 (measured at m = 64 .. 4300, gamma 0.5 .. 3)
 
 struct CondViews {
@@ -27,33 +35,22 @@ struct CondViews {
     float* w;         // [2][mpad]  Op^T Op v
     float* partial;   // [2][slabs][mpad]
     float* tri;       // [2][2][kLanczosSteps]  diagonal and off-diagonal of the Lanczos tridiagonal matrices
+    unsigned* done;   // [2]  CTAs of the current reduction that have finished (zero between launches)
 };
 
+// The start vector, as the only slab of a first reduction.
 __global__ void cond_init_kernel(CondViews v, uint64_t seed, uint32_t attempt)
 {
     const int z = blockIdx.y;
     const int i4 = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
+    if (i4 == 0) v.done[z] = 0;
     if (i4 >= v.mpad) return;
     float g[4];
     gaussian_block(seed, ((uint64_t)z * v.mpad + i4) >> 2, GELO_STREAM_POWER, attempt, g);
     for (int t = 0; t < 4; ++t) {
         const int i = i4 + t;
-        if (i >= v.mpad) break;
-        for (int s = 0; s < v.slabs; ++s)
-            v.partial[((size_t)z * v.slabs + s) * v.mpad + i] = (s == 0 && i < v.m) ? g[t] : 0.0f;
+        if (i < v.mpad) v.partial[(size_t)z * v.slabs * v.mpad + i] = i < v.m ? g[t] : 0.0f;
     }
-}
-
-// w = sum of slab partials (slabs ascend: fixed order), one thread per entry.
-__global__ void __launch_bounds__(kCondChunkCols) cond_reduce_kernel(CondViews v)
-{
-    const int z = blockIdx.y;
-    const int i = blockIdx.x * kCondChunkCols + threadIdx.x;
-    if (i >= v.m) return;
-    const float* p = v.partial + (size_t)z * v.slabs * v.mpad + i;
-    float s = 0.0f;
-    for (int k = 0; k < v.slabs; ++k) s += p[(size_t)k * v.mpad];
-    v.w[(size_t)z * v.mpad + i] = s;
 }
 
 // Sum over the CTA's threads in a fixed order; every thread receives it.
@@ -70,12 +67,11 @@ __device__ __forceinline__ float cond_block_sum(float local, float* red)
     return t;
 }
 
-// One CTA per operator.  step < 0: v = w / |w| (the start vector), vprev = 0.  Otherwise the Lanczos recurrence
+// step < 0: v = w / |w| (the start vector), vprev = 0.  Otherwise the Lanczos recurrence
 //   alpha = v . w,  r = w - alpha v - beta_prev vprev,  beta = |r|,  vprev <- v,  v <- r / beta.
-__global__ void __launch_bounds__(1024) cond_lanczos_kernel(CondViews v, int step)
+// Run by all 1024 threads of one CTA.
+__device__ __forceinline__ void cond_lanczos(const CondViews& v, int z, int step, float* red)
 {
-    __shared__ float red[32];
-    const int z = blockIdx.x;
     float* vc = v.v + (size_t)z * v.mpad;
     float* vp = v.vprev + (size_t)z * v.mpad;
     float* w = v.w + (size_t)z * v.mpad;
@@ -86,7 +82,7 @@ __global__ void __launch_bounds__(1024) cond_lanczos_kernel(CondViews v, int ste
         for (int i = threadIdx.x; i < v.m; i += 1024) local = fmaf(w[i], w[i], local);
         const float nrm = sqrtf(cond_block_sum(local, red));
         const float inv = nrm > 0.0f ? 1.0f / nrm : 0.0f;
-        for (int i = threadIdx.x; i < v.m; i += 1024) { vc[i] = w[i] * inv; vp[i] = 0.0f; }
+        for (int i = threadIdx.x; i < v.mpad; i += 1024) { vc[i] = i < v.m ? w[i] * inv : 0.0f; vp[i] = 0.0f; }
         return;
     }
     float local = 0.0f;
@@ -108,37 +104,85 @@ __global__ void __launch_bounds__(1024) cond_lanczos_kernel(CondViews v, int ste
     if (threadIdx.x == 0) { alpha[step] = a; beta[step] = b; }
 }
 
-// Largest eigenvalue of the symmetric tridiagonal matrix (alpha[0..k-1]; beta[0..k-2]) by bisection on the number of
-// eigenvalues below x (Sturm sequence), between 0 and the Gershgorin bound.  A breakdown (beta = 0) only decouples
-// the matrix: the count stays valid.
-__device__ double tridiagonal_lambda_max(const float* alpha, const float* beta, int k)
+// w = sum of `slabs` slab partials: kCondParts threads per entry take every kCondParts-th slab each, then their sums are
+// added in order.  The CTA that finishes last for an operator goes on with the recurrence.
+__global__ void __launch_bounds__(kCondChunkCols * kCondParts) cond_reduce_kernel(CondViews v, int slabs, int step)
 {
-    double hi = 0.0;
-    for (int i = 0; i < k; ++i) {
-        const double r = fabs((double)alpha[i]) + (i > 0 ? fabs((double)beta[i - 1]) : 0.0) + (i + 1 < k ? fabs((double)beta[i]) : 0.0);
-        if (r > hi) hi = r;
+    static_assert(kCondChunkCols * kCondParts == 1024, "cond_lanczos counts on 1024 threads");
+    __shared__ float part[kCondParts][kCondChunkCols];
+    __shared__ float red[32];
+    __shared__ int last;
+    const int z = blockIdx.y;
+    const int c = threadIdx.x % kCondChunkCols, q = threadIdx.x / kCondChunkCols;
+    const int i = blockIdx.x * kCondChunkCols + c;           // < mpad, a multiple of kCondChunkCols
+    const float* p = v.partial + (size_t)z * v.slabs * v.mpad + i;
+    float s = 0.0f;
+#pragma unroll 8
+    for (int k = q; k < slabs; k += kCondParts) s += p[(size_t)k * v.mpad];
+    part[q][c] = s;
+    __syncthreads();
+    if (q == 0 && i < v.m) {
+#pragma unroll
+        for (int t = 1; t < kCondParts; ++t) s += part[t][c];
+        v.w[(size_t)z * v.mpad + i] = s;
     }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        last = atomicAdd(v.done + z, 1u) + 1 == gridDim.x;
+        if (last) v.done[z] = 0;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    cond_lanczos(v, z, step, red);
+}
+
+// Largest eigenvalue of the symmetric tridiagonal matrix (alpha[0..k-1]; beta[0..k-2]), found by one warp that cuts the
+// interval from 0 to the Gershgorin bound into 33 at a time (twelve rounds: 2^-60 of the bound) by the number of
+// eigenvalues below each point (Sturm sequence).  A breakdown (beta = 0) only decouples the matrix: the count stays valid.
+__device__ double tridiagonal_lambda_max(const float* alpha, const float* beta)
+{
+    constexpr int k = kLanczosSteps;
+    double a[k], b2[k], hi = 0.0;
+#pragma unroll
+    for (int i = 0; i < k; ++i) {
+        a[i] = alpha[i];
+        const double bl = i > 0 ? fabs((double)beta[i - 1]) : 0.0, br = i + 1 < k ? fabs((double)beta[i]) : 0.0;
+        b2[i] = bl * bl;
+        hi = fmax(hi, fabs(a[i]) + bl + br);
+    }
+    const int lane = threadIdx.x & 31;
     double lo = 0.0;
-    for (int it = 0; it < 60; ++it) {
-        const double x = 0.5 * (lo + hi);
-        int below = 0;
+    for (int round = 0; round < 12; ++round) {
+        const double step = (hi - lo) * (1.0 / 33.0), x = lo + (lane + 1) * step;
+        bool all_below = true;                               // all k eigenvalues lie below x
         double q = 1.0;
+#pragma unroll
         for (int i = 0; i < k; ++i) {
-            const double b2 = i > 0 ? (double)beta[i - 1] * (double)beta[i - 1] : 0.0;
-            q = (double)alpha[i] - x - (i > 0 ? b2 / q : 0.0);
+            q = a[i] - x - (i > 0 ? b2[i] / q : 0.0);
             if (q == 0.0) q = -1e-300;
-            if (q < 0.0) ++below;
+            all_below = all_below && q < 0.0;
         }
-        if (below == k) hi = x; else lo = x;
+        const uint32_t mask = __ballot_sync(0xffffffffu, all_below);
+        const int first = mask ? __ffs(mask) - 1 : 32;       // the first point with everything below it
+        const double h = first < 32 ? lo + (first + 1) * step : hi;
+        lo = lo + first * step;
+        hi = h;
     }
     return 0.5 * (lo + hi);
 }
 
-__global__ void cond_verdict_kernel(CondViews v, float bound, float* cond_out, int* status, int deferred)
+// One warp per operator.
+__global__ void __launch_bounds__(64) cond_verdict_kernel(CondViews v, float bound, float* cond_out, int* status, int deferred)
 {
-    // lambda_max(Op^T Op) = sigma_max^2
-    const float c = (float)(sqrt(tridiagonal_lambda_max(v.tri, v.tri + kLanczosSteps, kLanczosSteps)) *
-                            sqrt(tridiagonal_lambda_max(v.tri + 2 * kLanczosSteps, v.tri + 3 * kLanczosSteps, kLanczosSteps)));
+    __shared__ double lam[2];
+    const int z = threadIdx.x >> 5;
+    const double l = tridiagonal_lambda_max(v.tri + z * 2 * kLanczosSteps, v.tri + z * 2 * kLanczosSteps + kLanczosSteps);
+    if ((threadIdx.x & 31) == 0) lam[z] = l;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    const float c = (float)(sqrt(lam[0]) * sqrt(lam[1]));    // lambda_max(Op^T Op) = sigma_max^2
     if (cond_out) cond_out[0] = c;
     const int ok = (c * 1.2f <= bound && c == c) ? 1 : 0;   // the estimate is a lower one (tests: >= 0.85 of the true value)
     status[1] = ok;
@@ -175,8 +219,9 @@ __device__ __forceinline__ void load8(const __half* p, float (&a)[8])
 }
 
 // One application Op^T (Op v) in a single pass over the operator: CTA (slab, z) first forms y_r =
-// Op[r, :] . xhat for its rows (one warp per row), then accumulates sum_r y_r Op[r, :] for every column; the
-// second read of the slab comes from L2.  partial[z][slab][:] receives the slab's contribution.
+// Op[r, :] . v for its rows (two rows per warp at a time, so that a vector load of v serves both), then accumulates
+// sum_r y_r Op[r, :] for every column; the second read of the slab comes from L1 or L2.  partial[z][slab][:] receives the
+// slab's contribution.
 template <typename T>
 __global__ void __launch_bounds__(256) cond_step_kernel(CondViews v)
 {
@@ -187,56 +232,72 @@ __global__ void __launch_bounds__(256) cond_step_kernel(CondViews v)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const T* op = static_cast<const T*>(v.op[z]);
     const float* x = v.v + (size_t)z * v.mpad;
-    const int groups = (v.m + 7) >> 3;
-    // loads are issued four at a time before anything is consumed: with one CTA's few warps per SM the kernel lives
-    // on memory-level parallelism
-    for (int r = r0 + warp; r < r1; r += 8) {
-        const T* a = op + (size_t)r * v.ld;
-        float s = 0.0f;
-        for (int g0 = lane; g0 < groups; g0 += 128) {
-            float e[4][8];
+    const int full = v.m >> 3, groups = (v.m + 7) >> 3;
+    for (int r = r0 + 2 * warp; r < r1; r += 16) {
+        const T* a0 = op + (size_t)r * v.ld;
+        const T* a1 = (r + 1 < r1) ? a0 + v.ld : a0;         // (an odd last row is read twice and counted once)
+        float s0 = 0.0f, s1 = 0.0f;
+#pragma unroll 4
+        for (int g = lane; g < full; g += 32) {
+            float e0[8], e1[8], xv[8];
+            load8(a0 + 8 * g, e0);
+            load8(a1 + 8 * g, e1);
+            load8(x + 8 * g, xv);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int g = g0 + 32 * u;
-                if (g < groups) load8(a + 8 * g, e[u]);
-            }
+            for (int t = 0; t < 8; ++t) { s0 = fmaf(e0[t], xv[t], s0); s1 = fmaf(e1[t], xv[t], s1); }
+        }
+        if (full < groups && lane == (full & 31)) {          // the columns past a multiple of 8
+            float e0[8], e1[8];
+            load8(a0 + 8 * full, e0);
+            load8(a1 + 8 * full, e1);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int g = g0 + 32 * u;
-                if (g < groups) {
-#pragma unroll
-                    for (int t = 0; t < 8; ++t)
-                        if (8 * g + t < v.m) s = fmaf(e[u][t], x[8 * g + t], s);
-                }
-            }
+            for (int t = 0; t < 8; ++t)
+                if (8 * full + t < v.m) { s0 = fmaf(e0[t], x[8 * full + t], s0); s1 = fmaf(e1[t], x[8 * full + t], s1); }
         }
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        if (lane == 0) ys[r - r0] = s;
+        for (int off = 16; off > 0; off >>= 1) {
+            s0 += __shfl_xor_sync(0xffffffffu, s0, off);
+            s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+        }
+        if (lane == 0) {
+            ys[r - r0] = s0;
+            if (r + 1 < r1) ys[r + 1 - r0] = s1;
+        }
     }
     __syncthreads();
     float* out = v.partial + ((size_t)z * v.slabs + slab) * v.mpad;
     for (int g = threadIdx.x; g < groups; g += 256) {
         float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int rb = r0; rb < r1; rb += 4) {
-            float e[4][8];
+        const T* a = op + (size_t)r0 * v.ld + 8 * g;
+        int r = 0;
+        for (; r + 8 <= r1 - r0; r += 8) {                   // rows ascend: the sum keeps its fixed order
+            float e[8][8];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (rb + u < r1) load8(op + (size_t)(rb + u) * v.ld + 8 * g, e[u]);
+            for (int u = 0; u < 8; ++u) load8(a + (size_t)(r + u) * v.ld, e[u]);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (rb + u < r1) {                           // rows ascend: the sum keeps its fixed order
-                    const float y = ys[rb + u - r0];
+            for (int u = 0; u < 8; ++u) {
+                const float y = ys[r + u];
 #pragma unroll
-                    for (int t = 0; t < 8; ++t) acc[t] = fmaf(e[u][t], y, acc[t]);
-                }
+                for (int t = 0; t < 8; ++t) acc[t] = fmaf(e[u][t], y, acc[t]);
             }
+        }
+        for (; r < r1 - r0; ++r) {
+            float e[8];
+            load8(a + (size_t)r * v.ld, e);
+            const float y = ys[r];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) acc[t] = fmaf(e[t], y, acc[t]);
         }
 #pragma unroll
         for (int t = 0; t < 8; ++t)
-            if (8 * g + t < v.m) out[8 * g + t] = acc[t];
+            if (8 * g + t >= v.m) acc[t] = 0.0f;             // (what stands past the last column is no data)
+        float4* o = reinterpret_cast<float4*>(out + 8 * g);
+        o[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        o[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
     }
 }
+
+int cond_slabs(int m) { return ceil_div(m, kCondRows) < kCondSlabsMax ? ceil_div(m, kCondRows) : kCondSlabsMax; }
 
 }  // namespace
 
@@ -244,7 +305,7 @@ CondScratch carve_cond(Arena& a, int m)
 {
     CondScratch s;
     const size_t mpad = (size_t)((m + 63) / 64) * 64;
-    s.vec = static_cast<float*>(a.take((6 + 2 * kCondSlabsMax) * mpad * sizeof(float)));
+    s.vec = static_cast<float*>(a.take((6 + 2 * (size_t)cond_slabs(m)) * mpad * sizeof(float)));
     s.scal = static_cast<float*>(a.take((16 + 4 * kLanczosSteps) * sizeof(float)));
     return s;
 }
@@ -255,33 +316,31 @@ int run_cond_estimate(gelo_ctx* ctx, int m, const void* A, const void* Ainv, int
     if ((ld % 8) || (reinterpret_cast<uintptr_t>(A) & 15u) || (reinterpret_cast<uintptr_t>(Ainv) & 15u)) return GELO_ERR_INVALID;
     CondViews v;
     v.op[0] = A; v.op[1] = Ainv; v.ld = ld; v.m = m; v.mpad = ((m + 63) / 64) * 64;
-    v.slabs = ceil_div(m, 32) < kCondSlabsMax ? ceil_div(m, 32) : kCondSlabsMax;
+    v.slabs = cond_slabs(m);
     v.rows_per = ceil_div(m, v.slabs);
     v.v = s.vec;
     v.vprev = s.vec + 2 * (size_t)v.mpad;
     v.w = s.vec + 4 * (size_t)v.mpad;
     v.partial = s.vec + 6 * (size_t)v.mpad;
     v.tri = s.scal + 16;
+    v.done = reinterpret_cast<unsigned*>(s.scal);
     const size_t ys_bytes = (size_t)v.rows_per * sizeof(float);
     if (ys_bytes > 48 * 1024) return GELO_ERR_UNSUPPORTED;
     dim3 gi(ceil_div(v.mpad, 4 * 256), 2);
     cond_init_kernel<<<gi, 256, 0, st>>>(v, 0x5eedull, 0u);
     GELO_TRY(after_launch(ctx));
-    const dim3 gr(ceil_div(m, kCondChunkCols), 2);
+    const dim3 gr(v.mpad / kCondChunkCols, 2), gs(ceil_div(m, v.rows_per), 2);
     for (int step = -1; step < kLanczosSteps; ++step) {
         if (step >= 0) {
-            dim3 g(v.slabs, 2);
-            if (dtype == GELO_BF16) cond_step_kernel<__nv_bfloat16><<<g, 256, ys_bytes, st>>>(v);
-            else if (dtype == GELO_F16) cond_step_kernel<__half><<<g, 256, ys_bytes, st>>>(v);
-            else cond_step_kernel<float><<<g, 256, ys_bytes, st>>>(v);
+            if (dtype == GELO_BF16) cond_step_kernel<__nv_bfloat16><<<gs, 256, ys_bytes, st>>>(v);
+            else if (dtype == GELO_F16) cond_step_kernel<__half><<<gs, 256, ys_bytes, st>>>(v);
+            else cond_step_kernel<float><<<gs, 256, ys_bytes, st>>>(v);
             GELO_TRY(after_launch(ctx));
         }
-        cond_reduce_kernel<<<gr, kCondChunkCols, 0, st>>>(v);
-        GELO_TRY(after_launch(ctx));
-        cond_lanczos_kernel<<<2, 1024, 0, st>>>(v, step);
+        cond_reduce_kernel<<<gr, kCondChunkCols * kCondParts, 0, st>>>(v, step < 0 ? 1 : (int)gs.x, step);
         GELO_TRY(after_launch(ctx));
     }
-    cond_verdict_kernel<<<1, 1, 0, st>>>(v, bound, cond_out, ctx->status_dev, deferred ? 1 : 0);
+    cond_verdict_kernel<<<1, 64, 0, st>>>(v, bound, cond_out, ctx->status_dev, deferred ? 1 : 0);
     return after_launch(ctx);
 }
 
