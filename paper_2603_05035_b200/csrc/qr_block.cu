@@ -8,7 +8,7 @@
 // (the compact WY form of Schreiber and Van Loan for the reflection that exchanges the orthonormal basis P R^-1 with -E;
 // T^-1 + T^-T = V^T V holds because B^T R = P^T P + (first b rows of P)^T R).  V differs from P in its top b x b block
 // only, so the reflectors stay where the panel was and no pass over the panel forms them.  What is serial in a block is
-// a 128 x 128 Cholesky factorisation and a 128 x 128 inverse in one CTA (block_factor_kernel); everything else is a
+// a 128 x 128 Cholesky factorisation and a 128 x 128 inverse (block_factor_kernel); everything else is a
 // product.  The update of columns C right of the block needs W' = T^T V^T C = T^T (P^T C) + D^T C1, D = R T = B^-T,
 // C1 = the first b rows of C: P^T C comes out of the same product as P^T P.
 // The last block, which would be square, is factorised by the one-launch Householder kernel.
@@ -19,26 +19,56 @@
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
+#include <type_traits>
+
 namespace gelo {
 
 namespace {
 
 constexpr int FB = kOuter;                     // block width
-constexpr int FS = FB + 4;                     // shared-memory row stride (16-byte rows, conflict-free column walks)
-// Two groups of 256 threads eliminate a 128 x 128 matrix each; thread (g, l) of a group (g = 0 .. 15, l = 0 .. 15) holds rows
-// g + 16 i and columns l + 16 q (i, q = 0 .. 7).  Step k then always finds its pivot row and column in registers of index
-// k / 16, a compile-time constant in a loop over the 16 steps that share it (the loops stay small enough for the
-// instruction cache), and the rows that are still to be eliminated are spread evenly over the warps.
-constexpr int kFactThreads = 512;
-constexpr int kRing = 16;                      // pivot rows in flight: one slot per step that shares a register index
+
+// ---- the 128 x 128 factorisation of a block, in a cluster of three CTAs -------------------------------------------
+//
+// CTA 0 eliminates the Gram matrix Z = R^T R (rows of R and of R^-T come out 16 at a time), CTA 1 inverts B = P1 + R by
+// Gauss-Jordan, CTA 2 applies the same row operations to R^-T and ends with B^-1 R^-T = T^T.  Each holds its matrix as fp32
+// accumulators of m16n8k16 matrix instructions in the registers of eight warps (32 rows x 64 columns each) and does eight
+// steps with 16 pivots p = 16 J .. 16 J + 15:
+//     publish    the rows p of the matrix (rows), and in CTA 1 its columns p (panel), go to shared memory
+//     U          = F * rows, F the inverse of the pivot block (CTA 0: of its Cholesky factor); in the columns p of an
+//                inverse that grows in place U is F itself
+//     update     a -= panel U, rows p <- U
+// A ninth warp runs ahead with the pivot blocks: as soon as the rows p are published it forms the next block (from its
+// published value, the panel and its 16 columns of U, straight from registers) and inverts it with shuffles while the
+// others are still busy with U and the update.  The rows of R and R^-T
+// are needed by the other CTAs only when their own step begins, because the elimination is linear in them: row p of B is
+// P1's until then.  They travel by bulk copies between the CTAs' shared memories into a slot per step, which is never
+// used twice, so nobody waits for space.
+//
+// The operands of the products are pairs of IEEE halves (x = hi + lo to 22 bits; hi hi + hi lo + lo hi, accumulated in fp32):
+// the caller scales the matrix to pivots around 1, so nothing leaves the range of a half, and the result has fp32 accuracy
+// (B^T D - I below 2e-6).  What bounds it is the chain of the 16-step inversions and, in CTA 1, the products (96 matrix
+// instructions per warp and step).  The same eliminations pivot by pivot in one CTA, with a broadcast each, took 57 us per launch;
+// fused multiply-adds on 8 x 8 tiles in this layout 36 us, bound by shared-memory reads; this form 25 us.
+constexpr int NB = 16;                         // pivots of a step
+constexpr int kSteps = FB / NB;
+constexpr int kFactCompute = 256;
+constexpr int kFactThreads = kFactCompute + 32;
+constexpr int kFactCtas = 3;
+constexpr int kPanelLd = NB + 8;               // row strides in halves: 16-byte rows, conflict-free matrix loads
+constexpr int kWideLd = FB + 8;
 struct FactShared {
-    float A[FB][FS];                           // R^-T (lower triangular)
-    float X[FB][FS];                           // R while B is eliminated, then D = B^-T
-    float row[2][kRing][FB + 4];               // pivot rows of the two groups; [FB]: reciprocal of the pivot
-    uint64_t full[2][kRing];                   // row slot published
-    uint64_t rready[8];                        // 16 rows of R complete
+    __half panel[kSteps][2][FB][kPanelLd];     // minus the columns p, hi and lo; CTA 0: the rows of R that it sends (fp32)
+    float got[kSteps][NB][FB];                 // CTA 1: rows of R, CTA 2: rows of R^-T; CTA 0: the rows of R^-T it sends
+    __half F[kSteps][2][NB][kPanelLd];
+    __half rows[2][2][NB][kWideLd];            // of even and of odd steps
+    __half U[2][NB][kWideLd];
+    float U32[NB][FB + 4];
+    float next[2][NB][NB + 4];                 // the next pivot block before the running update
+    uint64_t got_full[kSteps], panel_full[kSteps];
 };
 constexpr int kFactSmemBytes = (int)sizeof(FactShared);
+static_assert(kFactSmemBytes <= 227 * 1024, "shared memory budget");
+static_assert(sizeof(FactShared::panel) >= sizeof(float) * FB * FB, "CTA 0 keeps R there");
 
 __device__ __forceinline__ float fast_rcp(float x)
 {
@@ -58,190 +88,493 @@ __device__ __forceinline__ void fact_wait(const uint64_t* bar, uint32_t parity, 
     atomicCAS(status, 0, (int)GELO_ERR_TIMEOUT);
 }
 
-// Half warp g publishes its row of register index J: lane l the values of its columns as two float4.
-template <int J>
-__device__ __forceinline__ void publish_row(const float (&a)[8][8], float* slot, uint64_t* bar, int t, int g, int l)
+__device__ __forceinline__ void cluster_sync_all()
 {
-    if (g == t) {
-        *reinterpret_cast<float4*>(slot + 4 * l) = make_float4(a[J][0], a[J][1], a[J][2], a[J][3]);
-        *reinterpret_cast<float4*>(slot + 64 + 4 * l) = make_float4(a[J][4], a[J][5], a[J][6], a[J][7]);
-        if (l == t) slot[FB] = fast_rcp(a[J][J]);
-    }
-    __syncwarp();
-    if (g == t && l == 0) tcx::mbar_arrive(tcx::smem_u32(bar));
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Sixteen elimination steps with pivots k = 16 J + t:
-//     a_ij -= a_ik a_kj / a_kk   (j != k),      a_ik <- -a_ik / a_kk,
-// i.e. the inverse of the eliminating factor grows in the columns that are cleared.  kJordan: all rows i != k are
-// eliminated and row k becomes a_kj / a_kk, a_kk <- 1 / a_kk (the full inverse in the end); otherwise only the rows below k.
-// The special column and row ride along in the same multiply-adds: a_ik - a_ik (1 + 1 / a_kk) = -a_ik / a_kk and
-// a_kj - (a_kk - 1) (a_kj / a_kk) = a_kj / a_kk, exact enough because the caller scales the matrix to pivots around 1.
-// There is no barrier of all warps: a step waits for its pivot row only, and the owner of the next one updates and
-// publishes it before its other rows, so the latency from row to row is hidden behind the multiply-adds.  (A slot is
-// written again 16 steps later; every warp publishes twice in 16 steps and reads a step's row before it publishes the
-// next one, so by then all of them have read it.)
-template <int J, bool kJordan>
-__device__ __forceinline__ void sixteen_steps(float (&a)[8][8], float (*ring)[FB + 4], uint64_t* full, int g, int l, int* status)
+// Copies `bytes` of this CTA's shared memory to the place of `dst` in CTA `rank` and counts them on `bar` there.
+__device__ __forceinline__ void send_shared(const void* dst, const void* src, uint32_t bytes, const uint64_t* bar, int rank)
 {
-    const int half = threadIdx.x & 16;
-    if (g < 2) publish_row<J>(a, ring[0], full, 0, g, l);
-#pragma unroll 1
-    for (int t = 0; t < 16; ++t) {
-        float c[8];
+    uint32_t d, b;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(tcx::smem_u32(dst)), "r"(rank));
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(b) : "r"(tcx::smem_u32(bar)), "r"(rank));
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(d), "r"(tcx::smem_u32(src)), "r"(bytes), "r"(b) : "memory");
+}
+
+// Four 8 x 8 blocks of halves; lane i names row i % 8 of block i / 8.
+template <bool kTrans>
+__device__ __forceinline__ void ldsm4(uint32_t (&v)[4], const __half* p)
+{
+    const uint32_t addr = tcx::smem_u32(p);
+    if (kTrans)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(addr) : "memory");
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// Operand fragments as (hi, lo) pairs.  A (16 x 16): from a row-major array of rows, or (columns of U, CTA 0's panel)
+// from its transpose.  B (16 x 16, two column tiles): from an array of k rows.
+struct Pair4 { uint32_t hi[4], lo[4]; };
+__device__ __forceinline__ void load_a(Pair4& f, const __half* hi, const __half* lo, int ld, int lane)
+{
+    const int off = ((lane & 7) + ((lane >> 3) & 1) * 8) * ld + (lane >> 4) * 8;
+    ldsm4<false>(f.hi, hi + off);
+    ldsm4<false>(f.lo, lo + off);
+}
+__device__ __forceinline__ void load_a_transposed(Pair4& f, const __half* hi, const __half* lo, int ld, int lane)
+{
+    const int off = ((lane & 7) + (lane >> 4) * 8) * ld + ((lane >> 3) & 1) * 8;
+    ldsm4<true>(f.hi, hi + off);
+    ldsm4<true>(f.lo, lo + off);
+}
+__device__ __forceinline__ void load_b(Pair4& f, const __half* hi, const __half* lo, int ld, int lane)
+{
+    const int off = ((lane & 7) + ((lane >> 3) & 1) * 8) * ld + (lane >> 4) * 8;
+    ldsm4<true>(f.hi, hi + off);
+    ldsm4<true>(f.lo, lo + off);
+}
+__device__ __forceinline__ void negate(Pair4& f)
+{
 #pragma unroll
-        for (int i = kJordan ? 0 : J; i < 8; ++i) c[i] = __shfl_sync(0xffffffffu, a[i][J], half + t);
-        if (kJordan) c[J] -= (g == t) ? 1.0f : 0.0f;
-        else c[J] = (g <= t) ? 0.0f : c[J];
-        fact_wait(full + t, J & 1, status);
-        const float* slot = ring[t];
-        const float4 ra = *reinterpret_cast<const float4*>(slot + 4 * l), rb = *reinterpret_cast<const float4*>(slot + 64 + 4 * l);
-        const float rp = slot[FB];
-        float u[8] = {ra.x * rp, ra.y * rp, ra.z * rp, ra.w * rp, rb.x * rp, rb.y * rp, rb.z * rp, rb.w * rp};
-        if (l == t) u[J] = 1.0f + rp;
+    for (int t = 0; t < 4; ++t) { f.hi[t] ^= 0x80008000u; f.lo[t] ^= 0x80008000u; }
+}
+// c (16 x 16, two column tiles) += A B
+__device__ __forceinline__ void mma_pairs(float (&c)[2][4], const Pair4& a, const Pair4& b)
+{
 #pragma unroll
-        for (int q = 0; q < 8; ++q) a[J][q] = fmaf(-c[J], u[q], a[J][q]);
-        if (t < 15 && (g >> 1) == ((t + 1) >> 1)) publish_row<J>(a, ring[t + 1], full + t + 1, t + 1, g, l);
+    for (int t = 0; t < 2; ++t) mma16(c[t], a.lo, b.hi[2 * t], b.hi[2 * t + 1]);
 #pragma unroll
-        for (int i = kJordan ? 0 : J + 1; i < 8; ++i)
-            if (i != J) {
+    for (int t = 0; t < 2; ++t) mma16(c[t], a.hi, b.lo[2 * t], b.lo[2 * t + 1]);
 #pragma unroll
-                for (int q = 0; q < 8; ++q) a[i][q] = fmaf(-c[i], u[q], a[i][q]);
+    for (int t = 0; t < 2; ++t) mma16(c[t], a.hi, b.hi[2 * t], b.hi[2 * t + 1]);
+}
+// Accumulator tiles as an operand pair: x[t][2 i + e] = (row gid + 8 i, column 8 t + 2 tig + e).  As they stand they are
+// the A operand x; read as B (mma_pairs_t) they are x^T.
+__device__ __forceinline__ void pack_pairs(Pair4& p, const float (&x)[2][4])
+{
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const __half2 h = __floats2half2_rn(x[t][2 * i], x[t][2 * i + 1]);
+            const float2 f = __half22float2(h);
+            const __half2 l = __floats2half2_rn(x[t][2 * i] - f.x, x[t][2 * i + 1] - f.y);
+            p.hi[2 * t + i] = *reinterpret_cast<const uint32_t*>(&h);
+            p.lo[2 * t + i] = *reinterpret_cast<const uint32_t*>(&l);
+        }
+}
+// c += A x^T, both column tiles
+__device__ __forceinline__ void mma_pairs_t(float (&c)[2][4], const Pair4& a, const Pair4& x)
+{
+#pragma unroll
+    for (int t = 0; t < 2; ++t) mma16(c[t], a.lo, x.hi[t], x.hi[2 + t]);
+#pragma unroll
+    for (int t = 0; t < 2; ++t) mma16(c[t], a.hi, x.lo[t], x.lo[2 + t]);
+#pragma unroll
+    for (int t = 0; t < 2; ++t) mma16(c[t], a.hi, x.hi[t], x.hi[2 + t]);
+}
+__device__ __forceinline__ void store_pair(__half* hi, __half* lo, float x, float y)
+{
+    const __half2 h = __floats2half2_rn(x, y);
+    const float2 f = __half22float2(h);
+    *reinterpret_cast<__half2*>(hi) = h;
+    *reinterpret_cast<__half2*>(lo) = __floats2half2_rn(x - f.x, y - f.y);
+}
+
+// A warp's 16 x 16 block (two accumulator tiles: a[t][2 i + e] = row gid + 8 i, column 8 t + 2 tig + e) replaced by its inverse
+// by Gauss-Jordan steps, or (kChol) by the inverse of its Cholesky factor: elimination of the rows below the pivot
+// leaves L^-1 below the diagonal of L Delta L^T, which is scaled to Delta^-1/2 L^-1.  With p the pivot and u = (pivot row) / p,
+// a row x with f in the pivot column becomes x - f u, and f becomes -f / p.  The latter and the pivot row itself ride along:
+// f - f (1 + 1 / p) = -f / p and x - (p - 1) u = x / p, exact enough because the pivots are around 1.  The chain of a step would be
+// shuffle, reciprocal, product, update; every lane works the next pivot out for itself from the entries before the
+// update, so the reciprocal runs beside the rest.
+template <bool kChol>
+__device__ __forceinline__ void invert16(float (&a)[2][4], int gid, int tig, int* status)
+{
+    constexpr uint32_t all = 0xffffffffu;
+    float rp = fast_rcp(__shfl_sync(all, a[0][0], 0));
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {
+        const int kt = k >> 3, kg = k & 7, ke = k & 1, kc = (k & 7) >> 1;
+        float rn = 0.0f;
+        if (k + 1 < NB) {
+            const int nt = (k + 1) >> 3, ng = (k + 1) & 7, ne = (k + 1) & 1, nc = ng >> 1;
+            const float a11 = __shfl_sync(all, a[nt][2 * nt + ne], ng * 4 + nc), a10 = __shfl_sync(all, a[kt][2 * nt + ke], ng * 4 + kc);
+            const float a01 = __shfl_sync(all, a[nt][2 * kt + ne], kg * 4 + nc);
+            rn = fast_rcp(fmaf(-a10 * a01, rp, a11));
+        }
+        float u[2][2], f[2];
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) u[t][e] = __shfl_sync(all, a[t][2 * kt + e], kg * 4 + tig) * rp;
+        if (tig == kc) u[kt][ke] = 1.0f + rp;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) f[i] = __shfl_sync(all, a[kt][2 * i + ke], gid * 4 + kc);
+#pragma unroll
+        for (int i = kChol ? kt : 0; i < 2; ++i) {           // (Cholesky: rows above the pivot are done)
+            if (i == kt) {
+                if (kChol) f[i] = gid > kg ? f[i] : 0.0f;
+                else f[i] -= gid == kg ? 1.0f : 0.0f;
             }
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) a[t][2 * i + e] = fmaf(-f[i], u[t][e], a[t][2 * i + e]);
+        }
+        rp = rn;
+    }
+    if (kChol) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int r = gid + 8 * i;
+            const float d = __shfl_sync(all, (gid & 1) ? a[i][2 * i + 1] : a[i][2 * i], gid * 4 + (gid >> 1));   // pivot of row r
+            if (!(d > 0.0f)) atomicCAS(status, 0, (int)GELO_ERR_COND);           // a Gaussian block never gets here
+            const float rs = rsqrtf(d);
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int c = 8 * t + 2 * tig + e;
+                    a[t][2 * i + e] = c < r ? a[t][2 * i + e] * rs : (c == r ? rs : 0.0f);
+                }
+        }
     }
 }
 
-// The Gram group: elimination of G = L Delta L^T, then row 16 J + g of R = Delta^-1/2 (Delta L^T) and of R^-T = Delta^-1/2
-// L^-1, which are final after these steps.
-template <int J>
-__device__ __forceinline__ void gram_steps(float (&a)[8][8], FactShared& s, float* P1, int ld, int ob, float scale, int g, int l,
-                                           int* status)
+// f(v) with v as a compile-time constant, for values that choose registers.
+template <typename F>
+__device__ __forceinline__ void with_bit(int v, F&& f)
 {
-    sixteen_steps<J, false>(a, s.row[0], s.full[0], g, l, status);
-    const float d = __shfl_sync(0xffffffffu, a[J][J], (threadIdx.x & 16) + g);   // the row's diagonal entry: column l = g
-    const float rs = rsqrtf(d);
-    if (!(d > 0.0f)) atomicCAS(status, 0, (int)GELO_ERR_COND);                   // a Gaussian block never gets here
-    const int r = 16 * J + g;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const int c = l + 16 * q;
-        const float v = a[J][q] * rs;
-        s.A[r][c] = (c < r) ? v : ((c == r) ? rs : 0.0f);
-        s.X[r][c] = (c >= r) ? v : 0.0f;
-    }
-    __syncwarp();
-    if ((threadIdx.x & 31) == 0) tcx::mbar_arrive(tcx::smem_u32(&s.rready[J]));
-#pragma unroll
-    for (int q = J; q < 8; ++q) {                                                // B = P1 + R, the top block of V
-        const int c = l + 16 * q;
-        if (c >= r && c < ob) P1[(size_t)r * ld + c] += scale * (a[J][q] * rs);
-    }
+    if (v == 0) f(std::integral_constant<int, 0>{});
+    else f(std::integral_constant<int, 1>{});
 }
-
-// The other group: Gauss-Jordan inverse of B = P1 + R.  Rows of R are added when their steps begin; they add nothing to the
-// columns that earlier steps read.
-template <int J>
-__device__ __forceinline__ void inverse_steps(float (&b)[8][8], FactShared& s, int g, int l, int* status)
+template <typename F>
+__device__ __forceinline__ void with_quarter(int v, F&& f)
 {
-    fact_wait(&s.rready[J], 0, status);
-#pragma unroll
-    for (int q = J; q < 8; ++q) b[J][q] += s.X[16 * J + g][l + 16 * q];
-    sixteen_steps<J, true>(b, s.row[1], s.full[1], g, l, status);
+    if (v == 0) f(std::integral_constant<int, 0>{});
+    else if (v == 1) f(std::integral_constant<int, 1>{});
+    else if (v == 2) f(std::integral_constant<int, 2>{});
+    else f(std::integral_constant<int, 3>{});
 }
 
-// One CTA.  Z (ob x ob, stride ldz): the Gram matrix P^T P.  P1: the first ob rows of the panel (stride ld), overwritten
+enum FactRole { FACT_GRAM = 0, FACT_INVERSE = 1, FACT_FACTOR = 2 };
+
+// F, rows, panel and the next pivot block of a step are published (all warps) / U is (the eight warps).
+__device__ __forceinline__ void published_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(kFactThreads) : "memory"); }
+__device__ __forceinline__ void compute_barrier() { asm volatile("bar.sync 2, %0;" ::"n"(kFactCompute) : "memory"); }
+
+// The eight steps of the eight warps; a[mt][nt][2 i + e] = row 32 (w / 2) + 16 mt + gid + 8 i, column 64 (w % 2) + 8 nt + 2 tig + e.
+template <int kRole>
+__device__ __forceinline__ void fact_compute(float (&a)[2][8][4], FactShared& s, int* status)
+{
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
+    const int wr = w >> 1, wc = w & 1;
+    float* const R = reinterpret_cast<float*>(&s.panel[0][0][0][0]);             // CTA 0 only
+#pragma unroll 1
+    for (int J = 0; J < kSteps; ++J) {
+        // ---- publish ----
+        if (kRole != FACT_GRAM) {
+            fact_wait(&s.got_full[J], 0, status);
+            if (kRole == FACT_FACTOR) fact_wait(&s.panel_full[J], 0, status);
+        }
+        if (wr == (J >> 1))
+            with_bit(J & 1, [&](auto bit) {
+                constexpr int mt = decltype(bit)::value;
+#pragma unroll
+                for (int nt = 0; nt < 8; ++nt) {
+                    const int c = 64 * wc + 8 * nt + 2 * tig;
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        if (kRole != FACT_GRAM) {
+                            const float2 t = *reinterpret_cast<const float2*>(&s.got[J][gid + 8 * i][c]);
+                            a[mt][nt][2 * i] += t.x; a[mt][nt][2 * i + 1] += t.y;
+                        }
+                        store_pair(&s.rows[J & 1][0][gid + 8 * i][c], &s.rows[J & 1][1][gid + 8 * i][c], a[mt][nt][2 * i], a[mt][nt][2 * i + 1]);
+                    }
+                }
+            });
+        if (kRole != FACT_FACTOR) {
+            const int N = J + 1;
+            if (N < kSteps && wr == (N >> 1) && wc == (N >> 2))                  // the next pivot block, before this step's update
+                with_bit(N & 1, [&](auto bit) {
+                    with_quarter(N & 3, [&](auto quarter) {
+                        constexpr int mt = decltype(bit)::value, n0 = 2 * decltype(quarter)::value;
+#pragma unroll
+                        for (int t = 0; t < 2; ++t)
+#pragma unroll
+                            for (int i = 0; i < 2; ++i)
+                                *reinterpret_cast<float2*>(&s.next[N & 1][gid + 8 * i][8 * t + 2 * tig]) =
+                                    make_float2(a[mt][n0 + t][2 * i], a[mt][n0 + t][2 * i + 1]);
+                    });
+                });
+            if (wc == (J >> 2))                                                  // the columns p, which restart from zero
+                with_quarter(J & 3, [&](auto quarter) {
+                    constexpr int n0 = 2 * decltype(quarter)::value;
+#pragma unroll
+                    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                        for (int t = 0; t < 2; ++t)
+#pragma unroll
+                            for (int i = 0; i < 2; ++i) {
+                                float (&v)[4] = a[mt][n0 + t];
+                                const int r = 32 * wr + 16 * mt + gid + 8 * i, c = 8 * t + 2 * tig;
+                                if (kRole == FACT_INVERSE) store_pair(&s.panel[J][0][r][c], &s.panel[J][1][r][c], -v[2 * i], -v[2 * i + 1]);
+                                v[2 * i] = 0.0f; v[2 * i + 1] = 0.0f;
+                            }
+                });
+            if (kRole == FACT_INVERSE) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        }
+        published_barrier();
+        if (kRole == FACT_INVERSE && tid == 0) {
+            send_shared(s.panel[J], s.panel[J], sizeof(s.panel[J]), &s.panel_full[J], 2);
+            send_shared(s.F[J], s.F[J], sizeof(s.F[J]), &s.panel_full[J], 2);
+        }
+        // ---- U = F rows, 16 columns per warp (those of warp J are the columns p) ----
+        {
+            Pair4 f, x;
+            load_a(f, &s.F[J][0][0][0], &s.F[J][1][0][0], kPanelLd, lane);
+            load_b(x, &s.rows[J & 1][0][0][16 * w], &s.rows[J & 1][1][0][16 * w], kWideLd, lane);
+            float u[2][4] = {{0.0f, 0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f, 0.0f}};
+            mma_pairs(u, f, x);
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int r = gid + 8 * i, cp = 8 * t + 2 * tig, c = 16 * w + cp;
+                    float2 v = make_float2(u[t][2 * i], u[t][2 * i + 1]), fv = make_float2(0.0f, 0.0f);
+                    if (kRole != FACT_FACTOR && w == J) {
+                        const float2 fh = __half22float2(*reinterpret_cast<const __half2*>(&s.F[J][0][r][cp]));
+                        const float2 fl = __half22float2(*reinterpret_cast<const __half2*>(&s.F[J][1][r][cp]));
+                        fv = make_float2(fh.x + fl.x, fh.y + fl.y);
+                    }
+                    if (kRole == FACT_GRAM) {
+                        // row of R: U right of the pivots, the Cholesky factor above the diagonal of the pivot block
+                        float2 rv = v;
+                        if (w < J || (w == J && cp < r)) rv.x = 0.0f;
+                        if (w < J || (w == J && cp + 1 < r)) rv.y = 0.0f;
+                        *reinterpret_cast<float2*>(R + (J * NB + r) * FB + c) = rv;
+                        *reinterpret_cast<float2*>(&s.got[J][r][c]) = w < J ? v : fv;                            // row of R^-T
+                    }
+                    if (kRole != FACT_FACTOR && w == J) v = fv;
+                    store_pair(&s.U[0][r][c], &s.U[1][r][c], v.x, v.y);
+                    if (kRole != FACT_GRAM) *reinterpret_cast<float2*>(&s.U32[r][c]) = v;
+                }
+            if (kRole == FACT_GRAM) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        }
+        compute_barrier();
+        if (kRole == FACT_GRAM && tid == 0) {
+            send_shared(s.got[J], R + J * NB * FB, sizeof(s.got[J]), &s.got_full[J], 1);
+            send_shared(s.got[J], s.got[J], sizeof(s.got[J]), &s.got_full[J], 2);
+        }
+        // ---- update (CTA 0: the rows below the pivots only) ----
+        if (kRole != FACT_GRAM || 2 * wr + 1 > J) {
+            Pair4 c[2];
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+                const int r0 = 32 * wr + 16 * mt;
+                if (kRole == FACT_GRAM) {
+                    load_a_transposed(c[mt], &s.U[0][0][r0], &s.U[1][0][r0], kWideLd, lane);
+                    negate(c[mt]);
+                } else {
+                    load_a(c[mt], &s.panel[J][0][r0][0], &s.panel[J][1][r0][0], kPanelLd, lane);
+                }
+            }
+#pragma unroll
+            for (int np = 0; np < 4; ++np) {
+                Pair4 u;
+                load_b(u, &s.U[0][0][64 * wc + 16 * np], &s.U[1][0][64 * wc + 16 * np], kWideLd, lane);
+#pragma unroll
+                for (int e = 0; e < 3; ++e)                  // (four independent accumulators between dependent instructions)
+#pragma unroll
+                    for (int mt = 0; mt < 2; ++mt)
+                        if (kRole != FACT_GRAM || 2 * wr + mt > J) {
+                            const uint32_t (&x)[4] = e == 0 ? c[mt].lo : c[mt].hi;
+                            const uint32_t (&y)[4] = e == 1 ? u.lo : u.hi;
+                            mma16(a[mt][2 * np], x, y[0], y[1]);
+                            mma16(a[mt][2 * np + 1], x, y[2], y[3]);
+                        }
+            }
+        }
+        if (kRole != FACT_GRAM && wr == (J >> 1))
+            with_bit(J & 1, [&](auto bit) {
+                constexpr int mt = decltype(bit)::value;
+#pragma unroll
+                for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const float2 v = *reinterpret_cast<const float2*>(&s.U32[gid + 8 * i][64 * wc + 8 * nt + 2 * tig]);
+                        a[mt][nt][2 * i] = v.x; a[mt][nt][2 * i + 1] = v.y;
+                    }
+            });
+    }
+}
+
+// The ninth warp: the inverses of the pivot blocks.
+template <int kRole>
+__device__ __forceinline__ void fact_pivots(FactShared& s, int* status)
+{
+    const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
+    float a[2][4];
+    Pair4 f;
+#pragma unroll 1
+    for (int N = 0; N <= kSteps; ++N) {
+        if (N > 0) published_barrier();                      // of step N - 1
+        if (N == kSteps || kRole == FACT_FACTOR) continue;
+        Pair4 c, x;
+        if (N > 0) {
+            float ut[2][4] = {{0.0f, 0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f, 0.0f}};   // U^T = rows^T F^T, columns of the next block
+            const int sl = (N - 1) & 1;
+            load_a_transposed(c, &s.rows[sl][0][0][NB * N], &s.rows[sl][1][0][NB * N], kWideLd, lane);
+            mma_pairs_t(ut, c, f);
+            pack_pairs(x, ut);
+            if (kRole == FACT_GRAM) { c = x; negate(c); }
+            else load_a(c, &s.panel[N - 1][0][NB * N][0], &s.panel[N - 1][1][NB * N][0], kPanelLd, lane);
+        }
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float2 v = *reinterpret_cast<const float2*>(&s.next[N & 1][gid + 8 * i][8 * t + 2 * tig]);
+                a[t][2 * i] = v.x; a[t][2 * i + 1] = v.y;
+            }
+        if (N > 0) mma_pairs_t(a, c, x);
+        if (kRole == FACT_INVERSE) {
+            fact_wait(&s.got_full[N], 0, status);
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const float2 v = *reinterpret_cast<const float2*>(&s.got[N][gid + 8 * i][NB * N + 8 * t + 2 * tig]);
+                    a[t][2 * i] += v.x; a[t][2 * i + 1] += v.y;
+                }
+        }
+        invert16<kRole == FACT_GRAM>(a, gid, tig, status);
+        pack_pairs(f, a);
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                *reinterpret_cast<uint32_t*>(&s.F[N][0][gid + 8 * i][8 * t + 2 * tig]) = f.hi[2 * t + i];
+                *reinterpret_cast<uint32_t*>(&s.F[N][1][gid + 8 * i][8 * t + 2 * tig]) = f.lo[2 * t + i];
+            }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+}
+
+// Z (ob x ob, stride ldz): the Gram matrix P^T P.  P1: the first ob rows of the panel (stride ld), overwritten
 // with B = P1 + R.  T (stride ldt) = R^-1 B^-T and D (stride ldd) = dscale * B^-T, both rounded to tf32 if `round`.
 // ob <= 128, a multiple of 4; the kernel works on 128 x 128 with an identity in the part past ob.  `scale` is a power of
 // two close to the norm of a panel column.
-__global__ void __launch_bounds__(kFactThreads, 1)
+__global__ void __cluster_dims__(kFactCtas, 1, 1) __launch_bounds__(kFactThreads, 1)
 block_factor_kernel(const float* __restrict__ Z, int ldz, float* P1, int ld, int ob, float* __restrict__ T,
                     int ldt, float* __restrict__ D, int ldd, float scale, float dscale, int round, int* __restrict__ status)
 {
-    extern __shared__ __align__(16) uint8_t fsm[];
+    extern __shared__ __align__(128) uint8_t fsm[];
     FactShared& s = *reinterpret_cast<FactShared*>(fsm);
-    const int tid = threadIdx.x, g = (tid & 255) >> 4, l = tid & 15;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, gid = lane >> 2, tig = lane & 3;
+    const int wr = w >> 1, wc = w & 1;
+    const int role = blockIdx.x;
     const float s1 = 1.0f / scale, s2 = s1 * s1;
+    const bool compute = tid < kFactCompute;
 
     if (tid == 0) {
-        for (int i = 0; i < kRing; ++i) { tcx::mbar_init(tcx::smem_u32(&s.full[0][i]), 1); tcx::mbar_init(tcx::smem_u32(&s.full[1][i]), 1); }
-        for (int i = 0; i < 8; ++i) tcx::mbar_init(tcx::smem_u32(&s.rready[i]), 8);
+        for (int i = 0; i < kSteps; ++i) {
+            tcx::mbar_init(tcx::smem_u32(&s.got_full[i]), 1);
+            tcx::mbar_init(tcx::smem_u32(&s.panel_full[i]), 1);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    float a[8][8];
-    {
-        const float* src = tid < 256 ? Z : P1;
-        const int lds = tid < 256 ? ldz : ld;
-        const float f = tid < 256 ? s2 : s1, one = tid < 256 ? 1.0f : 0.0f;
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int r = g + 16 * i, c = l + 16 * q;
-                a[i][q] = (r < ob && c < ob) ? f * src[(size_t)r * lds + c] : (r == c ? one : 0.0f);
+        if (role != FACT_GRAM)
+            for (int i = 0; i < kSteps; ++i) {
+                tcx::mbar_expect_tx(tcx::smem_u32(&s.got_full[i]), sizeof(s.got[0]));
+                if (role == FACT_FACTOR) tcx::mbar_expect_tx(tcx::smem_u32(&s.panel_full[i]), sizeof(s.panel[0]) + sizeof(s.F[0]));
             }
     }
-    __syncthreads();
-    if (tid < 256) {
-        gram_steps<0>(a, s, P1, ld, ob, scale, g, l, status);
-        gram_steps<1>(a, s, P1, ld, ob, scale, g, l, status);
-        gram_steps<2>(a, s, P1, ld, ob, scale, g, l, status);
-        gram_steps<3>(a, s, P1, ld, ob, scale, g, l, status);
-        gram_steps<4>(a, s, P1, ld, ob, scale, g, l, status);
-        gram_steps<5>(a, s, P1, ld, ob, scale, g, l, status);
-        gram_steps<6>(a, s, P1, ld, ob, scale, g, l, status);
-        gram_steps<7>(a, s, P1, ld, ob, scale, g, l, status);
-        __syncthreads();
-    } else {
-        inverse_steps<0>(a, s, g, l, status);
-        inverse_steps<1>(a, s, g, l, status);
-        inverse_steps<2>(a, s, g, l, status);
-        inverse_steps<3>(a, s, g, l, status);
-        inverse_steps<4>(a, s, g, l, status);
-        inverse_steps<5>(a, s, g, l, status);
-        inverse_steps<6>(a, s, g, l, status);
-        inverse_steps<7>(a, s, g, l, status);
-        __syncthreads();                                                         // R has been read by everybody
+    float a[2][8][4];
+    if (compute) {
+        const float* src = role == FACT_GRAM ? Z : P1;
+        const int lds = role == FACT_GRAM ? ldz : ld;
+        const float f = role == FACT_GRAM ? s2 : s1, one = role == FACT_GRAM ? 1.0f : 0.0f;
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int q = 0; q < 8; ++q) s.X[l + 16 * q][g + 16 * i] = a[i][q];
+            for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int r = 32 * wr + 16 * mt + gid + 8 * i, c = 64 * wc + 8 * nt + 2 * tig;
+                    float2 v = make_float2(r == c ? one : 0.0f, r == c + 1 ? one : 0.0f);
+                    if (r < ob && c < ob) {                  // (ob is even: c + 1 < ob too)
+                        v = *reinterpret_cast<const float2*>(src + (size_t)r * lds + c);
+                        v.x *= f; v.y *= f;
+                    }
+                    a[mt][nt][2 * i] = role == FACT_FACTOR ? 0.0f : v.x;
+                    a[mt][nt][2 * i + 1] = role == FACT_FACTOR ? 0.0f : v.y;
+                    if (w == 0 && mt == 0 && nt < 2)         // the first pivot block
+                        *reinterpret_cast<float2*>(&s.next[0][r][c]) = v;
+                }
     }
-    __syncthreads();
-    auto out_val = [&](float v) { return round ? tcx::round_tf32(v) : v; };
-    const float ds = dscale * s1;
-    for (int idx = tid; idx < FB * FB / 4; idx += kFactThreads) {
-        const int r = idx >> 5, c = (idx & 31) * 4;
-        if (r < ob && c < ob) {
-            const float4 v = *reinterpret_cast<const float4*>(&s.X[r][c]);
-            *reinterpret_cast<float4*>(D + (size_t)r * ldd + c) =
-                make_float4(out_val(ds * v.x), out_val(ds * v.y), out_val(ds * v.z), out_val(ds * v.w));
+    __syncwarp();
+    cluster_sync_all();                                      // barriers initialised, P1 read, the first block published
+    if (!compute) {
+        if (role == FACT_GRAM) fact_pivots<FACT_GRAM>(s, status);
+        else if (role == FACT_INVERSE) fact_pivots<FACT_INVERSE>(s, status);
+        else fact_pivots<FACT_FACTOR>(s, status);
+    } else if (role == FACT_GRAM) {
+        fact_compute<FACT_GRAM>(a, s, status);
+        // B = P1 + R, the top block of V
+        const float* R = reinterpret_cast<const float*>(&s.panel[0][0][0][0]);
+#pragma unroll 4
+        for (int idx = tid; idx < FB * FB / 4; idx += kFactCompute) {
+            const int r = idx >> 5, c = (idx & 31) * 4;
+            if (r < ob && c < ob && c + 3 >= r) {
+                float4* p = reinterpret_cast<float4*>(P1 + (size_t)r * ld + c);
+                const float4 v = *reinterpret_cast<const float4*>(R + r * FB + c);
+                float4 o = *p;
+                o.x += scale * v.x; o.y += scale * v.y; o.z += scale * v.z; o.w += scale * v.w;
+                *p = o;
+            }
+        }
+    } else {
+        if (role == FACT_INVERSE) fact_compute<FACT_INVERSE>(a, s, status);
+        else fact_compute<FACT_FACTOR>(a, s, status);
+        // the transpose of the result, by way of the slots of got (all read by now); row q of the transpose is rotated
+        // by 8 (q / 2) so that a warp's writes fall into different banks
+        float* X = &s.got[0][0][0];
+        const float f = role == FACT_INVERSE ? dscale * s1 : s2;
+        compute_barrier();
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int r = 32 * wr + 16 * mt + gid + 8 * (e >> 1), q = 64 * wc + 8 * nt + 2 * tig + (e & 1);
+                    const float v = f * a[mt][nt][e];
+                    X[q * FB + ((r + 8 * (q >> 1)) & (FB - 1))] = round ? tcx::round_tf32(v) : v;
+                }
+        compute_barrier();
+        float* dst = role == FACT_INVERSE ? D : T;
+        const int ldo = role == FACT_INVERSE ? ldd : ldt;
+#pragma unroll 4
+        for (int idx = tid; idx < FB * FB / 4; idx += kFactCompute) {
+            const int q = idx >> 5, c = (idx & 31) * 4;
+            if (q < ob && c < ob)
+                *reinterpret_cast<float4*>(dst + (size_t)q * ldo + c) =
+                    *reinterpret_cast<const float4*>(X + q * FB + ((c + 8 * (q >> 1)) & (FB - 1)));
         }
     }
-    // ---- T = R^-1 D = (R^-T)^T D: 8 rows per warp, 4 columns per lane; a row block from row r0 on only meets rows
-    //      k >= r0, so short and long blocks are dealt evenly to the SM's four schedulers ----
-    const int warp = tid >> 5, n0 = 4 * (tid & 31);
-    const int r0 = 8 * ((warp & 4) ? (warp ^ 3) : warp);
-    float x[8][4];
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) x[i][q] = 0.0f;
-#pragma unroll 4
-    for (int k = r0; k < FB; ++k) {
-        const float4 u = *reinterpret_cast<const float4*>(&s.A[k][r0]), v = *reinterpret_cast<const float4*>(&s.A[k][r0 + 4]);
-        const float4 y = *reinterpret_cast<const float4*>(&s.X[k][n0]);
-        const float uu[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
-        const float yy[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) x[i][q] = fmaf(uu[i], yy[q], x[i][q]);
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-        if (r0 + i < ob && n0 < ob)
-            *reinterpret_cast<float4*>(T + (size_t)(r0 + i) * ldt + n0) =
-                make_float4(out_val(s2 * x[i][0]), out_val(s2 * x[i][1]), out_val(s2 * x[i][2]), out_val(s2 * x[i][3]));
+    __syncwarp();
+    cluster_sync_all();                                      // nobody's shared memory goes while a copy may still reach it
 }
 
 // Z = scale * (sum of the K slices of P^T [P | C]), in slice order; the first ob columns (the Gram matrix) stay fp32, the
@@ -369,7 +702,7 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
             float* Tb = Ts + (size_t)r * kSuper + r;
             float scale = 1.0f;                              // a power of two with scale^2 about nr
             while (2.0f * scale * scale < (float)nr) scale *= 2.0f;
-            block_factor_kernel<<<1, kFactThreads, kFactSmemBytes, st>>>(tc.w32[0], ld, P, ld, ob, Tb, kSuper, tc.t128, FB,
+            block_factor_kernel<<<kFactCtas, kFactThreads, kFactSmemBytes, st>>>(tc.w32[0], ld, P, ld, ob, Tb, kSuper, tc.t128, FB,
                                                                         scale, loss1, 1, ctx->status_dev);
             GELO_TRY(after_launch(ctx));
             if (send > bend) {
