@@ -17,7 +17,7 @@
 // * A segment names one A tensor map, one B tensor map and a starting k for each; the stacked
 //   operand of the mixing product is two segments, a split-precision product is three.  TMA's
 //   out-of-bounds zero fill handles every ragged edge (including a seam inside a k-block).
-// * Persistent CTAs (one per SM), warp-specialised: warp 0 issues TMA, warp 1 issues MMA and owns
+// * Persistent CTAs (one per SM, in pairs on 256 x 256 tiles where use_pair() says so), warp-specialised: warp 0 issues TMA, warp 1 issues MMA and owns
 //   the tensor-memory allocation, warps 2-9 drain the accumulator (two warps per TMEM lane
 //   quarter, half of the columns each).  Two accumulator stages let the epilogue of one tile
 //   overlap the main loop of the next.
@@ -77,18 +77,28 @@ struct TcParams {
 constexpr uint32_t kStageBoxBytes = 32 * 32 * 4;
 constexpr uint32_t kStagingBytes = kEpiWarps * 2 * kStageBoxBytes;
 
+// Store epilogue staging: 32 rows of 128 bytes per epilogue warp.
+constexpr uint32_t kStoreBytes = kEpiWarps * 32 * 128;
+
 // A stage holds 128 bytes of k per A row (64 bf16 or 32 tf32 values) and the matching B rows, so both kinds share
 // the shared-memory geometry: kTf32 only changes the element count per k-block, the box width of the N-major B tile
 // (128 bytes = 64 bf16 or 32 fp32 columns) and the instruction.  kAMn (tf32 only): the A tile arrives as four
 // boxes of 32 m-columns x 32 k-rows, i.e. laid out exactly like a 128-column B tile.
-template <int BN, int kStages, bool kStaging, bool kTf32 = false, bool kAMn = false, bool kF8 = false>
+// kPair: a cluster of two CTAs works on one 256-row tile (cta_group::2).  Each holds its 128 rows of A and one half of
+// the columns of B, and accumulates its 128 rows over all columns; CTA 0 issues the instructions for both.
+template <int BN, bool kStaging, bool kTf32 = false, bool kAMn = false, bool kF8 = false, bool kPair = false>
 struct TcCfg {
-    static constexpr uint32_t kStagingUsed = kStaging ? kStagingBytes : 0u;
+    static constexpr int kCols = kPair ? BN / 2 : BN;                      // columns of B that one CTA holds
+    static constexpr int kTileRows = kPair ? 2 * BM : BM;
+    static constexpr uint32_t kStagingUsed = kStaging ? kStagingBytes : kStoreBytes;
     static constexpr int kBKE = kF8 ? 128 : (kTf32 ? 32 : 64);             // elements of k per stage
     static constexpr int kBoxCols = kF8 ? 128 : (kTf32 ? 32 : 64);         // columns of one N-major box (128 bytes)
     static constexpr uint32_t kBoxBytes = (uint32_t)kBKE * 128u;           // one N-major box: kBKE rows of 128 bytes
-    static constexpr uint32_t kBBytes = (BN / kBoxCols) * kBoxBytes;
+    static constexpr uint32_t kBBytes = (kCols / kBoxCols) * kBoxBytes;
     static constexpr uint32_t kStageBytes = kABytes + kBBytes;
+    // as many stages as fit, six at most: 4 (3 with staging for the in-place subtraction) alone, 6 (5) in a pair
+    static constexpr int kFit = (int)((227u * 1024u - 1024u - 256u - kStagingUsed) / kStageBytes);
+    static constexpr int kStages = kFit > 6 ? 6 : kFit;
     static constexpr uint32_t kSmemBytes = kStages * kStageBytes + kStagingUsed + 1024 /*alignment slack*/ + 256 /*barriers*/;
     // k advance per instruction inside an N-major (or MN-major A) tile: 16 bf16 rows or 8 tf32 rows of 128 bytes
     static constexpr uint32_t kMnStep = kF8 ? 4096u : (kTf32 ? 1024u : 2048u);   // 32 e4m3 rows, 16 bf16 rows or 8 tf32 rows
@@ -97,12 +107,13 @@ struct TcCfg {
     static constexpr uint32_t kMnLayout = kTf32 ? 1u : 2u;
     static constexpr uint32_t kMnSbo = kTf32 ? 512u : 1024u;
     // Instruction descriptor: fp32 accumulate, operand formats (1 = bf16, 2 = tf32), A K-major or MN-major,
-    // B N-major, M = 128, N = BN.
+    // B N-major, M = 128 (256 in a pair), N = BN.
     static constexpr uint32_t kFmt = kF8 ? 0u : (kTf32 ? 2u : 1u);         // kind::f8f6f4: 0 = E4M3
     static constexpr uint32_t kInstrDesc = (1u << 4) | (kFmt << 7) | (kFmt << 10) | ((kAMn ? 1u : 0u) << 15) | (1u << 16) |
-                                           ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+                                           ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(kTileRows >> 4) << 24);
     static_assert(!kAMn || kTf32, "MN-major A is only wired up for the tf32 kind");
     static_assert(!(kF8 && kTf32), "one operand kind per instance");
+    static_assert(kCols % kBoxCols == 0, "a CTA's share of B is whole boxes");
 };
 
 // x = hi + lo with hi = bf16(x), lo = bf16(x - hi)
@@ -116,15 +127,16 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
 }
 
 // Row-tile and column-tile index of work item `tile`.  Ordinary products: row tiles fastest, then column tiles, then K
-// slices.  Symmetric products (prm.tri, 128 x 256 tiles): column tile nt owns the row tiles mt <= 2 nt + 1, i.e. those
-// whose first row is not below the tile's last column; they are enumerated column tile after column tile.
+// slices.  Symmetric products (prm.tri, 256 columns per tile): column tile nt owns the row tiles whose first row is not
+// below its last column, mt <= 2 nt + 1 (of 128 rows) or mt <= nt (of 256); they are enumerated column tile after column tile.
+template <bool kPair>
 __device__ __forceinline__ void tile_coords(const TcParams& prm, int tile, int m_tiles, int mn_tiles, int& mt, int& nt, int& slice)
 {
     if (prm.tri) {
         int t = tile;
         nt = 0;
         for (;;) {
-            const int cnt = min(m_tiles, 2 * nt + 2);
+            const int cnt = min(m_tiles, kPair ? nt + 1 : 2 * nt + 2);
             if (t < cnt) break;
             t -= cnt; ++nt;
         }
@@ -137,76 +149,130 @@ __device__ __forceinline__ void tile_coords(const TcParams& prm, int tile, int m
     nt = mn / m_tiles;
 }
 
-// One 8-column group of the epilogue: w[G*8 .. G*8+7] are the fp32 accumulator values of row gm, columns
-// gn..gn+7 (G is a template parameter so that the register array is indexed by constants only).
-template <int G>
-__device__ __forceinline__ void epilogue_group(const TcParams& prm, int gm, int gn, const uint32_t (&w)[32], int slice)
+// ---- the storing epilogue -----------------------------------------------------------------------------
+// A warp holds 32 rows of the tile, a lane one row each.  Written from there, every 16-byte store instruction would touch
+// 32 lines; so 128 bytes of every row at a time (64 columns of a 16-bit result, 32 of an fp32 one) go through 4 KiB of
+// shared memory (16-byte chunks swizzled by the row) and leave as whole lines: eight lanes per row, four rows per instruction.
+
+__device__ __forceinline__ uint32_t stage_addr(uint32_t buf, int row, int chunk) { return buf + row * 128 + ((chunk ^ (row & 7)) << 4); }
+__device__ __forceinline__ void stage_put(uint32_t buf, int row, int chunk, uint4 v)
 {
-    const uint32_t v[8] = {w[G * 8 + 0], w[G * 8 + 1], w[G * 8 + 2], w[G * 8 + 3],
-                           w[G * 8 + 4], w[G * 8 + 5], w[G * 8 + 6], w[G * 8 + 7]};
-    if (prm.mode == TC_STORE_BF16) {
-        const uint32_t (&v0)[8] = v;
-        const int chunk = gn / prm.csplit;
-        void* base = chunk == 0 ? prm.C0 : (chunk == 1 ? prm.C1 : prm.C2);
-        const size_t off = (size_t)gm * prm.ldc + (gn - chunk * prm.csplit);
-        uint32_t v[8] = {v0[0], v0[1], v0[2], v0[3], v0[4], v0[5], v0[6], v0[7]};
-        if (prm.scale_a) {
-            const float sc = prm.scale_a[0] * prm.scale_b[0];
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stage_addr(buf, row, chunk)), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ uint4 stage_get(uint32_t buf, int row, int chunk)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(stage_addr(buf, row, chunk)) : "memory");
+    return v;
+}
+
+// The staged rows (first one m0) to C, 128 bytes per row from column gn on; elements of kBytes bytes.
+template <int kBytes>
+__device__ __forceinline__ void write_staged(const TcParams& prm, uint32_t buf, int m0, int gn, int lane, long long offset)
+{
+    constexpr int kPer = 16 / kBytes;                         // elements per chunk
+    const int c = lane & 7, n = gn + kPer * c;
+    const int part = n / prm.csplit;                          // column block -> C0 / C1 / C2 (0 unless the output is split)
+    char* base = static_cast<char*>(part == 0 ? prm.C0 : (part == 1 ? prm.C1 : prm.C2));
+    char* dst = base + (offset + (long long)(m0 + (lane >> 3)) * prm.ldc + (n - part * prm.csplit)) * kBytes;
+    const size_t step = (size_t)4 * prm.ldc * kBytes;
+    if (n < prm.N) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = __float_as_uint(sc * __uint_as_float(v[j]));
+        for (int i = 0; i < 8; ++i) {
+            const int r = 4 * i + (lane >> 3);
+            if (m0 + r < prm.M) *reinterpret_cast<uint4*>(dst + i * step) = stage_get(buf, r, c);
         }
-        uint4 pk;
-        if (prm.out_f16) {
-            pk.x = pack_f16(v[0], v[1]); pk.y = pack_f16(v[2], v[3]);
-            pk.z = pack_f16(v[4], v[5]); pk.w = pack_f16(v[6], v[7]);
-        } else {
-            pk.x = pack_bf16(v[0], v[1]); pk.y = pack_bf16(v[2], v[3]);
-            pk.z = pack_bf16(v[4], v[5]); pk.w = pack_bf16(v[6], v[7]);
-        }
-        *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(base) + off) = pk;
-    } else if (prm.mode == TC_AFFINE16) {
-        float f[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-            f[j] = fmaf(prm.out_scale, __uint_as_float(v[j]), (gm == gn + j) ? prm.diag_sub : 0.0f);
-        if (prm.add) {
-            const uint4 raw = *reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(prm.add) + (size_t)gm * prm.ldadd + gn);
-            const uint32_t w2[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float2 t = prm.out_f16 ? __half22float2(*reinterpret_cast<const __half2*>(&w2[j]))
-                                             : __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w2[j]));
-                f[2 * j] += t.x; f[2 * j + 1] += t.y;
-            }
-        }
-        uint32_t o[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            o[j] = prm.out_f16 ? pack_f16(__float_as_uint(f[2 * j]), __float_as_uint(f[2 * j + 1]))
-                               : pack_bf16(__float_as_uint(f[2 * j]), __float_as_uint(f[2 * j + 1]));
-        *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(prm.C0) + (size_t)gm * prm.ldc + gn) = make_uint4(o[0], o[1], o[2], o[3]);
-    } else if (prm.mode == TC_STORE_F32) {
-        const int chunk = gn / prm.csplit;                    // column block -> C0 / C1 / C2 (0 unless the output is split)
-        float* base = static_cast<float*>(chunk == 0 ? prm.C0 : (chunk == 1 ? prm.C1 : prm.C2));
-        float4* dst = reinterpret_cast<float4*>(base + (size_t)slice * prm.plane + (size_t)gm * prm.ldc + (gn - chunk * prm.csplit));
-        float f[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const float a = __uint_as_float(v[j]);
-            f[j] = prm.round_tf32 ? round_tf32(prm.post_scale * (prm.out_scale * a - ((gm == gn + j) ? prm.diag_sub : 0.0f))) : a;
-        }
-        dst[0] = make_float4(f[0], f[1], f[2], f[3]);
-        dst[1] = make_float4(f[4], f[5], f[6], f[7]);
-    } else if (prm.mode == TC_EMIT_SPLIT) {
-        uint4 hi, lo;
-        split2(__uint_as_float(v[0]), __uint_as_float(v[1]), hi.x, lo.x);
-        split2(__uint_as_float(v[2]), __uint_as_float(v[3]), hi.y, lo.y);
-        split2(__uint_as_float(v[4]), __uint_as_float(v[5]), hi.z, lo.z);
-        split2(__uint_as_float(v[6]), __uint_as_float(v[7]), hi.w, lo.w);
-        const size_t off = (size_t)gm * prm.ldc + gn;
-        *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(prm.C0) + off) = hi;
-        *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(prm.C1) + off) = lo;
     }
+}
+
+// Accumulator columns [c, c + 64) of the tile as 64 16-bit values per row: product times the two scales (TC_STORE_BF16),
+// or out_scale * product + diag on the diagonal + the entry of `add` (TC_AFFINE16).
+__device__ __forceinline__ void store_tile16(const TcParams& prm, uint32_t taddr, uint32_t buf, int m0, int gn, int lane)
+{
+    const bool affine = prm.mode == TC_AFFINE16;
+    const int gm = m0 + lane;
+    const float sc = affine ? prm.out_scale : (prm.scale_a ? prm.scale_a[0] * prm.scale_b[0] : 1.0f);
+    if (affine && prm.add) {
+        const int n = gn + 8 * (lane & 7);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int r = 4 * i + (lane >> 3);
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (n < prm.N && m0 + r < prm.M)
+                v = *reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(prm.add) + (size_t)(m0 + r) * prm.ldadd + n);
+            stage_put(buf, r, lane & 7, v);
+        }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint32_t v[32];
+        tc_ld_32cols(taddr + 32 * h, v);
+        tc_ld_wait();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float f[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                f[j] = sc * __uint_as_float(v[8 * q + j]);
+                if (affine && gm == gn + 32 * h + 8 * q + j) f[j] += prm.diag_sub;
+            }
+            if (affine && prm.add) {
+                const uint4 raw = stage_get(buf, lane, 4 * h + q);
+                const uint32_t w2[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 t = prm.out_f16 ? __half22float2(*reinterpret_cast<const __half2*>(&w2[j]))
+                                                 : __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w2[j]));
+                    f[2 * j] += t.x; f[2 * j + 1] += t.y;
+                }
+            }
+            uint32_t o[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                o[j] = prm.out_f16 ? pack_f16(__float_as_uint(f[2 * j]), __float_as_uint(f[2 * j + 1]))
+                                   : pack_bf16(__float_as_uint(f[2 * j]), __float_as_uint(f[2 * j + 1]));
+            stage_put(buf, lane, 4 * h + q, make_uint4(o[0], o[1], o[2], o[3]));
+        }
+    }
+    __syncwarp();
+    write_staged<2>(prm, buf, m0, gn, lane, 0);
+    __syncwarp();
+}
+
+// 32 accumulator columns as fp32, plain or (round_tf32) scaled, shifted on the diagonal and rounded; K slice `slice` of
+// the output.
+__device__ __forceinline__ void store_tile32(const TcParams& prm, const uint32_t (&v)[32], uint32_t buf, int m0, int gn, int lane, int slice)
+{
+    const int gm = m0 + lane;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        float f[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float a = __uint_as_float(v[4 * q + j]);
+            f[j] = prm.round_tf32 ? round_tf32(prm.post_scale * (prm.out_scale * a - ((gm == gn + 4 * q + j) ? prm.diag_sub : 0.0f))) : a;
+        }
+        stage_put(buf, lane, q, make_uint4(__float_as_uint(f[0]), __float_as_uint(f[1]), __float_as_uint(f[2]), __float_as_uint(f[3])));
+    }
+    __syncwarp();
+    write_staged<4>(prm, buf, m0, gn, lane, (long long)slice * prm.plane);
+    __syncwarp();
+}
+
+// The product as a (hi, lo) bf16 pair, eight columns from gn on.
+template <int G>
+__device__ __forceinline__ void emit_split(const TcParams& prm, int gm, int gn, const uint32_t (&w)[32])
+{
+    if (gn >= prm.N) return;
+    uint4 hi, lo;
+    split2(__uint_as_float(w[G * 8 + 0]), __uint_as_float(w[G * 8 + 1]), hi.x, lo.x);
+    split2(__uint_as_float(w[G * 8 + 2]), __uint_as_float(w[G * 8 + 3]), hi.y, lo.y);
+    split2(__uint_as_float(w[G * 8 + 4]), __uint_as_float(w[G * 8 + 5]), hi.z, lo.z);
+    split2(__uint_as_float(w[G * 8 + 6]), __uint_as_float(w[G * 8 + 7]), hi.w, lo.w);
+    const size_t off = (size_t)gm * prm.ldc + gn;
+    *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(prm.C0) + off) = hi;
+    *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(prm.C1) + off) = lo;
 }
 
 // Symmetric result (TC_STORE_SYM16): 32 consecutive entries of row gm from column gn on, as
@@ -232,13 +298,14 @@ __device__ __forceinline__ void store_symmetric(const TcParams& prm, int gm, int
     }
 }
 
-template <int BN, int kStages, bool kStaging, bool kTf32, bool kAMn, bool kF8>
+template <int BN, bool kStaging, bool kTf32, bool kAMn, bool kF8, bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_a1,
                const __grid_constant__ CUtensorMap map_b0, const __grid_constant__ CUtensorMap map_b1,
                const __grid_constant__ CUtensorMap map_c, const TcParams prm)
 {
-    using Cfg = TcCfg<BN, kStages, kStaging, kTf32, kAMn, kF8>;
+    using Cfg = TcCfg<BN, kStaging, kTf32, kAMn, kF8, kPair>;
+    constexpr int kStages = Cfg::kStages;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t tiles_base = (raw + 1023u) & ~1023u;                 // swizzle atoms need 1024-byte alignment
@@ -257,25 +324,34 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
 
-    const int m_tiles = (prm.M + BM - 1) / BM;
+    const int rank = kPair ? (int)cluster_rank() : 0;         // CTA 0 of a pair leads
+    const int first_tile = kPair ? blockIdx.x >> 1 : blockIdx.x, tile_step = kPair ? gridDim.x >> 1 : gridDim.x;
+    const int m_tiles = (prm.M + Cfg::kTileRows - 1) / Cfg::kTileRows;
     const int n_tiles = (prm.N + BN - 1) / BN;
     const int mn_tiles = m_tiles * n_tiles;
     const int total_tiles = prm.tri ? prm.tri_tiles : mn_tiles * prm.ksplit;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-        for (int a = 0; a < kAccStages; ++a) { mbar_init(acc_full_bar(a), 1); mbar_init(acc_empty_bar(a), kEpiWarps); }
+        for (int a = 0; a < kAccStages; ++a) { mbar_init(acc_full_bar(a), 1); mbar_init(acc_empty_bar(a), kPair ? 2 * kEpiWarps : kEpiWarps); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32((const void*)tmem_slot)), "r"(kTmemCols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        if (kPair) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
+                         ::"r"(smem_u32((const void*)tmem_slot)), "r"(kTmemCols) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                         ::"r"(smem_u32((const void*)tmem_slot)), "r"(kTmemCols) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
     }
     tc_fence_before();
-    __syncthreads();
+    __syncwarp();
+    if (kPair) cluster_sync(); else __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
@@ -284,10 +360,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         if (lane == 0) {
             uint32_t it = 0;
             bool ok = true;
-            for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+            for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step) {
                 int mt, nt, slice;
-                tile_coords(prm, tile, m_tiles, mn_tiles, mt, nt, slice);
-                const int m0 = mt * BM, n0 = nt * BN;
+                tile_coords<kPair>(prm, tile, m_tiles, mn_tiles, mt, nt, slice);
+                const int m0 = mt * Cfg::kTileRows + rank * BM, n0 = nt * BN + rank * Cfg::kCols;
 #pragma unroll
                 for (int sg = 0; sg < 3; ++sg) {              // constant indices keep the parameters out of local memory
                     if (sg >= prm.nseg || !ok) break;
@@ -302,24 +378,32 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
                         if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, prm.wait_ns)) { ok = false; break; }
                         const uint32_t sa = tiles_base + s * Cfg::kStageBytes;
                         const uint32_t sb = sa + kABytes;
-                        mbar_expect_tx(full_bar(s), Cfg::kStageBytes);
+                        // in a pair the copies of both CTAs count on the leader's barrier
+                        if (rank == 0) mbar_expect_tx(full_bar(s), kPair ? 2 * Cfg::kStageBytes : Cfg::kStageBytes);
+                        const uint32_t bar = kPair ? map_rank(full_bar(s), 0) : full_bar(s);
+                        auto load_2d = [&](uint32_t dst, const CUtensorMap* map, int x, int y) {
+                            if (kPair) tma_load_2d_pair(dst, map, x, y, bar); else tma_load_2d(dst, map, x, y, bar);
+                        };
+                        auto load_3d = [&](uint32_t dst, const CUtensorMap* map, int x, int y, int z) {
+                            if (kPair) tma_load_3d_pair(dst, map, x, y, z, bar); else tma_load_3d(dst, map, x, y, z, bar);
+                        };
                         if (kAMn) {
                             if (prm.a3d) {
-                                tma_load_3d(sa, ma, 0, seg.a_k0 + kb * Cfg::kBKE, m0 / Cfg::kBoxCols, full_bar(s));
+                                load_3d(sa, ma, 0, seg.a_k0 + kb * Cfg::kBKE, m0 / Cfg::kBoxCols);
                             } else {
 #pragma unroll
                                 for (int j = 0; j < BM / Cfg::kBoxCols; ++j)
-                                    tma_load_2d(sa + j * Cfg::kBoxBytes, ma, m0 + j * Cfg::kBoxCols, seg.a_k0 + kb * Cfg::kBKE, full_bar(s));
+                                    load_2d(sa + j * Cfg::kBoxBytes, ma, m0 + j * Cfg::kBoxCols, seg.a_k0 + kb * Cfg::kBKE);
                             }
                         } else {
-                            tma_load_2d(sa, ma, seg.a_k0 + kb * Cfg::kBKE, m0, full_bar(s));
+                            load_2d(sa, ma, seg.a_k0 + kb * Cfg::kBKE, m0);
                         }
                         if (prm.b3d) {
-                            tma_load_3d(sb, mb, 0, seg.b_row0 + kb * Cfg::kBKE, n0 / Cfg::kBoxCols, full_bar(s));
+                            load_3d(sb, mb, 0, seg.b_row0 + kb * Cfg::kBKE, n0 / Cfg::kBoxCols);
                         } else {
 #pragma unroll
-                            for (int j = 0; j < BN / Cfg::kBoxCols; ++j)
-                                tma_load_2d(sb + j * Cfg::kBoxBytes, mb, n0 + j * Cfg::kBoxCols, seg.b_row0 + kb * Cfg::kBKE, full_bar(s));
+                            for (int j = 0; j < Cfg::kCols / Cfg::kBoxCols; ++j)
+                                load_2d(sb + j * Cfg::kBoxBytes, mb, n0 + j * Cfg::kBoxCols, seg.b_row0 + kb * Cfg::kBKE);
                         }
                     }
                 }
@@ -327,15 +411,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             if (!ok) { *abort_flag = 1; atomicCAS(prm.status, 0, (int)GELO_ERR_TIMEOUT); }
         }
     } else if (warp == 1) {
-        // ================= MMA issuer =================
-        if (lane == 0) {
+        // ================= MMA issuer (in a pair: of the leader) =================
+        if (lane == 0 && rank == 0) {
             uint32_t acc_it = 0;
             uint32_t s = 0, ph = 0;                   // operand stage and the parity of its "full" phase
             bool ready = false;                       // stage s is already known to be full (tested ahead, see tc_mma4_*_try)
             bool ok = true;
             // k advance per instruction in sixteen-byte units of the descriptors' start address
             constexpr uint64_t kAStep = kAMn ? (Cfg::kMnStep >> 4) : 2, kBStep = Cfg::kMnStep >> 4;
-            for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++acc_it) {
+            for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step, ++acc_it) {
                 const int slice = prm.tri ? 0 : tile / mn_tiles;
                 int kb_total = 0;
 #pragma unroll
@@ -361,14 +445,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
                     const uint32_t ns = (s + 1 == kStages) ? 0u : s + 1;
                     const uint32_t nph = (ns == 0u) ? (ph ^ 1u) : ph;
                     // four instructions of 32 bytes of k (16 bf16 / 8 tf32) per stage
-                    ready = kF8 ? tc_mma4_f8_try(tmem_d, da, db, kAStep, kBStep, prm.idesc, kb != 0 ? 1u : 0u, full_bar(ns), nph)
-                          : kTf32 ? tc_mma4_tf32_try(tmem_d, da, db, kAStep, kBStep, prm.idesc, kb != 0 ? 1u : 0u, full_bar(ns), nph)
-                                  : tc_mma4_bf16_try(tmem_d, da, db, kAStep, kBStep, prm.idesc, kb != 0 ? 1u : 0u, full_bar(ns), nph);
-                    tc_commit(empty_bar(s));          // frees the stage once these MMAs have read it
+                    ready = tc_mma4_try<kF8 ? 2 : (kTf32 ? 1 : 0), kPair>(tmem_d, da, db, kAStep, kBStep, prm.idesc, kb != 0 ? 1u : 0u,
+                                                                          full_bar(ns), nph);
+                    if (kPair) tc_commit_pair(empty_bar(s)); else tc_commit(empty_bar(s));   // frees the stage once these MMAs have read it
                     s = ns; ph = nph;
                 }
                 if (!ok) break;
-                tc_commit(acc_full_bar(a));           // accumulator complete
+                if (kPair) tc_commit_pair(acc_full_bar(a)); else tc_commit(acc_full_bar(a));   // accumulator complete
             }
             if (!ok) { *abort_flag = 1; atomicCAS(prm.status, 0, (int)GELO_ERR_TIMEOUT); }
         }
@@ -379,12 +462,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         constexpr int kHalfCols = BN / 2;
         uint32_t acc_it = 0, box_it = 0;
         bool ok = true;
-        for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++acc_it) {
+        for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step, ++acc_it) {
             const int a = acc_it % kAccStages;
             const uint32_t aph = (acc_it / kAccStages) & 1u;
             int mt, nt, slice;
-            tile_coords(prm, tile, m_tiles, mn_tiles, mt, nt, slice);
-            const int m0 = mt * BM, n0 = nt * BN;
+            tile_coords<kPair>(prm, tile, m_tiles, mn_tiles, mt, nt, slice);
+            const int m0 = mt * Cfg::kTileRows + rank * BM, n0 = nt * BN;
             const int gm = m0 + quarter * 32 + lane;
             const bool row_ok = gm < prm.M;
             if (kStaging && prm.mode == TC_SUB_F32) {
@@ -422,35 +505,48 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
                 if (!mbar_wait(acc_full_bar(a), aph, abort_flag, prm.wait_ns)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * BN);
+                const int c_end = min((half + 1) * kHalfCols, prm.N - n0);
+                const uint32_t buf = staging_base + (uint32_t)(warp - 2) * 4096u;
+                if (kHalfCols % 64 == 0 && (prm.mode == TC_STORE_BF16 || prm.mode == TC_AFFINE16)) {
 #pragma unroll 1
-                for (int c = half * kHalfCols; c < (half + 1) * kHalfCols; c += 32) {
-                    uint32_t v[32];
-                    tc_ld_32cols(taddr + c, v);
-                    tc_ld_wait();
-                    if (prm.mode == TC_STORE_SYM16) {
-                        if (row_ok) store_symmetric(prm, gm, n0 + c, v);
-                    } else if (row_ok) {
-                        const int gn = n0 + c;
-                        if (gn < prm.N) epilogue_group<0>(prm, gm, gn, v, slice);
-                        if (gn + 8 < prm.N) epilogue_group<1>(prm, gm, gn + 8, v, slice);
-                        if (gn + 16 < prm.N) epilogue_group<2>(prm, gm, gn + 16, v, slice);
-                        if (gn + 24 < prm.N) epilogue_group<3>(prm, gm, gn + 24, v, slice);
+                    for (int c = half * kHalfCols; c < c_end; c += 64) store_tile16(prm, taddr + c, buf, m0 + quarter * 32, n0 + c, lane);
+                } else {
+#pragma unroll 1
+                    for (int c = half * kHalfCols; c < c_end; c += 32) {
+                        uint32_t v[32];
+                        tc_ld_32cols(taddr + c, v);
+                        tc_ld_wait();
+                        if (prm.mode == TC_STORE_SYM16) {
+                            if (row_ok) store_symmetric(prm, gm, n0 + c, v);
+                        } else if (prm.mode == TC_STORE_F32) {
+                            store_tile32(prm, v, buf, m0 + quarter * 32, n0 + c, lane, slice);
+                        } else if (row_ok) {                  // TC_EMIT_SPLIT
+                            const int gn = n0 + c;
+                            emit_split<0>(prm, gm, gn, v);
+                            emit_split<1>(prm, gm, gn + 8, v);
+                            emit_split<2>(prm, gm, gn + 16, v);
+                            emit_split<3>(prm, gm, gn + 24, v);
+                        }
                     }
                 }
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(acc_empty_bar(a));
+            if (lane == 0) {
+                if (kPair) mbar_arrive_cluster(map_rank(acc_empty_bar(a), 0)); else mbar_arrive(acc_empty_bar(a));
+            }
         }
         if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // staged boxes fully written out
         if (!ok && lane == 0) { *abort_flag = 1; atomicCAS(prm.status, 0, (int)GELO_ERR_TIMEOUT); }
     }
 
     tc_fence_before();
-    __syncthreads();
+    __syncwarp();
+    if (kPair) cluster_sync(); else __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
+        if (kPair) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
+        else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
     }
 }
 
@@ -518,30 +614,83 @@ bool make_map_nmajor(gelo_ctx* ctx, CUtensorMap* map, const void* ptr, int elem_
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN, int kStages, bool kStaging, bool kTf32 = false, bool kAMn = false, bool kF8 = false>
-int launch_tiles(gelo_ctx* ctx, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0,
-                 const CUtensorMap& b1, const CUtensorMap& c, const TcParams& p, double flops, cudaStream_t st)
+// CTAs that one launch may use
+int launch_width(const gelo_ctx* ctx, int mode)
 {
-    using Cfg = TcCfg<BN, kStages, kStaging, kTf32, kAMn, kF8>;
+    return (mode != TC_STORE_BF16 && ctx->tc_update_ctas > 0 && ctx->tc_update_ctas < ctx->sm_count) ? ctx->tc_update_ctas : ctx->sm_count;
+}
+
+// Work items of a product: 256 columns, 128 rows (256 in a pair), times the K slices; symmetric products leave out what
+// lies below the diagonal.
+int tile_count(int M, int N, int slices, bool tri, bool pair)
+{
+    const int m_tiles = ceil_div(M, pair ? 2 * BM : BM), n_tiles = ceil_div(N, 256);
+    if (!tri) return m_tiles * n_tiles * slices;
+    int tiles = 0;
+    for (int nt = 0; nt < n_tiles; ++nt) {
+        const int own = pair ? nt + 1 : 2 * nt + 2;
+        tiles += m_tiles < own ? m_tiles : own;
+    }
+    return tiles;
+}
+
+// Whether a product runs on pairs of CTAs.  A 256 x 256 tile of a pair takes its two SMs no longer than a 128 x 256 tile takes
+// one (each SM stages half of B, a third less in all, in six stages instead of four), so the pair wins unless the coarser
+// tiles need more rounds.  Measured with the staged stores, single -> pair: 4300 x 12288 x 4096 in bf16 323 -> 292 us (1.34 -> 1.48
+// PFLOP/s), 2150 rows 196 -> 166 us, E4M3 operands 2.01 -> 2.37 PFLOP/s at 4300 rows; 1050 x 4096 x 1050, where 144 single tiles make
+// one round and 80 pair tiles two, stays single (18.5 us).
+bool use_pair(const gelo_ctx* ctx, int M, int N, int slices, bool tri, int mode)
+{
+    const int width = launch_width(ctx, mode);
+    if (M <= BM || width < 2) return false;
+    return ceil_div(tile_count(M, N, slices, tri, true), width / 2) <= ceil_div(tile_count(M, N, slices, tri, false), width);
+}
+
+template <int BN, bool kStaging, bool kTf32, bool kAMn, bool kF8, bool kPair>
+int launch_tiles_as(gelo_ctx* ctx, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0, const CUtensorMap& b1,
+                    const CUtensorMap& c, const TcParams& p, double flops, cudaStream_t st)
+{
+    using Cfg = TcCfg<BN, kStaging, kTf32, kAMn, kF8, kPair>;
     static_assert(Cfg::kSmemBytes <= 227 * 1024, "shared memory budget");
+    auto kernel = gemm_tc_kernel<BN, kStaging, kTf32, kAMn, kF8, kPair>;
     static bool attr_done[64] = {};
     if (ctx->device >= 0 && ctx->device < 64 && !attr_done[ctx->device]) {
-        GELO_CUDA_OK(cudaFuncSetAttribute(gemm_tc_kernel<BN, kStages, kStaging, kTf32, kAMn, kF8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)Cfg::kSmemBytes));
+        GELO_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmemBytes));
         attr_done[ctx->device] = true;
     }
-    const int tiles = ceil_div(p.M, BM) * ceil_div(p.N, BN) * p.ksplit;
-    int grid = tiles < ctx->sm_count ? tiles : ctx->sm_count;
-    if (p.mode != TC_STORE_BF16 && ctx->tc_update_ctas > 0 && grid > ctx->tc_update_ctas) grid = ctx->tc_update_ctas;
     TcParams q = p;
+    if (p.tri) q.tri_tiles = tile_count(p.M, p.N, 1, true, kPair);
+    const int tiles = p.tri ? q.tri_tiles : ceil_div(p.M, Cfg::kTileRows) * ceil_div(p.N, BN) * p.ksplit;
+    const int most = launch_width(ctx, p.mode) / (kPair ? 2 : 1);
+    const int grid = (tiles < most ? tiles : most) * (kPair ? 2 : 1);
     // both operands of a kind::f16 instruction have the same 16-bit format: 1 = bfloat16, 0 = IEEE half
     q.wait_ns = ctx->wait_limit_ns;
     q.idesc = (!kTf32 && !kF8 && p.out_f16) ? (Cfg::kInstrDesc & ~((7u << 7) | (7u << 10))) : Cfg::kInstrDesc;
     {
         ProfScope ps(ctx, PROF_GEMM_TC, flops, st);
-        gemm_tc_kernel<BN, kStages, kStaging, kTf32, kAMn, kF8><<<grid, kThreads, Cfg::kSmemBytes, st>>>(a0, a1, b0, b1, c, q);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = Cfg::kSmemBytes;
+        cfg.stream = st;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = kPair ? 1 : 0;
+        GELO_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, a0, a1, b0, b1, c, q));
     }
     return after_launch(ctx);
+}
+
+template <int BN, bool kStaging, bool kTf32 = false, bool kAMn = false, bool kF8 = false>
+int launch_tiles(gelo_ctx* ctx, bool pair, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0, const CUtensorMap& b1,
+                 const CUtensorMap& c, const TcParams& p, double flops, cudaStream_t st)
+{
+    if constexpr (BN == 256) {
+        if (pair) return launch_tiles_as<BN, kStaging, kTf32, kAMn, kF8, true>(ctx, a0, a1, b0, b1, c, p, flops, st);
+    }
+    return launch_tiles_as<BN, kStaging, kTf32, kAMn, kF8, false>(ctx, a0, a1, b0, b1, c, p, flops, st);
 }
 
 // fp32 tensor map of the matrix that the subtracting epilogue reduces into: 32 x 32 boxes, 128-byte swizzle.
@@ -582,12 +731,14 @@ int launch_gemm_tc(gelo_ctx* ctx, const GemmArgs& g, cudaStream_t st)
     if (!ctx->tmap_encode) return GELO_ERR_CUDA;
     constexpr int BN = 256;
     const int rows_first = g.B2 ? g.b_split : g.K;
+    const bool pair = use_pair(ctx, g.M, g.N, 1, false, TC_STORE_BF16);
+    const uint32_t cols = pair ? BN / 2 : BN;                 // columns of B per CTA
     CUtensorMap ma, mb, mb2;
     if (!make_map(ctx, &ma, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda, BK, BM)) return GELO_ERR_CUDA;
     bool b3d = false, b3d2 = false;
-    if (!make_map_nmajor(ctx, &mb, g.B, 2, false, (uint64_t)g.N, (uint64_t)rows_first, (uint64_t)g.ldb, BK, BN, &b3d)) return GELO_ERR_CUDA;
+    if (!make_map_nmajor(ctx, &mb, g.B, 2, false, (uint64_t)g.N, (uint64_t)rows_first, (uint64_t)g.ldb, BK, cols, &b3d)) return GELO_ERR_CUDA;
     if (g.B2) {
-        if (!make_map_nmajor(ctx, &mb2, g.B2, 2, false, (uint64_t)g.N, (uint64_t)(g.K - g.b_split), (uint64_t)g.ldb, BK, BN, &b3d2))
+        if (!make_map_nmajor(ctx, &mb2, g.B2, 2, false, (uint64_t)g.N, (uint64_t)(g.K - g.b_split), (uint64_t)g.ldb, BK, cols, &b3d2))
             return GELO_ERR_CUDA;
         if (b3d2 != b3d) return GELO_ERR_CUDA;                // same width and stride: the same decision
     } else {
@@ -610,7 +761,7 @@ int launch_gemm_tc(gelo_ctx* ctx, const GemmArgs& g, cudaStream_t st)
     p.C0 = g.C[0]; p.C1 = g.C[g.nsplit > 1 ? 1 : 0]; p.C2 = g.C[g.nsplit > 2 ? 2 : 0];
     p.ldc = g.ldc; p.csplit = g.N / g.nsplit; p.lde = 0;
     p.status = ctx->status_dev;
-    return launch_tiles<BN, 4, false>(ctx, ma, ma, mb, mb2, ma, p, 2.0 * g.M * (double)g.N * g.K, st);
+    return launch_tiles<BN, false>(ctx, pair, ma, ma, mb, mb2, ma, p, 2.0 * g.M * (double)g.N * g.K, st);
 }
 
 // Split-precision product for the factorisations.  A = Ahi + Alo (M x K, stride lda), B = Bhi + Blo
@@ -630,7 +781,8 @@ int launch_gemm_tc_split(gelo_ctx* ctx, int M, int N, int K, const void* Ahi, co
     if (emit_hi && ((lde % 8) || !aligned16(emit_hi) || !aligned16(emit_lo))) return GELO_ERR_INVALID;
     if (!sub_from && !emit_hi) return GELO_ERR_INVALID;
     CUtensorMap a0, a1, b0, b1;
-    const uint32_t tile_cols = (!sub_from && narrow_tiles) ? 64 : 256;
+    const bool pair = (sub_from || !narrow_tiles) && use_pair(ctx, M, N, 1, false, TC_SUB_F32);
+    const uint32_t tile_cols = (!sub_from && narrow_tiles) ? 64 : (pair ? 128 : 256);
     bool b3d = false, b3d1 = false;
     if (!make_map(ctx, &a0, Ahi, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, BM) ||
         !make_map(ctx, &a1, Alo, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, BM) ||
@@ -659,9 +811,9 @@ int launch_gemm_tc_split(gelo_ctx* ctx, int M, int N, int K, const void* Ahi, co
         p.C0 = emit_hi; p.C1 = emit_lo; p.ldc = lde; p.lde = lde;
     }
     const double flops = 6.0 * M * (double)N * K;
-    if (sub_from) return launch_tiles<256, 3, true>(ctx, a0, a1, b0, b1, mc, p, flops, st);
-    if (narrow_tiles) return launch_tiles<64, 4, false>(ctx, a0, a1, b0, b1, mc, p, flops, st);
-    return launch_tiles<256, 4, false>(ctx, a0, a1, b0, b1, mc, p, flops, st);
+    if (sub_from) return launch_tiles<256, true>(ctx, pair, a0, a1, b0, b1, mc, p, flops, st);
+    if (narrow_tiles) return launch_tiles<64, false>(ctx, pair, a0, a1, b0, b1, mc, p, flops, st);
+    return launch_tiles<256, false>(ctx, pair, a0, a1, b0, b1, mc, p, flops, st);
 }
 
 
@@ -675,17 +827,19 @@ int launch_gemm_tc_split_k(gelo_ctx* ctx, int M, int N, int K, const void* Ahi, 
     if ((lda % 8) || (ldb % 8) || (N % 8) || (ldp % 4) || !aligned16(Ahi) || !aligned16(Alo) || !aligned16(Bhi) ||
         !aligned16(Blo) || !aligned16(planes) || (plane % 4) || ksplit < 1)
         return GELO_ERR_INVALID;
-    CUtensorMap a0, a1, b0, b1;
-    bool b3d = false, b3d1 = false;
-    if (!make_map(ctx, &a0, Ahi, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, BM) ||
-        !make_map(ctx, &a1, Alo, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, BM) ||
-        !make_map_nmajor(ctx, &b0, Bhi, 2, false, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, BK, 256, &b3d) ||
-        !make_map_nmajor(ctx, &b1, Blo, 2, false, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, BK, 256, &b3d1) || b3d != b3d1)
-        return GELO_ERR_CUDA;
     const int kb = ceil_div(K, BK);
     if (ksplit > kb) ksplit = kb;
     const int per = ceil_div(kb, ksplit);
     ksplit = ceil_div(kb, per);                    // no empty slice
+    const bool pair = use_pair(ctx, M, N, ksplit, false, TC_STORE_F32);
+    const uint32_t cols = pair ? 128 : 256;
+    CUtensorMap a0, a1, b0, b1;
+    bool b3d = false, b3d1 = false;
+    if (!make_map(ctx, &a0, Ahi, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, BM) ||
+        !make_map(ctx, &a1, Alo, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, BM) ||
+        !make_map_nmajor(ctx, &b0, Bhi, 2, false, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, BK, cols, &b3d) ||
+        !make_map_nmajor(ctx, &b1, Blo, 2, false, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, BK, cols, &b3d1) || b3d != b3d1)
+        return GELO_ERR_CUDA;
     TcParams p = {};
     p.M = M; p.N = N;
     p.nseg = 3;
@@ -699,7 +853,7 @@ int launch_gemm_tc_split_k(gelo_ctx* ctx, int M, int N, int K, const void* Ahi, 
     p.C0 = planes; p.ldc = ldp; p.lde = 0;
     p.ksplit = ksplit; p.kb_per_split = per; p.plane = (long long)plane;
     if (used) *used = ksplit;
-    return launch_tiles<256, 4, false>(ctx, a0, a1, b0, b1, a0, p, 6.0 * M * (double)N * K, st);
+    return launch_tiles<256, false>(ctx, pair, a0, a1, b0, b1, a0, p, 6.0 * M * (double)N * K, st);
 }
 
 // One-product tf32 GEMM on fp32 matrices, fp32 accumulation:  P = op(A) (M x K) * B (K x N, row-major, stride ldb).
@@ -719,15 +873,25 @@ int launch_gemm_tf32(gelo_ctx* ctx, int M, int N, int K, const float* A, int lda
     if ((lda % 4) || (ldb % 4) || (ldc % 4) || !aligned16(A) || !aligned16(B) || !aligned16(C) || !C) return GELO_ERR_INVALID;
     if (!subtract && (N % 8)) return GELO_ERR_INVALID;
     if (subtract && ksplit > 1) return GELO_ERR_INVALID;
+    const int kb = ceil_div(K, 32);
+    int per = kb;
+    if (ksplit > 1) {
+        if (ksplit > kb) ksplit = kb;
+        per = ceil_div(kb, ksplit);
+        ksplit = ceil_div(kb, per);                // no empty slice
+    } else {
+        ksplit = 1;
+    }
+    const bool pair = use_pair(ctx, M, N, ksplit, false, subtract ? TC_SUB_F32 : TC_STORE_F32);
+    const uint32_t cols = pair ? 128 : 256;
     CUtensorMap ma, mb, mc;
     bool a3d = false, b3d = false;
     const bool a_ok = a_mn ? make_map_nmajor(ctx, &ma, A, 4, true, (uint64_t)M, (uint64_t)K, (uint64_t)lda, 32, BM, &a3d)
                            : make_map_f32_box(ctx, &ma, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BM);
-    if (!a_ok || !make_map_nmajor(ctx, &mb, B, 4, true, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, 32, 256, &b3d)) return GELO_ERR_CUDA;
+    if (!a_ok || !make_map_nmajor(ctx, &mb, B, 4, true, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, 32, cols, &b3d)) return GELO_ERR_CUDA;
     mc = ma;
     TcParams p = {};
     p.M = M; p.N = N;
-    const int kb = ceil_div(K, 32);
     p.nseg = 1;
     p.seg[0] = TcSegment{0, 0, 0, 0, kb};
     p.status = ctx->status_dev;
@@ -741,19 +905,14 @@ int launch_gemm_tf32(gelo_ctx* ctx, int M, int N, int K, const float* A, int lda
     if (subtract) {
         if (!make_map_f32_box(ctx, &mc, C, (uint64_t)N, (uint64_t)M, (uint64_t)ldc, 32)) return GELO_ERR_CUDA;
         p.mode = TC_SUB_F32;
-        return a_mn ? launch_tiles<256, 3, true, true, true>(ctx, ma, ma, mb, mb, mc, p, flops, st)
-                    : launch_tiles<256, 3, true, true, false>(ctx, ma, ma, mb, mb, mc, p, flops, st);
+        return a_mn ? launch_tiles<256, true, true, true>(ctx, pair, ma, ma, mb, mb, mc, p, flops, st)
+                    : launch_tiles<256, true, true, false>(ctx, pair, ma, ma, mb, mb, mc, p, flops, st);
     }
     p.mode = TC_STORE_F32;
-    if (ksplit > 1) {
-        if (ksplit > kb) ksplit = kb;
-        const int per = ceil_div(kb, ksplit);
-        ksplit = ceil_div(kb, per);                // no empty slice
-        p.ksplit = ksplit; p.kb_per_split = per; p.plane = (long long)plane;
-    }
+    if (ksplit > 1) { p.ksplit = ksplit; p.kb_per_split = per; p.plane = (long long)plane; }
     if (used) *used = p.ksplit;
-    return a_mn ? launch_tiles<256, 4, false, true, true>(ctx, ma, ma, mb, mb, mc, p, flops, st)
-                : launch_tiles<256, 4, false, true, false>(ctx, ma, ma, mb, mb, mc, p, flops, st);
+    return a_mn ? launch_tiles<256, false, true, true>(ctx, pair, ma, ma, mb, mb, mc, p, flops, st)
+                : launch_tiles<256, false, true, false>(ctx, pair, ma, ma, mb, mb, mc, p, flops, st);
 }
 
 // C = out_scale * (A0^T B0 + A1^T B1) rounded to tf32: two products of the same sizes in one accumulator.
@@ -765,12 +924,14 @@ int launch_gemm_tf32_dual(gelo_ctx* ctx, int M, int N, int K, const float* A0, i
     if ((lda0 % 4) || (lda1 % 4) || (ldb0 % 4) || (ldb1 % 4) || (ldc % 4) || (N % 8) || !aligned16(A0) || !aligned16(A1) ||
         !aligned16(B0) || !aligned16(B1) || !aligned16(C))
         return GELO_ERR_INVALID;
+    const bool pair = use_pair(ctx, M, N, 1, false, TC_STORE_F32);
+    const uint32_t cols = pair ? 128 : 256;
     CUtensorMap a0, a1, b0, b1;
     bool a3d = false, a3d1 = false, b3d = false, b3d1 = false;
     if (!make_map_nmajor(ctx, &a0, A0, 4, true, (uint64_t)M, (uint64_t)K, (uint64_t)lda0, 32, BM, &a3d) ||
         !make_map_nmajor(ctx, &a1, A1, 4, true, (uint64_t)M, (uint64_t)K, (uint64_t)lda1, 32, BM, &a3d1) ||
-        !make_map_nmajor(ctx, &b0, B0, 4, true, (uint64_t)N, (uint64_t)K, (uint64_t)ldb0, 32, 256, &b3d) ||
-        !make_map_nmajor(ctx, &b1, B1, 4, true, (uint64_t)N, (uint64_t)K, (uint64_t)ldb1, 32, 256, &b3d1) || a3d != a3d1 || b3d != b3d1)
+        !make_map_nmajor(ctx, &b0, B0, 4, true, (uint64_t)N, (uint64_t)K, (uint64_t)ldb0, 32, cols, &b3d) ||
+        !make_map_nmajor(ctx, &b1, B1, 4, true, (uint64_t)N, (uint64_t)K, (uint64_t)ldb1, 32, cols, &b3d1) || a3d != a3d1 || b3d != b3d1)
         return GELO_ERR_CUDA;
     TcParams p = {};
     p.M = M; p.N = N;
@@ -786,7 +947,7 @@ int launch_gemm_tf32_dual(gelo_ctx* ctx, int M, int N, int K, const float* A0, i
     p.out_scale = out_scale; p.post_scale = 1.0f;
     p.C0 = C; p.ldc = ldc;
     p.mode = TC_STORE_F32;
-    return launch_tiles<256, 4, false, true, true>(ctx, a0, a1, b0, b1, a0, p, 4.0 * M * (double)N * K, st);
+    return launch_tiles<256, false, true, true>(ctx, pair, a0, a1, b0, b1, a0, p, 4.0 * M * (double)N * K, st);
 }
 
 // D (m x m bf16, stride ldd) = post_scale * (out_scale * Q^T Q - diag_sub I) for a row-major fp32 Q (stride ld): one
@@ -799,10 +960,12 @@ int launch_gram_sym_bf16(gelo_ctx* ctx, int m, const float* Q, int ld, void* D, 
     if (!ctx->tmap_encode) return GELO_ERR_CUDA;
     const int m8 = (m + 7) & ~7;
     if ((ld % 4) || ld < m8 || (ldd % 8) || ldd < m8 || !aligned16(Q) || !aligned16(D)) return GELO_ERR_INVALID;
+    const bool pair = use_pair(ctx, m, m8, 1, true, TC_STORE_SYM16);
+    const uint32_t cols = pair ? 128 : 256;
     CUtensorMap ma, mb;
     bool a3d = false, b3d = false;
     if (!make_map_nmajor(ctx, &ma, Q, 4, true, (uint64_t)m, (uint64_t)m, (uint64_t)ld, 32, BM, &a3d) ||
-        !make_map_nmajor(ctx, &mb, Q, 4, true, (uint64_t)m8, (uint64_t)m, (uint64_t)ld, 32, 256, &b3d))
+        !make_map_nmajor(ctx, &mb, Q, 4, true, (uint64_t)m8, (uint64_t)m, (uint64_t)ld, 32, cols, &b3d))
         return GELO_ERR_CUDA;
     TcParams p = {};
     p.M = m; p.N = m8;
@@ -816,11 +979,7 @@ int launch_gram_sym_bf16(gelo_ctx* ctx, int m, const float* Q, int ld, void* D, 
     p.C0 = D; p.ldc = ldd;
     p.mode = TC_STORE_SYM16;
     p.tri = 1;
-    const int m_tiles = ceil_div(m, BM), n_tiles = ceil_div(m8, 256);
-    int tiles = 0;
-    for (int nt = 0; nt < n_tiles; ++nt) tiles += (m_tiles < 2 * nt + 2) ? m_tiles : 2 * nt + 2;
-    p.tri_tiles = tiles;
-    return launch_tiles<256, 4, false, true, true>(ctx, ma, ma, mb, mb, ma, p, 2.0 * m * (double)m * m, st);
+    return launch_tiles<256, false, true, true>(ctx, pair, ma, ma, mb, mb, ma, p, 2.0 * m * (double)m * m, st);
 }
 
 // C (M x N fp32, stride ldc) -= A (M x K bf16, stride lda) * B (K x N bf16, stride ldb), in place by TMA reduce-add.
@@ -830,10 +989,12 @@ int launch_gemm_bf16_sub(gelo_ctx* ctx, int M, int N, int K, const void* A, int 
     if (M <= 0 || N <= 0 || K <= 0) return GELO_OK;
     if (!ctx->tmap_encode) return GELO_ERR_CUDA;
     if ((lda % 8) || (ldb % 8) || (ldc % 4) || !aligned16(A) || !aligned16(B) || !aligned16(C)) return GELO_ERR_INVALID;
+    const bool pair = use_pair(ctx, M, N, 1, false, TC_SUB_F32);
+    const uint32_t cols = pair ? 128 : 256;
     CUtensorMap ma, mb, mc;
     bool b3d = false;
     if (!make_map(ctx, &ma, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, BM) ||
-        !make_map_nmajor(ctx, &mb, B, 2, false, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, BK, 256, &b3d) ||
+        !make_map_nmajor(ctx, &mb, B, 2, false, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, BK, cols, &b3d) ||
         !make_map_f32_box(ctx, &mc, C, (uint64_t)N, (uint64_t)M, (uint64_t)ldc))
         return GELO_ERR_CUDA;
     TcParams p = {};
@@ -846,7 +1007,7 @@ int launch_gemm_bf16_sub(gelo_ctx* ctx, int M, int N, int K, const void* A, int 
     p.ksplit = 1; p.kb_per_split = 1 << 30; p.plane = 0;
     p.mode = TC_SUB_F32;
     p.C0 = C; p.ldc = ldc;
-    return launch_tiles<256, 3, true>(ctx, ma, ma, mb, mb, mc, p, 2.0 * M * (double)N * K, st);
+    return launch_tiles<256, true>(ctx, pair, ma, ma, mb, mb, mc, p, 2.0 * M * (double)N * K, st);
 }
 
 // C (M x N, 16-bit type of the operands) = sign * A (M x K) B (K x N) + diag I + add (optional, M x N)
@@ -858,10 +1019,12 @@ int launch_gemm_affine16(gelo_ctx* ctx, int dtype, int M, int N, int K, const vo
     if ((lda % 8) || (ldb % 8) || (ldc % 8) || (N % 8) || (ldadd % 8) || !aligned16(A) || !aligned16(B) || !aligned16(C) ||
         !aligned16(add))
         return GELO_ERR_INVALID;
+    const bool pair = use_pair(ctx, M, N, 1, false, TC_AFFINE16);
+    const uint32_t cols = pair ? 128 : 256;
     CUtensorMap ma, mb;
     bool b3d = false;
     if (!make_map(ctx, &ma, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, BM) ||
-        !make_map_nmajor(ctx, &mb, B, 2, false, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, BK, 256, &b3d))
+        !make_map_nmajor(ctx, &mb, B, 2, false, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, BK, cols, &b3d))
         return GELO_ERR_CUDA;
     TcParams p = {};
     p.M = M; p.N = N;
@@ -875,7 +1038,7 @@ int launch_gemm_affine16(gelo_ctx* ctx, int dtype, int M, int N, int K, const vo
     p.add = add; p.ldadd = ldadd;
     p.C0 = C; p.ldc = ldc; p.csplit = N;
     p.status = ctx->status_dev;
-    return launch_tiles<256, 4, false>(ctx, ma, ma, mb, mb, ma, p, 2.0 * M * (double)N * K, st);
+    return launch_tiles<256, false>(ctx, pair, ma, ma, mb, mb, ma, p, 2.0 * M * (double)N * K, st);
 }
 
 // Y (M x N, bf16) = (sa sb) A8 (M x K, E4M3, row stride lda bytes) * B8 (K x N, E4M3, row stride ldb bytes): the offloaded
@@ -889,6 +1052,7 @@ int launch_gemm_e4m3(gelo_ctx* ctx, int M, int N, int K, const void* A8, int lda
     if ((lda % 16) || (ldb % 16) || (ldc % 8) || (N % 8) || !aligned16(A8) || !aligned16(B8) || !aligned16(C) || !sa || !sb)
         return GELO_ERR_INVALID;
     EncodeTiledFn enc = reinterpret_cast<EncodeTiledFn>(ctx->tmap_encode);
+    const bool pair = use_pair(ctx, M, N, 1, false, TC_STORE_BF16);
     CUtensorMap ma, mb;
     {
         const cuuint64_t dims[2] = { (cuuint64_t)K, (cuuint64_t)M };
@@ -900,7 +1064,7 @@ int launch_gemm_e4m3(gelo_ctx* ctx, int M, int N, int K, const void* A8, int lda
             return GELO_ERR_CUDA;
     }
     bool b3d = false;
-    if (!make_map_nmajor(ctx, &mb, B8, 1, false, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, 128, 256, &b3d)) return GELO_ERR_CUDA;
+    if (!make_map_nmajor(ctx, &mb, B8, 1, false, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, 128, pair ? 128 : 256, &b3d)) return GELO_ERR_CUDA;
     TcParams p = {};
     p.M = M; p.N = N;
     p.nseg = 1;
@@ -912,7 +1076,7 @@ int launch_gemm_e4m3(gelo_ctx* ctx, int M, int N, int K, const void* A8, int lda
     p.ldc = ldc; p.csplit = N;
     p.scale_a = sa; p.scale_b = sb;
     p.status = ctx->status_dev;
-    return launch_tiles<256, 4, false, false, false, true>(ctx, ma, ma, mb, mb, ma, p, 2.0 * M * (double)N * K, st);
+    return launch_tiles<256, false, false, false, true>(ctx, pair, ma, ma, mb, mb, ma, p, 2.0 * M * (double)N * K, st);
 }
 
 int launch_gemm_tf32x3(gelo_ctx* ctx, int M, int N, int K, const float* Ahi, const float* Alo, int lda, const float* Bhi,
@@ -925,16 +1089,21 @@ int launch_gemm_tf32x3(gelo_ctx* ctx, int M, int N, int K, const float* Ahi, con
         return GELO_ERR_INVALID;
     for (int q = 0; q < nsplit; ++q)
         if (!C[q] || !aligned16(C[q])) return GELO_ERR_INVALID;
+    const int kb = ceil_div(K, 32);
+    // (N a multiple of 8, so the planes' rows are whole chunks)
+    const bool sliced = planes && kb >= 2 * kTf32x3Slices && aligned16(planes);
+    const int per = sliced ? ceil_div(kb, kTf32x3Slices) : kb;
+    const bool pair = use_pair(ctx, M, N, ceil_div(kb, per), false, TC_STORE_F32);
+    const uint32_t cols = pair ? 128 : 256;
     CUtensorMap a0, a1, b0, b1;
     bool b3d = false, b3d1 = false;
     if (!make_map_f32_box(ctx, &a0, Ahi, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BM) ||
         !make_map_f32_box(ctx, &a1, Alo, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BM) ||
-        !make_map_nmajor(ctx, &b0, Bhi, 4, true, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, 32, 256, &b3d) ||
-        !make_map_nmajor(ctx, &b1, Blo, 4, true, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, 32, 256, &b3d1) || b3d != b3d1)
+        !make_map_nmajor(ctx, &b0, Bhi, 4, true, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, 32, cols, &b3d) ||
+        !make_map_nmajor(ctx, &b1, Blo, 4, true, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, 32, cols, &b3d1) || b3d != b3d1)
         return GELO_ERR_CUDA;
     TcParams p = {};
     p.M = M; p.N = N;
-    const int kb = ceil_div(K, 32);
     p.nseg = 3;
     p.seg[0] = TcSegment{0, 0, 0, 0, kb};
     p.seg[1] = TcSegment{0, 1, 0, 0, kb};
@@ -945,16 +1114,15 @@ int launch_gemm_tf32x3(gelo_ctx* ctx, int M, int N, int K, const float* Ahi, con
     p.mode = TC_STORE_F32;
     p.out_scale = 1.0f; p.post_scale = 1.0f;
     float* const Cq[3] = { C[0], C[nsplit > 1 ? 1 : 0], C[nsplit > 2 ? 2 : 0] };
-    if (planes && kb >= 2 * kTf32x3Slices && aligned16(planes) && (N % 4) == 0) {
-        const int per = ceil_div(kb, kTf32x3Slices);
+    if (sliced) {
         p.ksplit = ceil_div(kb, per); p.kb_per_split = per; p.plane = (long long)M * N;
         p.C0 = planes; p.C1 = planes; p.C2 = planes; p.ldc = N; p.csplit = N;
-        GELO_TRY((launch_tiles<256, 4, false, true, false>(ctx, a0, a1, b0, b1, a0, p, 6.0 * M * (double)N * K, st)));
+        GELO_TRY((launch_tiles<256, false, true, false>(ctx, pair, a0, a1, b0, b1, a0, p, 6.0 * M * (double)N * K, st)));
         return launch_sum_planes_routed(ctx, planes, (size_t)M * N, p.ksplit, M, N, Cq, ldc, N / nsplit, st);
     }
     p.C0 = Cq[0]; p.C1 = Cq[1]; p.C2 = Cq[2];
     p.ldc = ldc; p.csplit = N / nsplit;
-    return launch_tiles<256, 4, false, true, false>(ctx, a0, a1, b0, b1, a0, p, 6.0 * M * (double)N * K, st);
+    return launch_tiles<256, false, true, false>(ctx, pair, a0, a1, b0, b1, a0, p, 6.0 * M * (double)N * K, st);
 }
 
 }  // namespace gelo

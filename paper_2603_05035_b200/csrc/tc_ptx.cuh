@@ -73,12 +73,57 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
 }
 
+// Copies of a CTA pair: `bar` is a shared::cluster address and may lie in the other CTA.
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
+}
+
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
+}
+
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// The address of `addr` (this CTA's shared memory) in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 __device__ __forceinline__ void tc_commit(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// ... arriving at the barrier at this place in both CTAs of a pair
+__device__ __forceinline__ void tc_commit_pair(uint32_t bar)
+{
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 ::"r"(bar), "h"((uint16_t)3) : "memory");
 }
 
 __device__ __forceinline__ void tc_mma_bf16(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc,
@@ -105,16 +150,16 @@ __device__ __forceinline__ void tc_mma_tf32(uint32_t tmem_d, uint64_t desc_a, ui
 // start address), with a barrier test tucked in front of them: the test of the NEXT stage's "full" barrier takes about
 // a hundred cycles to answer, and asked here its answer arrives while the four instructions issue instead of holding
 // up the next stage.  Returns whether that barrier phase had completed.
-#define GELO_TC_MMA4_TRY(KIND)                                                                                          \
+#define GELO_TC_MMA4_TRY(GROUP, KIND)                                                                                   \
     uint32_t ready;                                                                                                     \
     asm volatile(                                                                                                       \
-        "{\n\t.reg .pred q, p;\n\t"                                                                                    \
+        "{\n\t.reg .pred q, p;\n\t"                                                                                     \
         "mbarrier.try_wait.parity.shared::cta.b64 q, [%8], %9;\n\t"                                                     \
         "setp.ne.b32 p, %7, 0;\n\t"                                                                                     \
-        "tcgen05.mma.cta_group::1.kind::" KIND " [%1], %2, %3, %6, p;\n\t"                                              \
-        "tcgen05.mma.cta_group::1.kind::" KIND " [%1], %4, %5, %6, 1;\n\t"                                              \
-        "tcgen05.mma.cta_group::1.kind::" KIND " [%1], %10, %11, %6, 1;\n\t"                                            \
-        "tcgen05.mma.cta_group::1.kind::" KIND " [%1], %12, %13, %6, 1;\n\t"                                            \
+        "tcgen05.mma.cta_group::" GROUP ".kind::" KIND " [%1], %2, %3, %6, p;\n\t"                                      \
+        "tcgen05.mma.cta_group::" GROUP ".kind::" KIND " [%1], %4, %5, %6, 1;\n\t"                                      \
+        "tcgen05.mma.cta_group::" GROUP ".kind::" KIND " [%1], %10, %11, %6, 1;\n\t"                                    \
+        "tcgen05.mma.cta_group::" GROUP ".kind::" KIND " [%1], %12, %13, %6, 1;\n\t"                                    \
         "selp.u32 %0, 1, 0, q;\n\t}"                                                                                    \
         : "=r"(ready)                                                                                                   \
         : "r"(tmem_d), "l"(da), "l"(db), "l"(da + astep), "l"(db + bstep), "r"(idesc), "r"(accumulate), "r"(next_bar),  \
@@ -122,20 +167,20 @@ __device__ __forceinline__ void tc_mma_tf32(uint32_t tmem_d, uint64_t desc_a, ui
         : "memory");                                                                                                    \
     return ready != 0;
 
-__device__ __forceinline__ bool tc_mma4_bf16_try(uint32_t tmem_d, uint64_t da, uint64_t db, uint64_t astep, uint64_t bstep,
-                                                 uint32_t idesc, uint32_t accumulate, uint32_t next_bar, uint32_t next_parity)
+// kKind: 0 = f16 / bf16, 1 = tf32, 2 = 8-bit; kPair: the instruction of a CTA pair
+template <int kKind, bool kPair>
+__device__ __forceinline__ bool tc_mma4_try(uint32_t tmem_d, uint64_t da, uint64_t db, uint64_t astep, uint64_t bstep, uint32_t idesc,
+                                            uint32_t accumulate, uint32_t next_bar, uint32_t next_parity)
 {
-    GELO_TC_MMA4_TRY("f16")
-}
-__device__ __forceinline__ bool tc_mma4_tf32_try(uint32_t tmem_d, uint64_t da, uint64_t db, uint64_t astep, uint64_t bstep,
-                                                 uint32_t idesc, uint32_t accumulate, uint32_t next_bar, uint32_t next_parity)
-{
-    GELO_TC_MMA4_TRY("tf32")
-}
-__device__ __forceinline__ bool tc_mma4_f8_try(uint32_t tmem_d, uint64_t da, uint64_t db, uint64_t astep, uint64_t bstep,
-                                               uint32_t idesc, uint32_t accumulate, uint32_t next_bar, uint32_t next_parity)
-{
-    GELO_TC_MMA4_TRY("f8f6f4")
+    if constexpr (kPair) {
+        if constexpr (kKind == 0) { GELO_TC_MMA4_TRY("2", "f16") }
+        else if constexpr (kKind == 1) { GELO_TC_MMA4_TRY("2", "tf32") }
+        else { GELO_TC_MMA4_TRY("2", "f8f6f4") }
+    } else {
+        if constexpr (kKind == 0) { GELO_TC_MMA4_TRY("1", "f16") }
+        else if constexpr (kKind == 1) { GELO_TC_MMA4_TRY("1", "tf32") }
+        else { GELO_TC_MMA4_TRY("1", "f8f6f4") }
+    }
 }
 #undef GELO_TC_MMA4_TRY
 
