@@ -915,7 +915,7 @@ int launch_gemm_tf32(gelo_ctx* ctx, int M, int N, int K, const float* A, int lda
                 : launch_tiles<256, false, true, false>(ctx, pair, ma, ma, mb, mb, mc, p, flops, st);
 }
 
-// C = out_scale * (A0^T B0 + A1^T B1) rounded to tf32: two products of the same sizes in one accumulator.
+// C = out_scale * (A0 B0 + A1 B1) rounded to tf32: two products of the same sizes in one accumulator.
 int launch_gemm_tf32_dual(gelo_ctx* ctx, int M, int N, int K, const float* A0, int lda0, const float* B0, int ldb0, const float* A1,
                           int lda1, const float* B1, int ldb1, float* C, int ldc, float out_scale, cudaStream_t st)
 {
@@ -927,11 +927,11 @@ int launch_gemm_tf32_dual(gelo_ctx* ctx, int M, int N, int K, const float* A0, i
     const bool pair = use_pair(ctx, M, N, 1, false, TC_STORE_F32);
     const uint32_t cols = pair ? 128 : 256;
     CUtensorMap a0, a1, b0, b1;
-    bool a3d = false, a3d1 = false, b3d = false, b3d1 = false;
-    if (!make_map_nmajor(ctx, &a0, A0, 4, true, (uint64_t)M, (uint64_t)K, (uint64_t)lda0, 32, BM, &a3d) ||
-        !make_map_nmajor(ctx, &a1, A1, 4, true, (uint64_t)M, (uint64_t)K, (uint64_t)lda1, 32, BM, &a3d1) ||
+    bool b3d = false, b3d1 = false;
+    if (!make_map_f32_box(ctx, &a0, A0, (uint64_t)K, (uint64_t)M, (uint64_t)lda0, BM) ||
+        !make_map_f32_box(ctx, &a1, A1, (uint64_t)K, (uint64_t)M, (uint64_t)lda1, BM) ||
         !make_map_nmajor(ctx, &b0, B0, 4, true, (uint64_t)N, (uint64_t)K, (uint64_t)ldb0, 32, cols, &b3d) ||
-        !make_map_nmajor(ctx, &b1, B1, 4, true, (uint64_t)N, (uint64_t)K, (uint64_t)ldb1, 32, cols, &b3d1) || a3d != a3d1 || b3d != b3d1)
+        !make_map_nmajor(ctx, &b1, B1, 4, true, (uint64_t)N, (uint64_t)K, (uint64_t)ldb1, 32, cols, &b3d1) || b3d != b3d1)
         return GELO_ERR_CUDA;
     TcParams p = {};
     p.M = M; p.N = N;
@@ -942,12 +942,12 @@ int launch_gemm_tf32_dual(gelo_ctx* ctx, int M, int N, int K, const float* A0, i
     p.status = ctx->status_dev;
     p.csplit = N;
     p.ksplit = 1; p.kb_per_split = 1 << 30; p.plane = 0;
-    p.a3d = a3d ? 1 : 0; p.b3d = b3d ? 1 : 0;
+    p.b3d = b3d ? 1 : 0;
     p.round_tf32 = 1;
     p.out_scale = out_scale; p.post_scale = 1.0f;
     p.C0 = C; p.ldc = ldc;
     p.mode = TC_STORE_F32;
-    return launch_tiles<256, false, true, true>(ctx, pair, a0, a1, b0, b1, a0, p, 4.0 * M * (double)N * K, st);
+    return launch_tiles<256, false, true, false>(ctx, pair, a0, a1, b0, b1, a0, p, 4.0 * M * (double)N * K, st);
 }
 
 // D (m x m bf16, stride ldd) = post_scale * (out_scale * Q^T Q - diag_sub I) for a row-major fp32 Q (stride ld): one

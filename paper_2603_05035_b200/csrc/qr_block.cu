@@ -11,6 +11,11 @@
 // a 128 x 128 Cholesky factorisation and a 128 x 128 inverse (block_factor_kernel); everything else is a
 // product.  The update of columns C right of the block needs W' = T^T V^T C = T^T (P^T C) + D^T C1, D = R T = B^-T,
 // C1 = the first b rows of C: P^T C comes out of the same product as P^T P.
+// Blocks are grouped four by four into superblocks whose merged reflector, I - V_s T_s V_s^T, is all that the rest of the matrix
+// and Q ever see.  A block's row of T_s^T left of the diagonal is -X^T T_<^T with X^T = T^T V^T V_<, which is W' with the
+// earlier reflectors V_< of the superblock in place of C.  So a block's two products, P^T [V_< P C] and the one that gives
+// W', run over all columns of the superblock, and a merge is a single small product more (as products of its own with its sum
+// it was five dependent launches, 50 us per block).
 // The last block, which would be square, is factorised by the one-launch Householder kernel.
 //
 // Against 32-column Householder panels in registers (70 us per 32 columns of serial column steps, and rank-32 updates
@@ -473,12 +478,12 @@ __device__ __forceinline__ void fact_pivots(FactShared& s, int* status)
 }
 
 // Z (ob x ob, stride ldz): the Gram matrix P^T P.  P1: the first ob rows of the panel (stride ld), overwritten
-// with B = P1 + R.  T (stride ldt) = R^-1 B^-T and D (stride ldd) = dscale * B^-T, both rounded to tf32 if `round`.
+// with B = P1 + R.  Tt (stride ldt) = T^T = B^-1 R^-T and Dt (stride ldd) = dscale * B^-1, both rounded to tf32.
 // ob <= 128, a multiple of 4; the kernel works on 128 x 128 with an identity in the part past ob.  `scale` is a power of
 // two close to the norm of a panel column.
 __global__ void __cluster_dims__(kFactCtas, 1, 1) __launch_bounds__(kFactThreads, 1)
-block_factor_kernel(const float* __restrict__ Z, int ldz, float* P1, int ld, int ob, float* __restrict__ T,
-                    int ldt, float* __restrict__ D, int ldd, float scale, float dscale, int round, int* __restrict__ status)
+block_factor_kernel(const float* __restrict__ Z, int ldz, float* P1, int ld, int ob, float* __restrict__ Tt,
+                    int ldt, float* __restrict__ Dt, int ldd, float scale, float dscale, int* __restrict__ status)
 {
     extern __shared__ __align__(128) uint8_t fsm[];
     FactShared& s = *reinterpret_cast<FactShared*>(fsm);
@@ -547,41 +552,30 @@ block_factor_kernel(const float* __restrict__ Z, int ldz, float* P1, int ld, int
     } else {
         if (role == FACT_INVERSE) fact_compute<FACT_INVERSE>(a, s, status);
         else fact_compute<FACT_FACTOR>(a, s, status);
-        // the transpose of the result, by way of the slots of got (all read by now); row q of the transpose is rotated
-        // by 8 (q / 2) so that a warp's writes fall into different banks
-        float* X = &s.got[0][0][0];
+        float* dst = role == FACT_INVERSE ? Dt : Tt;
+        const int ldo = role == FACT_INVERSE ? ldd : ldt;
         const float f = role == FACT_INVERSE ? dscale * s1 : s2;
-        compute_barrier();
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int r = 32 * wr + 16 * mt + gid + 8 * (e >> 1), q = 64 * wc + 8 * nt + 2 * tig + (e & 1);
-                    const float v = f * a[mt][nt][e];
-                    X[q * FB + ((r + 8 * (q >> 1)) & (FB - 1))] = round ? tcx::round_tf32(v) : v;
+                for (int i = 0; i < 2; ++i) {
+                    const int r = 32 * wr + 16 * mt + gid + 8 * i, c = 64 * wc + 8 * nt + 2 * tig;
+                    if (r < ob && c < ob)
+                        *reinterpret_cast<float2*>(dst + (size_t)r * ldo + c) =
+                            make_float2(tcx::round_tf32(f * a[mt][nt][2 * i]), tcx::round_tf32(f * a[mt][nt][2 * i + 1]));
                 }
-        compute_barrier();
-        float* dst = role == FACT_INVERSE ? D : T;
-        const int ldo = role == FACT_INVERSE ? ldd : ldt;
-#pragma unroll 4
-        for (int idx = tid; idx < FB * FB / 4; idx += kFactCompute) {
-            const int q = idx >> 5, c = (idx & 31) * 4;
-            if (q < ob && c < ob)
-                *reinterpret_cast<float4*>(dst + (size_t)q * ldo + c) =
-                    *reinterpret_cast<const float4*>(X + q * FB + ((c + 8 * (q >> 1)) & (FB - 1)));
-        }
     }
     __syncwarp();
     cluster_sync_all();                                      // nobody's shared memory goes while a copy may still reach it
 }
 
-// Z = scale * (sum of the K slices of P^T [P | C]), in slice order; the first ob columns (the Gram matrix) stay fp32, the
-// others are rounded to tf32 (they feed the next product).  Also clears the rows above the block (z_rows x ob) where the
-// superblock's reflectors are zero.
+// Z = scale * (sum of the K slices of P^T [V_< | P | C]), in slice order; columns c0 .. c0 + ob - 1 (the Gram matrix) stay
+// fp32, the others are rounded to tf32 (they feed the next product).  Also clears the rows above the block (z_rows x ob)
+// where the superblock's reflectors are zero.
 __global__ void __launch_bounds__(256)
-block_sum_kernel(const float* __restrict__ planes, size_t plane, int parts, int ldp, int rows, int cols, int ob, float scale,
+block_sum_kernel(const float* __restrict__ planes, size_t plane, int parts, int ldp, int rows, int cols, int c0, int ob, float scale,
                  float* __restrict__ Z, int ldz, float* __restrict__ zero, int z_rows, int ld)
 {
     const int idx = blockIdx.x * 256 + threadIdx.x;
@@ -595,7 +589,7 @@ block_sum_kernel(const float* __restrict__ planes, size_t plane, int parts, int 
             acc.x += t.x; acc.y += t.y; acc.z += t.z; acc.w += t.w;
         }
         acc.x *= scale; acc.y *= scale; acc.z *= scale; acc.w *= scale;
-        if (c >= ob) {
+        if (c < c0 || c >= c0 + ob) {
             acc.x = tcx::round_tf32(acc.x); acc.y = tcx::round_tf32(acc.y);
             acc.z = tcx::round_tf32(acc.z); acc.w = tcx::round_tf32(acc.w);
         }
@@ -650,8 +644,8 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
         int want = (2 * tiles >= width) ? 1 : ceil_div(2 * width, tiles);
         return want > most ? most : want;
     };
-    // C (rows from r0) <- (I - V op(T) V^T) C for the merged reflectors of a superblock (kv columns from c0)
-    auto apply = [&](int c0, int kv, const float* T, float* C, int nc, bool transpose_t) -> int {
+    // C (rows from c0) <- (I - V op(T^T) V^T) C for the merged reflectors of a superblock (kv columns from c0)
+    auto apply = [&](int c0, int kv, const float* Tt, float* C, int nc, bool transpose) -> int {
         const int nr = m - c0;
         const int nc8 = (nc + 7) & ~7;
         const float* V = G + (size_t)c0 * ld + c0;
@@ -665,7 +659,7 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
             GELO_TRY(launch_sum_planes(ctx, tc.wf32, plane, used, ld, kv, nc8, loss2, tc.w32[0], ld, st));
         }
         // (the factor loss1 makes up for the truncation of V in the last product)
-        GELO_TRY(launch_gemm_tf32(ctx, kv, nc8, kv, T, kSuper, transpose_t, tc.w32[0], ld, false, tc.w32[1], ld, true, loss1, 1, 0,
+        GELO_TRY(launch_gemm_tf32(ctx, kv, nc8, kv, Tt, kSuper, transpose, tc.w32[0], ld, false, tc.w32[1], ld, true, loss1, 1, 0,
                                   nullptr, st));
         return launch_gemm_tf32(ctx, nr, nc, kv, V, ld, false, tc.w32[1], ld, true, C, ld, false, 1.0f, 1, 0, nullptr, st);
     };
@@ -681,51 +675,44 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
     const int nblocks = (int)start.size() - 1;
     const int per = kSuper / FB;
     // ---- factorisation ----
+    GELO_CUDA_OK(cudaMemsetAsync(tc.tsuper, 0, (size_t)ceil_div(nblocks, per) * kSuper * kSuper * sizeof(float), st));
     for (int s = 0; s < nblocks; s += per) {
         const int e = (s + per < nblocks) ? s + per : nblocks;
         const int s0 = start[s], send = start[e];
-        float* Ts = tc.tsuper + (size_t)(s / per) * kSuper * kSuper;
-        GELO_CUDA_OK(cudaMemsetAsync(Ts, 0, (size_t)kSuper * kSuper * sizeof(float), st));
+        float* Ts = tc.tsuper + (size_t)(s / per) * kSuper * kSuper;     // T^T, lower triangular
         for (int b = s; b < e; ++b) {
             const int b0 = start[b], ob = start[b + 1] - b0, bend = b0 + ob;
             const int nr = m - b0, r = b0 - s0;
-            const int ncs = (send - b0 + 7) & ~7;            // the block and the superblock's columns right of it
+            const int ncs = (send - s0 + 7) & ~7;            // the superblock's columns
             float* P = G + (size_t)b0 * ld + b0;
+            float* rows = G + (size_t)b0 * ld + s0;          // the block's rows of [V_< | P | C]
+            float* Wb = tc.w32[1] + (size_t)(b - s) * FB * ld;
             int used = 0;
             const size_t plane = (size_t)FB * ld;
-            GELO_TRY(launch_gemm_tf32(ctx, ob, ncs, nr, P, ld, true, P, ld, false, tc.wf32, ld, false, 1.0f,
+            GELO_TRY(launch_gemm_tf32(ctx, ob, ncs, nr, P, ld, true, rows, ld, false, tc.wf32, ld, false, 1.0f,
                                       slices(ob, ncs, kMaxKSplit), plane, &used, st));
             const int work = ob * (ncs >> 2) + r * (ob >> 2);
-            block_sum_kernel<<<ceil_div(work, 256), 256, 0, st>>>(tc.wf32, plane, used, ld, ob, ncs, ob, loss2, tc.w32[0], ld,
+            block_sum_kernel<<<ceil_div(work, 256), 256, 0, st>>>(tc.wf32, plane, used, ld, ob, ncs, r, ob, loss2, tc.w32[0], ld,
                                                                  G + (size_t)s0 * ld + b0, r, ld);
             GELO_TRY(after_launch(ctx));
             float* Tb = Ts + (size_t)r * kSuper + r;
             float scale = 1.0f;                              // a power of two with scale^2 about nr
             while (2.0f * scale * scale < (float)nr) scale *= 2.0f;
-            block_factor_kernel<<<kFactCtas, kFactThreads, kFactSmemBytes, st>>>(tc.w32[0], ld, P, ld, ob, Tb, kSuper, tc.t128, FB,
-                                                                        scale, loss1, 1, ctx->status_dev);
+            block_factor_kernel<<<kFactCtas, kFactThreads, kFactSmemBytes, st>>>(tc.w32[0] + r, ld, P, ld, ob, Tb, kSuper, tc.t128, FB,
+                                                                                scale, loss1, ctx->status_dev);
             GELO_TRY(after_launch(ctx));
-            if (send > bend) {
-                // W' = T^T (P^T C) + D^T C1, then C -= V W'
-                const int nc = send - bend, nc8 = (nc + 7) & ~7;
-                GELO_TRY(launch_gemm_tf32_dual(ctx, ob, nc8, ob, Tb, kSuper, tc.w32[0] + ob, ld, tc.t128, FB, P + ob, ld, tc.w32[1], ld,
-                                               loss1, st));
-                GELO_TRY(launch_gemm_tf32(ctx, nr, nc, ob, P, ld, false, tc.w32[1], ld, true, P + ob, ld, false, 1.0f, 1, 0, nullptr,
-                                          st));
+            if (e - s > 1) {
+                // [X^T | . | W'] = T^T Z + D^T [V_< | . | C1], scaled up for the truncation of V in the next product
+                GELO_TRY(launch_gemm_tf32_dual(ctx, ob, ncs, ob, Tb, kSuper, tc.w32[0], ld, tc.t128, FB, rows, ld, Wb, ld, loss1, st));
             }
-            if (r > 0) {
-                // merge into the superblock's factor: T[0:r, r:r+ob] = -T[0:r, 0:r] (V_<^T V_b) T_b
-                const float* Vl = G + (size_t)b0 * ld + s0;
-                GELO_TRY(launch_gemm_tf32(ctx, r, (ob + 7) & ~7, nr, Vl, ld, true, P, ld, false, tc.wf32, FB, false, 1.0f,
-                                          slices(r, ob, kMaxKSplit), (size_t)r * FB, &used, st));
-                GELO_TRY(launch_sum_planes(ctx, tc.wf32, (size_t)r * FB, used, FB, r, ob, loss2, tc.sx, FB, st));
-                GELO_TRY(launch_gemm_tf32(ctx, r, (ob + 7) & ~7, ob, tc.sx, FB, false, Tb, kSuper, false, tc.xb, FB, true, 1.0f, 1, 0,
+            if (send > bend)                                 // C -= V W'
+                GELO_TRY(launch_gemm_tf32(ctx, nr, send - bend, ob, P, ld, false, Wb + (bend - s0), ld, true, P + ob, ld, false, 1.0f, 1, 0,
                                           nullptr, st));
-                GELO_TRY(launch_gemm_tf32(ctx, r, (ob + 7) & ~7, r, Ts, kSuper, false, tc.xb, FB, false, Ts + r, kSuper, true, -1.0f,
-                                          1, 0, nullptr, st));
-            }
+            if (r > 0)                                       // T^T[r:r+ob, 0:r] = -X^T T_<^T
+                GELO_TRY(launch_gemm_tf32(ctx, ob, r, r, Wb, ld, false, Ts, kSuper, false, Ts + (size_t)r * kSuper, kSuper, true,
+                                          -1.0f / loss1, 1, 0, nullptr, st));
         }
-        GELO_TRY(apply(s0, send - s0, Ts, G + (size_t)s0 * ld + send, m - send, true));
+        GELO_TRY(apply(s0, send - s0, Ts, G + (size_t)s0 * ld + send, m - send, false));
     }
     // ---- the square that is left, and Q accumulated backwards, one superblock at a time ----
     GELO_TRY(launch_qr_small(ctx, m - bf, G + (size_t)bf * ld + bf, ld, Q + (size_t)bf * ld + bf, st));
@@ -734,7 +721,7 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
     for (int s = (nblocks - 1) / per * per; s >= 0; s -= per) {
         const int e = (s + per < nblocks) ? s + per : nblocks;
         const int s0 = start[s];
-        GELO_TRY(apply(s0, start[e] - s0, tc.tsuper + (size_t)(s / per) * kSuper * kSuper, Q + (size_t)s0 * ld + s0, m - s0, false));
+        GELO_TRY(apply(s0, start[e] - s0, tc.tsuper + (size_t)(s / per) * kSuper * kSuper, Q + (size_t)s0 * ld + s0, m - s0, true));
     }
     return GELO_OK;
 }
