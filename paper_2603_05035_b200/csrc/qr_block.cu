@@ -664,12 +664,15 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
         return launch_gemm_tf32(ctx, nr, nc, kv, V, ld, false, tc.w32[1], ld, true, C, ld, false, 1.0f, 1, 0, nullptr, st);
     };
 
-    // block columns: 128 wide while at least twice as many rows are left, then one that leaves a square of at most 128
+    // Block columns: 128 wide while at least twice as many rows are left, then narrower ones (half of the rows at most) (multiples of eight) down to a
+    // square of at most 96 rows for the Householder kernel, which takes 45 us for 64 rows, 97 for 96 and 183 for 128, against about
+    // 50 us for a block.
     std::vector<int> start;
     int bf = 0;                                              // first column of the square that is left for Householder
-    while (m - bf > FB) {
+    while (m - bf > 96) {
+        const int left = m - bf;
         start.push_back(bf);
-        bf += (m - bf >= 2 * FB) ? FB : ((m - bf - FB + 3) & ~3);
+        bf += left >= 2 * FB ? FB : (left <= 192 ? (left >> 1) & ~7 : (left - 121) & ~7);
     }
     start.push_back(bf);
     const int nblocks = (int)start.size() - 1;

@@ -23,8 +23,8 @@ def _sample(m, kind, seed, dt):
     return f64(A[:, :m]), f64(X[:, :m])
 
 
-# 256: the first size of the route, one full block and a square of 128; 257: a block of four columns; 383 .. 385: the block
-# before the square is as wide as it gets, full, or four columns again; 513, 641: a second group of blocks begins
+# 256: the first size of the route, blocks of 128 and 64 columns and a square of 64; 257: a square of an odd size; 383 .. 385: three
+# blocks whose middle one is as wide as it gets, full, or full with an odd square; 513, 641: a second group of blocks begins
 @pytest.mark.parametrize("m", [256, 257, 383, 384, 385, 513, 641])
 def test_block_qr_of_a_gaussian(oracle, m):
     a, x = _sample(m, ORTHOGONAL, 900 + m, "f16")
@@ -34,12 +34,14 @@ def test_block_qr_of_a_gaussian(oracle, m):
     d = a.T @ a - np.eye(m)
     assert np.linalg.norm(d) / np.sqrt(m) <= 6e-4
     assert abs(np.trace(d)) / m <= 1e-4
-    # the factor itself: tf32 products err by 2^-11 sqrt(2/3) = 4e-4 per block and the first half of the columns sees at
-    # most m / 256 of them; the last columns are conditioned like the Gaussian itself, so they are only aligned
+    # the factor itself: tf32 products err by 2^-11 sqrt(2/3) = 4e-4 per block.  Four blocks at a time act as one merged reflector,
+    # in which the blocks right of a column cancel only as well as those products do, so a column of the first half
+    # meets the errors of all m / 128 blocks, beside those of its own triangular factor and of Q; the last columns are conditioned like
+    # the Gaussian itself, so they are only aligned
     G64 = oracle.gaussian(900 + m, 0, 0, m, m).astype(np.float32).astype(np.float64)
     q_ref, _ = oracle.householder_qr(G64)
     h = m // 2
-    assert np.linalg.norm(a[:, :h] - q_ref[:, :h]) / np.sqrt(h) <= 4e-4 * (2 + m / 256)
+    assert np.linalg.norm(a[:, :h] - q_ref[:, :h]) / np.sqrt(h) <= 4e-4 * (2 + m / 128)
     assert np.median(np.sum(a * q_ref, axis=0)) > 1 - 1e-4
 
 
