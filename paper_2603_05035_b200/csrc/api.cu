@@ -14,7 +14,14 @@ namespace {
 
 inline cudaStream_t as_stream(void* s) { return static_cast<cudaStream_t>(s); }
 inline int round_up(int x, int to) { return (x + to - 1) / to * to; }
-constexpr int kTcMinRows = 256;   // below this the factorisations are latency-bound anyway
+constexpr int kTcMinRows = 256;   // below this the factorisations are latency-bound anyway, and stay in fp32
+// Up to here fp32 samples (and 16-bit ones of less than kTcMinRows rows) take the block QR in fp32 multiply-adds instead of
+// 32-column Householder panels: orthogonal sample at 512 rows 1.52 -> 0.45 ms, 1075 rows 3.59 -> 1.19 ms, 3000 rows 12.4 -> 9.4 ms.
+constexpr int kExactBlockRows = 3072;
+// And up to here Newton's iteration in fp32 multiply-adds instead of the LU, whose latency its ten products undercut:
+// non-orthogonal sample at 512 rows 3.61 -> 0.70 ms; |A^-1 A - I| / sqrt(m) there 1.1e-5 -> 4e-7.  At 1075 rows alone it is 8.09 -> 2.16 ms,
+// but 32 calls on 16 lanes lose 6%: that much arithmetic on the FMA pipes is no longer hidden.
+constexpr int kExactNewtonRows = 768;
 
 // How a factorisation of an m x m sample stored as `dtype` runs its level-3 updates: 0 = fp32 FMA kernels,
 // 2 = tensor cores with three bf16 products of split operands, 3 = tensor cores with one tf32 product.
@@ -156,17 +163,31 @@ int sample_attempt(gelo_ctx* ctx, const Layout& L, int m, int kind, uint64_t see
     GELO_TRY(launch_gaussian(ctx, m, m, ldi, seed, GELO_STREAM_G0, attempt, 1.0f, nullptr, L.G, st, seed_dev));
     const int l3 = level3_kind(ctx, m, dtype, true);
     // the block route signs its columns itself; the others leave that to the copy (by the diagonal of R, in L.G)
-    const bool blocks = l3 == 3 && gaussian_qr_supports(m);
+    // (fp32 storage and small matrices, l3 = 0: the same in fp32 multiply-adds)
+    const bool exact = ctx->level3 == 0 && l3 == 0 && m <= kExactBlockRows;
+    const bool blocks = (l3 == 3 || exact) && gaussian_qr_supports(m);
     const float* sign = blocks ? nullptr : L.G;
-    if (blocks) GELO_TRY(run_gaussian_qr(ctx, m, L.G, ldi, L.Qraw, L.tc, st));
+    if (blocks) GELO_TRY(run_gaussian_qr(ctx, m, L.G, ldi, L.Qraw, L.tc, exact, st));
     else if (l3 == 3) GELO_TRY(run_householder_qr_tf32(ctx, m, L.G, ldi, L.Qraw, L.qr, L.tc, st));
     else if (l3) GELO_TRY(run_householder_qr_tc(ctx, m, L.G, ldi, L.Qraw, L.qr, L.tc, st));
     else GELO_TRY(run_householder_qr(ctx, m, L.G, ldi, L.Qraw, L.qr, st));
     if (kind == GELO_ORTHOGONAL) {
         // tf32 updates: polish Q (A32 and X32 are free for this kind).  The non-orthogonal kind skips it: there Q0 only
         // has to keep A = Q0 + gamma G1 well conditioned, and A^-1 comes from the LU of the stored A.
+        const float* Q = L.Qraw;
         if (l3 == 3) GELO_TRY(polish_orthogonal_tf32(ctx, m, L.Qraw, ldi, L.X32, L.A32, st));
-        GELO_TRY(launch_finish_mixing(ctx, m, L.Qraw, ldi, sign, ldi, dtype, A_out, Ainv_out, lda, st));
+        if (blocks && exact) {
+            // the same step in fp32, from the 4e-6 that the Gram matrices leave: Q (3 I - Q^T Q) / 2
+            GemmArgs g;
+            g.M = m; g.N = m; g.K = m;
+            g.A = L.Qraw; g.lda = ldi; g.transA = true; g.B = L.Qraw; g.ldb = ldi;
+            g.C[0] = L.X32; g.ldc = ldi; g.alpha = -0.5f; g.diag = 1.5f;
+            GELO_TRY(launch_gemm_simt(ctx, g, st));
+            g.transA = false; g.B = L.X32; g.C[0] = L.A32; g.alpha = 1.0f; g.diag = 0.0f;
+            GELO_TRY(launch_gemm_simt(ctx, g, st));
+            Q = L.A32;
+        }
+        GELO_TRY(launch_finish_mixing(ctx, m, Q, ldi, sign, ldi, dtype, A_out, Ainv_out, lda, st));
         if (cond_dev) {
             set_scalar_kernel<<<1, 1, 0, st>>>(cond_dev, 1.0f);
             GELO_TRY(after_launch(ctx));
@@ -186,6 +207,15 @@ int sample_attempt(gelo_ctx* ctx, const Layout& L, int m, int kind, uint64_t see
         GELO_TRY(launch_gaussian(ctx, m, m, ldi, seed, GELO_STREAM_G1, attempt, s, Q0, L.A32, st, seed_dev));
         GELO_TRY(launch_narrow(ctx, m, L.A32, ldi, dtype, A_out, lda, st));
         GELO_TRY(run_newton_inverse(ctx, m, dtype, A_out, lda, g16, g16 + half, x16, ldi, Ainv_out, lda, st));
+    } else if (blocks && exact && m <= kExactNewtonRows && ctx->gamma <= 0.55f) {
+        // in fp32 from the stored A, and rounded once
+        GELO_TRY(launch_finish_mixing(ctx, m, Q0, ldi, nullptr, ldi, GELO_F32, L.X32, L.G, ldi, st));
+        GELO_TRY(launch_gaussian(ctx, m, m, ldi, seed, GELO_STREAM_G1, attempt, s, Q0, L.A32, st, seed_dev));
+        GELO_TRY(launch_narrow(ctx, m, L.A32, ldi, dtype, A_out, lda, st, dtype != GELO_F32 ? L.A32 : nullptr, ldi));
+        const bool direct = dtype == GELO_F32;
+        GELO_TRY(run_newton_inverse_f32(ctx, m, L.A32, ldi, L.G, L.X32, L.lu.M, ldi, direct ? static_cast<float*>(Ainv_out) : L.Qraw,
+                                        direct ? lda : ldi, st));
+        if (!direct) GELO_TRY(launch_narrow(ctx, m, L.Qraw, ldi, dtype, Ainv_out, lda, st));
     } else {
         GELO_TRY(launch_gaussian(ctx, m, m, ldi, seed, GELO_STREAM_G1, attempt, s, Q0, L.A32, st, seed_dev));
         // the inverse is that of the stored A: round, and carry on from the rounded values

@@ -146,6 +146,8 @@ struct GemmArgs {
     void* C[3] = {nullptr, nullptr, nullptr}; int ldc = 0;       // column block c / (N / nsplit) selects C[...]
     int nsplit = 1;
     float alpha = 1.0f, beta = 0.0f;
+    float diag = 0.0f;                                           // FMA kernel: added to the diagonal entries
+    int ksplit = 1; size_t plane = 0;                            // FMA kernel: K slices, written to consecutive planes of C (stride in elements)
     int dtype = GELO_F32;                                        // storage type of A, B and C
 };
 int launch_gemm_simt(gelo_ctx*, const GemmArgs&, cudaStream_t);
@@ -270,11 +272,11 @@ int run_householder_qr_tc(gelo_ctx*, int m, float* R, int ld, float* Q, const Qr
 // applied to the columns right of the group and, later, to Q, so the big matrices stream through the GPU once per
 // 512 columns instead of once per 128.
 int run_householder_qr_tf32(gelo_ctx*, int m, float* R, int ld, float* Q, const QrScratch&, const TcScratch&, cudaStream_t);
-// The orthogonal factor of a GAUSSIAN matrix on tf32 products, blocks factorised through their Gram matrices
-// (qr_block.cu; relies on the blocks being well conditioned).  G is overwritten with the reflectors; Q receives the
-// factor whose R has a positive diagonal.
+// The orthogonal factor of a GAUSSIAN matrix, blocks factorised through their Gram matrices (qr_block.cu; relies on the
+// blocks being well conditioned), on tf32 products or (exact) on fp32 multiply-adds.  G is overwritten with the reflectors; Q
+// receives the factor whose R has a positive diagonal.
 bool gaussian_qr_supports(int m);
-int run_gaussian_qr(gelo_ctx*, int m, float* G, int ld, float* Q, const TcScratch&, cudaStream_t);
+int run_gaussian_qr(gelo_ctx*, int m, float* G, int ld, float* Q, const TcScratch&, bool exact, cudaStream_t);
 // One Newton-Schulz step Q <- Q - Q (Q^T Q - I) / 2 on the tensor cores in tf32: squares the orthogonality defect
 // that tf32 updates leave in Q.  D and Qold are m x ld scratch matrices.
 int polish_orthogonal_tf32(gelo_ctx*, int m, float* Q, int ld, float* D, float* Qold, cudaStream_t);
@@ -296,6 +298,9 @@ int run_lu_inverse_tc(gelo_ctx*, int m, const float* A, int ld, float* Ainv, con
 bool newton_inverse_supports(int m, int dtype, float gamma);
 int run_newton_inverse(gelo_ctx*, int m, int dtype, const void* A, int lda, void* X0, void* X1, void* Y, int ld, void* Ainv, int ldi,
                        cudaStream_t);
+// the same in fp32 on multiply-adds
+int run_newton_inverse_f32(gelo_ctx*, int m, const float* A, int lda, float* X0, float* X1, float* Y, int ld, float* Ainv, int ldi,
+                           cudaStream_t);
 
 struct CondScratch {
     float* vec = nullptr;     // iterate, image and row-slab partial sums for both operators
@@ -327,9 +332,9 @@ int launch_split_pair(gelo_ctx*, const float* A, int lda, int rows_a, int cols_a
 
 int launch_sum_split(gelo_ctx*, const float* planes, size_t plane, int parts, int ld, int rows, int cols, void* hi,
                      void* lo, int ldo, cudaStream_t);
-// out = scale * (sum of `parts` fp32 planes in plane order), rounded to tf32 (cols a multiple of 4)
+// out = scale * (sum of `parts` fp32 planes in plane order), rounded to tf32 unless round is false (cols a multiple of 4)
 int launch_sum_planes(gelo_ctx*, const float* planes, size_t plane, int parts, int ld, int rows, int cols, float scale,
-                      float* out, int ldo, cudaStream_t);
+                      float* out, int ldo, cudaStream_t, bool round = true);
 
 // Scratch of the tensor-core level-3 updates (outer blocks of kOuter columns).
 constexpr int kOuter = 128;

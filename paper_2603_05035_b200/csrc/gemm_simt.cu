@@ -3,6 +3,8 @@
 // (Eq. 1-3) and the workhorse of the trailing updates in the blocked QR and LU.
 // The B operand may be the vertical stack of two matrices (Eq. 8: H_full = [H; S])
 // and the output may be split into column thirds (Q | K | V).
+//
+// Two kernels: gemm_f32_kernel for fp32 matrices with 16-byte rows, gemm_simt_kernel for everything else.
 #include "common.cuh"
 
 namespace gelo {
@@ -18,7 +20,8 @@ struct GemmParams {
     const void* B; int ldb;
     const void* B2; int b_split;
     void* C0; void* C1; void* C2; int ldc; int csplit;
-    float alpha, beta;
+    float alpha, beta, diag;
+    int kper; size_t plane;                                  // K slice blockIdx.z covers [z kper, z kper + kper) and writes plane z
 };
 
 __device__ __forceinline__ float ldf(const float* p) { return __ldg(p); }
@@ -98,11 +101,12 @@ __global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmParams pr
         }
     };
 
-    fetch(0);
-    for (int k0 = 0; k0 < prm.K; k0 += BK) {
+    const int k_lo = blockIdx.z * prm.kper, k_hi = min(prm.K, k_lo + prm.kper);
+    fetch(k_lo);
+    for (int k0 = k_lo; k0 < k_hi; k0 += BK) {
         stash();
         __syncthreads();
-        if (k0 + BK < prm.K) fetch(k0 + BK);
+        if (k0 + BK < k_hi) fetch(k0 + BK);
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
             float a[RM * 4], b[RN * 4];
@@ -134,22 +138,180 @@ __global__ void __launch_bounds__(kThreads) gemm_simt_kernel(const GemmParams pr
             const int gn = n0 + tx * 4 + (j >> 2) * 64 + (j & 3);
             if (gn >= prm.N) continue;
             const int chunk = gn / prm.csplit;
-            T* p = Cs[chunk] + (size_t)gm * prm.ldc + (gn - chunk * prm.csplit);
-            float v = prm.alpha * acc[i][j];
+            T* p = Cs[chunk] + blockIdx.z * prm.plane + (size_t)gm * prm.ldc + (gn - chunk * prm.csplit);
+            float v = prm.alpha * acc[i][j] + (gm == gn ? prm.diag : 0.0f);
             if (prm.beta != 0.0f) v += prm.beta * ldc(p);
             stf(p, v);
         }
     }
 }
 
+// ---- fp32, 64 x kN tiles, the k range of a stage shared out to four groups of threads ---------------------------
+//
+// A warp's 16-byte read of shared memory takes four cycles whatever it broadcasts, so what counts is values read per multiply-add:
+// 8 x 8 entries per thread read a value per four multiply-adds, which balances the two pipes, 4 x 4 entries twice that.  A
+// 64 x 64 tile then has only 64 threads; four such groups take 16 of the 64 k of a stage each and their sums are added at the end
+// (in order), which also shortens the chain of a product with a deep K and few tiles.  32 columns per tile where 64 would leave SMs idle.
+// 512 x 512 x 512: 39 us with 4 x 4 entries per thread and single-word loads, 15 us.
+constexpr int kF32K = 64;                      // k of a stage
+constexpr int kF32M = 64;
+
+template <int kN>
+struct F32Shared {
+    float A[2][kF32K][kF32M + 4];
+    float B[2][kF32K][kN + 4];
+};
+
+template <bool TA, int kN>
+__global__ void __launch_bounds__(kThreads) gemm_f32_kernel(const GemmParams prm)
+{
+    constexpr int kC = kN / 32;                // column quads per thread
+    extern __shared__ __align__(16) uint8_t f32_smem[];
+    F32Shared<kN>& s = *reinterpret_cast<F32Shared<kN>*>(f32_smem);
+    const float* __restrict__ A = static_cast<const float*>(prm.A);
+    const float* __restrict__ B = static_cast<const float*>(prm.B);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int group = tid >> 6, ty = (tid & 63) >> 3, tx = tid & 7;
+    const int m0 = blockIdx.y * kF32M, n0 = blockIdx.x * kN;
+    const int k_lo = blockIdx.z * prm.kper, k_hi = min(prm.K, k_lo + prm.kper);
+
+    float4 ra[4], rb[2 * kC];
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            ra[i] = zero;
+            if (TA) {                          // 16 quads of columns, 16 rows of k at a time
+                const int k = k0 + 16 * i + (tid >> 4), c = m0 + 4 * (tid & 15);
+                if (k < k_hi && c < prm.M) ra[i] = *reinterpret_cast<const float4*>(A + (size_t)k * prm.lda + c);
+            } else {                           // a row per lane, so that the transposed stores fall into different banks
+                const int k = k0 + 16 * i + 4 * (warp >> 1), r = m0 + 32 * (warp & 1) + lane;
+                if (k < k_hi && r < prm.M) {
+                    ra[i] = *reinterpret_cast<const float4*>(A + (size_t)r * prm.lda + k);
+                    if (k + 1 >= k_hi) ra[i].y = 0.0f;
+                    if (k + 2 >= k_hi) ra[i].z = 0.0f;
+                    if (k + 3 >= k_hi) ra[i].w = 0.0f;
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 2 * kC; ++i) {
+            const int idx = tid + kThreads * i, k = k0 + idx / (kN / 4), c = n0 + 4 * (idx % (kN / 4));
+            rb[i] = (k < k_hi && c < prm.N) ? *reinterpret_cast<const float4*>(B + (size_t)k * prm.ldb + c) : zero;
+        }
+    };
+    auto stash = [&](int b) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (TA) {
+                *reinterpret_cast<float4*>(&s.A[b][16 * i + (tid >> 4)][4 * (tid & 15)]) = ra[i];
+            } else {
+                const int k = 16 * i + 4 * (warp >> 1), r = 32 * (warp & 1) + lane;
+                s.A[b][k][r] = ra[i].x; s.A[b][k + 1][r] = ra[i].y; s.A[b][k + 2][r] = ra[i].z; s.A[b][k + 3][r] = ra[i].w;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 2 * kC; ++i) {
+            const int idx = tid + kThreads * i;
+            *reinterpret_cast<float4*>(&s.B[b][idx / (kN / 4)][4 * (idx % (kN / 4))]) = rb[i];
+        }
+    };
+
+    float acc[8][4 * kC];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4 * kC; ++j) acc[i][j] = 0.0f;
+
+    fetch(k_lo);
+    stash(0);
+    __syncthreads();
+    int b = 0;
+    for (int k0 = k_lo; k0 < k_hi; k0 += kF32K, b ^= 1) {
+        const bool more = k0 + kF32K < k_hi;
+        if (more) fetch(k0 + kF32K);
+#pragma unroll
+        for (int kk = 0; kk < 16; ++kk) {
+            const int k = 16 * group + kk;
+            float x[8], y[4 * kC];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float4 v = *reinterpret_cast<const float4*>(&s.A[b][k][32 * h + 4 * ty]);
+                x[4 * h] = v.x; x[4 * h + 1] = v.y; x[4 * h + 2] = v.z; x[4 * h + 3] = v.w;
+            }
+#pragma unroll
+            for (int h = 0; h < kC; ++h) {
+                const float4 v = *reinterpret_cast<const float4*>(&s.B[b][k][32 * h + 4 * tx]);
+                y[4 * h] = v.x; y[4 * h + 1] = v.y; y[4 * h + 2] = v.z; y[4 * h + 3] = v.w;
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < 4 * kC; ++j) acc[i][j] = fmaf(x[i], y[j], acc[i][j]);
+        }
+        if (more) stash(b ^ 1);
+        __syncthreads();
+    }
+
+    // ---- the four groups' sums, tile by tile in shared memory; then 256 threads add and store quads of columns ----
+    float* const sum = &s.A[0][0][0];          // 4 tiles of 64 x kN (the operands have been read)
+    static_assert(sizeof(F32Shared<kN>) >= 4 * kF32M * kN * sizeof(float), "the sums fit where the operands were");
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int h = 0; h < kC; ++h)
+            *reinterpret_cast<float4*>(sum + (group * kF32M + 32 * (i >> 2) + 4 * ty + (i & 3)) * kN + 32 * h + 4 * tx) =
+                make_float4(acc[i][4 * h], acc[i][4 * h + 1], acc[i][4 * h + 2], acc[i][4 * h + 3]);
+    __syncthreads();
+    float* const Cs[3] = { static_cast<float*>(prm.C0), static_cast<float*>(prm.C1), static_cast<float*>(prm.C2) };
+    for (int idx = tid; idx < kF32M * kN / 4; idx += kThreads) {
+        const int r = idx / (kN / 4), c = 4 * (idx % (kN / 4)), gm = m0 + r, gn = n0 + c;
+        if (gm >= prm.M || gn >= prm.N) continue;
+        float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 t = *reinterpret_cast<const float4*>(sum + (q * kF32M + r) * kN + c);
+            v[0] += t.x; v[1] += t.y; v[2] += t.z; v[3] += t.w;
+        }
+        const int part = gn / prm.csplit;      // (a multiple of four)
+        float* p = Cs[part] + blockIdx.z * prm.plane + (size_t)gm * prm.ldc + (gn - part * prm.csplit);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            v[j] = prm.alpha * v[j] + (gm == gn + j ? prm.diag : 0.0f);
+            if (prm.beta != 0.0f && gn + j < prm.N) v[j] += prm.beta * p[j];
+        }
+        if (gn + 3 < prm.N) {
+            *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (gn + j < prm.N) p[j] = v[j];
+        }
+    }
+}
+
+template <bool TA, int kN>
+int launch_f32(gelo_ctx* ctx, const GemmParams& p, int slices, cudaStream_t st)
+{
+    static bool attr_done[64] = {};
+    if (ctx->device >= 0 && ctx->device < 64 && !attr_done[ctx->device]) {
+        GELO_CUDA_OK(cudaFuncSetAttribute(gemm_f32_kernel<TA, kN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(F32Shared<kN>)));
+        attr_done[ctx->device] = true;
+    }
+    gemm_f32_kernel<TA, kN><<<dim3(ceil_div(p.N, kN), ceil_div(p.M, kF32M), slices), kThreads, sizeof(F32Shared<kN>), st>>>(p);
+    return after_launch(ctx);
+}
+
+bool aligned_rows(const void* p, int ld) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (ld % 4) == 0; }
+
 template <typename T, bool TA, bool TB>
-void launch_tiles(const GemmParams& p, bool small, cudaStream_t st)
+void launch_tiles(const GemmParams& p, bool small, int slices, cudaStream_t st)
 {
     if (small) {
-        dim3 grid(ceil_div(p.N, 64), ceil_div(p.M, 64));
+        dim3 grid(ceil_div(p.N, 64), ceil_div(p.M, 64), slices);
         gemm_simt_kernel<T, TA, TB, 64, 64><<<grid, kThreads, 0, st>>>(p);
     } else {
-        dim3 grid(ceil_div(p.N, 128), ceil_div(p.M, 128));
+        dim3 grid(ceil_div(p.N, 128), ceil_div(p.M, 128), slices);
         gemm_simt_kernel<T, TA, TB, 128, 128><<<grid, kThreads, 0, st>>>(p);
     }
 }
@@ -162,6 +324,7 @@ int launch_gemm_simt(gelo_ctx* ctx, const GemmArgs& g, cudaStream_t st)
     if (g.K < 0 || !g.A || !g.B || !g.C[0] || g.nsplit < 1 || g.nsplit > 3 || g.N % g.nsplit != 0)
         return GELO_ERR_INVALID;
     if (g.B2 && g.transB) return GELO_ERR_INVALID;
+    if (g.ksplit < 1 || (g.ksplit > 1 && (g.beta != 0.0f || g.nsplit != 1))) return GELO_ERR_INVALID;
     for (int i = 0; i < g.nsplit; ++i)
         if (!g.C[i]) return GELO_ERR_INVALID;
     GemmParams p;
@@ -170,20 +333,30 @@ int launch_gemm_simt(gelo_ctx* ctx, const GemmArgs& g, cudaStream_t st)
     p.B2 = g.B2 ? g.B2 : g.B; p.b_split = g.B2 ? g.b_split : g.K;
     p.C0 = g.C[0]; p.C1 = g.C[g.nsplit > 1 ? 1 : 0]; p.C2 = g.C[g.nsplit > 2 ? 2 : 0];
     p.ldc = g.ldc; p.csplit = g.N / g.nsplit;
-    p.alpha = g.alpha; p.beta = g.beta;
-    const long tiles128 = (long)ceil_div(g.M, 128) * ceil_div(g.N, 128);
+    p.alpha = g.alpha; p.beta = g.beta; p.diag = g.diag;
+    p.kper = ceil_div(ceil_div(g.K, g.ksplit), BK) * BK;      // (the caller's slices: whole steps, none of them empty)
+    p.plane = g.plane;
+    const int slices = g.ksplit;
+    if (g.dtype == GELO_F32 && !g.transB && !g.B2 && aligned_rows(g.A, g.lda) && aligned_rows(g.B, g.ldb) && aligned_rows(g.C[0], g.ldc) &&
+        (g.nsplit == 1 || (p.csplit % 4 == 0 && aligned_rows(p.C1, g.ldc) && aligned_rows(p.C2, g.ldc))) && g.plane % 4 == 0) {
+        // rows of A and B are read in whole quads: the last one of a row may reach past its end, but not past its stride
+        const bool wide = (long)ceil_div(g.N, 64) * ceil_div(g.M, kF32M) * slices >= ctx->sm_count;
+        if (g.transA) return wide ? launch_f32<true, 64>(ctx, p, slices, st) : launch_f32<true, 32>(ctx, p, slices, st);
+        return wide ? launch_f32<false, 64>(ctx, p, slices, st) : launch_f32<false, 32>(ctx, p, slices, st);
+    }
+    const long tiles128 = (long)ceil_div(g.M, 128) * ceil_div(g.N, 128) * slices;
     const bool small = g.M <= 64 || g.N <= 64 || tiles128 < 2L * ctx->sm_count;
     if (g.dtype == GELO_BF16) {
         if (g.transA || g.transB) return GELO_ERR_UNSUPPORTED;
-        launch_tiles<__nv_bfloat16, false, false>(p, small, st);
+        launch_tiles<__nv_bfloat16, false, false>(p, small, slices, st);
     } else if (g.dtype == GELO_F16) {
         if (g.transA || g.transB) return GELO_ERR_UNSUPPORTED;
-        launch_tiles<__half, false, false>(p, small, st);
+        launch_tiles<__half, false, false>(p, small, slices, st);
     } else {
-        if (!g.transA && !g.transB) launch_tiles<float, false, false>(p, small, st);
-        else if (g.transA && !g.transB) launch_tiles<float, true, false>(p, small, st);
-        else if (!g.transA && g.transB) launch_tiles<float, false, true>(p, small, st);
-        else launch_tiles<float, true, true>(p, small, st);
+        if (!g.transA && !g.transB) launch_tiles<float, false, false>(p, small, slices, st);
+        else if (g.transA && !g.transB) launch_tiles<float, true, false>(p, small, slices, st);
+        else if (!g.transA && g.transB) launch_tiles<float, false, true>(p, small, slices, st);
+        else launch_tiles<float, true, true>(p, small, slices, st);
     }
     return after_launch(ctx);
 }

@@ -19,7 +19,7 @@
 namespace gelo {
 
 // gamma: beyond 0.55 the fourth step no longer reaches 1e-4 (0.55^16 = 7e-5), and from 1 on the iteration diverges.
-// m: below 256 the eigenvalues scatter around the disc by more than a tenth of its radius, and the fp32 routes take those.
+// m: smaller matrices take the fp32 iteration.
 bool newton_inverse_supports(int m, int dtype, float gamma) { return dtype != GELO_F32 && m >= 256 && gamma <= 0.55f; }
 
 int run_newton_inverse(gelo_ctx* ctx, int m, int dtype, const void* A, int lda, void* X0, void* X1, void* Y, int ld, void* Ainv, int ldi,
@@ -33,6 +33,26 @@ int run_newton_inverse(gelo_ctx* ctx, int m, int dtype, const void* A, int lda, 
     }
     GELO_TRY(launch_gemm_affine16(ctx, dtype, m, m8, m, A, lda, X0, ld, -1.0f, 1.0f, nullptr, 0, Y, ld, st));
     return launch_gemm_affine16(ctx, dtype, m, m8, m, X0, ld, Y, ld, 1.0f, 0.0f, X0, ld, Ainv, ldi, st);
+}
+
+// fp32: five steps (gamma^32 = 2e-10) of products on the FMA pipes.
+int run_newton_inverse_f32(gelo_ctx* ctx, int m, const float* A, int lda, float* X0, float* X1, float* Y, int ld, float* Ainv, int ldi,
+                           cudaStream_t st)
+{
+    auto product = [&](const float* a, int la, const float* b, int lb, float alpha, float diag, float* c, int lc) -> int {
+        GemmArgs g;
+        g.M = m; g.N = m; g.K = m;
+        g.A = a; g.lda = la; g.B = b; g.ldb = lb;
+        g.C[0] = c; g.ldc = lc; g.alpha = alpha; g.diag = diag;
+        return launch_gemm_simt(ctx, g, st);
+    };
+    for (int step = 0; step < 5; ++step) {
+        GELO_TRY(product(A, lda, X0, ld, -1.0f, 2.0f, Y, ld));
+        if (step == 4) return product(X0, ld, Y, ld, 1.0f, 0.0f, Ainv, ldi);
+        GELO_TRY(product(X0, ld, Y, ld, 1.0f, 0.0f, X1, ld));
+        float* t = X0; X0 = X1; X1 = t;
+    }
+    return GELO_OK;
 }
 
 }  // namespace gelo

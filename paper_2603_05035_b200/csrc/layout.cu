@@ -155,11 +155,11 @@ __global__ void __launch_bounds__(256) sum_split_kernel(const float* __restrict_
     *reinterpret_cast<uint2*>(lo + (size_t)r * ldo + c4) = *reinterpret_cast<const uint2*>(l);
 }
 
-// Sum of `parts` fp32 planes (fixed order), rounded to tf32: the second half of a split-K tf32 product whose
+// Sum of `parts` fp32 planes (fixed order), rounded to tf32 if `round`: the second half of a split-K tf32 product whose
 // result feeds the next tf32 product.
 __global__ void __launch_bounds__(256) sum_planes_kernel(const float* __restrict__ planes, size_t plane, int parts,
                                                          int ld, int rows, int cols, float scale, float* __restrict__ out,
-                                                         int ldo)
+                                                         int ldo, int round)
 {
     const int c4 = (blockIdx.x * 256 + threadIdx.x) * 4;
     const int r = blockIdx.y;
@@ -168,6 +168,10 @@ __global__ void __launch_bounds__(256) sum_planes_kernel(const float* __restrict
     for (int q = 0; q < parts; ++q) {
         const float4 t = *reinterpret_cast<const float4*>(planes + q * plane + (size_t)r * ld + c4);
         acc.x += t.x; acc.y += t.y; acc.z += t.z; acc.w += t.w;
+    }
+    if (!round) {
+        *reinterpret_cast<float4*>(out + (size_t)r * ldo + c4) = make_float4(scale * acc.x, scale * acc.y, scale * acc.z, scale * acc.w);
+        return;
     }
     uint32_t o[4];
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(o[0]) : "f"(scale * acc.x));
@@ -363,11 +367,11 @@ int launch_split_tf32(gelo_ctx* ctx, const float* src, int lds, int rows, int co
 }
 
 int launch_sum_planes(gelo_ctx* ctx, const float* planes, size_t plane, int parts, int ld, int rows, int cols, float scale,
-                      float* out, int ldo, cudaStream_t st)
+                      float* out, int ldo, cudaStream_t st, bool round)
 {
     if (rows <= 0 || cols <= 0) return GELO_OK;
     dim3 grid(ceil_div(cols, 1024), rows);
-    sum_planes_kernel<<<grid, 256, 0, st>>>(planes, plane, parts, ld, rows, cols, scale, out, ldo);
+    sum_planes_kernel<<<grid, 256, 0, st>>>(planes, plane, parts, ld, rows, cols, scale, out, ldo, round ? 1 : 0);
     return after_launch(ctx);
 }
 

@@ -18,9 +18,11 @@
 // it was five dependent launches, 50 us per block).
 // The last block, which would be square, is factorised by the one-launch Householder kernel.
 //
+// The products run in tf32 or, for fp32 storage and small matrices (`exact`), on the FMA pipes.
+//
 // Against 32-column Householder panels in registers (70 us per 32 columns of serial column steps, and rank-32 updates
-// between them), which the sampler used before: 2048 + 102 rows, orthogonal, calls back to back 2.80 -> 1.21 ms; the 32-layer
-// sweep at 4300 rows 126 -> 114 ms.
+// between them), which the sampler used before: 2048 + 102 rows, orthogonal, one call alone 8.9 -> 1.8 ms; 512 rows in fp32, the sample
+// 1.52 -> 0.45 ms.
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -478,12 +480,12 @@ __device__ __forceinline__ void fact_pivots(FactShared& s, int* status)
 }
 
 // Z (ob x ob, stride ldz): the Gram matrix P^T P.  P1: the first ob rows of the panel (stride ld), overwritten
-// with B = P1 + R.  Tt (stride ldt) = T^T = B^-1 R^-T and Dt (stride ldd) = dscale * B^-1, both rounded to tf32.
+// with B = P1 + R.  Tt (stride ldt) = T^T = B^-1 R^-T and Dt (stride ldd) = dscale * B^-1, both rounded to tf32 if `round`.
 // ob <= 128, a multiple of 4; the kernel works on 128 x 128 with an identity in the part past ob.  `scale` is a power of
 // two close to the norm of a panel column.
 __global__ void __cluster_dims__(kFactCtas, 1, 1) __launch_bounds__(kFactThreads, 1)
 block_factor_kernel(const float* __restrict__ Z, int ldz, float* P1, int ld, int ob, float* __restrict__ Tt,
-                    int ldt, float* __restrict__ Dt, int ldd, float scale, float dscale, int* __restrict__ status)
+                    int ldt, float* __restrict__ Dt, int ldd, float scale, float dscale, int round, int* __restrict__ status)
 {
     extern __shared__ __align__(128) uint8_t fsm[];
     FactShared& s = *reinterpret_cast<FactShared*>(fsm);
@@ -555,6 +557,7 @@ block_factor_kernel(const float* __restrict__ Z, int ldz, float* P1, int ld, int
         float* dst = role == FACT_INVERSE ? Dt : Tt;
         const int ldo = role == FACT_INVERSE ? ldd : ldt;
         const float f = role == FACT_INVERSE ? dscale * s1 : s2;
+        auto out_val = [&](float v) { return round ? tcx::round_tf32(f * v) : f * v; };
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
@@ -563,8 +566,7 @@ block_factor_kernel(const float* __restrict__ Z, int ldz, float* P1, int ld, int
                 for (int i = 0; i < 2; ++i) {
                     const int r = 32 * wr + 16 * mt + gid + 8 * i, c = 64 * wc + 8 * nt + 2 * tig;
                     if (r < ob && c < ob)
-                        *reinterpret_cast<float2*>(dst + (size_t)r * ldo + c) =
-                            make_float2(tcx::round_tf32(f * a[mt][nt][2 * i]), tcx::round_tf32(f * a[mt][nt][2 * i + 1]));
+                        *reinterpret_cast<float2*>(dst + (size_t)r * ldo + c) = make_float2(out_val(a[mt][nt][2 * i]), out_val(a[mt][nt][2 * i + 1]));
                 }
     }
     __syncwarp();
@@ -572,10 +574,10 @@ block_factor_kernel(const float* __restrict__ Z, int ldz, float* P1, int ld, int
 }
 
 // Z = scale * (sum of the K slices of P^T [V_< | P | C]), in slice order; columns c0 .. c0 + ob - 1 (the Gram matrix) stay
-// fp32, the others are rounded to tf32 (they feed the next product).  Also clears the rows above the block (z_rows x ob)
+// fp32, the others are rounded to tf32 if `round` (they feed the next product).  Also clears the rows above the block (z_rows x ob)
 // where the superblock's reflectors are zero.
 __global__ void __launch_bounds__(256)
-block_sum_kernel(const float* __restrict__ planes, size_t plane, int parts, int ldp, int rows, int cols, int c0, int ob, float scale,
+block_sum_kernel(const float* __restrict__ planes, size_t plane, int parts, int ldp, int rows, int cols, int c0, int ob, float scale, int round,
                  float* __restrict__ Z, int ldz, float* __restrict__ zero, int z_rows, int ld)
 {
     const int idx = blockIdx.x * 256 + threadIdx.x;
@@ -589,7 +591,7 @@ block_sum_kernel(const float* __restrict__ planes, size_t plane, int parts, int 
             acc.x += t.x; acc.y += t.y; acc.z += t.z; acc.w += t.w;
         }
         acc.x *= scale; acc.y *= scale; acc.z *= scale; acc.w *= scale;
-        if (c < c0 || c >= c0 + ob) {
+        if (round && (c < c0 || c >= c0 + ob)) {
             acc.x = tcx::round_tf32(acc.x); acc.y = tcx::round_tf32(acc.y);
             acc.z = tcx::round_tf32(acc.z); acc.w = tcx::round_tf32(acc.w);
         }
@@ -628,21 +630,40 @@ start_q_kernel(float* __restrict__ Q, int ld, int m, int bf, const float* __rest
 
 bool gaussian_qr_supports(int m) { return m > FB; }
 
-int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcScratch& tc, cudaStream_t st)
+int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcScratch& tc, bool exact, cudaStream_t st)
 {
     static bool attr_done[64] = {};
     if (ctx->device >= 0 && ctx->device < 64 && !attr_done[ctx->device]) {
         GELO_CUDA_OK(cudaFuncSetAttribute(block_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFactSmemBytes));
         attr_done[ctx->device] = true;
     }
-    const float loss1 = 1.0f + kTf32TruncLoss, loss2 = loss1 * loss1;
+    const float loss1 = exact ? 1.0f : 1.0f + kTf32TruncLoss, loss2 = loss1 * loss1;
     const int width = ctx->tc_update_ctas > 0 ? ctx->tc_update_ctas : ctx->sm_count;   // CTAs one launch may use
+    const int round = exact ? 0 : 1;
 
     // V^T C with few output tiles: the rows are cut into slices whose partial products are summed in a fixed order
     auto slices = [&](int M, int N, int most) {
-        const int tiles = ceil_div(M, 128) * ceil_div(N, 256);
+        const int tiles = exact ? ceil_div(M, 64) * ceil_div(N, 64) : ceil_div(M, 128) * ceil_div(N, 256);
         int want = (2 * tiles >= width) ? 1 : ceil_div(2 * width, tiles);
         return want > most ? most : want;
+    };
+    // C = scale * op(A) B or C -= op(A) B, as launch_gemm_tf32 or in fp32
+    auto gemm = [&](int M, int N, int K, const float* A, int lda, bool a_mn, const float* B, int ldb, bool subtract, float* C, int ldc,
+                    bool round_out, float scale, int ksplit, size_t plane, int* used) -> int {
+        if (!exact) return launch_gemm_tf32(ctx, M, N, K, A, lda, a_mn, B, ldb, subtract, C, ldc, round_out, scale, ksplit, plane, used, st);
+        if (M <= 0 || N <= 0 || K <= 0) return GELO_OK;
+        GemmArgs g;
+        g.M = M; g.N = N; g.K = K;
+        g.A = A; g.lda = lda; g.transA = a_mn; g.B = B; g.ldb = ldb;
+        g.C[0] = C; g.ldc = ldc;
+        g.alpha = subtract ? -1.0f : scale; g.beta = subtract ? 1.0f : 0.0f;
+        if (ksplit > 1) {
+            const int steps = ceil_div(K, 16), per = ceil_div(steps, ksplit < steps ? ksplit : steps);
+            g.ksplit = ceil_div(steps, per);       // no empty slice
+            g.plane = plane;
+        }
+        if (used) *used = g.ksplit;
+        return launch_gemm_simt(ctx, g, st);
     };
     // C (rows from c0) <- (I - V op(T^T) V^T) C for the merged reflectors of a superblock (kv columns from c0)
     auto apply = [&](int c0, int kv, const float* Tt, float* C, int nc, bool transpose) -> int {
@@ -651,17 +672,16 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
         const float* V = G + (size_t)c0 * ld + c0;
         const int want = slices(kv, nc8, kSuperKSplit);
         if (want <= 1) {
-            GELO_TRY(launch_gemm_tf32(ctx, kv, nc8, nr, V, ld, true, C, ld, false, tc.w32[0], ld, true, loss2, 1, 0, nullptr, st));
+            GELO_TRY(gemm(kv, nc8, nr, V, ld, true, C, ld, false, tc.w32[0], ld, true, loss2, 1, 0, nullptr));
         } else {
             int used = 0;
             const size_t plane = (size_t)kv * ld;
-            GELO_TRY(launch_gemm_tf32(ctx, kv, nc8, nr, V, ld, true, C, ld, false, tc.wf32, ld, false, 1.0f, want, plane, &used, st));
-            GELO_TRY(launch_sum_planes(ctx, tc.wf32, plane, used, ld, kv, nc8, loss2, tc.w32[0], ld, st));
+            GELO_TRY(gemm(kv, nc8, nr, V, ld, true, C, ld, false, tc.wf32, ld, false, 1.0f, want, plane, &used));
+            GELO_TRY(launch_sum_planes(ctx, tc.wf32, plane, used, ld, kv, nc8, loss2, tc.w32[0], ld, st, !exact));
         }
         // (the factor loss1 makes up for the truncation of V in the last product)
-        GELO_TRY(launch_gemm_tf32(ctx, kv, nc8, kv, Tt, kSuper, transpose, tc.w32[0], ld, false, tc.w32[1], ld, true, loss1, 1, 0,
-                                  nullptr, st));
-        return launch_gemm_tf32(ctx, nr, nc, kv, V, ld, false, tc.w32[1], ld, true, C, ld, false, 1.0f, 1, 0, nullptr, st);
+        GELO_TRY(gemm(kv, nc8, kv, Tt, kSuper, transpose, tc.w32[0], ld, false, tc.w32[1], ld, true, loss1, 1, 0, nullptr));
+        return gemm(nr, nc, kv, V, ld, false, tc.w32[1], ld, true, C, ld, false, 1.0f, 1, 0, nullptr);
     };
 
     // Block columns: 128 wide while at least twice as many rows are left, then narrower ones (half of the rows at most) (multiples of eight) down to a
@@ -692,28 +712,35 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
             float* Wb = tc.w32[1] + (size_t)(b - s) * FB * ld;
             int used = 0;
             const size_t plane = (size_t)FB * ld;
-            GELO_TRY(launch_gemm_tf32(ctx, ob, ncs, nr, P, ld, true, rows, ld, false, tc.wf32, ld, false, 1.0f,
-                                      slices(ob, ncs, kMaxKSplit), plane, &used, st));
+            GELO_TRY(gemm(ob, ncs, nr, P, ld, true, rows, ld, false, tc.wf32, ld, false, 1.0f, slices(ob, ncs, kMaxKSplit), plane, &used));
             const int work = ob * (ncs >> 2) + r * (ob >> 2);
-            block_sum_kernel<<<ceil_div(work, 256), 256, 0, st>>>(tc.wf32, plane, used, ld, ob, ncs, r, ob, loss2, tc.w32[0], ld,
+            block_sum_kernel<<<ceil_div(work, 256), 256, 0, st>>>(tc.wf32, plane, used, ld, ob, ncs, r, ob, loss2, round, tc.w32[0], ld,
                                                                  G + (size_t)s0 * ld + b0, r, ld);
             GELO_TRY(after_launch(ctx));
             float* Tb = Ts + (size_t)r * kSuper + r;
             float scale = 1.0f;                              // a power of two with scale^2 about nr
             while (2.0f * scale * scale < (float)nr) scale *= 2.0f;
             block_factor_kernel<<<kFactCtas, kFactThreads, kFactSmemBytes, st>>>(tc.w32[0] + r, ld, P, ld, ob, Tb, kSuper, tc.t128, FB,
-                                                                                scale, loss1, ctx->status_dev);
+                                                                                scale, loss1, round, ctx->status_dev);
             GELO_TRY(after_launch(ctx));
             if (e - s > 1) {
                 // [X^T | . | W'] = T^T Z + D^T [V_< | . | C1], scaled up for the truncation of V in the next product
-                GELO_TRY(launch_gemm_tf32_dual(ctx, ob, ncs, ob, Tb, kSuper, tc.w32[0], ld, tc.t128, FB, rows, ld, Wb, ld, loss1, st));
+                if (exact) {
+                    GELO_TRY(gemm(ob, ncs, ob, Tb, kSuper, false, tc.w32[0], ld, false, Wb, ld, false, 1.0f, 1, 0, nullptr));
+                    GemmArgs g;
+                    g.M = ob; g.N = ncs; g.K = ob;
+                    g.A = tc.t128; g.lda = FB; g.B = rows; g.ldb = ld;
+                    g.C[0] = Wb; g.ldc = ld; g.beta = 1.0f;
+                    GELO_TRY(launch_gemm_simt(ctx, g, st));
+                } else {
+                    GELO_TRY(launch_gemm_tf32_dual(ctx, ob, ncs, ob, Tb, kSuper, tc.w32[0], ld, tc.t128, FB, rows, ld, Wb, ld, loss1, st));
+                }
             }
             if (send > bend)                                 // C -= V W'
-                GELO_TRY(launch_gemm_tf32(ctx, nr, send - bend, ob, P, ld, false, Wb + (bend - s0), ld, true, P + ob, ld, false, 1.0f, 1, 0,
-                                          nullptr, st));
+                GELO_TRY(gemm(nr, send - bend, ob, P, ld, false, Wb + (bend - s0), ld, true, P + ob, ld, false, 1.0f, 1, 0, nullptr));
             if (r > 0)                                       // T^T[r:r+ob, 0:r] = -X^T T_<^T
-                GELO_TRY(launch_gemm_tf32(ctx, ob, r, r, Wb, ld, false, Ts, kSuper, false, Ts + (size_t)r * kSuper, kSuper, true,
-                                          -1.0f / loss1, 1, 0, nullptr, st));
+                GELO_TRY(gemm(ob, r, r, Wb, ld, false, Ts, kSuper, false, Ts + (size_t)r * kSuper, kSuper, true, -1.0f / loss1, 1, 0,
+                              nullptr));
         }
         GELO_TRY(apply(s0, send - s0, Ts, G + (size_t)s0 * ld + send, m - send, false));
     }

@@ -64,3 +64,20 @@ def test_inverse_of_the_nonorthogonal_sample(m, gamma, dt):
     # a binade: 2^-9 / sqrt(3) * 1.5 = 1.7e-3 (bf16), 2.1e-4 (half); the LU adds up to 1.3e-3
     bound = {"bf16": 2.0e-3, "f16": 2.5e-4}[dt] + (1.3e-3 if gamma > 0.55 else 0.0)
     assert np.linalg.norm(x - ref) / np.linalg.norm(ref) <= bound
+
+
+# the fp32 route: 129: its first size, one block of 64; 250: an odd split; 700: two groups of blocks; half at 200 rows takes it too
+@pytest.mark.parametrize("m,dt", [(129, "f32"), (250, "f32"), (700, "f32"), (200, "f16")])
+def test_exact_block_route(oracle, m, dt):
+    a, x = _sample(m, ORTHOGONAL, 300 + m, dt)
+    assert np.array_equal(x, a.T)
+    # fp32: sums of m products with eps = 2^-24 each leave sqrt(m) eps = 1.6e-6 at most in an entry of A^T A; half: its own rounding
+    bound = 2.0e-6 if dt == "f32" else 4e-4
+    assert np.linalg.norm(a.T @ a - np.eye(m)) / np.sqrt(m) <= bound
+    G64 = oracle.gaussian(300 + m, 0, 0, m, m).astype(np.float32).astype(np.float64)
+    q_ref, _ = oracle.householder_qr(G64)
+    h = m // 2
+    # 2e-6 per block from its factor (the Gram matrix squares a condition of at most 6), times at most m / 100 blocks
+    assert np.linalg.norm(a[:, :h] - q_ref[:, :h]) / np.sqrt(h) <= (2e-6 * (2 + m / 100) if dt == "f32" else 4e-4)
+    a, x = _sample(m, NONORTHOGONAL, 300 + m, dt)
+    assert np.linalg.norm(x @ a - np.eye(m)) / np.sqrt(m) <= (3e-6 if dt == "f32" else 5e-4)
