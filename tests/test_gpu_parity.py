@@ -1129,3 +1129,17 @@ def test_e4m3_projection_full_size_and_chain(ctx, oracle):
     drows = sample_rows(n, 32, seed=4)
     err = oracle.rel_fro(y[drows], oracle.rows_times_w(f64(H), f64(W), drows))
     assert 0.02 < err <= 0.2
+
+
+@pytest.mark.parametrize("n,k,kind", [(255, 12, 0), (300, 1, 1)])
+def test_fp32_products_of_any_depth(ctx, oracle, n, k, kind):
+    """Shield rows and a K that is no multiple of four on the tf32 pairs (products above 1 GFLOP); 300 + 1 rows end a quad after one."""
+    d, p = 2048, 6144
+    H = inputs.make_hidden(n, d, "f32", 5, True, "cuda"); W = inputs.make_weight(d, p, "f32", 6, "cuda")
+    ctx.ensure_workspace(n, k, d, p, "f32")
+    Q = torch.empty((n, p), device="cuda")
+    ctx.qkv_offload(H, W, n, k, d, p, kind, 77, 10.0, "f32", Q, None, None)
+    torch.cuda.synchronize()
+    ref = H.double() @ W.double()
+    # the fp32 path's tolerance
+    assert ((Q.double() - ref).norm() / ref.norm()).item() <= TOL["f32"]
