@@ -52,9 +52,9 @@ struct gelo_ctx {
     float gamma = 0.5f;
     float cond_bound = 100.0f;
     int max_attempts = 8;
-    int lane_tc_share = 4;        // batches with at least this many lanes give each level-3 update 1/share of the SMs
-    int tc_update_ctas = 0;       // CTAs of a level-3 tensor-core launch (0: one per SM); batches with many lanes use fewer,
-                                  // so that the updates of several lanes run side by side instead of queueing
+    int lane_tc_share = 4;        // batches with at least this many lanes plan each level-3 update for 1/share of the SMs
+    int tc_update_ctas = 0;       // CTAs that a level-3 tensor-core launch is planned for (0: one per SM): with many lanes fewer K slices
+                                  // do, because the updates of several lanes run side by side
     int level3 = 0;               // 0: tf32 tensor-core updates for bf16 calls with m >= 256; 1: always fp32 FMA;
                                   // 2: always tensor cores, three bf16 products of split operands; 3: always tensor cores, tf32
     long long launches = 0;

@@ -17,7 +17,10 @@
 // * A segment names one A tensor map, one B tensor map and a starting k for each; the stacked
 //   operand of the mixing product is two segments, a split-precision product is three.  TMA's
 //   out-of-bounds zero fill handles every ragged edge (including a seam inside a k-block).
-// * Persistent CTAs (one per SM, in pairs on 256 x 256 tiles where use_pair() says so), warp-specialised: warp 0 issues TMA, warp 1 issues MMA and owns
+// * CTAs (one per SM, in pairs on 256 x 256 tiles where use_pair() says so) that take tile after tile from the hardware's queue
+//   (cluster launch control), so that one which starts late because another stream's kernel held its SM finds less
+//   left to do instead of a fixed share: the 32-layer sweep 87 -> 81.5 ms, 32 fp32 calls at 1075 rows on 16 lanes 99 -> 54 ms (one
+//   call alone at 4300 rows 5.70 -> 5.75 ms); warp-specialised: warp 0 issues TMA, warp 1 issues MMA and owns
 //   the tensor-memory allocation, warps 2-9 drain the accumulator (two warps per TMEM lane
 //   quarter, half of the columns each).  Two accumulator stages let the epilogue of one tile
 //   overlap the main loop of the next.
@@ -42,6 +45,8 @@ constexpr int kEpiWarps = 8;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr uint32_t kABytes = BM * BK * 2;            // 16 KiB
 constexpr uint32_t kTmemCols = 512;
+constexpr uint32_t kBarBytes = 640;                  // barriers and the ring of tiles
+constexpr int kRing = 16;                            // tiles the roles of a CTA may be apart, see next_tile()
 
 enum TcMode { TC_STORE_BF16 = 0, TC_STORE_F32 = 1, TC_SUB_F32 = 2, TC_EMIT_SPLIT = 3, TC_STORE_SYM16 = 4, TC_AFFINE16 = 5 };
 
@@ -97,9 +102,9 @@ struct TcCfg {
     static constexpr uint32_t kBBytes = (kCols / kBoxCols) * kBoxBytes;
     static constexpr uint32_t kStageBytes = kABytes + kBBytes;
     // as many stages as fit, six at most: 4 (3 with staging for the in-place subtraction) alone, 6 (5) in a pair
-    static constexpr int kFit = (int)((227u * 1024u - 1024u - 256u - kStagingUsed) / kStageBytes);
+    static constexpr int kFit = (int)((227u * 1024u - 1024u - kBarBytes - kStagingUsed) / kStageBytes);
     static constexpr int kStages = kFit > 6 ? 6 : kFit;
-    static constexpr uint32_t kSmemBytes = kStages * kStageBytes + kStagingUsed + 1024 /*alignment slack*/ + 256 /*barriers*/;
+    static constexpr uint32_t kSmemBytes = kStages * kStageBytes + kStagingUsed + 1024 /*alignment slack*/ + kBarBytes;
     // k advance per instruction inside an N-major (or MN-major A) tile: 16 bf16 rows or 8 tf32 rows of 128 bytes
     static constexpr uint32_t kMnStep = kF8 ? 4096u : (kTf32 ? 1024u : 2048u);   // 32 e4m3 rows, 16 bf16 rows or 8 tf32 rows
     // N-major tiles: bf16 in the 16-byte-chunk swizzle (atoms of 8 k-rows, 1024 bytes), fp32 in the 32-byte-chunk
@@ -318,22 +323,29 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     auto empty_bar = [&](int s) { return bar_base + 8u * (kStages + s); };
     auto acc_full_bar = [&](int a) { return bar_base + 8u * (2 * kStages + a); };
     auto acc_empty_bar = [&](int a) { return bar_base + 8u * (2 * kStages + kAccStages + a); };
-    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bar_gen + 8 * (2 * kStages + 2 * kAccStages));
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_gen + 8 * (2 * kStages + 2 * kAccStages) + 8);
+    constexpr uint32_t kMisc = 8 * (2 * kStages + 2 * kAccStages);
+    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bar_gen + kMisc);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_gen + kMisc + 8);
+    const uint32_t clc_bar = bar_base + kMisc + 16, clc_slot = bar_base + ((kMisc + 24 + 15) & ~15u);
+    const uint32_t ring_off = ((kMisc + 24 + 15) & ~15u) + 16;
+    auto tile_bar = [&](int i) { return bar_base + ring_off + 8u * i; };
+    const uint32_t ring_base = bar_base + ring_off + 8u * kRing;
+    static_assert(kMisc + 24 + 15 + 16 + 12 * kRing <= kBarBytes, "barriers and ring fit");
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
 
     const int rank = kPair ? (int)cluster_rank() : 0;         // CTA 0 of a pair leads
-    const int first_tile = kPair ? blockIdx.x >> 1 : blockIdx.x, tile_step = kPair ? gridDim.x >> 1 : gridDim.x;
+    const int first_tile = kPair ? blockIdx.x >> 1 : blockIdx.x;
     const int m_tiles = (prm.M + Cfg::kTileRows - 1) / Cfg::kTileRows;
     const int n_tiles = (prm.N + BN - 1) / BN;
     const int mn_tiles = m_tiles * n_tiles;
-    const int total_tiles = prm.tri ? prm.tri_tiles : mn_tiles * prm.ksplit;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
         for (int a = 0; a < kAccStages; ++a) { mbar_init(acc_full_bar(a), 1); mbar_init(acc_empty_bar(a), kPair ? 2 * kEpiWarps : kEpiWarps); }
+        mbar_init(clc_bar, 1);
+        for (int i = 0; i < kRing; ++i) mbar_init(tile_bar(i), 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -355,12 +367,27 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
+    // The tiles of a CTA (pair): the one it was launched for, then whatever the leader's producer gets from the hardware's
+    // queue of CTAs not yet launched.  It hands each on through a ring; -1 ends.  The roles are at most kStages + 3 tiles apart (a tile
+    // has at least one stage of operands, and two accumulators), so a ring of kRing never overruns.
+    auto next_tile = [&](uint32_t it, bool& ok) -> int {
+        const int i = it % kRing;
+        const uint32_t parity = (it / kRing) & 1u;
+        if (!(kPair ? mbar_wait_cluster(tile_bar(i), parity, abort_flag, prm.wait_ns) : mbar_wait(tile_bar(i), parity, abort_flag, prm.wait_ns))) {
+            ok = false;
+            return -1;
+        }
+        int t;
+        asm volatile("ld.shared.s32 %0, [%1];" : "=r"(t) : "r"(ring_base + 4u * i) : "memory");
+        return t;
+    };
+
     if (warp == 0) {
         // ================= TMA producer =================
         if (lane == 0) {
-            uint32_t it = 0;
-            bool ok = true;
-            for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step) {
+            uint32_t it = 0, tile_it = 0;
+            bool ok = true, asked = false;
+            for (int tile = first_tile; tile >= 0 && ok; ++tile_it) {
                 int mt, nt, slice;
                 tile_coords<kPair>(prm, tile, m_tiles, mn_tiles, mt, nt, slice);
                 const int m0 = mt * Cfg::kTileRows + rank * BM, n0 = nt * BN + rank * Cfg::kCols;
@@ -405,7 +432,28 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
                             for (int j = 0; j < Cfg::kCols / Cfg::kBoxCols; ++j)
                                 load_2d(sb + j * Cfg::kBoxBytes, mb, n0 + j * Cfg::kBoxCols, seg.b_row0 + kb * Cfg::kBKE);
                         }
+                        if (rank == 0 && !asked) {            // the next tile, while this one's operands come in
+                            mbar_expect_tx(clc_bar, 16);
+                            clc_try_cancel(clc_slot, clc_bar);
+                            asked = true;
+                        }
                     }
+                }
+                if (rank == 0) {
+                    if (asked && !mbar_wait(clc_bar, tile_it & 1u, abort_flag, prm.wait_ns)) ok = false;
+                    if (!ok) break;
+                    asked = false;
+                    const int x = clc_answer(clc_slot);
+                    tile = kPair && x >= 0 ? x >> 1 : x;
+                    const uint32_t slot = ring_base + 4u * (tile_it % kRing), bar = tile_bar(tile_it % kRing);
+                    asm volatile("st.shared.s32 [%0], %1;" ::"r"(slot), "r"(tile) : "memory");
+                    if (kPair) {
+                        asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(map_rank(slot, 1)), "r"(tile) : "memory");
+                        mbar_arrive_cluster(map_rank(bar, 1));
+                    }
+                    mbar_arrive(bar);
+                } else {
+                    tile = next_tile(tile_it, ok);
                 }
             }
             if (!ok) { *abort_flag = 1; atomicCAS(prm.status, 0, (int)GELO_ERR_TIMEOUT); }
@@ -419,7 +467,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             bool ok = true;
             // k advance per instruction in sixteen-byte units of the descriptors' start address
             constexpr uint64_t kAStep = kAMn ? (Cfg::kMnStep >> 4) : 2, kBStep = Cfg::kMnStep >> 4;
-            for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step, ++acc_it) {
+            for (int tile = first_tile; tile >= 0 && ok; tile = next_tile(acc_it, ok), ++acc_it) {
                 const int slice = prm.tri ? 0 : tile / mn_tiles;
                 int kb_total = 0;
 #pragma unroll
@@ -462,7 +510,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
         constexpr int kHalfCols = BN / 2;
         uint32_t acc_it = 0, box_it = 0;
         bool ok = true;
-        for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step, ++acc_it) {
+        for (int tile = first_tile; tile >= 0 && ok; tile = next_tile(acc_it, ok), ++acc_it) {
             const int a = acc_it % kAccStages;
             const uint32_t aph = (acc_it / kAccStages) & 1u;
             int mt, nt, slice;
@@ -614,7 +662,8 @@ bool make_map_nmajor(gelo_ctx* ctx, CUtensorMap* map, const void* ptr, int elem_
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// CTAs that one launch may use
+// CTAs that a launch should plan for: all SMs, or a lane's share of them in a batch (no limit: the tiles go wherever an SM is
+// free)
 int launch_width(const gelo_ctx* ctx, int mode)
 {
     return (mode != TC_STORE_BF16 && ctx->tc_update_ctas > 0 && ctx->tc_update_ctas < ctx->sm_count) ? ctx->tc_update_ctas : ctx->sm_count;
@@ -661,15 +710,13 @@ int launch_tiles_as(gelo_ctx* ctx, const CUtensorMap& a0, const CUtensorMap& a1,
     TcParams q = p;
     if (p.tri) q.tri_tiles = tile_count(p.M, p.N, 1, true, kPair);
     const int tiles = p.tri ? q.tri_tiles : ceil_div(p.M, Cfg::kTileRows) * ceil_div(p.N, BN) * p.ksplit;
-    const int most = launch_width(ctx, p.mode) / (kPair ? 2 : 1);
-    const int grid = (tiles < most ? tiles : most) * (kPair ? 2 : 1);
     // both operands of a kind::f16 instruction have the same 16-bit format: 1 = bfloat16, 0 = IEEE half
     q.wait_ns = ctx->wait_limit_ns;
     q.idesc = (!kTf32 && !kF8 && p.out_f16) ? (Cfg::kInstrDesc & ~((7u << 7) | (7u << 10))) : Cfg::kInstrDesc;
     {
         ProfScope ps(ctx, PROF_GEMM_TC, flops, st);
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(grid);
+        cfg.gridDim = dim3(tiles * (kPair ? 2 : 1));
         cfg.blockDim = dim3(kThreads);
         cfg.dynamicSmemBytes = Cfg::kSmemBytes;
         cfg.stream = st;
