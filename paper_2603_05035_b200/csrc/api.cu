@@ -206,7 +206,7 @@ int sample_attempt(gelo_ctx* ctx, const Layout& L, int m, int kind, uint64_t see
         GELO_TRY(launch_finish_mixing(ctx, m, Q0, ldi, nullptr, ldi, dtype, x16, g16, ldi, st));
         GELO_TRY(launch_gaussian(ctx, m, m, ldi, seed, GELO_STREAM_G1, attempt, s, Q0, L.A32, st, seed_dev));
         GELO_TRY(launch_narrow(ctx, m, L.A32, ldi, dtype, A_out, lda, st));
-        GELO_TRY(run_newton_inverse(ctx, m, dtype, A_out, lda, g16, g16 + half, x16, ldi, Ainv_out, lda, st));
+        GELO_TRY(run_newton_inverse(ctx, m, dtype, ctx->gamma, A_out, lda, g16, g16 + half, x16, x16 + half, ldi, Ainv_out, lda, st));
     } else if (blocks && exact && m <= kExactNewtonRows && ctx->gamma <= 0.55f) {
         // in fp32 from the stored A, and rounded once
         GELO_TRY(launch_finish_mixing(ctx, m, Q0, ldi, nullptr, ldi, GELO_F32, L.X32, L.G, ldi, st));

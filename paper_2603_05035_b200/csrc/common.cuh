@@ -182,9 +182,9 @@ int launch_gram_sym_bf16(gelo_ctx*, int m, const float* Q, int ld, void* D, int 
 // C (fp32) -= A (bf16) B (bf16), in place
 int launch_gemm_bf16_sub(gelo_ctx*, int M, int N, int K, const void* A, int lda, const void* B, int ldb, float* C, int ldc,
                          cudaStream_t);
-// C (M x N, 16-bit type) = sign * A B + diag I + add (optional)
+// C (M x N, 16-bit type) = sign * A B + diag I + add_scale * add (optional)
 int launch_gemm_affine16(gelo_ctx*, int dtype, int M, int N, int K, const void* A, int lda, const void* B, int ldb, float sign,
-                         float diag, const void* add, int ldadd, void* C, int ldc, cudaStream_t);
+                         float diag, const void* add, int ldadd, float add_scale, void* C, int ldc, cudaStream_t);
 // ---- E4M3 operands for the offloaded product (fp8.cu, gemm_tc.cu) ----
 int launch_quantize_e4m3(gelo_ctx*, const void* x, int rows, int cols, int ld, int dtype, void* out, int ldo, float* scale,
                          cudaStream_t);
@@ -294,10 +294,11 @@ struct TcScratch;
 int run_lu_inverse_tc(gelo_ctx*, int m, const float* A, int ld, float* Ainv, const LuScratch&, const TcScratch&,
                       bool tf32, cudaStream_t);
 
-// A^-1 of A = Q0 + gamma G1 / sqrt(m) (m x m, 16-bit, stride lda) by Newton's iteration from X0 = Q0^T (inverse.cu)
+// A^-1 of A = Q0 + gamma G1 / sqrt(m) (m x m, 16-bit, stride lda) by Newton's iteration from X0 = Q0^T (inverse.cu); X0, T1, T2 and
+// X are scratch of stride ld
 bool newton_inverse_supports(int m, int dtype, float gamma);
-int run_newton_inverse(gelo_ctx*, int m, int dtype, const void* A, int lda, void* X0, void* X1, void* Y, int ld, void* Ainv, int ldi,
-                       cudaStream_t);
+int run_newton_inverse(gelo_ctx*, int m, int dtype, float gamma, const void* A, int lda, void* X0, void* T1, void* T2, void* X, int ld,
+                       void* Ainv, int ldi, cudaStream_t);
 // the same in fp32 on multiply-adds
 int run_newton_inverse_f32(gelo_ctx*, int m, const float* A, int lda, float* X0, float* X1, float* Y, int ld, float* Ainv, int ldi,
                            cudaStream_t);

@@ -69,7 +69,7 @@ struct TcParams {
     int out_f16;                    // TC_STORE_BF16: operands and output are IEEE half instead of bfloat16
     const float* scale_a;           // TC_STORE_BF16 with 8-bit operands: the per-tensor scales (device scalars); the
     const float* scale_b;           //   accumulator is multiplied by their product before it is rounded
-    const void* add; int ldadd;     // TC_AFFINE16: out = out_scale * acc + diag_sub on the diagonal + the entry of `add` (optional)
+    const void* add; int ldadd;     // TC_AFFINE16: out = out_scale * acc + diag_sub on the diagonal + post_scale * the entry of `add` (optional)
     int tri, tri_tiles;             // TC_STORE_SYM16: the result is symmetric; only the tri_tiles tiles that reach the diagonal or lie
                                     // above it are computed, and what lies below them is filled in by mirroring
     uint32_t idesc;                 // instruction descriptor (filled in by the launcher)
@@ -191,7 +191,7 @@ __device__ __forceinline__ void write_staged(const TcParams& prm, uint32_t buf, 
 }
 
 // Accumulator columns [c, c + 64) of the tile as 64 16-bit values per row: product times the two scales (TC_STORE_BF16),
-// or out_scale * product + diag on the diagonal + the entry of `add` (TC_AFFINE16).
+// or out_scale * product + diag on the diagonal + post_scale * the entry of `add` (TC_AFFINE16).
 __device__ __forceinline__ void store_tile16(const TcParams& prm, uint32_t taddr, uint32_t buf, int m0, int gn, int lane)
 {
     const bool affine = prm.mode == TC_AFFINE16;
@@ -229,7 +229,7 @@ __device__ __forceinline__ void store_tile16(const TcParams& prm, uint32_t taddr
                 for (int j = 0; j < 4; ++j) {
                     const float2 t = prm.out_f16 ? __half22float2(*reinterpret_cast<const __half2*>(&w2[j]))
                                                  : __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w2[j]));
-                    f[2 * j] += t.x; f[2 * j + 1] += t.y;
+                    f[2 * j] = fmaf(prm.post_scale, t.x, f[2 * j]); f[2 * j + 1] = fmaf(prm.post_scale, t.y, f[2 * j + 1]);
                 }
             }
             uint32_t o[4];
@@ -1057,9 +1057,9 @@ int launch_gemm_bf16_sub(gelo_ctx* ctx, int M, int N, int K, const void* A, int 
     return launch_tiles<256, true>(ctx, pair, ma, ma, mb, mb, mc, p, 2.0 * M * (double)N * K, st);
 }
 
-// C (M x N, 16-bit type of the operands) = sign * A (M x K) B (K x N) + diag I + add (optional, M x N)
+// C (M x N, 16-bit type of the operands) = sign * A (M x K) B (K x N) + diag I + add_scale * add (optional, M x N)
 int launch_gemm_affine16(gelo_ctx* ctx, int dtype, int M, int N, int K, const void* A, int lda, const void* B, int ldb, float sign,
-                         float diag, const void* add, int ldadd, void* C, int ldc, cudaStream_t st)
+                         float diag, const void* add, int ldadd, float add_scale, void* C, int ldc, cudaStream_t st)
 {
     if (M <= 0 || N <= 0 || K <= 0) return GELO_OK;
     if (!ctx->tmap_encode) return GELO_ERR_CUDA;
@@ -1081,7 +1081,7 @@ int launch_gemm_affine16(gelo_ctx* ctx, int dtype, int M, int N, int K, const vo
     p.mode = TC_AFFINE16;
     p.b3d = b3d ? 1 : 0;
     p.out_f16 = dtype == GELO_F16 ? 1 : 0;
-    p.out_scale = sign; p.diag_sub = diag;
+    p.out_scale = sign; p.diag_sub = diag; p.post_scale = add_scale;
     p.add = add; p.ldadd = ldadd;
     p.C0 = C; p.ldc = ldc; p.csplit = N;
     p.status = ctx->status_dev;

@@ -2,37 +2,54 @@
 // batch").
 //
 // The sampler's A = Q0 + gamma G1 / sqrt(m) comes with a good first guess of its inverse: with X0 = Q0^T the residual
-// I - A X0 = -gamma G1 Q0^T / sqrt(m) is a Gaussian matrix whose eigenvalues fill the disc of radius gamma (the circular
-// law), so its 2^k-th power, which k steps of
-//     X <- X (2 I - A X)
-// leave, has Frobenius norm gamma^(2^k) sqrt(m): 0.4% of the identity's after three steps at gamma = 1/2.  Every step is two
-// products of 16-bit operands, and a step corrects the rounding of the one before, because it starts from A and the stored
-// X.  The last step keeps what is left of the residual small instead of adding it to the identity before it is rounded,
-//     R = I - A X,   A^-1 = X + X R   (rounded once, to the storage type),
-// and ends at gamma^16 = 1.5e-5 and 2^-9 |R| = 2e-5 (bfloat16), below what the storage type resolves.
+// R = I - A X0 = -gamma G1 Q0^T / sqrt(m) is a Gaussian matrix whose eigenvalues fill the disc of radius gamma (the circular
+// law), and A^-1 = X0 (I + R + R^2 + ...).  The k-th power of such a matrix has Frobenius norm gamma^k sqrt(m).
 //
-// Eight products at the 16-bit rate of the tensor cores replace the pivoted LU and its two triangular solves, which were bound
-// by some 1000 dependent launches: 4300 rows, one call alone 30.4 -> 8.6 ms, the 32-layer sweep (16 of them) 114 -> 98.5 ms, and
-// A^-1 A - I falls from 1.3e-3 to what rounding A^-1 leaves (half: 2.7e-4).
+// Products of 16-bit operands, in two parts.  First X = X0 (I + R + R^2 + R^3 + R^4) in four products, the polynomial by
+// completing squares: with S = R + I/4 and N = S^2 + 5/16 I it is N^2 + 5/8 S + 45/64 I.  What is missing, R^5, and all rounding so
+// far is then the residual of the stored X, which a last part computes and corrects:
+//     R = I - A X,   A^-1 = X + X R                   (two products, ends at gamma^10),
+//     R = I - A X,   Z = R^2 + R,   A^-1 = X + X Z    (three, gamma^15),
+// with R or Z kept small instead of added to the identity before it is rounded, and A^-1 rounded once.  The second leaves
+// 3e-5 at gamma = 1/2, nothing beside the rounding of A^-1 (bfloat16 1.66e-3, half 2.1e-4).  The first leaves 2^-10, a total of 1.93e-3 in
+// bfloat16; it serves bfloat16 from 4096 rows up, where that is what the pivoted LU had (1.96e-3 at 4300 rows, growing
+// with m) and a product costs 0.11 ms.
+//
+// Six or seven products at the 16-bit rate of the tensor cores replace the pivoted LU and its two triangular solves, which were
+// bound by some 1000 dependent launches: 4300 rows, one call alone 30.4 -> 8.6 ms (with eight products, four Newton steps from
+// X0), the 32-layer sweep (16 of them) 114 -> 98.5 ms; six products instead of eight: 81.5 -> 78 ms later.
 #include "common.cuh"
 
 namespace gelo {
 
-// gamma: beyond 0.55 the fourth step no longer reaches 1e-4 (0.55^16 = 7e-5), and from 1 on the iteration diverges.
+// gamma: beyond 0.55 even two corrections leave more than rounding does, and from 1 on the series diverges.
 // m: smaller matrices take the fp32 iteration.
 bool newton_inverse_supports(int m, int dtype, float gamma) { return dtype != GELO_F32 && m >= 256 && gamma <= 0.55f; }
 
-int run_newton_inverse(gelo_ctx* ctx, int m, int dtype, const void* A, int lda, void* X0, void* X1, void* Y, int ld, void* Ainv, int ldi,
-                       cudaStream_t st)
+int run_newton_inverse(gelo_ctx* ctx, int m, int dtype, float gamma, const void* A, int lda, void* X0, void* T1, void* T2, void* X, int ld,
+                       void* Ainv, int ldi, cudaStream_t st)
 {
     const int m8 = (m + 7) & ~7;
-    for (int step = 0; step < 3; ++step) {
-        GELO_TRY(launch_gemm_affine16(ctx, dtype, m, m8, m, A, lda, X0, ld, -1.0f, 2.0f, nullptr, 0, Y, ld, st));
-        GELO_TRY(launch_gemm_affine16(ctx, dtype, m, m8, m, X0, ld, Y, ld, 1.0f, 0.0f, nullptr, 0, X1, ld, st));
-        void* t = X0; X0 = X1; X1 = t;
+    auto product = [&](const void* a, int la, const void* b, float sign, float diag, const void* add, float add_scale, void* c, int lc) -> int {
+        return launch_gemm_affine16(ctx, dtype, m, m8, m, a, la, b, ld, sign, diag, add, ld, add_scale, c, lc, st);
+    };
+    GELO_TRY(product(A, lda, X0, -1.0f, 1.25f, nullptr, 0.0f, T1, ld));                       // S
+    GELO_TRY(product(T1, ld, T1, 1.0f, 0.3125f, nullptr, 0.0f, T2, ld));                      // N
+    GELO_TRY(product(T2, ld, T2, 1.0f, 0.703125f, T1, 0.625f, X, ld));                        // the polynomial
+    GELO_TRY(product(X0, ld, X, 1.0f, 0.0f, nullptr, 0.0f, T1, ld));
+    void* x = T1;
+    void* r = T2;
+    if (gamma > 0.5f) {                                                                       // gamma^10 first, then its square
+        GELO_TRY(product(A, lda, x, -1.0f, 1.0f, nullptr, 0.0f, r, ld));
+        GELO_TRY(product(x, ld, r, 1.0f, 0.0f, x, 1.0f, X0, ld));
+        x = X0;
     }
-    GELO_TRY(launch_gemm_affine16(ctx, dtype, m, m8, m, A, lda, X0, ld, -1.0f, 1.0f, nullptr, 0, Y, ld, st));
-    return launch_gemm_affine16(ctx, dtype, m, m8, m, X0, ld, Y, ld, 1.0f, 0.0f, X0, ld, Ainv, ldi, st);
+    GELO_TRY(product(A, lda, x, -1.0f, 1.0f, nullptr, 0.0f, r, ld));
+    if (gamma <= 0.5f && !(dtype == GELO_BF16 && m >= 4096)) {
+        GELO_TRY(product(r, ld, r, 1.0f, 0.0f, r, 1.0f, X, ld));
+        r = X;
+    }
+    return product(x, ld, r, 1.0f, 0.0f, x, 1.0f, Ainv, ldi);
 }
 
 // fp32: five steps (gamma^32 = 2e-10) of products on the FMA pipes.
