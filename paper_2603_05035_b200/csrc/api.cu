@@ -231,6 +231,57 @@ int sample_attempt(gelo_ctx* ctx, const Layout& L, int m, int kind, uint64_t see
                              st, deferred);
 }
 
+__global__ void set_seed_kernel(uint64_t* slot, uint64_t seed) { *slot = seed; }
+
+void drop_graphs(gelo_ctx* ctx)
+{
+    for (auto& g : ctx->graphs) cudaGraphExecDestroy(g.exec);
+    ctx->graphs.clear();
+}
+
+// Samples (A, A^-1) of one batched call on a lane stream by replaying a launch graph of the whole sampling
+// sequence (about a thousand dependent launches): one host call instead of a thousand, so a single host thread
+// keeps all lanes busy.  The seed reaches the kernels through the lane's device slot.  The first use of a
+// (lane scratch, kind, size, type) combination records the graph by stream capture.
+int sample_on_lane(gelo_ctx* ctx, const Layout& L, int lane, int m, int kind, uint64_t seed, int dtype, cudaStream_t ls,
+                   bool deferred = true)
+{
+    uint64_t* slot = ctx->lane_seed_dev + lane * 8;
+    set_seed_kernel<<<1, 1, 0, ls>>>(slot, seed);
+    GELO_TRY(after_launch(ctx));
+    if (ctx->prof_on)      // per-launch timing needs real launches
+        return sample_attempt(ctx, L, m, kind, seed, 0u, dtype, L.A, L.Ainv, L.ldi, nullptr, ls, deferred, slot);
+    for (auto& g : ctx->graphs) {
+        if (g.key_ptr == L.G && g.m == m && g.kind == kind && g.dtype == dtype && g.level3 == ctx->level3 &&
+            g.tc_ctas == ctx->tc_update_ctas && g.deferred == deferred) {
+            GELO_CUDA_OK(cudaGraphLaunch(g.exec, ls));
+            ctx->launches += g.launches;
+            return GELO_OK;
+        }
+    }
+    const long long before = ctx->launches;
+    GELO_CUDA_OK(cudaStreamBeginCapture(ls, cudaStreamCaptureModeRelaxed));
+    ctx->recording = true;
+    const int rc = sample_attempt(ctx, L, m, kind, seed, 0u, dtype, L.A, L.Ainv, L.ldi, nullptr, ls, deferred, slot);
+    ctx->recording = false;
+    cudaGraph_t graph = nullptr;
+    const cudaError_t ce = cudaStreamEndCapture(ls, &graph);
+    if (rc != GELO_OK || ce != cudaSuccess || !graph) {
+        if (graph) cudaGraphDestroy(graph);
+        return rc != GELO_OK ? rc : GELO_ERR_CUDA;
+    }
+    gelo_ctx::SampleGraph g;
+    g.key_ptr = L.G; g.m = m; g.kind = kind; g.dtype = dtype; g.level3 = ctx->level3; g.tc_ctas = ctx->tc_update_ctas; g.deferred = deferred;
+    g.launches = ctx->launches - before;
+    g.exec = nullptr;
+    const cudaError_t ie = cudaGraphInstantiate(&g.exec, graph, 0);
+    cudaGraphDestroy(graph);
+    if (ie != cudaSuccess) return GELO_ERR_CUDA;
+    ctx->graphs.push_back(g);
+    GELO_CUDA_OK(cudaGraphLaunch(g.exec, ls));
+    return GELO_OK;
+}
+
 int sample_mixing_impl(gelo_ctx* ctx, const Layout& L, int m, int kind, uint64_t seed, int dtype,
                        void* A_out, void* Ainv_out, int lda, float* cond_dev, cudaStream_t st)
 {
@@ -339,64 +390,39 @@ int check_split(int p, const void* Q, const void* K, const void* V)
     return GELO_OK;
 }
 
+// One whole call on the caller's stream.  A non-orthogonal pair is verified: the first attempt replays the recorded sampling
+// graph on a lane's stream beside the shield rows, the products are enqueued behind it, and the host waits for the verdict only;
+// a sample that misses the bound (never seen) is drawn again, and the products repeated.
 int offload_impl(gelo_ctx* ctx, const Layout& L, const void* H, const void* W, int n, int k, int d, int p,
                  int kind, uint64_t seed, float shield_scale, int dtype, void* Q, void* K, void* V,
                  cudaStream_t st)
 {
     const int m = n + k;
-    GELO_TRY(sample_mixing_impl(ctx, L, m, kind, seed, dtype, L.A, L.Ainv, L.ldi, nullptr, st));
-    GELO_TRY(run_shield_rows(ctx, H, n, d, k, shield_scale, seed, dtype, L.S, L.sh, st, ctx->shield_nu));
-    GELO_TRY(mix_impl(ctx, L.A, L.ldi, H, k > 0 ? L.S : nullptr, n, k, d, dtype, L.U, st, &L.t3));
-    return project_and_unmix(ctx, L.U, W, L.Ainv, L.ldi, L.Yp, n, k, d, p, dtype, Q, K, V, st, &L.t3);
-}
-
-
-__global__ void set_seed_kernel(uint64_t* slot, uint64_t seed) { *slot = seed; }
-
-void drop_graphs(gelo_ctx* ctx)
-{
-    for (auto& g : ctx->graphs) cudaGraphExecDestroy(g.exec);
-    ctx->graphs.clear();
-}
-
-// Samples (A, A^-1) of one batched call on a lane stream by replaying a launch graph of the whole sampling
-// sequence (about a thousand dependent launches): one host call instead of a thousand, so a single host thread
-// keeps all lanes busy.  The seed reaches the kernels through the lane's device slot.  The first use of a
-// (lane scratch, kind, size, type) combination records the graph by stream capture.
-int sample_on_lane(gelo_ctx* ctx, const Layout& L, int lane, int m, int kind, uint64_t seed, int dtype, cudaStream_t ls)
-{
-    uint64_t* slot = ctx->lane_seed_dev + lane * 8;
-    set_seed_kernel<<<1, 1, 0, ls>>>(slot, seed);
-    GELO_TRY(after_launch(ctx));
-    if (ctx->prof_on)      // per-launch timing needs real launches
-        return sample_attempt(ctx, L, m, kind, seed, 0u, dtype, L.A, L.Ainv, L.ldi, nullptr, ls, true, slot);
-    for (auto& g : ctx->graphs) {
-        if (g.key_ptr == L.G && g.m == m && g.kind == kind && g.dtype == dtype && g.level3 == ctx->level3 &&
-            g.tc_ctas == ctx->tc_update_ctas) {
-            GELO_CUDA_OK(cudaGraphLaunch(g.exec, ls));
-            ctx->launches += g.launches;
-            return GELO_OK;
-        }
+    auto shields = [&]() -> int { return run_shield_rows(ctx, H, n, d, k, shield_scale, seed, dtype, L.S, L.sh, st, ctx->shield_nu); };
+    auto products = [&]() -> int {
+        GELO_TRY(mix_impl(ctx, L.A, L.ldi, H, k > 0 ? L.S : nullptr, n, k, d, dtype, L.U, st, &L.t3));
+        return project_and_unmix(ctx, L.U, W, L.Ainv, L.ldi, L.Yp, n, k, d, p, dtype, Q, K, V, st, &L.t3);
+    };
+    if (kind == GELO_ORTHOGONAL || ctx->prof_on) {
+        GELO_TRY(sample_mixing_impl(ctx, L, m, kind, seed, dtype, L.A, L.Ainv, L.ldi, nullptr, st));
+        GELO_TRY(shields());
+        return products();
     }
-    const long long before = ctx->launches;
-    GELO_CUDA_OK(cudaStreamBeginCapture(ls, cudaStreamCaptureModeRelaxed));
-    const int rc = sample_attempt(ctx, L, m, kind, seed, 0u, dtype, L.A, L.Ainv, L.ldi, nullptr, ls, true, slot);
-    cudaGraph_t graph = nullptr;
-    const cudaError_t ce = cudaStreamEndCapture(ls, &graph);
-    if (rc != GELO_OK || ce != cudaSuccess || !graph) {
-        if (graph) cudaGraphDestroy(graph);
-        return rc != GELO_OK ? rc : GELO_ERR_CUDA;
+    for (int attempt = 0; attempt < ctx->max_attempts; ++attempt) {
+        cudaStream_t ls = ctx->lane_stream[0];
+        GELO_CUDA_OK(cudaEventRecord(ctx->batch_start, st));
+        GELO_CUDA_OK(cudaStreamWaitEvent(ls, ctx->batch_start, 0));
+        if (attempt == 0) GELO_TRY(sample_on_lane(ctx, L, 0, m, kind, seed, dtype, ls, false));
+        else GELO_TRY(sample_attempt(ctx, L, m, kind, seed, (uint32_t)attempt, dtype, L.A, L.Ainv, L.ldi, nullptr, ls));
+        GELO_CUDA_OK(cudaMemcpyAsync(ctx->status_host, ctx->status_dev, kStatusWords * sizeof(int), cudaMemcpyDeviceToHost, ls));
+        GELO_CUDA_OK(cudaEventRecord(ctx->lane_ready[0], ls));
+        if (attempt == 0) GELO_TRY(shields());
+        GELO_CUDA_OK(cudaStreamWaitEvent(st, ctx->lane_ready[0], 0));
+        GELO_TRY(products());
+        GELO_CUDA_OK(cudaEventSynchronize(ctx->lane_ready[0]));
+        if (ctx->status_host[1] == 1) return GELO_OK;
     }
-    gelo_ctx::SampleGraph g;
-    g.key_ptr = L.G; g.m = m; g.kind = kind; g.dtype = dtype; g.level3 = ctx->level3; g.tc_ctas = ctx->tc_update_ctas;
-    g.launches = ctx->launches - before;
-    g.exec = nullptr;
-    const cudaError_t ie = cudaGraphInstantiate(&g.exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (ie != cudaSuccess) return GELO_ERR_CUDA;
-    ctx->graphs.push_back(g);
-    GELO_CUDA_OK(cudaGraphLaunch(g.exec, ls));
-    return GELO_OK;
+    return GELO_ERR_COND;
 }
 
 // The whole path for a batch of independent calls.  Sampling A depends only on the seed, so up to

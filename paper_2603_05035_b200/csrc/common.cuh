@@ -78,8 +78,9 @@ struct gelo_ctx {
     int chain_lanes = 0;
     int chain_shape[6] = {0, 0, 0, 0, 0, 0};   // n, k, d, p, dtype, host staging of the batch a later one may chain onto
     // replayable launch graphs of the sampling sequence, one per (lane scratch, kind, size, type)
-    struct SampleGraph { const void* key_ptr; int m, kind, dtype, level3, tc_ctas; cudaGraphExec_t exec; long long launches; };
+    struct SampleGraph { const void* key_ptr; int m, kind, dtype, level3, tc_ctas; bool deferred; cudaGraphExec_t exec; long long launches; };
     std::vector<SampleGraph> graphs;
+    bool recording = false;                         // the launches go into such a graph
     uint64_t* lane_seed_dev = nullptr;              // one seed slot per lane
     // the batched host variant moves activations in and results out on streams of their own, through two staging pairs
     cudaStream_t copy_in = nullptr, copy_out = nullptr;
@@ -107,6 +108,30 @@ namespace gelo {
 static inline int after_launch(gelo_ctx* ctx) {
     ctx->launches += 1;
     return cudaPeekAtLastError() == cudaSuccess ? GELO_OK : GELO_ERR_CUDA;
+}
+
+// Launches that follow one another in a call wait for each other on the device (programmatic dependent launch): a kernel
+// lets its successor be set up as soon as all of its own CTAs run (chain_next) and itself touches memory only after
+// chain_wait, which returns when its predecessor has finished and its results are visible.  A kernel that is launched this way always
+// waits, so the order is that of the stream.  For launches into a stream: 4300 rows non-orthogonal 5.55 -> 5.08 ms, 350 rows staged
+// 629 -> 540 us.  Not in recorded graphs, which have that already (no difference), and not with many lanes, where CTAs that only wait
+// would keep SMs from other lanes' work.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+static inline bool chain_launches(const gelo_ctx* ctx) { return ctx->tc_update_ctas == 0 && !ctx->prof_on && !ctx->recording; }
+
+template <typename... P, typename... A>
+int launch_chained(gelo_ctx* ctx, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = chain_launches(ctx) ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) == cudaSuccess ? GELO_OK : GELO_ERR_CUDA;
 }
 
 // Brackets one launch with CUDA events on its stream while per-launch timing is on.

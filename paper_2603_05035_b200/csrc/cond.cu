@@ -41,6 +41,8 @@ struct CondViews {
 // The start vector, as the only slab of a first reduction.
 __global__ void cond_init_kernel(CondViews v, uint64_t seed, uint32_t attempt)
 {
+    chain_next();
+    chain_wait();
     const int z = blockIdx.y;
     const int i4 = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (i4 == 0) v.done[z] = 0;
@@ -108,6 +110,8 @@ __device__ __forceinline__ void cond_lanczos(const CondViews& v, int z, int step
 // added in order.  The CTA that finishes last for an operator goes on with the recurrence.
 __global__ void __launch_bounds__(kCondChunkCols * kCondParts) cond_reduce_kernel(CondViews v, int slabs, int step)
 {
+    chain_next();
+    chain_wait();
     static_assert(kCondChunkCols * kCondParts == 1024, "cond_lanczos counts on 1024 threads");
     __shared__ float part[kCondParts][kCondChunkCols];
     __shared__ float red[32];
@@ -176,6 +180,8 @@ __device__ double tridiagonal_lambda_max(const float* alpha, const float* beta)
 // One warp per operator.
 __global__ void __launch_bounds__(64) cond_verdict_kernel(CondViews v, float bound, float* cond_out, int* status, int deferred)
 {
+    chain_next();
+    chain_wait();
     __shared__ double lam[2];
     const int z = threadIdx.x >> 5;
     const double l = tridiagonal_lambda_max(v.tri + z * 2 * kLanczosSteps, v.tri + z * 2 * kLanczosSteps + kLanczosSteps);
@@ -225,6 +231,8 @@ __device__ __forceinline__ void load8(const __half* p, float (&a)[8])
 template <typename T>
 __global__ void __launch_bounds__(256) cond_step_kernel(CondViews v)
 {
+    chain_next();
+    chain_wait();
     extern __shared__ float ys[];
     const int z = blockIdx.y, slab = blockIdx.x;
     const int r0 = slab * v.rows_per;
@@ -327,20 +335,21 @@ int run_cond_estimate(gelo_ctx* ctx, int m, const void* A, const void* Ainv, int
     const size_t ys_bytes = (size_t)v.rows_per * sizeof(float);
     if (ys_bytes > 48 * 1024) return GELO_ERR_UNSUPPORTED;
     dim3 gi(ceil_div(v.mpad, 4 * 256), 2);
-    cond_init_kernel<<<gi, 256, 0, st>>>(v, 0x5eedull, 0u);
+    GELO_TRY(launch_chained(ctx, cond_init_kernel, gi, 256, 0, st, v, 0x5eedull, 0u));
     GELO_TRY(after_launch(ctx));
     const dim3 gr(v.mpad / kCondChunkCols, 2), gs(ceil_div(m, v.rows_per), 2);
     for (int step = -1; step < kLanczosSteps; ++step) {
         if (step >= 0) {
-            if (dtype == GELO_BF16) cond_step_kernel<__nv_bfloat16><<<gs, 256, ys_bytes, st>>>(v);
-            else if (dtype == GELO_F16) cond_step_kernel<__half><<<gs, 256, ys_bytes, st>>>(v);
-            else cond_step_kernel<float><<<gs, 256, ys_bytes, st>>>(v);
+            if (dtype == GELO_BF16) GELO_TRY(launch_chained(ctx, cond_step_kernel<__nv_bfloat16>, gs, 256, ys_bytes, st, v));
+            else if (dtype == GELO_F16) GELO_TRY(launch_chained(ctx, cond_step_kernel<__half>, gs, 256, ys_bytes, st, v));
+            else GELO_TRY(launch_chained(ctx, cond_step_kernel<float>, gs, 256, ys_bytes, st, v));
             GELO_TRY(after_launch(ctx));
         }
-        cond_reduce_kernel<<<gr, kCondChunkCols * kCondParts, 0, st>>>(v, step < 0 ? 1 : (int)gs.x, step);
+        GELO_TRY(launch_chained(ctx, cond_reduce_kernel, gr, kCondChunkCols * kCondParts, 0, st, v, step < 0 ? 1 : (int)gs.x,
+                               step));
         GELO_TRY(after_launch(ctx));
     }
-    cond_verdict_kernel<<<1, 64, 0, st>>>(v, bound, cond_out, ctx->status_dev, deferred ? 1 : 0);
+    GELO_TRY(launch_chained(ctx, cond_verdict_kernel, 1, 64, 0, st, v, bound, cond_out, ctx->status_dev, deferred ? 1 : 0));
     return after_launch(ctx);
 }
 

@@ -298,6 +298,7 @@ int launch_f32(gelo_ctx* ctx, const GemmParams& p, int slices, cudaStream_t st)
         GELO_CUDA_OK(cudaFuncSetAttribute(gemm_f32_kernel<TA, kN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(F32Shared<kN>)));
         attr_done[ctx->device] = true;
     }
+    // (not chained: 512 rows in fp32, non-orthogonal sample 700 us like this, 753 us chained)
     gemm_f32_kernel<TA, kN><<<dim3(ceil_div(p.N, kN), ceil_div(p.M, kF32M), slices), kThreads, sizeof(F32Shared<kN>), st>>>(p);
     return after_launch(ctx);
 }

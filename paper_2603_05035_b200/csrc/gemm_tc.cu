@@ -341,6 +341,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     const int n_tiles = (prm.N + BN - 1) / BN;
     const int mn_tiles = m_tiles * n_tiles;
 
+    chain_next();
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
         for (int a = 0; a < kAccStages; ++a) { mbar_init(acc_full_bar(a), 1); mbar_init(acc_empty_bar(a), kPair ? 2 * kEpiWarps : kEpiWarps); }
@@ -366,6 +367,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     if (kPair) cluster_sync(); else __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    chain_wait();
 
     // The tiles of a CTA (pair): the one it was launched for, then whatever the leader's producer gets from the hardware's
     // queue of CTAs not yet launched.  It hands each on through a ring; -1 ends.  The roles are at most kStages + 3 tiles apart (a tile
@@ -720,11 +722,13 @@ int launch_tiles_as(gelo_ctx* ctx, const CUtensorMap& a0, const CUtensorMap& a1,
         cfg.blockDim = dim3(kThreads);
         cfg.dynamicSmemBytes = Cfg::kSmemBytes;
         cfg.stream = st;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = kPair ? 1 : 0;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = chain_launches(ctx) ? 1 : 0;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = 2; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = kPair ? 2 : 1;
         GELO_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, a0, a1, b0, b1, c, q));
     }
     return after_launch(ctx);

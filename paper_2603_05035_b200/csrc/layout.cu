@@ -21,6 +21,8 @@ __global__ void __launch_bounds__(256) finish_mixing_kernel(int m, const float* 
                                                             const float* __restrict__ sign_diag, int ldg,
                                                             T* __restrict__ dst, T* __restrict__ dstT, int ldd)
 {
+    chain_next();
+    chain_wait();
     __shared__ float tile[32][33];
     const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -77,6 +79,8 @@ template <typename TS, typename TD>
 __global__ void __launch_bounds__(256) convert_kernel(int m, const TS* __restrict__ src, int lds, TD* __restrict__ dst, int ldd,
                                                       float* __restrict__ back, int ldb)
 {
+    chain_next();
+    chain_wait();
     const int c4 = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
     const int r = blockIdx.y;
     if (c4 >= m) return;
@@ -161,6 +165,8 @@ __global__ void __launch_bounds__(256) sum_planes_kernel(const float* __restrict
                                                          int ld, int rows, int cols, float scale, float* __restrict__ out,
                                                          int ldo, int round)
 {
+    chain_next();
+    chain_wait();
     const int c4 = (blockIdx.x * 256 + threadIdx.x) * 4;
     const int r = blockIdx.y;
     if (c4 >= cols) return;
@@ -312,6 +318,8 @@ int launch_sum_split(gelo_ctx* ctx, const float* planes, size_t plane, int parts
 __global__ void __launch_bounds__(256) split_tf32_kernel(const float* __restrict__ src, int lds, int rows, int cols,
                                                          float* __restrict__ hi, float* __restrict__ lo, int ldo)
 {
+    chain_next();
+    chain_wait();
     const int c4 = (blockIdx.x * 256 + threadIdx.x) * 4;
     if (c4 >= cols) return;
     for (int r = blockIdx.y; r < rows; r += gridDim.y) {
@@ -332,6 +340,8 @@ __global__ void __launch_bounds__(256) sum_planes_routed_kernel(const float* __r
                                                                 int cols, float* __restrict__ C0, float* __restrict__ C1,
                                                                 float* __restrict__ C2, int ldc, int csplit)
 {
+    chain_next();
+    chain_wait();
     const int c4 = (blockIdx.x * 256 + threadIdx.x) * 4;
     const int r = blockIdx.y;
     if (c4 >= cols) return;
@@ -350,7 +360,8 @@ int launch_sum_planes_routed(gelo_ctx* ctx, const float* planes, size_t plane, i
 {
     if (rows <= 0 || cols <= 0) return GELO_OK;
     dim3 grid(ceil_div(cols, 1024), rows);
-    sum_planes_routed_kernel<<<grid, 256, 0, st>>>(planes, plane, parts, cols, C[0], C[1], C[2], ldc, csplit);
+    GELO_TRY(launch_chained(ctx, sum_planes_routed_kernel, grid, 256, 0, st, planes, plane, parts, cols, C[0], C[1], C[2],
+                           ldc, csplit));
     return after_launch(ctx);
 }
 
@@ -362,7 +373,7 @@ int launch_split_tf32(gelo_ctx* ctx, const float* src, int lds, int rows, int co
         (reinterpret_cast<uintptr_t>(hi) & 15u) || (reinterpret_cast<uintptr_t>(lo) & 15u))
         return GELO_ERR_INVALID;
     dim3 grid(ceil_div(cols, 1024), rows < 4096 ? rows : 4096);
-    split_tf32_kernel<<<grid, 256, 0, st>>>(src, lds, rows, cols, hi, lo, ldo);
+    GELO_TRY(launch_chained(ctx, split_tf32_kernel, grid, 256, 0, st, src, lds, rows, cols, hi, lo, ldo));
     return after_launch(ctx);
 }
 
@@ -371,7 +382,8 @@ int launch_sum_planes(gelo_ctx* ctx, const float* planes, size_t plane, int part
 {
     if (rows <= 0 || cols <= 0) return GELO_OK;
     dim3 grid(ceil_div(cols, 1024), rows);
-    sum_planes_kernel<<<grid, 256, 0, st>>>(planes, plane, parts, ld, rows, cols, scale, out, ldo, round ? 1 : 0);
+    GELO_TRY(launch_chained(ctx, sum_planes_kernel, grid, 256, 0, st, planes, plane, parts, ld, rows, cols, scale, out, ldo,
+                           round ? 1 : 0));
     return after_launch(ctx);
 }
 
@@ -380,14 +392,14 @@ int launch_finish_mixing(gelo_ctx* ctx, int m, const float* src, int lds, const 
 {
     dim3 grid(ceil_div(m, 32), ceil_div(m, 32));
     if (dtype == GELO_BF16)
-        finish_mixing_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(m, src, lds, sign_diag, ldg,
-            static_cast<__nv_bfloat16*>(dst), static_cast<__nv_bfloat16*>(dstT), ldd);
+        GELO_TRY(launch_chained(ctx, finish_mixing_kernel<__nv_bfloat16>, grid, 256, 0, st, m, src, lds, sign_diag, ldg,
+                               static_cast<__nv_bfloat16*>(dst), static_cast<__nv_bfloat16*>(dstT), ldd));
     else if (dtype == GELO_F16)
-        finish_mixing_kernel<__half><<<grid, 256, 0, st>>>(m, src, lds, sign_diag, ldg,
-            static_cast<__half*>(dst), static_cast<__half*>(dstT), ldd);
+        GELO_TRY(launch_chained(ctx, finish_mixing_kernel<__half>, grid, 256, 0, st, m, src, lds, sign_diag, ldg,
+                               static_cast<__half*>(dst), static_cast<__half*>(dstT), ldd));
     else
-        finish_mixing_kernel<float><<<grid, 256, 0, st>>>(m, src, lds, sign_diag, ldg,
-            static_cast<float*>(dst), static_cast<float*>(dstT), ldd);
+        GELO_TRY(launch_chained(ctx, finish_mixing_kernel<float>, grid, 256, 0, st, m, src, lds, sign_diag, ldg,
+                               static_cast<float*>(dst), static_cast<float*>(dstT), ldd));
     return after_launch(ctx);
 }
 
@@ -399,11 +411,14 @@ int launch_narrow(gelo_ctx* ctx, int m, const float* src, int lds, int dtype, vo
         return GELO_ERR_INVALID;
     dim3 grid(ceil_div(m, 1024), m);
     if (dtype == GELO_BF16)
-        convert_kernel<float, __nv_bfloat16><<<grid, 256, 0, st>>>(m, src, lds, static_cast<__nv_bfloat16*>(dst), ldd, back, ldb);
+        GELO_TRY(launch_chained(ctx, convert_kernel<float, __nv_bfloat16>, grid, 256, 0, st, m, src, lds,
+                               static_cast<__nv_bfloat16*>(dst), ldd, back, ldb));
     else if (dtype == GELO_F16)
-        convert_kernel<float, __half><<<grid, 256, 0, st>>>(m, src, lds, static_cast<__half*>(dst), ldd, back, ldb);
+        GELO_TRY(launch_chained(ctx, convert_kernel<float, __half>, grid, 256, 0, st, m, src, lds, static_cast<__half*>(dst),
+                               ldd, back, ldb));
     else
-        convert_kernel<float, float><<<grid, 256, 0, st>>>(m, src, lds, static_cast<float*>(dst), ldd, back, ldb);
+        GELO_TRY(launch_chained(ctx, convert_kernel<float, float>, grid, 256, 0, st, m, src, lds, static_cast<float*>(dst),
+                               ldd, back, ldb));
     return after_launch(ctx);
 }
 

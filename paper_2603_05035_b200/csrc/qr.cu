@@ -501,6 +501,8 @@ template <int RM>
 __global__ void __launch_bounds__(8 * RM, 1)
 qr_small_kernel(float* __restrict__ G, int ld, int m, float* __restrict__ Q)
 {
+    chain_next();
+    chain_wait();
     constexpr int RPT = RM / 8;
     extern __shared__ float qs_smem[];
     float* Vs = qs_smem;                      // RM x RM: row j = reflector j over the rows
@@ -591,7 +593,7 @@ int launch_qr_small_rm(gelo_ctx* ctx, int m, float* G, int ld, float* Q, cudaStr
         GELO_CUDA_OK(cudaFuncSetAttribute(qr_small_kernel<RM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
         attr_done[ctx->device] = true;
     }
-    qr_small_kernel<RM><<<1, 8 * RM, smem, st>>>(G, ld, m, Q);
+    GELO_TRY(launch_chained(ctx, qr_small_kernel<RM>, 1, 8 * RM, smem, st, G, ld, m, Q));
     return after_launch(ctx);
 }
 

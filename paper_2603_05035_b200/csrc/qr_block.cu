@@ -487,6 +487,8 @@ __global__ void __cluster_dims__(kFactCtas, 1, 1) __launch_bounds__(kFactThreads
 block_factor_kernel(const float* __restrict__ Z, int ldz, float* P1, int ld, int ob, float* __restrict__ Tt,
                     int ldt, float* __restrict__ Dt, int ldd, float scale, float dscale, int round, int* __restrict__ status)
 {
+    chain_next();
+    chain_wait();
     extern __shared__ __align__(128) uint8_t fsm[];
     FactShared& s = *reinterpret_cast<FactShared*>(fsm);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, gid = lane >> 2, tig = lane & 3;
@@ -580,6 +582,8 @@ __global__ void __launch_bounds__(256)
 block_sum_kernel(const float* __restrict__ planes, size_t plane, int parts, int ldp, int rows, int cols, int c0, int ob, float scale, int round,
                  float* __restrict__ Z, int ldz, float* __restrict__ zero, int z_rows, int ld)
 {
+    chain_next();
+    chain_wait();
     const int idx = blockIdx.x * 256 + threadIdx.x;
     const int c4n = cols >> 2, o4n = ob >> 2;
     if (idx < rows * c4n) {
@@ -609,6 +613,8 @@ block_sum_kernel(const float* __restrict__ planes, size_t plane, int parts, int 
 __global__ void __launch_bounds__(256)
 start_q_kernel(float* __restrict__ Q, int ld, int m, int bf, const float* __restrict__ R)
 {
+    chain_next();
+    chain_wait();
     const int r = blockIdx.y;
     const int c = (blockIdx.x * 256 + threadIdx.x) * 4;
     if (c >= ld) return;
@@ -714,14 +720,14 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
             const size_t plane = (size_t)FB * ld;
             GELO_TRY(gemm(ob, ncs, nr, P, ld, true, rows, ld, false, tc.wf32, ld, false, 1.0f, slices(ob, ncs, kMaxKSplit), plane, &used));
             const int work = ob * (ncs >> 2) + r * (ob >> 2);
-            block_sum_kernel<<<ceil_div(work, 256), 256, 0, st>>>(tc.wf32, plane, used, ld, ob, ncs, r, ob, loss2, round, tc.w32[0], ld,
-                                                                 G + (size_t)s0 * ld + b0, r, ld);
+            GELO_TRY(launch_chained(ctx, block_sum_kernel, ceil_div(work, 256), 256, 0, st, tc.wf32, plane, used, ld, ob,
+                                   ncs, r, ob, loss2, round, tc.w32[0], ld, G + (size_t)s0 * ld + b0, r, ld));
             GELO_TRY(after_launch(ctx));
             float* Tb = Ts + (size_t)r * kSuper + r;
             float scale = 1.0f;                              // a power of two with scale^2 about nr
             while (2.0f * scale * scale < (float)nr) scale *= 2.0f;
-            block_factor_kernel<<<kFactCtas, kFactThreads, kFactSmemBytes, st>>>(tc.w32[0] + r, ld, P, ld, ob, Tb, kSuper, tc.t128, FB,
-                                                                                scale, loss1, round, ctx->status_dev);
+            GELO_TRY(launch_chained(ctx, block_factor_kernel, kFactCtas, kFactThreads, kFactSmemBytes, st, tc.w32[0] + r, ld,
+                                   P, ld, ob, Tb, kSuper, tc.t128, FB, scale, loss1, round, ctx->status_dev));
             GELO_TRY(after_launch(ctx));
             if (e - s > 1) {
                 // [X^T | . | W'] = T^T Z + D^T [V_< | . | C1], scaled up for the truncation of V in the next product
@@ -746,7 +752,7 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
     }
     // ---- the square that is left, and Q accumulated backwards, one superblock at a time ----
     GELO_TRY(launch_qr_small(ctx, m - bf, G + (size_t)bf * ld + bf, ld, Q + (size_t)bf * ld + bf, st));
-    start_q_kernel<<<dim3(ceil_div(ld, 1024), m), 256, 0, st>>>(Q, ld, m, bf, G);
+    GELO_TRY(launch_chained(ctx, start_q_kernel, dim3(ceil_div(ld, 1024), m), 256, 0, st, Q, ld, m, bf, G));
     GELO_TRY(after_launch(ctx));
     for (int s = (nblocks - 1) / per * per; s >= 0; s -= per) {
         const int e = (s + per < nblocks) ? s + per : nblocks;

@@ -30,6 +30,8 @@ __global__ void gaussian_kernel(int rows, int cols, int ld, uint64_t seed_value,
                                 uint32_t stream_id, uint32_t attempt, float scale, const float* __restrict__ base,
                                 float* __restrict__ out)
 {
+    chain_next();
+    chain_wait();
     // a replayed launch graph cannot change by-value arguments, so the seed may come from device memory
     const uint64_t seed = seed_ptr ? *seed_ptr : seed_value;
     const uint64_t total = (uint64_t)rows * (uint64_t)cols;
@@ -84,7 +86,8 @@ int launch_gaussian(gelo_ctx* ctx, int rows, int cols, int ld, uint64_t seed, ui
     const unsigned threads = 256;
     const uint64_t grid = ((total + 3) / 4 + threads - 1) / threads;
     if (grid > 0x7fffffffull) return GELO_ERR_INVALID;
-    gaussian_kernel<<<(unsigned)grid, threads, 0, st>>>(rows, cols, ld, seed, seed_dev, stream_id, attempt, scale, base, out);
+    GELO_TRY(launch_chained(ctx, gaussian_kernel, (unsigned)grid, threads, 0, st, rows, cols, ld, seed, seed_dev, stream_id,
+                           attempt, scale, base, out));
     return after_launch(ctx);
 }
 

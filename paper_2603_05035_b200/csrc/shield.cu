@@ -75,6 +75,8 @@ __device__ __forceinline__ float warp_row_norm(const T* __restrict__ h, int d, i
 template <typename T>
 __global__ void __launch_bounds__(256) row_norm_kernel(const T* __restrict__ H, int n, int d, float* __restrict__ norms)
 {
+    chain_next();
+    chain_wait();
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (row >= n) return;
@@ -85,6 +87,8 @@ __global__ void __launch_bounds__(256) row_norm_kernel(const T* __restrict__ H, 
 // med[0], med[1] = the elements of rank (n-1)/2 and n/2 (ties broken by index).
 __global__ void __launch_bounds__(256) median_rank_kernel(const float* __restrict__ norms, int n, float* __restrict__ med)
 {
+    chain_next();
+    chain_wait();
     __shared__ float tile[256];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const float mine = (i < n) ? norms[i] : 0.0f;
@@ -133,6 +137,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) shield_fill_kernel(T* __restrict__ S, int k, int d, float scale,
                                                           const float* __restrict__ med, uint64_t seed, int nu)
 {
+    chain_next();
+    chain_wait();
     const uint64_t total = (uint64_t)k * d;
     const uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t e0 = q << 2;
@@ -252,22 +258,28 @@ int run_shield_rows(gelo_ctx* ctx, const void* H, int n, int d, int k, float sca
         return launch_shield_small<float>(ctx, H, n, d, k, scale, seed, S, nu, st);
     }
     if (dtype == GELO_BF16)
-        row_norm_kernel<__nv_bfloat16><<<ceil_div(n, 8), 256, 0, st>>>(static_cast<const __nv_bfloat16*>(H), n, d, s.norms);
+        GELO_TRY(launch_chained(ctx, row_norm_kernel<__nv_bfloat16>, ceil_div(n, 8), 256, 0, st, static_cast<const
+                               __nv_bfloat16*>(H), n, d, s.norms));
     else if (dtype == GELO_F16)
-        row_norm_kernel<__half><<<ceil_div(n, 8), 256, 0, st>>>(static_cast<const __half*>(H), n, d, s.norms);
+        GELO_TRY(launch_chained(ctx, row_norm_kernel<__half>, ceil_div(n, 8), 256, 0, st, static_cast<const __half*>(H), n,
+                               d, s.norms));
     else
-        row_norm_kernel<float><<<ceil_div(n, 8), 256, 0, st>>>(static_cast<const float*>(H), n, d, s.norms);
+        GELO_TRY(launch_chained(ctx, row_norm_kernel<float>, ceil_div(n, 8), 256, 0, st, static_cast<const float*>(H), n, d,
+                               s.norms));
     GELO_TRY(after_launch(ctx));
-    median_rank_kernel<<<ceil_div(n, 256), 256, 0, st>>>(s.norms, n, s.med);
+    GELO_TRY(launch_chained(ctx, median_rank_kernel, ceil_div(n, 256), 256, 0, st, s.norms, n, s.med));
     GELO_TRY(after_launch(ctx));
     const uint64_t blocks = ((uint64_t)k * d + 3) / 4;
     const unsigned grid = (unsigned)((blocks + 255) / 256);
     if (dtype == GELO_BF16)
-        shield_fill_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(static_cast<__nv_bfloat16*>(S), k, d, scale, s.med, seed, nu);
+        GELO_TRY(launch_chained(ctx, shield_fill_kernel<__nv_bfloat16>, grid, 256, 0, st, static_cast<__nv_bfloat16*>(S), k,
+                               d, scale, s.med, seed, nu));
     else if (dtype == GELO_F16)
-        shield_fill_kernel<__half><<<grid, 256, 0, st>>>(static_cast<__half*>(S), k, d, scale, s.med, seed, nu);
+        GELO_TRY(launch_chained(ctx, shield_fill_kernel<__half>, grid, 256, 0, st, static_cast<__half*>(S), k, d, scale,
+                               s.med, seed, nu));
     else
-        shield_fill_kernel<float><<<grid, 256, 0, st>>>(static_cast<float*>(S), k, d, scale, s.med, seed, nu);
+        GELO_TRY(launch_chained(ctx, shield_fill_kernel<float>, grid, 256, 0, st, static_cast<float*>(S), k, d, scale, s.med,
+                               seed, nu));
     return after_launch(ctx);
 }
 
