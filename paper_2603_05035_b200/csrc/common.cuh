@@ -198,6 +198,8 @@ int launch_gemm_tc_split_k(gelo_ctx*, int M, int N, int K, const void* Ahi, cons
 int launch_gemm_tf32(gelo_ctx*, int M, int N, int K, const float* A, int lda, bool a_mn, const float* B, int ldb,
                      bool subtract, float* C, int ldc, bool round_out, float out_scale, int ksplit, size_t plane, int* used,
                      cudaStream_t, float diag_sub = 0.0f, float post_scale = 1.0f);
+// columns per tile that the tensor-core products choose (gemm_tc.cu)
+int gemm_tile_cols(const gelo_ctx*, int M, int N, int K, int slices, int bytes, bool lanes_share, int least);
 // C (M x N) = out_scale * (A0 B0 + A1 B1) rounded to tf32; A0, A1: M x K, B0, B1: K x N, row-major
 int launch_gemm_tf32_dual(gelo_ctx*, int M, int N, int K, const float* A0, int lda0, const float* B0, int ldb0, const float* A1,
                           int lda1, const float* B1, int ldb1, float* C, int ldc, float out_scale, cudaStream_t);

@@ -744,6 +744,16 @@ int launch_tiles(gelo_ctx* ctx, bool pair, const CUtensorMap& a0, const CUtensor
     return launch_tiles_as<BN, kStaging, kTf32, kAMn, kF8, false>(ctx, a0, a1, b0, b1, c, p, flops, st);
 }
 
+// tf32 products on tiles of 64, 128 or 256 columns
+template <bool kStaging, bool kAMn>
+int launch_tf32_cols(gelo_ctx* ctx, int cols, bool pair, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0,
+                     const CUtensorMap& b1, const CUtensorMap& c, const TcParams& p, double flops, cudaStream_t st)
+{
+    if (cols == 64) return launch_tiles<64, kStaging, true, kAMn>(ctx, false, a0, a1, b0, b1, c, p, flops, st);
+    if (cols == 128) return launch_tiles<128, kStaging, true, kAMn>(ctx, false, a0, a1, b0, b1, c, p, flops, st);
+    return launch_tiles<256, kStaging, true, kAMn>(ctx, pair, a0, a1, b0, b1, c, p, flops, st);
+}
+
 // fp32 tensor map of the matrix that the subtracting epilogue reduces into: 32 x 32 boxes, 128-byte swizzle.
 bool make_map_f32_box(gelo_ctx* ctx, CUtensorMap* map, const void* ptr, uint64_t cols, uint64_t rows, uint64_t ld,
                       uint32_t box_rows = 32, bool chunk32 = false)
@@ -762,6 +772,22 @@ bool make_map_f32_box(gelo_ctx* ctx, CUtensorMap* map, const void* ptr, uint64_t
 }
 
 }  // namespace
+
+// Columns of a tile of an M x N x K product of elements of `bytes` bytes.  A product that fills no more than a part of the GPU is
+// bound by what one tile takes from its first copy to its last store, and most of that goes with the columns: 128 x 512 x (2 x 128)
+// in tf32 takes 11.4 us on 256 columns per tile and 7.7 us on 64.  So the narrowest tiles that still run in one round are
+// taken, as long as what all of them read, which narrow tiles multiply, does not become the bound (512 x 1638 x 2150 reads 170 MB on
+// 64 columns: 27 us, against 17 us on 256 with the depth in four slices).  In the lanes of a batch SM time counts, and 256 columns
+// use it best.
+int gemm_tile_cols(const gelo_ctx* ctx, int M, int N, int K, int slices, int bytes, bool lanes_share, int least)
+{
+    if (ctx->tc_update_ctas > 0 && lanes_share) return 256;
+    for (int cols = least; cols < 256; cols *= 2) {
+        const long tiles = (long)ceil_div(M, BM) * ceil_div(N, cols);
+        if (tiles * slices <= ctx->sm_count && (double)tiles * K * (BM + cols) * bytes <= 48e6) return cols;
+    }
+    return 256;
+}
 
 bool gemm_tc_supports(const GemmArgs& g)
 {
@@ -782,8 +808,9 @@ int launch_gemm_tc(gelo_ctx* ctx, const GemmArgs& g, cudaStream_t st)
     if (!ctx->tmap_encode) return GELO_ERR_CUDA;
     constexpr int BN = 256;
     const int rows_first = g.B2 ? g.b_split : g.K;
-    const bool pair = use_pair(ctx, g.M, g.N, 1, false, TC_STORE_BF16);
-    const uint32_t cols = pair ? BN / 2 : BN;                 // columns of B per CTA
+    const int wide = gemm_tile_cols(ctx, g.M, g.N, g.K, 1, 2, false, 128);
+    const bool pair = wide == BN && use_pair(ctx, g.M, g.N, 1, false, TC_STORE_BF16);
+    const uint32_t cols = pair ? BN / 2 : wide;               // columns of B per CTA
     CUtensorMap ma, mb, mb2;
     if (!make_map(ctx, &ma, g.A, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda, BK, BM)) return GELO_ERR_CUDA;
     bool b3d = false, b3d2 = false;
@@ -812,6 +839,7 @@ int launch_gemm_tc(gelo_ctx* ctx, const GemmArgs& g, cudaStream_t st)
     p.C0 = g.C[0]; p.C1 = g.C[g.nsplit > 1 ? 1 : 0]; p.C2 = g.C[g.nsplit > 2 ? 2 : 0];
     p.ldc = g.ldc; p.csplit = g.N / g.nsplit; p.lde = 0;
     p.status = ctx->status_dev;
+    if (wide == 128) return launch_tiles<128, false>(ctx, false, ma, ma, mb, mb2, ma, p, 2.0 * g.M * (double)g.N * g.K, st);
     return launch_tiles<BN, false>(ctx, pair, ma, ma, mb, mb2, ma, p, 2.0 * g.M * (double)g.N * g.K, st);
 }
 
@@ -933,8 +961,9 @@ int launch_gemm_tf32(gelo_ctx* ctx, int M, int N, int K, const float* A, int lda
     } else {
         ksplit = 1;
     }
-    const bool pair = use_pair(ctx, M, N, ksplit, false, subtract ? TC_SUB_F32 : TC_STORE_F32);
-    const uint32_t cols = pair ? 128 : 256;
+    const int wide = gemm_tile_cols(ctx, M, N, K, ksplit, 4, true, 64);
+    const bool pair = wide == 256 && use_pair(ctx, M, N, ksplit, false, subtract ? TC_SUB_F32 : TC_STORE_F32);
+    const uint32_t cols = pair ? 128 : wide;
     CUtensorMap ma, mb, mc;
     bool a3d = false, b3d = false;
     const bool a_ok = a_mn ? make_map_nmajor(ctx, &ma, A, 4, true, (uint64_t)M, (uint64_t)K, (uint64_t)lda, 32, BM, &a3d)
@@ -956,14 +985,14 @@ int launch_gemm_tf32(gelo_ctx* ctx, int M, int N, int K, const float* A, int lda
     if (subtract) {
         if (!make_map_f32_box(ctx, &mc, C, (uint64_t)N, (uint64_t)M, (uint64_t)ldc, 32)) return GELO_ERR_CUDA;
         p.mode = TC_SUB_F32;
-        return a_mn ? launch_tiles<256, true, true, true>(ctx, pair, ma, ma, mb, mb, mc, p, flops, st)
-                    : launch_tiles<256, true, true, false>(ctx, pair, ma, ma, mb, mb, mc, p, flops, st);
+        return a_mn ? launch_tf32_cols<true, true>(ctx, wide, pair, ma, ma, mb, mb, mc, p, flops, st)
+                    : launch_tf32_cols<true, false>(ctx, wide, pair, ma, ma, mb, mb, mc, p, flops, st);
     }
     p.mode = TC_STORE_F32;
     if (ksplit > 1) { p.ksplit = ksplit; p.kb_per_split = per; p.plane = (long long)plane; }
     if (used) *used = p.ksplit;
-    return a_mn ? launch_tiles<256, false, true, true>(ctx, pair, ma, ma, mb, mb, mc, p, flops, st)
-                : launch_tiles<256, false, true, false>(ctx, pair, ma, ma, mb, mb, mc, p, flops, st);
+    return a_mn ? launch_tf32_cols<false, true>(ctx, wide, pair, ma, ma, mb, mb, mc, p, flops, st)
+                : launch_tf32_cols<false, false>(ctx, wide, pair, ma, ma, mb, mb, mc, p, flops, st);
 }
 
 // C = out_scale * (A0 B0 + A1 B1) rounded to tf32: two products of the same sizes in one accumulator.
@@ -975,8 +1004,9 @@ int launch_gemm_tf32_dual(gelo_ctx* ctx, int M, int N, int K, const float* A0, i
     if ((lda0 % 4) || (lda1 % 4) || (ldb0 % 4) || (ldb1 % 4) || (ldc % 4) || (N % 8) || !aligned16(A0) || !aligned16(A1) ||
         !aligned16(B0) || !aligned16(B1) || !aligned16(C))
         return GELO_ERR_INVALID;
-    const bool pair = use_pair(ctx, M, N, 1, false, TC_STORE_F32);
-    const uint32_t cols = pair ? 128 : 256;
+    const int wide = gemm_tile_cols(ctx, M, N, 2 * K, 1, 4, true, 64);
+    const bool pair = wide == 256 && use_pair(ctx, M, N, 1, false, TC_STORE_F32);
+    const uint32_t cols = pair ? 128 : wide;
     CUtensorMap a0, a1, b0, b1;
     bool b3d = false, b3d1 = false;
     if (!make_map_f32_box(ctx, &a0, A0, (uint64_t)K, (uint64_t)M, (uint64_t)lda0, BM) ||
@@ -998,7 +1028,7 @@ int launch_gemm_tf32_dual(gelo_ctx* ctx, int M, int N, int K, const float* A0, i
     p.out_scale = out_scale; p.post_scale = 1.0f;
     p.C0 = C; p.ldc = ldc;
     p.mode = TC_STORE_F32;
-    return launch_tiles<256, false, true, false>(ctx, pair, a0, a1, b0, b1, a0, p, 4.0 * M * (double)N * K, st);
+    return launch_tf32_cols<false, false>(ctx, wide, pair, a0, a1, b0, b1, a0, p, 4.0 * M * (double)N * K, st);
 }
 
 // D (m x m bf16, stride ldd) = post_scale * (out_scale * Q^T Q - diag_sub I) for a row-major fp32 Q (stride ld): one
@@ -1070,8 +1100,9 @@ int launch_gemm_affine16(gelo_ctx* ctx, int dtype, int M, int N, int K, const vo
     if ((lda % 8) || (ldb % 8) || (ldc % 8) || (N % 8) || (ldadd % 8) || !aligned16(A) || !aligned16(B) || !aligned16(C) ||
         !aligned16(add))
         return GELO_ERR_INVALID;
-    const bool pair = use_pair(ctx, M, N, 1, false, TC_AFFINE16);
-    const uint32_t cols = pair ? 128 : 256;
+    const int wide = gemm_tile_cols(ctx, M, N, K, 1, 2, true, 128);
+    const bool pair = wide == 256 && use_pair(ctx, M, N, 1, false, TC_AFFINE16);
+    const uint32_t cols = pair ? 128 : wide;
     CUtensorMap ma, mb;
     bool b3d = false;
     if (!make_map(ctx, &ma, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, BM) ||
@@ -1089,6 +1120,7 @@ int launch_gemm_affine16(gelo_ctx* ctx, int dtype, int M, int N, int K, const vo
     p.add = add; p.ldadd = ldadd;
     p.C0 = C; p.ldc = ldc; p.csplit = N;
     p.status = ctx->status_dev;
+    if (wide == 128) return launch_tiles<128, false>(ctx, false, ma, ma, mb, mb, ma, p, 2.0 * M * (double)N * K, st);
     return launch_tiles<256, false>(ctx, pair, ma, ma, mb, mb, ma, p, 2.0 * M * (double)N * K, st);
 }
 

@@ -648,10 +648,15 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
     const int round = exact ? 0 : 1;
 
     // V^T C with few output tiles: the rows are cut into slices whose partial products are summed in a fixed order
-    auto slices = [&](int M, int N, int most) {
-        const int tiles = exact ? ceil_div(M, 64) * ceil_div(N, 64) : ceil_div(M, 128) * ceil_div(N, 256);
-        int want = (2 * tiles >= width) ? 1 : ceil_div(2 * width, tiles);
-        return want > most ? most : want;
+    auto slices = [&](int M, int N, int K, int most) {
+        int want;
+        if (!exact && gemm_tile_cols(ctx, M, N, K, 1, 4, true, 64) == 64) {
+            want = width / (ceil_div(M, 128) * ceil_div(N, 64));      // one round of narrow tiles
+        } else {
+            const int tiles = exact ? ceil_div(M, 64) * ceil_div(N, 64) : ceil_div(M, 128) * ceil_div(N, 256);
+            want = (2 * tiles >= width) ? 1 : ceil_div(2 * width, tiles);
+        }
+        return want < 1 ? 1 : (want > most ? most : want);
     };
     // C = scale * op(A) B or C -= op(A) B, as launch_gemm_tf32 or in fp32
     auto gemm = [&](int M, int N, int K, const float* A, int lda, bool a_mn, const float* B, int ldb, bool subtract, float* C, int ldc,
@@ -676,7 +681,7 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
         const int nr = m - c0;
         const int nc8 = (nc + 7) & ~7;
         const float* V = G + (size_t)c0 * ld + c0;
-        const int want = slices(kv, nc8, kSuperKSplit);
+        const int want = slices(kv, nc8, nr, kSuperKSplit);
         if (want <= 1) {
             GELO_TRY(gemm(kv, nc8, nr, V, ld, true, C, ld, false, tc.w32[0], ld, true, loss2, 1, 0, nullptr));
         } else {
@@ -718,7 +723,7 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
             float* Wb = tc.w32[1] + (size_t)(b - s) * FB * ld;
             int used = 0;
             const size_t plane = (size_t)FB * ld;
-            GELO_TRY(gemm(ob, ncs, nr, P, ld, true, rows, ld, false, tc.wf32, ld, false, 1.0f, slices(ob, ncs, kMaxKSplit), plane, &used));
+            GELO_TRY(gemm(ob, ncs, nr, P, ld, true, rows, ld, false, tc.wf32, ld, false, 1.0f, slices(ob, ncs, nr, kMaxKSplit), plane, &used));
             const int work = ob * (ncs >> 2) + r * (ob >> 2);
             GELO_TRY(launch_chained(ctx, block_sum_kernel, ceil_div(work, 256), 256, 0, st, tc.wf32, plane, used, ld, ob,
                                    ncs, r, ob, loss2, round, tc.w32[0], ld, G + (size_t)s0 * ld + b0, r, ld));
