@@ -117,9 +117,21 @@ Layout carve(Arena& a, int n, int k, int d, int p, int dtype, bool host_staging)
     return L;
 }
 
-// Lanes other than the first hold only what sampling needs, except for small batches (m <= 128), whose lanes also
-// form their own shield rows and mixed matrix: those get an S and a U of their own (d columns wide).
-inline int lane_width(int n, int k, int d) { return (n + k <= 128) ? d : 0; }
+// Lanes other than the first hold only what sampling needs, except where whole calls run on the lanes: small batches
+// (m <= 128, S and U of d columns) and 16-bit calls of up to kLaneCallRows rows (S, U and Y').
+// kLaneCallRows: up to here a product leaves SMs idle in its first and last tiles and the shield rows are three short launches,
+// so one call after the other on the caller's stream is a chain of its own: 32 layers of 315 rows on 16 lanes 3.50 -> 2.62 ms, 2150
+// rows on 32 lanes 22.0 -> 20.2 ms, eight of 1050 rows 1.95 -> 1.78 ms.  Beyond, the products fill the GPU by themselves, and Y' alone is
+// 106 MB per lane at 4300 rows.  With four lanes or less the lanes are the bound and only sample (2150 rows 27.6 ms like that,
+// 28.0 ms with whole calls).
+constexpr int kLaneCallRows = 2304;
+inline bool lane_calls(int m, int dtype) { return dtype != GELO_F32 && m > 128 && m <= kLaneCallRows; }
+inline Layout carve_lane(Arena& a, int n, int k, int d, int p, int dtype)
+{
+    const int m = n + k;
+    const bool whole = lane_calls(m, dtype);
+    return carve(a, n, k, (whole || m <= 128) ? d : 0, whole ? p : 0, dtype, false);
+}
 
 bool carve_ctx(gelo_ctx* ctx, int n, int k, int d, int p, int dtype, bool host_staging, Layout* out)
 {
@@ -444,7 +456,7 @@ int offload_batch_impl(gelo_ctx* ctx, int calls, const void* const* H, const voi
     a.cap = ctx->ws_bytes;
     Layout L[kMaxLanes];
     L[0] = carve(a, n, k, d, p, dtype, host);
-    for (int i = 1; i < D; ++i) L[i] = carve(a, n, k, lane_width(n, k, d), 0, dtype, false);
+    for (int i = 1; i < D; ++i) L[i] = carve_lane(a, n, k, d, p, dtype);
     if (!a.ok) return GELO_ERR_WORKSPACE;
     const size_t es = elem_size(dtype);
     const bool split = K[0] != nullptr;
@@ -452,9 +464,10 @@ int offload_batch_impl(gelo_ctx* ctx, int calls, const void* const* H, const voi
     // A small batch (the decode shape) is a stream of W per call and little else; its other launches are short and
     // latency-bound.  There the WHOLE call runs on its lane (sampling, shield rows, mixing, fused projection + unmixing,
     // on the lane's own S and U): the weight streams of different calls overlap at their seams and the caller's stream
-    // only joins the lanes at the end of the batch.
-    bool small = !host && D > 1 && ctx->fuse_small && lane_width(n, k, d) > 0 && mix_small_supports(n, k, d, dtype) &&
-                 project_unmix_supports(ctx, n, k, d, p, dtype, L[0].ldi, split ? 3 : 1);
+    // only joins the lanes at the end of the batch.  So do 16-bit calls of a medium size (see kLaneCallRows).
+    bool small = !host && D > 1 &&
+                 ((D > 4 && lane_calls(m, dtype)) || (ctx->fuse_small && m <= 128 && mix_small_supports(n, k, d, dtype) &&
+                                           project_unmix_supports(ctx, n, k, d, p, dtype, L[0].ldi, split ? 3 : 1)));
     for (int i = 0; i < calls && small; ++i) small = !misaligned(H[i]);
     if (small) {
         // calls that share an output buffer are promised call order: keep those on the caller's stream
@@ -504,7 +517,7 @@ int offload_batch_impl(gelo_ctx* ctx, int calls, const void* const* H, const voi
             if (chained && i < D) GELO_CUDA_OK(cudaStreamWaitEvent(ls, ctx->batch_start, 0));
             GELO_TRY(run_shield_rows(ctx, H[i], n, d, k, shield_scale, seeds[i], dtype, L[l].S, L[l].sh, ls, ctx->shield_nu));
             GELO_TRY(mix_impl(ctx, L[l].A, L[l].ldi, H[i], k > 0 ? L[l].S : nullptr, n, k, d, dtype, L[l].U, ls, nullptr));
-            GELO_TRY(project_and_unmix(ctx, L[l].U, W[i], L[l].Ainv, L[l].ldi, nullptr, n, k, d, p, dtype, Q[i],
+            GELO_TRY(project_and_unmix(ctx, L[l].U, W[i], L[l].Ainv, L[l].ldi, L[l].Yp, n, k, d, p, dtype, Q[i],
                                        split ? K[i] : nullptr, split ? V[i] : nullptr, ls, nullptr));
         }
         for (int l = 0; l < D; ++l) {
@@ -663,30 +676,41 @@ int offload_blockdiag_impl(gelo_ctx* ctx, int calls, const void* const* H, const
         cudaStream_t ls = ctx->lane_stream[l];
         if (v >= D) GELO_CUDA_OK(cudaStreamWaitEvent(ls, ctx->lane_free[l], 0));
         const uint64_t seed = seeds[c] ^ (0x9E3779B97F4A7C15ull * (uint64_t)(j + 1));     // a fresh A_j per group and call
-        GELO_TRY(sample_on_lane(ctx, L[l], l, P.nd[j] + P.ns[j], GELO_ORTHOGONAL, seed, dtype, ls));
-        GELO_CUDA_OK(cudaEventRecord(ctx->lane_ready[l], ls));
-        return GELO_OK;
+        return sample_on_lane(ctx, L[l], l, P.nd[j] + P.ns[j], GELO_ORTHOGONAL, seed, dtype, ls);
     };
     for (long long v = 0; v < total && v < D; ++v) GELO_TRY(enqueue_sample(v));
     for (int c = 0; c < calls; ++c) {
         const char* Hc = static_cast<const char*>(H[c]);
         GELO_TRY(run_shield_rows(ctx, Hc, n, d, k, shield_scale, seeds[c], dtype, S, sh, st, ctx->shield_nu));
+        // the groups' mixing and unmixing products are short: each goes to its lane, beside those of the other groups
+        GELO_CUDA_OK(cudaEventRecord(ctx->batch_start, st));
         for (int j = 0; j < P.nb; ++j) {
             const int l = (int)(((long long)c * P.nb + j) % D);
             const int u0 = P.d0[j] + P.s0[j];
-            GELO_CUDA_OK(cudaStreamWaitEvent(st, ctx->lane_ready[l], 0));
+            cudaStream_t ls = ctx->lane_stream[l];
+            GELO_CUDA_OK(cudaStreamWaitEvent(ls, ctx->batch_start, 0));
             GELO_TRY(mix_impl(ctx, L[l].A, L[l].ldi, Hc + (size_t)P.d0[j] * d * es, P.ns[j] ? S + (size_t)P.s0[j] * d * es : nullptr,
-                              P.nd[j], P.ns[j], d, dtype, U + (size_t)u0 * d * es, st));
+                              P.nd[j], P.ns[j], d, dtype, U + (size_t)u0 * d * es, ls));
+            GELO_CUDA_OK(cudaEventRecord(ctx->lane_ready[l], ls));
+            GELO_CUDA_OK(cudaStreamWaitEvent(st, ctx->lane_ready[l], 0));
         }
         GELO_TRY(project_impl(ctx, U, W[c], m, d, p, dtype, Yp, st));
+        GELO_CUDA_OK(cudaEventRecord(ctx->batch_start, st));
         for (int j = 0; j < P.nb; ++j) {
             const int l = (int)(((long long)c * P.nb + j) % D);
             const int u0 = P.d0[j] + P.s0[j];
             const size_t qoff = (size_t)P.d0[j] * qcols * es;
+            cudaStream_t ls = ctx->lane_stream[l];
+            GELO_CUDA_OK(cudaStreamWaitEvent(ls, ctx->batch_start, 0));
             GELO_TRY(unmix_impl(ctx, L[l].Ainv, L[l].ldi, Yp + (size_t)u0 * p * es, P.nd[j], P.ns[j], p, dtype,
                                 static_cast<char*>(Q[c]) + qoff, split ? static_cast<char*>(K[c]) + qoff : nullptr,
-                                split ? static_cast<char*>(V[c]) + qoff : nullptr, st));
-            GELO_CUDA_OK(cudaEventRecord(ctx->lane_free[l], st));
+                                split ? static_cast<char*>(V[c]) + qoff : nullptr, ls));
+            GELO_CUDA_OK(cudaEventRecord(ctx->lane_free[l], ls));
+        }
+        // (the next call's shield rows and projection reuse S, U and Y')
+        for (int j = 0; j < P.nb; ++j) {
+            const int l = (int)(((long long)c * P.nb + j) % D);
+            GELO_CUDA_OK(cudaStreamWaitEvent(st, ctx->lane_free[l], 0));
         }
         for (int j = 0; j < P.nb; ++j) {
             const long long v = (long long)c * P.nb + j + D;
@@ -722,7 +746,7 @@ size_t batch_workspace(int n, int k, int d, int p, int dtype, int lanes)
     Arena a;
     a.cap = ~size_t(0) >> 1;
     carve(a, n, k, d, p, dtype, true);
-    for (int i = 1; i < lanes; ++i) carve(a, n, k, lane_width(n, k, d), 0, dtype, false);
+    for (int i = 1; i < lanes; ++i) carve_lane(a, n, k, d, p, dtype);
     return a.off + 256;
 }
 

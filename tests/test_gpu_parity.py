@@ -1143,3 +1143,28 @@ def test_fp32_products_of_any_depth(ctx, oracle, n, k, kind):
     ref = H.double() @ W.double()
     # the fp32 path's tolerance
     assert ((Q.double() - ref).norm() / ref.norm()).item() <= TOL["f32"]
+
+
+# whole calls on the lanes: one over the small path, the last size that takes it and the first that does not; fewer calls than
+# lanes, a second round per lane, results in one buffer that every call overwrites (call order is promised)
+@pytest.mark.parametrize("n,k,calls,shared", [(120, 9, 6, False), (2200, 104, 5, False), (2201, 104, 5, False), (300, 15, 13, False), (300, 15, 7, True)])
+def test_medium_batches_match_single_calls(n, k, calls, shared):
+    d, p, dt = 256, 384, "bf16"
+    c = binding.Context(0)
+    c.set_lanes(6)
+    c.ensure_batch_workspace(n, k, d, p, dt, 6)
+    H = [inputs.make_hidden(n, d, dt, 40 + i, True, "cuda") for i in range(calls)]
+    W = [inputs.make_weight(d, p, dt, 90 + i, "cuda") for i in range(calls)]
+    out = torch.zeros((1 if shared else calls, 3, n, p // 3), dtype=torch.bfloat16, device="cuda")
+    pick = lambda j: [out[0 if shared else i, j] for i in range(calls)]
+    kinds = [(ORTHOGONAL, NONORTHOGONAL)[i % 2] for i in range(calls)]
+    seeds = [500 + i for i in range(calls)]
+    for _ in range(2):                                            # the second batch chains onto the first
+        c.qkv_offload_batch(H, W, n, k, d, p, kinds, seeds, 10.0, dt, pick(0), pick(1), pick(2))
+    torch.cuda.synchronize()
+    assert c.last_status() == binding.OK
+    for i in ([calls - 1] if shared else range(calls)):
+        ref = H[i].double() @ W[i].double()
+        got = torch.cat([out[0 if shared else i, j] for j in range(3)], dim=1).double()
+        assert ((got - ref).norm() / ref.norm()).item() <= TOL[dt]
+    c.close()
