@@ -783,6 +783,9 @@ int gelo_create(gelo_ctx** out, int device)
                    cudaEventCreateWithFlags(&ctx->lane_ready[l], cudaEventDisableTiming) == cudaSuccess &&
                    cudaEventCreateWithFlags(&ctx->lane_free[l], cudaEventDisableTiming) == cudaSuccess;
     lanes_ok = lanes_ok && cudaMalloc(&ctx->lane_seed_dev, kMaxLanes * 8 * sizeof(uint64_t)) == cudaSuccess;
+    lanes_ok = lanes_ok && cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking) == cudaSuccess &&
+               cudaEventCreateWithFlags(&ctx->side_from, cudaEventDisableTiming) == cudaSuccess &&
+               cudaEventCreateWithFlags(&ctx->side_done, cudaEventDisableTiming) == cudaSuccess;
     lanes_ok = lanes_ok && cudaStreamCreateWithFlags(&ctx->copy_in, cudaStreamNonBlocking) == cudaSuccess &&
                cudaStreamCreateWithFlags(&ctx->copy_out, cudaStreamNonBlocking) == cudaSuccess;
     for (int b = 0; b < 2 && lanes_ok; ++b)
@@ -810,6 +813,9 @@ int gelo_destroy(gelo_ctx* ctx)
         if (ctx->lane_free[l]) cudaEventDestroy(ctx->lane_free[l]);
     }
     drop_graphs(ctx);
+    if (ctx->side) cudaStreamDestroy(ctx->side);
+    if (ctx->side_from) cudaEventDestroy(ctx->side_from);
+    if (ctx->side_done) cudaEventDestroy(ctx->side_done);
     if (ctx->copy_in) { cudaStreamSynchronize(ctx->copy_in); cudaStreamDestroy(ctx->copy_in); }
     if (ctx->copy_out) { cudaStreamSynchronize(ctx->copy_out); cudaStreamDestroy(ctx->copy_out); }
     for (int b = 0; b < 2; ++b) {

@@ -70,6 +70,8 @@ struct gelo_ctx {
     cudaEvent_t lane_ready[gelo::kMaxLanes] = {};   // A and A^-1 of the lane are complete
     cudaEvent_t lane_free[gelo::kMaxLanes] = {};    // the products that read them have been enqueued and finished
     cudaEvent_t batch_start = nullptr;
+    cudaStream_t side = nullptr;                    // branches of recorded sampling graphs
+    cudaEvent_t side_from = nullptr, side_done = nullptr;
     // a batched call may chain onto the previous one (lanes wait for their own lane_free events only) when
     // nothing else has touched the workspace in between
     bool chain_valid = false;

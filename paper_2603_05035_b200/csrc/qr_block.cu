@@ -609,15 +609,15 @@ block_sum_kernel(const float* __restrict__ planes, size_t plane, int parts, int 
 
 // Q <- diag(-I, Q_f S): the columns of the blocks start as -e_j (their R has a negative diagonal, and A takes the
 // factor whose R is positive), the last f columns as the Householder factor Qf (f x f at its place in Q) with the
-// columns flipped where its R (diagonal of Rf) is negative.  Everything else is cleared.
+// columns flipped where its R (diagonal of Rf) is negative.  Everything else is cleared.  Columns c0 .. c_end - 1 of it.
 __global__ void __launch_bounds__(256)
-start_q_kernel(float* __restrict__ Q, int ld, int m, int bf, const float* __restrict__ R)
+start_q_kernel(float* __restrict__ Q, int ld, int m, int bf, const float* __restrict__ R, int c0, int c_end)
 {
     chain_next();
     chain_wait();
     const int r = blockIdx.y;
-    const int c = (blockIdx.x * 256 + threadIdx.x) * 4;
-    if (c >= ld) return;
+    const int c = c0 + (blockIdx.x * 256 + threadIdx.x) * 4;   // (c0, bf and c_end are multiples of four)
+    if (c >= c_end) return;
     float v[4];
     float* p = Q + (size_t)r * ld + c;
 #pragma unroll
@@ -646,6 +646,22 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
     const float loss1 = exact ? 1.0f : 1.0f + kTf32TruncLoss, loss2 = loss1 * loss1;
     const int width = ctx->tc_update_ctas > 0 ? ctx->tc_update_ctas : ctx->sm_count;   // CTAs one launch may use
     const int round = exact ? 0 : 1;
+    // In a recorded graph of a call that runs alone, what nobody waits for yet goes into branches of the graph (on the context's side
+    // stream): the merges, which are needed at the end of a superblock, and the last square with its columns of Q.
+    // 2150 rows orthogonal, one call 1.61 -> 1.56 ms; 4300 non-orthogonal 4.51 -> 4.41 ms.
+    const bool fork = ctx->recording && ctx->tc_update_ctas == 0;
+    cudaStream_t cur = st;                                   // where the products go
+    auto branch = [&]() -> int {
+        GELO_CUDA_OK(cudaEventRecord(ctx->side_from, st));
+        GELO_CUDA_OK(cudaStreamWaitEvent(ctx->side, ctx->side_from, 0));
+        cur = ctx->side;
+        return GELO_OK;
+    };
+    auto join = [&]() -> int {
+        GELO_CUDA_OK(cudaEventRecord(ctx->side_done, ctx->side));
+        GELO_CUDA_OK(cudaStreamWaitEvent(st, ctx->side_done, 0));
+        return GELO_OK;
+    };
 
     // V^T C with few output tiles: the rows are cut into slices whose partial products are summed in a fixed order
     auto slices = [&](int M, int N, int K, int most) {
@@ -661,7 +677,7 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
     // C = scale * op(A) B or C -= op(A) B, as launch_gemm_tf32 or in fp32
     auto gemm = [&](int M, int N, int K, const float* A, int lda, bool a_mn, const float* B, int ldb, bool subtract, float* C, int ldc,
                     bool round_out, float scale, int ksplit, size_t plane, int* used) -> int {
-        if (!exact) return launch_gemm_tf32(ctx, M, N, K, A, lda, a_mn, B, ldb, subtract, C, ldc, round_out, scale, ksplit, plane, used, st);
+        if (!exact) return launch_gemm_tf32(ctx, M, N, K, A, lda, a_mn, B, ldb, subtract, C, ldc, round_out, scale, ksplit, plane, used, cur);
         if (M <= 0 || N <= 0 || K <= 0) return GELO_OK;
         GemmArgs g;
         g.M = M; g.N = N; g.K = K;
@@ -674,28 +690,29 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
             g.plane = plane;
         }
         if (used) *used = g.ksplit;
-        return launch_gemm_simt(ctx, g, st);
+        return launch_gemm_simt(ctx, g, cur);
     };
-    // C (rows from c0) <- (I - V op(T^T) V^T) C for the merged reflectors of a superblock (kv columns from c0)
-    auto apply = [&](int c0, int kv, const float* Tt, float* C, int nc, bool transpose) -> int {
+    // C (rows from c0) <- (I - V op(T^T) V^T) C for the merged reflectors of a superblock (kv columns from c0); scratch from column
+    // `at` on
+    auto apply = [&](int c0, int kv, const float* Tt, float* C, int nc, bool transpose, int at = 0) -> int {
         const int nr = m - c0;
         const int nc8 = (nc + 7) & ~7;
         const float* V = G + (size_t)c0 * ld + c0;
         const int want = slices(kv, nc8, nr, kSuperKSplit);
         if (want <= 1) {
-            GELO_TRY(gemm(kv, nc8, nr, V, ld, true, C, ld, false, tc.w32[0], ld, true, loss2, 1, 0, nullptr));
+            GELO_TRY(gemm(kv, nc8, nr, V, ld, true, C, ld, false, tc.w32[0] + at, ld, true, loss2, 1, 0, nullptr));
         } else {
             int used = 0;
             const size_t plane = (size_t)kv * ld;
-            GELO_TRY(gemm(kv, nc8, nr, V, ld, true, C, ld, false, tc.wf32, ld, false, 1.0f, want, plane, &used));
-            GELO_TRY(launch_sum_planes(ctx, tc.wf32, plane, used, ld, kv, nc8, loss2, tc.w32[0], ld, st, !exact));
+            GELO_TRY(gemm(kv, nc8, nr, V, ld, true, C, ld, false, tc.wf32 + at, ld, false, 1.0f, want, plane, &used));
+            GELO_TRY(launch_sum_planes(ctx, tc.wf32 + at, plane, used, ld, kv, nc8, loss2, tc.w32[0] + at, ld, cur, !exact));
         }
         // (the factor loss1 makes up for the truncation of V in the last product)
-        GELO_TRY(gemm(kv, nc8, kv, Tt, kSuper, transpose, tc.w32[0], ld, false, tc.w32[1], ld, true, loss1, 1, 0, nullptr));
-        return gemm(nr, nc, kv, V, ld, false, tc.w32[1], ld, true, C, ld, false, 1.0f, 1, 0, nullptr);
+        GELO_TRY(gemm(kv, nc8, kv, Tt, kSuper, transpose, tc.w32[0] + at, ld, false, tc.w32[1] + at, ld, true, loss1, 1, 0, nullptr));
+        return gemm(nr, nc, kv, V, ld, false, tc.w32[1] + at, ld, true, C, ld, false, 1.0f, 1, 0, nullptr);
     };
 
-    // Block columns: 128 wide while at least twice as many rows are left, then narrower ones (half of the rows at most) (multiples of eight) down to a
+    // Block columns: 128 wide while at least twice as many rows are left, then narrower ones (half of the rows, a multiple of eight) down to a
     // square of at most 96 rows for the Householder kernel, which takes 45 us for 64 rows, 97 for 96 and 183 for 128, against about
     // 50 us for a block.
     std::vector<int> start;
@@ -747,23 +764,45 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
                     GELO_TRY(launch_gemm_tf32_dual(ctx, ob, ncs, ob, Tb, kSuper, tc.w32[0], ld, tc.t128, FB, rows, ld, Wb, ld, loss1, st));
                 }
             }
-            if (send > bend)                                 // C -= V W'
-                GELO_TRY(gemm(nr, send - bend, ob, P, ld, false, Wb + (bend - s0), ld, true, P + ob, ld, false, 1.0f, 1, 0, nullptr));
-            if (r > 0)                                       // T^T[r:r+ob, 0:r] = -X^T T_<^T
+            if (r > 0) {                                     // T^T[r:r+ob, 0:r] = -X^T T_<^T
+                if (fork) GELO_TRY(branch());
                 GELO_TRY(gemm(ob, r, r, Wb, ld, false, Ts, kSuper, false, Ts + (size_t)r * kSuper, kSuper, true, -1.0f / loss1, 1, 0,
                               nullptr));
+                cur = st;
+            }
+            if (send > bend)                                 // C -= V W'
+                GELO_TRY(gemm(nr, send - bend, ob, P, ld, false, Wb + (bend - s0), ld, true, P + ob, ld, false, 1.0f, 1, 0, nullptr));
         }
+        if (fork && e - s > 1) GELO_TRY(join());
         GELO_TRY(apply(s0, send - s0, Ts, G + (size_t)s0 * ld + send, m - send, false));
     }
     // ---- the square that is left, and Q accumulated backwards, one superblock at a time ----
-    GELO_TRY(launch_qr_small(ctx, m - bf, G + (size_t)bf * ld + bf, ld, Q + (size_t)bf * ld + bf, st));
-    GELO_TRY(launch_chained(ctx, start_q_kernel, dim3(ceil_div(ld, 1024), m), 256, 0, st, Q, ld, m, bf, G));
-    GELO_TRY(after_launch(ctx));
-    for (int s = (nblocks - 1) / per * per; s >= 0; s -= per) {
-        const int e = (s + per < nblocks) ? s + per : nblocks;
-        const int s0 = start[s];
-        GELO_TRY(apply(s0, start[e] - s0, tc.tsuper + (size_t)(s / per) * kSuper * kSuper, Q + (size_t)s0 * ld + s0, m - s0, true));
+    auto form_q = [&](int c0, int c1) -> int {               // columns c0 .. c1 - 1
+        const int c_end = c1 == m ? ld : c1;                 // (the padding is cleared)
+        GELO_TRY(launch_chained(ctx, start_q_kernel, dim3(ceil_div(c_end - c0, 1024), m), 256, 0, cur, Q, ld, m, bf, G, c0, c_end));
+        GELO_TRY(after_launch(ctx));
+        for (int s = (nblocks - 1) / per * per; s >= 0; s -= per) {
+            const int e = (s + per < nblocks) ? s + per : nblocks;
+            const int s0 = start[s], from = c0 > s0 ? c0 : s0;
+            GELO_TRY(apply(s0, start[e] - s0, tc.tsuper + (size_t)(s / per) * kSuper * kSuper, Q + (size_t)s0 * ld + from, c1 - from, true,
+                           c0));
+        }
+        return GELO_OK;
+    };
+    float* Gf = G + (size_t)bf * ld + bf;
+    float* Qf = Q + (size_t)bf * ld + bf;
+    if (!fork) {
+        GELO_TRY(launch_qr_small(ctx, m - bf, Gf, ld, Qf, st));
+        return form_q(0, m);
     }
+    // (the columns of the square only have it in common with the others that the reflectors come next: c1 - from <= bf in the
+    // first call, so the second's scratch, from column bf on, is its own)
+    GELO_TRY(branch());
+    GELO_TRY(launch_qr_small(ctx, m - bf, Gf, ld, Qf, cur));
+    GELO_TRY(form_q(bf, m));
+    cur = st;
+    GELO_TRY(form_q(0, bf));
+    GELO_TRY(join());
     return GELO_OK;
 }
 
