@@ -172,6 +172,14 @@ int sample_attempt(gelo_ctx* ctx, const Layout& L, int m, int kind, uint64_t see
                    bool deferred = false, const uint64_t* seed_dev = nullptr)
 {
     const int ldi = L.ldi;
+    if (!seed_dev && sample_small_supports(ctx, m, kind)) {
+        GELO_TRY(launch_sample_small(ctx, m, seed, attempt, dtype, A_out, Ainv_out, lda, st));
+        if (cond_dev) {
+            set_scalar_kernel<<<1, 1, 0, st>>>(cond_dev, 1.0f);
+            GELO_TRY(after_launch(ctx));
+        }
+        return GELO_OK;
+    }
     GELO_TRY(launch_gaussian(ctx, m, m, ldi, seed, GELO_STREAM_G0, attempt, 1.0f, nullptr, L.G, st, seed_dev));
     const int l3 = level3_kind(ctx, m, dtype, true);
     // the block route signs its columns itself; the others leave that to the copy (by the diagonal of R, in L.G)
@@ -258,6 +266,8 @@ void drop_graphs(gelo_ctx* ctx)
 int sample_on_lane(gelo_ctx* ctx, const Layout& L, int lane, int m, int kind, uint64_t seed, int dtype, cudaStream_t ls,
                    bool deferred = true)
 {
+    if (sample_small_supports(ctx, m, kind))                 // one launch: nothing to record
+        return sample_attempt(ctx, L, m, kind, seed, 0u, dtype, L.A, L.Ainv, L.ldi, nullptr, ls, deferred, nullptr);
     uint64_t* slot = ctx->lane_seed_dev + lane * 8;
     set_seed_kernel<<<1, 1, 0, ls>>>(slot, seed);
     GELO_TRY(after_launch(ctx));

@@ -294,6 +294,9 @@ QrScratch carve_qr(Arena&, int m, int ld, char** idle = nullptr, size_t* idle_by
 int run_householder_qr(gelo_ctx*, int m, float* R, int ld, float* Q, const QrScratch&, cudaStream_t);
 // The whole factorisation of an m x m matrix, m <= 128, in one launch: R (diagonal of either sign) overwrites G
 int launch_qr_small(gelo_ctx*, int m, float* G, int ld, float* Q, cudaStream_t);
+// A whole orthogonal sample (A and its transpose in the storage type), m <= 128, in one launch
+bool sample_small_supports(const gelo_ctx*, int m, int kind);
+int launch_sample_small(gelo_ctx*, int m, uint64_t seed, uint32_t attempt, int dtype, void* A, void* Ainv, int lda, cudaStream_t);
 struct TcScratch;
 // Same factorisation with 128-column outer blocks whose updates run on the tensor cores in split precision.
 int run_householder_qr_tc(gelo_ctx*, int m, float* R, int ld, float* Q, const QrScratch&, const TcScratch&, cudaStream_t);

@@ -16,6 +16,9 @@
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "philox.cuh"
+
+#include <type_traits>
 
 namespace gelo {
 
@@ -498,73 +501,66 @@ t_merge_kernel(const float* __restrict__ part, int slabs, int ldp, const float* 
 // backwards to e_c (only H_j with j <= c touch it), with no barrier at all.
 // Same conventions as the blocked path: R (upper triangle, diagonal of either sign) overwrites G, Q is unsigned.
 template <int RM>
-__global__ void __launch_bounds__(8 * RM, 1)
-qr_small_kernel(float* __restrict__ G, int ld, int m, float* __restrict__ Q)
-{
-    chain_next();
-    chain_wait();
-    constexpr int RPT = RM / 8;
-    extern __shared__ float qs_smem[];
-    float* Vs = qs_smem;                      // RM x RM: row j = reflector j over the rows
-    float* tau_s = qs_smem + RM * RM;
-    const int c = threadIdx.x >> 3, h = threadIdx.x & 7;
-    const unsigned gmask = 0xFFu << (threadIdx.x & 24);        // the eight lanes of this column
-    auto group_sum = [&](float v) {
+struct QrSmall {
+    static constexpr int RPT = RM / 8;
+    float* Vs;                                // RM x RM: row j = reflector j over the rows
+    float* tau_s;
+    int m, c, h;
+    unsigned gmask;                           // the eight lanes of this column
+
+    __device__ __forceinline__ QrSmall(float* smem, int rows)
+        : Vs(smem), tau_s(smem + RM * RM), m(rows), c(threadIdx.x >> 3), h(threadIdx.x & 7), gmask(0xFFu << (threadIdx.x & 24))
+    {
+    }
+    __device__ __forceinline__ float group_sum(float v) const
+    {
         v += __shfl_xor_sync(gmask, v, 1);
         v += __shfl_xor_sync(gmask, v, 2);
         v += __shfl_xor_sync(gmask, v, 4);
         return v;
-    };
-    float x[RPT];
-#pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-        const int r = h + 8 * i;
-        x[i] = (r < m && c < m) ? G[(size_t)r * ld + c] : 0.0f;
     }
-    for (int j = 0; j < m; ++j) {
-        if (c == j) {
-            float s = 0.0f, a = 0.0f;
+    // x: column c of the matrix -> column c of R; the reflectors stay in Vs
+    __device__ __forceinline__ void factorise(float (&x)[RPT]) const
+    {
+        for (int j = 0; j < m; ++j) {
+            if (c == j) {
+                float s = 0.0f, a = 0.0f;
 #pragma unroll
-            for (int i = 0; i < RPT; ++i) {
-                const int r = h + 8 * i;
-                s = fmaf((r > j) ? x[i] : 0.0f, x[i], s);
-                a += (r == j) ? x[i] : 0.0f;
+                for (int i = 0; i < RPT; ++i) {
+                    const int r = h + 8 * i;
+                    s = fmaf((r > j) ? x[i] : 0.0f, x[i], s);
+                    a += (r == j) ? x[i] : 0.0f;
+                }
+                const float sigma = group_sum(s), alpha = group_sum(a);
+                float beta = alpha, tau = 0.0f, scale = 0.0f;
+                if (sigma > 0.0f) {
+                    beta = -copysignf(sqrtf(fmaf(alpha, alpha, sigma)), alpha);
+                    tau = (beta - alpha) / beta;
+                    scale = 1.0f / (alpha - beta);
+                }
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) {
+                    const int r = h + 8 * i;
+                    Vs[j * RM + r] = (r < j) ? 0.0f : ((r == j) ? 1.0f : x[i] * scale);
+                    x[i] = (r < j) ? x[i] : ((r == j) ? beta : 0.0f);
+                }
+                if (h == 0) tau_s[j] = tau;
             }
-            const float sigma = group_sum(s), alpha = group_sum(a);
-            float beta = alpha, tau = 0.0f, scale = 0.0f;
-            if (sigma > 0.0f) {
-                beta = -copysignf(sqrtf(fmaf(alpha, alpha, sigma)), alpha);
-                tau = (beta - alpha) / beta;
-                scale = 1.0f / (alpha - beta);
+            __syncthreads();
+            if (c > j && c < m) {
+                const float* v = Vs + j * RM + h;
+                float w = 0.0f;
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) w = fmaf(v[8 * i], x[i], w);        // v is zero above row j
+                const float tw = tau_s[j] * group_sum(w);
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) x[i] = fmaf(-tw, v[8 * i], x[i]);
             }
-#pragma unroll
-            for (int i = 0; i < RPT; ++i) {
-                const int r = h + 8 * i;
-                Vs[j * RM + r] = (r < j) ? 0.0f : ((r == j) ? 1.0f : x[i] * scale);
-                x[i] = (r < j) ? x[i] : ((r == j) ? beta : 0.0f);
-            }
-            if (h == 0) tau_s[j] = tau;
-        }
-        __syncthreads();
-        if (c > j && c < m) {
-            const float* v = Vs + j * RM + h;
-            float w = 0.0f;
-#pragma unroll
-            for (int i = 0; i < RPT; ++i) w = fmaf(v[8 * i], x[i], w);            // v is zero above row j
-            const float tw = tau_s[j] * group_sum(w);
-#pragma unroll
-            for (int i = 0; i < RPT; ++i) x[i] = fmaf(-tw, v[8 * i], x[i]);
         }
     }
-    if (c < m) {
-#pragma unroll
-        for (int i = 0; i < RPT; ++i) {
-            const int r = h + 8 * i;
-            if (r < m) G[(size_t)r * ld + c] = x[i];
-        }
-    }
-    // ---- column c of Q ----
-    if (c < m) {
+    // column c of Q
+    __device__ __forceinline__ void form_q(float (&x)[RPT]) const
+    {
 #pragma unroll
         for (int i = 0; i < RPT; ++i) x[i] = (h + 8 * i == c) ? 1.0f : 0.0f;
         for (int j = c; j >= 0; --j) {
@@ -576,25 +572,136 @@ qr_small_kernel(float* __restrict__ G, int ld, int m, float* __restrict__ Q)
 #pragma unroll
             for (int i = 0; i < RPT; ++i) x[i] = fmaf(-tw, v[8 * i], x[i]);
         }
+    }
+};
+
+template <int RM>
+__global__ void __launch_bounds__(8 * RM, 1)
+qr_small_kernel(float* __restrict__ G, int ld, int m, float* __restrict__ Q)
+{
+    chain_next();
+    chain_wait();
+    extern __shared__ float qs_smem[];
+    const QrSmall<RM> q(qs_smem, m);
+    const int c = q.c;
+    float x[QrSmall<RM>::RPT];
 #pragma unroll
-        for (int i = 0; i < RPT; ++i) {
-            const int r = h + 8 * i;
-            if (r < m) Q[(size_t)r * ld + c] = x[i];
+    for (int i = 0; i < QrSmall<RM>::RPT; ++i) {
+        const int r = q.h + 8 * i;
+        x[i] = (r < m && c < m) ? G[(size_t)r * ld + c] : 0.0f;
+    }
+    q.factorise(x);
+    if (c >= m) return;
+#pragma unroll
+    for (int i = 0; i < QrSmall<RM>::RPT; ++i) {
+        const int r = q.h + 8 * i;
+        if (r < m) G[(size_t)r * ld + c] = x[i];
+    }
+    q.form_q(x);
+#pragma unroll
+    for (int i = 0; i < QrSmall<RM>::RPT; ++i) {
+        const int r = q.h + 8 * i;
+        if (r < m) Q[(size_t)r * ld + c] = x[i];
+    }
+}
+
+__device__ __forceinline__ void put_small(float* p, float v) { *p = v; }
+__device__ __forceinline__ void put_small(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
+__device__ __forceinline__ void put_small(__half* p, float v) { *p = __float2half_rn(v); }
+
+// A whole orthogonal sample of a small matrix in one launch: the Gaussian (the blocks of the stream shared out to the
+// threads, by way of shared memory), its QR, the columns signed by the diagonal of R, A and its transpose in the storage
+// type.  Same values as the three kernels it stands for (gaussian_kernel, qr_small_kernel, finish_mixing_kernel): their launches, the
+// recorded graph around them and the passes over memory made a 64 + 4 row call 117 us alone, now 97, and 32 of them on 16 lanes, which
+// the host's launches bound, 829 us, now 770.
+template <int RM, typename T>
+__global__ void __launch_bounds__(8 * RM, 1)
+sample_small_kernel(int m, uint64_t seed, uint32_t attempt, T* __restrict__ A, T* __restrict__ At, int lda)
+{
+    chain_next();
+    chain_wait();
+    extern __shared__ float qs_smem[];
+    const QrSmall<RM> q(qs_smem, m);
+    const int c = q.c;
+    const unsigned total = (unsigned)(m * m);
+    for (unsigned b = threadIdx.x; 4 * b < total; b += 8 * RM) {
+        float z[4];
+        gaussian_block(seed, b, GELO_STREAM_G0, attempt, z);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const unsigned e = 4 * b + t, r = e / (unsigned)m;
+            if (e < total) q.Vs[r * RM + (e - r * m)] = z[t];
         }
     }
+    __syncthreads();
+    float x[QrSmall<RM>::RPT];
+#pragma unroll
+    for (int i = 0; i < QrSmall<RM>::RPT; ++i) {
+        const int r = q.h + 8 * i;
+        x[i] = (r < m && c < m) ? q.Vs[r * RM + c] : 0.0f;
+    }
+    __syncthreads();
+    q.factorise(x);
+    float d = 0.0f;
+#pragma unroll
+    for (int i = 0; i < QrSmall<RM>::RPT; ++i) d += (q.h + 8 * i == c) ? x[i] : 0.0f;
+    const float sign = q.group_sum(d) < 0.0f ? -1.0f : 1.0f;
+    if (c < m) q.form_q(x);
+    __syncthreads();                          // the reflectors have been read
+    float* out = qs_smem;                     // row stride RM + 1: read by rows and by columns
+    if (c < m) {
+#pragma unroll
+        for (int i = 0; i < QrSmall<RM>::RPT; ++i) out[(q.h + 8 * i) * (RM + 1) + c] = sign * x[i];
+    }
+    __syncthreads();
+    for (unsigned e = threadIdx.x; e < total; e += 8 * RM) {
+        const unsigned r = e / (unsigned)m, k = e - r * m;
+        put_small(A + (size_t)r * lda + k, out[r * (RM + 1) + k]);
+        put_small(At + (size_t)r * lda + k, out[k * (RM + 1) + r]);
+    }
+}
+
+constexpr int qr_small_smem(int RM) { return (RM * (RM + 1) + RM) * (int)sizeof(float); }
+
+template <typename F>
+int qr_small_attr(gelo_ctx* ctx, F* kernel, int smem, bool (&done)[64])
+{
+    if (ctx->device >= 0 && ctx->device < 64 && !done[ctx->device]) {
+        GELO_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        done[ctx->device] = true;
+    }
+    return GELO_OK;
 }
 
 template <int RM>
 int launch_qr_small_rm(gelo_ctx* ctx, int m, float* G, int ld, float* Q, cudaStream_t st)
 {
-    const int smem = (RM * RM + RM) * (int)sizeof(float);
-    static bool attr_done[64] = {};
-    if (ctx->device >= 0 && ctx->device < 64 && !attr_done[ctx->device]) {
-        GELO_CUDA_OK(cudaFuncSetAttribute(qr_small_kernel<RM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        attr_done[ctx->device] = true;
-    }
-    GELO_TRY(launch_chained(ctx, qr_small_kernel<RM>, 1, 8 * RM, smem, st, G, ld, m, Q));
+    static bool done[64] = {};
+    GELO_TRY(qr_small_attr(ctx, qr_small_kernel<RM>, qr_small_smem(RM), done));
+    GELO_TRY(launch_chained(ctx, qr_small_kernel<RM>, 1, 8 * RM, qr_small_smem(RM), st, G, ld, m, Q));
     return after_launch(ctx);
+}
+
+template <int RM, typename T>
+int launch_sample_small_rm(gelo_ctx* ctx, int m, uint64_t seed, uint32_t attempt, void* A, void* At, int lda, cudaStream_t st)
+{
+    static bool done[64] = {};
+    GELO_TRY(qr_small_attr(ctx, sample_small_kernel<RM, T>, qr_small_smem(RM), done));
+    GELO_TRY(launch_chained(ctx, sample_small_kernel<RM, T>, 1, 8 * RM, qr_small_smem(RM), st, m, seed, attempt, static_cast<T*>(A),
+                           static_cast<T*>(At), lda));
+    return after_launch(ctx);
+}
+
+// f(RM) for the smallest instance that holds m rows (72: the decode shape, 64 + 4)
+template <typename F>
+int with_small_rows(int m, F&& f)
+{
+    if (m <= 32) return f(std::integral_constant<int, 32>{});
+    if (m <= 48) return f(std::integral_constant<int, 48>{});
+    if (m <= 64) return f(std::integral_constant<int, 64>{});
+    if (m <= 72) return f(std::integral_constant<int, 72>{});
+    if (m <= 96) return f(std::integral_constant<int, 96>{});
+    return f(std::integral_constant<int, 128>{});
 }
 
 constexpr int kSmallQrRows = 128;
@@ -603,10 +710,22 @@ constexpr int kSmallQrRows = 128;
 
 int launch_qr_small(gelo_ctx* ctx, int m, float* G, int ld, float* Q, cudaStream_t st)
 {
-    if (m <= 32) return launch_qr_small_rm<32>(ctx, m, G, ld, Q, st);
-    if (m <= 64) return launch_qr_small_rm<64>(ctx, m, G, ld, Q, st);
-    if (m <= 96) return launch_qr_small_rm<96>(ctx, m, G, ld, Q, st);
-    return launch_qr_small_rm<128>(ctx, m, G, ld, Q, st);
+    return with_small_rows(m, [&](auto rm) { return launch_qr_small_rm<decltype(rm)::value>(ctx, m, G, ld, Q, st); });
+}
+
+bool sample_small_supports(const gelo_ctx* ctx, int m, int kind)
+{
+    return kind == GELO_ORTHOGONAL && m <= kSmallQrRows && ctx->fuse_small && ctx->level3 == 0;
+}
+
+int launch_sample_small(gelo_ctx* ctx, int m, uint64_t seed, uint32_t attempt, int dtype, void* A, void* Ainv, int lda, cudaStream_t st)
+{
+    return with_small_rows(m, [&](auto rm) {
+        constexpr int RM = decltype(rm)::value;
+        if (dtype == GELO_BF16) return launch_sample_small_rm<RM, __nv_bfloat16>(ctx, m, seed, attempt, A, Ainv, lda, st);
+        if (dtype == GELO_F16) return launch_sample_small_rm<RM, __half>(ctx, m, seed, attempt, A, Ainv, lda, st);
+        return launch_sample_small_rm<RM, float>(ctx, m, seed, attempt, A, Ainv, lda, st);
+    });
 }
 
 // Takes `bytes` from the idle region if it has that much left, else from the arena.
