@@ -223,9 +223,8 @@ int sample_attempt(gelo_ctx* ctx, const Layout& L, int m, int kind, uint64_t see
         const size_t half = (size_t)m * ldi;
         uint16_t* g16 = reinterpret_cast<uint16_t*>(L.G);
         uint16_t* x16 = reinterpret_cast<uint16_t*>(L.X32);
-        GELO_TRY(launch_finish_mixing(ctx, m, Q0, ldi, nullptr, ldi, dtype, x16, g16, ldi, st));
-        GELO_TRY(launch_gaussian(ctx, m, m, ldi, seed, GELO_STREAM_G1, attempt, s, Q0, L.A32, st, seed_dev));
-        GELO_TRY(launch_narrow(ctx, m, L.A32, ldi, dtype, A_out, lda, st));
+        GELO_TRY(launch_finish_mixing(ctx, m, Q0, ldi, nullptr, ldi, dtype, nullptr, g16, ldi, st));
+        GELO_TRY(launch_gaussian_to(ctx, dtype, m, m, seed, GELO_STREAM_G1, attempt, s, Q0, ldi, A_out, lda, st, seed_dev));
         GELO_TRY(run_newton_inverse(ctx, m, dtype, ctx->gamma, A_out, lda, g16, g16 + half, x16, x16 + half, ldi, Ainv_out, lda, st));
     } else if (blocks && exact && m <= kExactNewtonRows && ctx->gamma <= 0.55f) {
         // in fp32 from the stored A, and rounded once

@@ -163,6 +163,10 @@ int launch_gaussian(gelo_ctx*, int rows, int cols, int ld, uint64_t seed, uint32
                     uint32_t attempt, float scale, const float* base, float* out, cudaStream_t,
                     const uint64_t* seed_dev = nullptr);
 
+// the same into a matrix of type `dtype` with a stride of its own, rounded once
+int launch_gaussian_to(gelo_ctx*, int dtype, int rows, int cols, uint64_t seed, uint32_t stream_id, uint32_t attempt, float scale,
+                       const float* base, int ldb, void* out, int ld, cudaStream_t, const uint64_t* seed_dev = nullptr);
+
 // ---- fp32 SIMT GEMM ----------------------------------------------------------------
 
 struct GemmArgs {
@@ -347,7 +351,7 @@ int run_cond_estimate(gelo_ctx*, int m, const void* A, const void* Ainv, int ld,
 
 // ---- layout helpers ----------------------------------------------------------------------
 
-// dst (rows x cols, stride ldd, dtype) = colscale-signed copy of src (fp32); dstT = its transpose.
+// dst (rows x cols, stride ldd, dtype) = colscale-signed copy of src (fp32); dstT = its transpose.  Either may be null.
 // sign_diag (optional, fp32 matrix with stride lds): column j is multiplied by sign(sign_diag[j*lds + j]).
 int launch_finish_mixing(gelo_ctx*, int m, const float* src, int lds_src, const float* sign_diag,
                          int lds_diag, int dtype, void* dst, void* dstT, int ldd, cudaStream_t);
