@@ -1168,3 +1168,25 @@ def test_medium_batches_match_single_calls(n, k, calls, shared):
         got = torch.cat([out[0 if shared else i, j] for j in range(3)], dim=1).double()
         assert ((got - ref).norm() / ref.norm()).item() <= TOL[dt]
     c.close()
+
+
+# the median of the norms: the first size past the one-launch path, one value past a round of the CTA, more rounds, norms over six orders
+# of magnitude, all norms equal, half of them equal on either side of the middle
+@pytest.mark.parametrize("n,shape", [(257, "spread"), (1025, "spread"), (4096, "equal"), (3000, "half"), (2999, "half"), (5001, "spread")])
+def test_shield_scale_is_the_median(ctx, oracle, n, shape):
+    d, k = 16, 3
+    g = torch.Generator(device="cuda"); g.manual_seed(n)
+    H = torch.randn((n, d), generator=g, device="cuda")
+    if shape == "spread":
+        H = H * torch.exp(14.0 * torch.rand((n, 1), generator=g, device="cuda") - 7.0)
+    elif shape == "equal":
+        H = H[:1].repeat(n, 1)
+    else:
+        H[: n // 2] = H[0] * 3.0
+        H[n // 2:] = H[n // 2] * 5.0
+    H = H.contiguous()
+    ctx.ensure_workspace(n, k, d, 48, "f32")
+    S = torch.empty((k, d), device="cuda")
+    ctx.shield_rows(H, n, d, k, 10.0, 91, "f32", S)
+    ref = oracle.shield_rows(f64(H), k, 10.0, 91)
+    assert np.max(np.abs(f64(S) - ref)) <= 2e-5 * np.max(np.abs(ref))     # an fp32 norm and one product, as in test_shield_rows
