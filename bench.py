@@ -399,7 +399,7 @@ def run_ours(args):
         alu_peak = 148 * 128 * 2 * 1.965e9 / 1e12
         descr = {"rank_update": "rank_update_kernel: C -= A B inside the QR / LU outer blocks",
                  "vtc": "vtc_partial_kernel: V^T C inside the QR outer blocks",
-                 "gemm_tc": "gemm_tc_kernel: tcgen05 GEMM (mix / project / unmix and the level-3 QR / LU updates)",
+                 "gemm_tc": "gemm_tc_kernel: tcgen05 GEMM (mix / project / unmix and the products of the QR and of the inverse)",
                  "qr_panel": "qr_panel_cluster_kernel: 32-column Householder panel in registers across a cluster of <= 8 CTAs",
                  "lu_panel": "lu_panel_cluster_kernel: 32-column pivoted LU panel in registers across a cluster of <= 8 CTAs"}
         roofline = {"kernel": descr[dominant], "achieved": dk["achieved"], "unit": dk["unit"],
@@ -441,9 +441,8 @@ def run_ours(args):
                        "peak_source": peaks["source"] + " bf16 GEMM x nominal tf32/bf16 ratio 0.5",
                        # ncu: dram read 82.1 MB + write 9.0 MB per launch (algorithmic 147 MB, half of C stays in L2)
                        "traffic": 91.1e6,
-                       "note": "largest share of SM time among the sampling kernels; "
-                               "510 tiles of 16 k-blocks on 148 CTAs: fp32 operands re-read from L2 for every 128 x 256 tile (8.8 TB/s L2 -> SM) "
-                               "and the 3.45-wave quantisation; 630 TFLOP/s sustained at large K"}
+                       "note": "the subtracting update reads and writes C at the L2 (8 bytes per entry for 1024 flop); "
+                               "710 TFLOP/s at large K"}
         per_call_ms = ms_max / args.steps / calls
         chain_tflops = chain_flops / (chain_ms * 1e-3) / 1e12
         # all arithmetic of a sweep against the time the sweep takes with every lane busy: the Householder QR of every
