@@ -17,6 +17,9 @@
 // N-major without swizzle, i.e. core matrices of 8 k-rows x 8 columns (128 contiguous bytes), 8-row groups 128 bytes
 // apart, 8-column groups kpad * 16 bytes apart - which is what a thread holding one row of the accumulator can write
 // as 16-byte pieces without bank conflicts.
+// Behind the shield rows and the mixing it is set up while they run (launch_chained; the three of a 64-row call 42.7 -> 35.9 us, the
+// call 44.8 -> 39.5 us back to back).  The weight could be asked for before the wait as well: its first stages gave nothing (39.5 -> 39.7 us),
+// an L2 prefetch of the rest cost 3.5 us, because the mixing kernel's own loads then queue behind it.
 // Warp roles: warp 0 issues TMA, warps 1-2 issue MMA for alternate k-blocks (warp 1 owns tensor memory), warps 3-6 are
 // the epilogue (one per tensor-memory lane quarter).  Every barrier wait is bounded in time as in gemm_tc.cu.
 #include <cuda.h>
@@ -124,6 +127,7 @@ project_unmix_kernel(const __grid_constant__ CUtensorMap map_u, const __grid_con
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    chain_wait();                                        // before any role looks at the clock
     // instruction descriptor: fp32 accumulate, both operands bf16 (1) or half (0), A K-major, B N-major, M = 128, N = ncols
     const uint32_t fmt = prm.out_f16 ? 0u : 1u;
     const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | (1u << 16) | ((uint32_t)(ncols >> 3) << 17) | ((128u >> 4) << 24);
@@ -356,6 +360,8 @@ mix_small_kernel(const T* __restrict__ A, int lda, const T* __restrict__ H, cons
     // All global loads of a thread are issued before any of them is used (16 bytes each; the row stride of A is a
     // multiple of 8 elements, so a group that starts inside a row may run into its padding, which is read and dropped).
     const int ga = (m + 7) >> 3;                             // 16-byte groups per row of A
+    chain_next();
+    chain_wait();
     constexpr int kMaxA = (128 * 16 + 255) / 256, kMaxH = (128 * 4 + 255) / 256;
     uint4 ra[kMaxA], rh[kMaxH];
 #pragma unroll
@@ -445,13 +451,12 @@ int launch_mix_small(gelo_ctx* ctx, const void* A, int lda, const void* H, const
         attr_done[ctx->device] = true;
     }
     if (dtype == GELO_F16) {
-        mix_small_kernel<__half><<<grid, 256, smem, st>>>(static_cast<const __half*>(A), lda, static_cast<const __half*>(H),
-                                                          static_cast<const __half*>(S), n, k, d, static_cast<__half*>(U));
+        GELO_TRY(launch_chained(ctx, mix_small_kernel<__half>, grid, 256, smem, st, static_cast<const __half*>(A), lda,
+                                static_cast<const __half*>(H), static_cast<const __half*>(S), n, k, d, static_cast<__half*>(U)));
     } else {
-        mix_small_kernel<__nv_bfloat16><<<grid, 256, smem, st>>>(static_cast<const __nv_bfloat16*>(A), lda,
-                                                                 static_cast<const __nv_bfloat16*>(H),
-                                                                 static_cast<const __nv_bfloat16*>(S), n, k, d,
-                                                                 static_cast<__nv_bfloat16*>(U));
+        GELO_TRY(launch_chained(ctx, mix_small_kernel<__nv_bfloat16>, grid, 256, smem, st, static_cast<const __nv_bfloat16*>(A), lda,
+                                static_cast<const __nv_bfloat16*>(H), static_cast<const __nv_bfloat16*>(S), n, k, d,
+                                static_cast<__nv_bfloat16*>(U)));
     }
     return after_launch(ctx);
 }
@@ -531,7 +536,7 @@ int launch_project_unmix(gelo_ctx* ctx, const void* U, const void* W, const void
     }
     {
         ProfScope ps(ctx, PROF_GEMM_TC, 2.0 * m * (double)d * p + 2.0 * n * (double)m * p, st);
-        project_unmix_kernel<<<ncta, kDecThreads, smem, st>>>(mu, mww, mwn, ma, prm);
+        GELO_TRY(launch_chained(ctx, project_unmix_kernel, ncta, kDecThreads, smem, st, mu, mww, mwn, ma, prm));
     }
     return after_launch(ctx);
 }

@@ -233,6 +233,8 @@ shield_small_kernel(const T* __restrict__ H, int n, int d, int k, float scale, u
     const int rank = (int)cluster.block_rank();
     __shared__ float norms_s[kShieldSmallRows];
     __shared__ float med_s[2];
+    chain_next();
+    chain_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int row = rank * 32 + warp;
     if (row < n) {
@@ -267,11 +269,13 @@ int launch_shield_small(gelo_ctx* ctx, const void* H, int n, int d, int k, float
     cfg.blockDim = dim3(1024, 1, 1);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cs; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = chain_launches(ctx) ? 2 : 1;
     if (cudaLaunchKernelEx(&cfg, shield_small_kernel<T>, static_cast<const T*>(H), n, d, k, scale, seed, static_cast<T*>(S), nu) != cudaSuccess)
         return GELO_ERR_CUDA;
     return after_launch(ctx);
