@@ -261,7 +261,7 @@ void drop_graphs(gelo_ctx* ctx)
 // Samples (A, A^-1) of one batched call on a lane stream by replaying a launch graph of the whole sampling
 // sequence (about a thousand dependent launches): one host call instead of a thousand, so a single host thread
 // keeps all lanes busy.  The seed reaches the kernels through the lane's device slot.  The first use of a
-// (lane scratch, kind, size, type) combination records the graph by stream capture.
+// combination of places, sizes and settings (SampleKey) records the graph by stream capture.
 int sample_on_lane(gelo_ctx* ctx, const Layout& L, int lane, int m, int kind, uint64_t seed, int dtype, cudaStream_t ls,
                    bool deferred = true)
 {
@@ -272,9 +272,9 @@ int sample_on_lane(gelo_ctx* ctx, const Layout& L, int lane, int m, int kind, ui
     GELO_TRY(after_launch(ctx));
     if (ctx->prof_on)      // per-launch timing needs real launches
         return sample_attempt(ctx, L, m, kind, seed, 0u, dtype, L.A, L.Ainv, L.ldi, nullptr, ls, deferred, slot);
+    const gelo_ctx::SampleKey key = { L.G, L.A, L.Ainv, L.cond_val, slot, L.m, m, kind, dtype, ctx->level3, ctx->tc_update_ctas, deferred };
     for (auto& g : ctx->graphs) {
-        if (g.key_ptr == L.G && g.m == m && g.kind == kind && g.dtype == dtype && g.level3 == ctx->level3 &&
-            g.tc_ctas == ctx->tc_update_ctas && g.deferred == deferred) {
+        if (g.key == key) {
             GELO_CUDA_OK(cudaGraphLaunch(g.exec, ls));
             ctx->launches += g.launches;
             return GELO_OK;
@@ -292,7 +292,7 @@ int sample_on_lane(gelo_ctx* ctx, const Layout& L, int lane, int m, int kind, ui
         return rc != GELO_OK ? rc : GELO_ERR_CUDA;
     }
     gelo_ctx::SampleGraph g;
-    g.key_ptr = L.G; g.m = m; g.kind = kind; g.dtype = dtype; g.level3 = ctx->level3; g.tc_ctas = ctx->tc_update_ctas; g.deferred = deferred;
+    g.key = key;
     g.launches = ctx->launches - before;
     g.exec = nullptr;
     const cudaError_t ie = cudaGraphInstantiate(&g.exec, graph, 0);

@@ -79,8 +79,20 @@ struct gelo_ctx {
     const void* chain_key = nullptr;
     int chain_lanes = 0;
     int chain_shape[6] = {0, 0, 0, 0, 0, 0};   // n, k, d, p, dtype, host staging of the batch a later one may chain onto
-    // replayable launch graphs of the sampling sequence, one per (lane scratch, kind, size, type)
-    struct SampleGraph { const void* key_ptr; int m, kind, dtype, level3, tc_ctas; bool deferred; cudaGraphExec_t exec; long long launches; };
+    // Replayable launch graphs of the sampling sequence.  A graph belongs to all that its launches were given: the places it works in
+    // and writes to, the sizes, and the settings that choose its kernels (gamma, the bound on kappa_2 and the wait limit drop all graphs).
+    // Where G lies and for how many rows the scratch was carved say where the rest of the scratch lies, but not A, A^-1 and
+    // the estimate: they stand behind the row norms of the data rows, so they move with n at equal m.
+    struct SampleKey {
+        const void *G, *A, *Ainv, *cond, *seed;
+        int rows, m, kind, dtype, level3, tc_ctas, deferred;
+        bool operator==(const SampleKey& o) const
+        {
+            return G == o.G && A == o.A && Ainv == o.Ainv && cond == o.cond && seed == o.seed && rows == o.rows && m == o.m && kind == o.kind &&
+                   dtype == o.dtype && level3 == o.level3 && tc_ctas == o.tc_ctas && deferred == o.deferred;
+        }
+    };
+    struct SampleGraph { SampleKey key; cudaGraphExec_t exec; long long launches; };
     std::vector<SampleGraph> graphs;
     bool recording = false;                         // the launches go into such a graph
     uint64_t* lane_seed_dev = nullptr;              // one seed slot per lane

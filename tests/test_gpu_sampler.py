@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2603_05035_b200 import binding
+from paper_2603_05035_b200 import binding, inputs
 from gpu_util import f64, padded
 
 pytestmark = pytest.mark.gpu
@@ -81,3 +81,35 @@ def test_exact_block_route(oracle, m, dt):
     assert np.linalg.norm(a[:, :h] - q_ref[:, :h]) / np.sqrt(h) <= (2e-6 * (2 + m / 100) if dt == "f32" else 4e-4)
     a, x = _sample(m, NONORTHOGONAL, 300 + m, dt)
     assert np.linalg.norm(x @ a - np.eye(m)) / np.sqrt(m) <= (3e-6 if dt == "f32" else 5e-4)
+
+
+# The buffers of a call lie elsewhere where n and k split the same m differently, or where the rows are a group of a block-diagonal call.
+# 330 rows: the size at which the first three differ; every call after the first finds recordings of the others in the context.
+@pytest.mark.parametrize("kind", [ORTHOGONAL, NONORTHOGONAL])
+@pytest.mark.parametrize("entry", ["call", "batch"])
+def test_calls_of_equal_m_in_one_context(entry, kind):
+    d, p, dt, calls = 256, 768, "bf16", 6 if entry == "batch" else 1
+    c = binding.Context(0)
+    c.set_lanes(6)
+    c.ensure_blockdiag_workspace(660, 0, d, p, dt, 384, 6)
+    c.ensure_batch_workspace(330, 60, d, p, dt, 6)
+    out = torch.zeros((calls, 3, 660, p // 3), dtype=TDT[dt], device="cuda")
+    for n, k, block in ((300, 30, 0), (330, 0, 0), (660, 0, 384), (300, 30, 0), (330, 0, 0), (270, 60, 0)):
+        H = [inputs.make_hidden(n, d, dt, n + i, True, "cuda") for i in range(calls)]
+        W = [inputs.make_weight(d, p, dt, n + i, "cuda") for i in range(calls)]
+        o = [[out[i, j, :n] for i in range(calls)] for j in range(3)]
+        seeds = [7 + i for i in range(calls)]
+        if block:
+            c.qkv_offload_blockdiag_batch(H, W, n, k, d, p, block, seeds, 10.0, dt, *o)
+        elif entry == "batch":
+            c.qkv_offload_batch(H, W, n, k, d, p, [kind] * calls, seeds, 10.0, dt, *o)
+        else:
+            c.qkv_offload(H[0], W[0], n, k, d, p, kind, seeds[0], 10.0, dt, o[0][0], o[1][0], o[2][0])
+        torch.cuda.synchronize()
+        assert c.last_status() == binding.OK
+        for i in range(calls):
+            ref = H[i].double() @ W[i].double()
+            got = torch.cat([out[i, j, :n] for j in range(3)], dim=1).double()
+            assert ((got - ref).norm() / ref.norm()).item() <= 2e-2, (n, k, block, i)        # the bf16 path's tolerance
+        out.zero_()
+    c.close()
