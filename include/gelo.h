@@ -256,8 +256,9 @@ int gelo_set_small_batch_fusion(gelo_ctx* ctx, int on);
 /* ---- the whole call --------------------------------------------------------------------- */
 
 /* sample -> shields -> mix -> project -> unmix for one batch, all from workspace scratch.
- * H_dev n x d, W_dev d x p; outputs as in gelo_unmix.  Waits for `stream` only when
- * kind is GELO_NONORTHOGONAL (condition-number verdict). */
+ * H_dev n x d, W_dev d x p; outputs as in gelo_unmix.  GELO_NONORTHOGONAL WAITS until the verdict on
+ * the condition number is known (the last product runs on after the return); with GELO_ERR_COND the
+ * outputs are untouched. */
 int gelo_qkv_offload(gelo_ctx* ctx, const void* H_dev, const void* W_dev, int n, int k, int d,
                      int p, int kind, uint64_t seed, float shield_scale, int dtype,
                      void* Q_dev, void* K_dev, void* V_dev, void* stream);

@@ -394,10 +394,15 @@ const Tf32x3Scratch* stage_pairs(gelo_ctx* ctx, int rows, int k, int d, int p, i
 
 // Eq. 2 and Eq. 3 of one call: one fused launch for a small batch (the weight is streamed once and Y' stays on chip),
 // otherwise the two products with Y' in workspace memory.
+bool fused_projection(const gelo_ctx* ctx, int n, int k, int d, int p, int dtype, int lda, const void* K)
+{
+    return ctx->fuse_small && project_unmix_supports(ctx, n, k, d, p, dtype, lda, K ? 3 : 1);
+}
+
 int project_and_unmix(gelo_ctx* ctx, const void* U, const void* W, const void* Ainv, int lda, void* Yp, int n, int k, int d,
                       int p, int dtype, void* Q, void* K, void* V, cudaStream_t st, const Tf32x3Scratch* t3)
 {
-    if (ctx->fuse_small && project_unmix_supports(ctx, n, k, d, p, dtype, lda, (K || V) ? 3 : 1))
+    if (fused_projection(ctx, n, k, d, p, dtype, lda, K))
         return launch_project_unmix(ctx, U, W, Ainv, lda, n, k, d, p, dtype, Q, K, V, st);
     GELO_TRY(project_impl(ctx, U, W, n + k, d, p, dtype, Yp, st, t3));
     return unmix_impl(ctx, Ainv, lda, Yp, n, k, p, dtype, Q, K, V, st, t3);
@@ -411,37 +416,61 @@ int check_split(int p, const void* Q, const void* K, const void* V)
     return GELO_OK;
 }
 
+// Orders the caller's stream after what a lane has been given when an entry point returns early, so that whatever the caller enqueues
+// next (or frees) waits for the launches that went out before the error.
+struct LaneJoin {
+    gelo_ctx* ctx; cudaStream_t st; int lanes;
+    LaneJoin(gelo_ctx* c, cudaStream_t s, int n) : ctx(c), st(s), lanes(n) {}
+    LaneJoin(const LaneJoin&) = delete;
+    void done() { lanes = 0; }
+    ~LaneJoin()
+    {
+        for (int l = 0; l < lanes; ++l)
+            if (cudaEventRecord(ctx->lane_ready[l], ctx->lane_stream[l]) == cudaSuccess) cudaStreamWaitEvent(st, ctx->lane_ready[l], 0);
+    }
+};
+
 // One whole call on the caller's stream.  A non-orthogonal pair is verified: the first attempt replays the recorded sampling
-// graph on a lane's stream beside the shield rows, the products are enqueued behind it, and the host waits for the verdict only;
-// a sample that misses the bound (never seen) is drawn again, and the products repeated.
+// graph on a lane's stream beside the shield rows, and what needs the pair but only writes to the workspace (mixing, and the
+// projection where it is a launch of its own) is enqueued behind it.  The host waits for the verdict, which comes in while
+// those run, and the launch that writes the results follows only then: results of a rejected pair never reach the caller's buffers,
+// and a sample that is drawn again (never seen at gamma = 1/2) still finds the caller's H as it was, even where a result overwrites it.
 int offload_impl(gelo_ctx* ctx, const Layout& L, const void* H, const void* W, int n, int k, int d, int p,
                  int kind, uint64_t seed, float shield_scale, int dtype, void* Q, void* K, void* V,
                  cudaStream_t st)
 {
     const int m = n + k;
+    const bool fused = fused_projection(ctx, n, k, d, p, dtype, L.ldi, K);
     auto shields = [&]() -> int { return run_shield_rows(ctx, H, n, d, k, shield_scale, seed, dtype, L.S, L.sh, st, ctx->shield_nu); };
-    auto products = [&]() -> int {
+    auto to_workspace = [&]() -> int {
         GELO_TRY(mix_impl(ctx, L.A, L.ldi, H, k > 0 ? L.S : nullptr, n, k, d, dtype, L.U, st, &L.t3));
-        return project_and_unmix(ctx, L.U, W, L.Ainv, L.ldi, L.Yp, n, k, d, p, dtype, Q, K, V, st, &L.t3);
+        return fused ? GELO_OK : project_impl(ctx, L.U, W, m, d, p, dtype, L.Yp, st, &L.t3);
+    };
+    auto results = [&]() -> int {
+        return fused ? launch_project_unmix(ctx, L.U, W, L.Ainv, L.ldi, n, k, d, p, dtype, Q, K, V, st)
+                     : unmix_impl(ctx, L.Ainv, L.ldi, L.Yp, n, k, p, dtype, Q, K, V, st, &L.t3);
     };
     if (kind == GELO_ORTHOGONAL || ctx->prof_on) {
         GELO_TRY(sample_mixing_impl(ctx, L, m, kind, seed, dtype, L.A, L.Ainv, L.ldi, nullptr, st));
         GELO_TRY(shields());
-        return products();
+        GELO_TRY(to_workspace());
+        return results();
     }
+    cudaStream_t ls = ctx->lane_stream[0];
     for (int attempt = 0; attempt < ctx->max_attempts; ++attempt) {
-        cudaStream_t ls = ctx->lane_stream[0];
         GELO_CUDA_OK(cudaEventRecord(ctx->batch_start, st));
         GELO_CUDA_OK(cudaStreamWaitEvent(ls, ctx->batch_start, 0));
+        LaneJoin join(ctx, st, 1);
         if (attempt == 0) GELO_TRY(sample_on_lane(ctx, L, 0, m, kind, seed, dtype, ls, false));
         else GELO_TRY(sample_attempt(ctx, L, m, kind, seed, (uint32_t)attempt, dtype, L.A, L.Ainv, L.ldi, nullptr, ls));
         GELO_CUDA_OK(cudaMemcpyAsync(ctx->status_host, ctx->status_dev, kStatusWords * sizeof(int), cudaMemcpyDeviceToHost, ls));
         GELO_CUDA_OK(cudaEventRecord(ctx->lane_ready[0], ls));
         if (attempt == 0) GELO_TRY(shields());
         GELO_CUDA_OK(cudaStreamWaitEvent(st, ctx->lane_ready[0], 0));
-        GELO_TRY(products());
+        join.done();
+        GELO_TRY(to_workspace());
         GELO_CUDA_OK(cudaEventSynchronize(ctx->lane_ready[0]));
-        if (ctx->status_host[1] == 1) return GELO_OK;
+        if (ctx->status_host[1] == 1) return results();
     }
     return GELO_ERR_COND;
 }

@@ -204,6 +204,42 @@ def test_condition_bound_resampling(oracle):
     c.last_status()
     c.close()
 
+def test_results_only_from_accepted_pairs():
+    """A rejected pair writes nothing to the caller's buffers, and a redraw starts from the caller's H even where the results go there:
+    sizes with the fused projection and with products of their own."""
+    for n, k, d, dt in ((64, 4, 256, "bf16"), (300, 15, 256, "bf16"), (200, 0, 128, "f32")):
+        m, p = n + k, d
+        c = binding.Context(0)
+        c.ensure_workspace(n, k, d, p, dt)
+        H = inputs.make_hidden(n, d, dt, 3, True, "cuda")
+        W = inputs.make_weight(d, p, dt, 3, "cuda")
+        Y = torch.full((n, p), 7.0, device="cuda", dtype=TDT[dt])
+        c.set_nonorthogonal(0.5, 1.0, 3)                        # kappa_2 is about 4.7: no attempt can pass
+        with pytest.raises(binding.GeloError) as e:
+            c.qkv_offload(H, W, n, k, d, p, NONORTHOGONAL, 5, 10.0, dt, Y)
+        assert e.value.status == binding.ERR_COND
+        torch.cuda.synchronize()
+        assert (Y == 7.0).all()
+        # a seed whose first estimate is above its second, and a bound between the two (times the 1.2 that the check applies)
+        ld = c.mixing_ld(m)
+        A = padded(m, ld, TDT[dt]); X = padded(m, ld, TDT[dt]); cond = torch.zeros(1, device="cuda")
+        for seed in range(20):
+            c.set_nonorthogonal(0.5, 100.0, 1)
+            c.sample_mixing(m, NONORTHOGONAL, seed, dt, A, X, ld, cond)
+            first = cond.item()
+            c.set_nonorthogonal(0.5, 1.2 * first * 0.995, 2)
+            try:
+                c.sample_mixing(m, NONORTHOGONAL, seed, dt, A, X, ld, cond)
+                break
+            except binding.GeloError:
+                continue
+        ref = H.double() @ W.double()
+        c.qkv_offload(H, W, n, k, d, p, NONORTHOGONAL, seed, 10.0, dt, H)        # (p = d: the result replaces H)
+        torch.cuda.synchronize()
+        assert cond.item() < 0.995 * first and c.last_status() == binding.OK
+        assert ((H.double() - ref).norm() / ref.norm()).item() <= TOL[dt]
+        c.close()
+
 
 # ------------------------------------------------------------------------- shields
 
