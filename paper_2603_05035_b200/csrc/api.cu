@@ -475,6 +475,32 @@ int offload_impl(gelo_ctx* ctx, const Layout& L, const void* H, const void* W, i
     return GELO_ERR_COND;
 }
 
+// Whether the results of one call overlap those of another (they are promised in call order) or what another one reads (which sees
+// the results of the calls before it): such batches keep to the caller's stream.
+bool calls_depend(int calls, const void* const* H, size_t h_bytes, const void* const* W, size_t w_bytes, void* const* Q, void* const* K,
+                  void* const* V, size_t out_bytes)
+{
+    struct Piece { uintptr_t lo, hi; int call; };
+    std::vector<Piece> out;
+    out.reserve((size_t)calls * 3);
+    for (int i = 0; i < calls; ++i)
+        for (const void* q : { Q[i], K[i], V[i] })
+            if (q) out.push_back({ reinterpret_cast<uintptr_t>(q), reinterpret_cast<uintptr_t>(q) + out_bytes, i });
+    std::sort(out.begin(), out.end(), [](const Piece& a, const Piece& b) { return a.lo < b.lo; });
+    for (size_t i = 1; i < out.size(); ++i)
+        if (out[i].lo < out[i - 1].hi) return true;
+    auto reads_anothers = [&](const void* p, size_t bytes, int call) {
+        const uintptr_t lo = reinterpret_cast<uintptr_t>(p), hi = lo + bytes;
+        auto it = std::upper_bound(out.begin(), out.end(), lo, [](uintptr_t v, const Piece& o) { return v < o.hi; });   // (disjoint: the ends ascend too)
+        for (; it != out.end() && it->lo < hi; ++it)
+            if (it->call != call) return true;
+        return false;
+    };
+    for (int i = 0; i < calls; ++i)
+        if (reads_anothers(H[i], h_bytes, i) || reads_anothers(W[i], w_bytes, i)) return true;
+    return false;
+}
+
 // The whole path for a batch of independent calls.  Sampling A depends only on the seed, so up to
 // `lanes` calls sample their mixing pairs concurrently on the context's lane streams (each with its
 // own scratch) while the main stream runs shields and the three products of earlier calls.
@@ -507,21 +533,7 @@ int offload_batch_impl(gelo_ctx* ctx, int calls, const void* const* H, const voi
                  ((D > 4 && lane_calls(m, dtype)) || (ctx->fuse_small && m <= 128 && mix_small_supports(n, k, d, dtype) &&
                                            project_unmix_supports(ctx, n, k, d, p, dtype, L[0].ldi, split ? 3 : 1)));
     for (int i = 0; i < calls && small; ++i) small = !misaligned(H[i]);
-    if (small) {
-        // calls that share an output buffer are promised call order: keep those on the caller's stream
-        std::vector<std::pair<uintptr_t, uintptr_t>> out;
-        out.reserve((size_t)calls * 3);
-        const size_t bytes = split ? third : (size_t)n * p * es;
-        for (int i = 0; i < calls; ++i) {
-            out.emplace_back(reinterpret_cast<uintptr_t>(Q[i]), reinterpret_cast<uintptr_t>(Q[i]) + bytes);
-            if (split) {
-                out.emplace_back(reinterpret_cast<uintptr_t>(K[i]), reinterpret_cast<uintptr_t>(K[i]) + bytes);
-                out.emplace_back(reinterpret_cast<uintptr_t>(V[i]), reinterpret_cast<uintptr_t>(V[i]) + bytes);
-            }
-        }
-        std::sort(out.begin(), out.end());
-        for (size_t i = 1; i < out.size() && small; ++i) small = out[i].first >= out[i - 1].second;
-    }
+    if (small && calls > 1) small = !calls_depend(calls, H, (size_t)n * d * es, W, (size_t)d * p * es, Q, K, V, split ? third : (size_t)n * p * es);
     // with several lanes in flight each level-3 update takes a share of the SMs (ctx->lane_tc_share-th of them)
     ctx->tc_update_ctas = (D >= ctx->lane_tc_share && ctx->lane_tc_share > 1) ? ctx->sm_count / ctx->lane_tc_share : 0;
 

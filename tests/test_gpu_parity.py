@@ -668,6 +668,31 @@ def test_small_batch_with_shared_outputs_keeps_call_order():
     c.close()
 
 
+# a call that reads the result of the one before it, on the sizes whose calls run on their lanes (fused, and with products of their own)
+# and on one that never does
+@pytest.mark.parametrize("n,k", [(64, 4), (300, 15), (2300, 20)])
+def test_batched_calls_that_read_earlier_results_run_in_call_order(n, k):
+    d, dt, calls = 256, "bf16", 7
+    c = binding.Context(0)
+    c.set_lanes(6)
+    c.ensure_batch_workspace(n, k, d, d, dt, 6)
+    W = [inputs.make_weight(d, d, dt, 90 + i, "cuda") * 3.0 for i in range(calls)]       # (keeps the scale of the rows)
+    chain = torch.zeros((calls + 1, n, d), dtype=torch.bfloat16, device="cuda")
+    for _ in range(2):
+        chain.zero_()
+        chain[0] = inputs.make_hidden(n, d, dt, 40, True, "cuda")
+        rows = [chain[i] for i in range(calls + 1)]
+        torch.cuda._sleep(20_000_000)                # every call is enqueued before the first one starts
+        c.qkv_offload_batch(rows[:-1], W, n, k, d, d, [ORTHOGONAL] * calls, [500 + i for i in range(calls)], 10.0, dt, rows[1:])
+        torch.cuda.synchronize()
+        assert c.last_status() == binding.OK
+        for i in range(calls):
+            ref = chain[i].double() @ W[i].double()
+            assert ref.norm() > 0 and ((chain[i + 1].double() - ref).norm() / ref.norm()).item() <= TOL[dt]
+    c.close()
+
+
+
 def test_batched_offload_full_size(oracle):
     w = inputs.WORKLOADS["prefill_bf16"]
     n, k, d, p = w.n, w.k, w.d, w.p
