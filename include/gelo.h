@@ -99,7 +99,7 @@ int gelo_set_level3(gelo_ctx* ctx, int mode);
 int gelo_mixing_ld(int m);
 
 /* Limit, in nanoseconds of the GPU's global timer, of every device-side wait on a pipeline
- * barrier in the tensor-core kernels (default 2e9 = two seconds).  When a wait runs out the
+ * barrier in the tensor-core kernels and in the sampler's block factor (default 2e9 = two seconds).  When a wait runs out the
  * CTA records GELO_ERR_TIMEOUT in the status word, stops issuing work, frees its tensor
  * memory and returns, and the outputs of that call are invalid.  A limit of 0 makes every
  * such kernel give up before it issues its first copy or MMA: a diagnostic setting that lets

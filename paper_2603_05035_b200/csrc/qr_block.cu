@@ -72,6 +72,7 @@ struct FactShared {
     float U32[NB][FB + 4];
     float next[2][NB][NB + 4];                 // the next pivot block before the running update
     uint64_t got_full[kSteps], panel_full[kSteps];
+    int abort;                                 // a wait ran out somewhere in the cluster
 };
 constexpr int kFactSmemBytes = (int)sizeof(FactShared);
 static_assert(kFactSmemBytes <= 227 * 1024, "shared memory budget");
@@ -84,15 +85,19 @@ __device__ __forceinline__ float fast_rcp(float x)
     return r;
 }
 
-// Bounded wait for a phase of a barrier of this CTA (a block that runs out of patience sets the status word and goes on:
-// nothing it does afterwards can hang).
-__device__ __forceinline__ void fact_wait(const uint64_t* bar, uint32_t parity, int* status)
+// Wait for a phase of a barrier of this CTA, bounded in time.  A wait that runs out sets the status word and the flag of all three CTAs and
+// goes on (with values that nobody will use): every copy is still sent and every barrier reached, the other waits give up at
+// their next look at the flag, and the copies that are still on their way are waited for at the end.
+__device__ __forceinline__ void fact_wait(const uint64_t* bar, FactShared& s, unsigned long long limit_ns, int* status)
 {
     const uint32_t addr = tcx::smem_u32(bar);
 #pragma unroll 1
-    for (int spin = 0; spin < (1 << 22); ++spin)
-        if (tcx::mbar_try(addr, parity)) return;
+    for (int spin = 0; spin < 256; ++spin)
+        if (tcx::mbar_try(addr, 0)) return;
+    if (tcx::mbar_wait(addr, 0, &s.abort, limit_ns)) return;
     atomicCAS(status, 0, (int)GELO_ERR_TIMEOUT);
+    for (int r = 0; r < kFactCtas; ++r)
+        asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(tcx::map_rank(tcx::smem_u32(&s.abort), r)), "r"(1) : "memory");
 }
 
 __device__ __forceinline__ void cluster_sync_all()
@@ -283,7 +288,7 @@ __device__ __forceinline__ void compute_barrier() { asm volatile("bar.sync 2, %0
 
 // The eight steps of the eight warps; a[mt][nt][2 i + e] = row 32 (w / 2) + 16 mt + gid + 8 i, column 64 (w % 2) + 8 nt + 2 tig + e.
 template <int kRole>
-__device__ __forceinline__ void fact_compute(float (&a)[2][8][4], FactShared& s, int* status)
+__device__ __forceinline__ void fact_compute(float (&a)[2][8][4], FactShared& s, unsigned long long wait_ns, int* status)
 {
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
     const int wr = w >> 1, wc = w & 1;
@@ -292,8 +297,8 @@ __device__ __forceinline__ void fact_compute(float (&a)[2][8][4], FactShared& s,
     for (int J = 0; J < kSteps; ++J) {
         // ---- publish ----
         if (kRole != FACT_GRAM) {
-            fact_wait(&s.got_full[J], 0, status);
-            if (kRole == FACT_FACTOR) fact_wait(&s.panel_full[J], 0, status);
+            fact_wait(&s.got_full[J], s, wait_ns, status);
+            if (kRole == FACT_FACTOR) fact_wait(&s.panel_full[J], s, wait_ns, status);
         }
         if (wr == (J >> 1))
             with_bit(J & 1, [&](auto bit) {
@@ -429,7 +434,7 @@ __device__ __forceinline__ void fact_compute(float (&a)[2][8][4], FactShared& s,
 
 // The ninth warp: the inverses of the pivot blocks.
 template <int kRole>
-__device__ __forceinline__ void fact_pivots(FactShared& s, int* status)
+__device__ __forceinline__ void fact_pivots(FactShared& s, unsigned long long wait_ns, int* status)
 {
     const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
     float a[2][4];
@@ -457,7 +462,7 @@ __device__ __forceinline__ void fact_pivots(FactShared& s, int* status)
             }
         if (N > 0) mma_pairs_t(a, c, x);
         if (kRole == FACT_INVERSE) {
-            fact_wait(&s.got_full[N], 0, status);
+            fact_wait(&s.got_full[N], s, wait_ns, status);
 #pragma unroll
             for (int t = 0; t < 2; ++t)
 #pragma unroll
@@ -485,10 +490,15 @@ __device__ __forceinline__ void fact_pivots(FactShared& s, int* status)
 // two close to the norm of a panel column.
 __global__ void __cluster_dims__(kFactCtas, 1, 1) __launch_bounds__(kFactThreads, 1)
 block_factor_kernel(const float* __restrict__ Z, int ldz, float* P1, int ld, int ob, float* __restrict__ Tt,
-                    int ldt, float* __restrict__ Dt, int ldd, float scale, float dscale, int round, int* __restrict__ status)
+                    int ldt, float* __restrict__ Dt, int ldd, float scale, float dscale, int round, unsigned long long wait_ns,
+                    int* __restrict__ status)
 {
     chain_next();
     chain_wait();
+    if (wait_ns == 0) {                                      // give up before any copy is on its way
+        if (blockIdx.x == 0 && threadIdx.x == 0) atomicCAS(status, 0, (int)GELO_ERR_TIMEOUT);
+        return;
+    }
     extern __shared__ __align__(128) uint8_t fsm[];
     FactShared& s = *reinterpret_cast<FactShared*>(fsm);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, gid = lane >> 2, tig = lane & 3;
@@ -498,6 +508,7 @@ block_factor_kernel(const float* __restrict__ Z, int ldz, float* P1, int ld, int
     const bool compute = tid < kFactCompute;
 
     if (tid == 0) {
+        s.abort = 0;
         for (int i = 0; i < kSteps; ++i) {
             tcx::mbar_init(tcx::smem_u32(&s.got_full[i]), 1);
             tcx::mbar_init(tcx::smem_u32(&s.panel_full[i]), 1);
@@ -535,11 +546,11 @@ block_factor_kernel(const float* __restrict__ Z, int ldz, float* P1, int ld, int
     __syncwarp();
     cluster_sync_all();                                      // barriers initialised, P1 read, the first block published
     if (!compute) {
-        if (role == FACT_GRAM) fact_pivots<FACT_GRAM>(s, status);
-        else if (role == FACT_INVERSE) fact_pivots<FACT_INVERSE>(s, status);
-        else fact_pivots<FACT_FACTOR>(s, status);
+        if (role == FACT_GRAM) fact_pivots<FACT_GRAM>(s, wait_ns, status);
+        else if (role == FACT_INVERSE) fact_pivots<FACT_INVERSE>(s, wait_ns, status);
+        else fact_pivots<FACT_FACTOR>(s, wait_ns, status);
     } else if (role == FACT_GRAM) {
-        fact_compute<FACT_GRAM>(a, s, status);
+        fact_compute<FACT_GRAM>(a, s, wait_ns, status);
         // B = P1 + R, the top block of V
         const float* R = reinterpret_cast<const float*>(&s.panel[0][0][0][0]);
 #pragma unroll 4
@@ -554,8 +565,8 @@ block_factor_kernel(const float* __restrict__ Z, int ldz, float* P1, int ld, int
             }
         }
     } else {
-        if (role == FACT_INVERSE) fact_compute<FACT_INVERSE>(a, s, status);
-        else fact_compute<FACT_FACTOR>(a, s, status);
+        if (role == FACT_INVERSE) fact_compute<FACT_INVERSE>(a, s, wait_ns, status);
+        else fact_compute<FACT_FACTOR>(a, s, wait_ns, status);
         float* dst = role == FACT_INVERSE ? Dt : Tt;
         const int ldo = role == FACT_INVERSE ? ldd : ldt;
         const float f = role == FACT_INVERSE ? dscale * s1 : s2;
@@ -573,6 +584,17 @@ block_factor_kernel(const float* __restrict__ Z, int ldz, float* P1, int ld, int
     }
     __syncwarp();
     cluster_sync_all();                                      // nobody's shared memory goes while a copy may still reach it
+    if (*static_cast<volatile int*>(&s.abort)) {             // (the same in all three CTAs) not every copy has been waited for
+        if (tid == 0 && role != FACT_GRAM) {
+            int on = 0;                                      // a flag that stays zero: these waits only end in time
+            for (int i = 0; i < kSteps; ++i) {
+                tcx::mbar_wait(tcx::smem_u32(&s.got_full[i]), 0, &on, wait_ns);
+                if (role == FACT_FACTOR) tcx::mbar_wait(tcx::smem_u32(&s.panel_full[i]), 0, &on, wait_ns);
+            }
+        }
+        __syncwarp();
+        cluster_sync_all();
+    }
 }
 
 // Z = scale * (sum of the K slices of P^T [V_< | P | C]), in slice order; columns c0 .. c0 + ob - 1 (the Gram matrix) stay
@@ -749,7 +771,7 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
             float scale = 1.0f;                              // a power of two with scale^2 about nr
             while (2.0f * scale * scale < (float)nr) scale *= 2.0f;
             GELO_TRY(launch_chained(ctx, block_factor_kernel, kFactCtas, kFactThreads, kFactSmemBytes, st, tc.w32[0] + r, ld,
-                                   P, ld, ob, Tb, kSuper, tc.t128, FB, scale, loss1, round, ctx->status_dev));
+                                   P, ld, ob, Tb, kSuper, tc.t128, FB, scale, loss1, round, ctx->wait_limit_ns, ctx->status_dev));
             GELO_TRY(after_launch(ctx));
             if (e - s > 1) {
                 // [X^T | . | W'] = T^T Z + D^T [V_< | . | C1], scaled up for the truncation of V in the next product

@@ -113,3 +113,22 @@ def test_calls_of_equal_m_in_one_context(entry, kind):
             assert ((got - ref).norm() / ref.norm()).item() <= 2e-2, (n, k, block, i)        # the bf16 path's tolerance
         out.zero_()
     c.close()
+
+
+# The block factor's copies between CTAs are waited for as long as the context says: with a limit of zero it gives up before it sends any, which
+# the fp32 route (no tensor-core kernel in it) reports by itself.
+def test_zero_wait_limit_reaches_the_block_factor():
+    m, dt = 300, "f32"
+    c = binding.Context(0)
+    c.ensure_workspace(m, 0, 8, 24, dt)
+    ld = c.mixing_ld(m)
+    A = padded(m, ld, TDT[dt]); X = padded(m, ld, TDT[dt])
+    c.set_wait_limit_ns(0)
+    c.sample_mixing(m, ORTHOGONAL, 5, dt, A, X, ld)
+    assert c.last_status() == binding.ERR_TIMEOUT
+    c.set_wait_limit_ns(2_000_000_000)
+    c.sample_mixing(m, ORTHOGONAL, 5, dt, A, X, ld)
+    assert c.last_status() == binding.OK
+    a = f64(A[:, :m])
+    assert np.linalg.norm(a.T @ a - np.eye(m)) / np.sqrt(m) <= 2e-6
+    c.close()
