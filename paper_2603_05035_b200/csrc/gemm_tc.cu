@@ -26,7 +26,7 @@
 //   overlap the main loop of the next.
 // * Every wait on an mbarrier is bounded in time (the context's wait limit, two seconds by default,
 //   measured on the GPU's global timer); on expiry the CTA records GELO_ERR_TIMEOUT in the
-//   context's status word, stops issuing work, releases tensor memory and returns.
+//   context's status word, stops issuing work, lets what is in flight arrive, releases tensor memory and returns.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -593,7 +593,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     tc_fence_before();
     __syncwarp();
     if (kPair) cluster_sync(); else __syncthreads();
+    settle(abort_flag, prm.wait_ns);
     if (warp == 1) {
+        __syncwarp();
         tc_fence_after();
         if (kPair) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
         else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
