@@ -98,6 +98,7 @@ int launch_gaussian_as(gelo_ctx* ctx, int rows, int cols, int ldb, int ld, uint6
     const uint64_t blocks = ((uint64_t)rows * cols + 3) >> 2;
     const int threads = 256;
     const uint64_t grid = (blocks + threads - 1) / threads;
+    if (grid > 0x7fffffffull) return GELO_ERR_INVALID;
     GELO_TRY(launch_chained(ctx, gaussian_kernel<T>, (unsigned)grid, threads, 0, st, rows, cols, ldb, ld, seed, seed_dev, stream_id, attempt,
                            scale, base, static_cast<T*>(out)));
     return after_launch(ctx);

@@ -53,6 +53,14 @@ def test_gaussian_matches_oracle(ctx, oracle, rows, cols, ld):
         assert torch.isnan(out[:, cols:]).all()      # padding columns are never written
 
 
+def test_gaussian_refuses_more_than_a_grid(ctx):
+    # 2^42 elements are 2^32 thread blocks, more than one launch can have
+    out = torch.zeros(64, device="cuda")
+    with pytest.raises(binding.GeloError) as e:
+        ctx.sample_gaussian(1 << 21, 1 << 21, 1 << 21, 1, 0, 0, 1.0, out)
+    assert e.value.status == binding.ERR_INVALID and (out == 0).all()
+
+
 def test_gaussian_statistics(ctx):
     out = torch.empty((2048, 2048), device="cuda", dtype=torch.float32)
     ctx.sample_gaussian(2048, 2048, 2048, 5, 0, 0, 1.0, out)
