@@ -33,7 +33,9 @@
  *   - All other matrices are dense: H n x d, S k x d, U m x d, W d x p, Y' m x p,
  *     Q/K/V n x (p/3).  d and p must be multiples of 8.
  *   - Scratch memory comes from the caller through gelo_set_workspace; no entry point
- *     except gelo_create / gelo_destroy allocates or frees device memory.
+ *     except gelo_create / gelo_destroy allocates or frees device memory of its own.  The driver
+ *     keeps what it needs for recorded launch graphs (the whole-call entry points replay their
+ *     sampling; 0.3 to 4 MB each, 128 per context at most, from the second call of a size on).
  */
 #ifndef GELO_H
 #define GELO_H

@@ -261,25 +261,35 @@ void drop_graphs(gelo_ctx* ctx)
 // Samples (A, A^-1) of one batched call on a lane stream by replaying a launch graph of the whole sampling
 // sequence (about a thousand dependent launches): one host call instead of a thousand, so a single host thread
 // keeps all lanes busy.  The seed reaches the kernels through the lane's device slot.  The first use of a
-// combination of places, sizes and settings (SampleKey) records the graph by stream capture.
+// combination of places, sizes and settings (SampleKey) records the graph by stream capture, that of a call by itself (`single`) only the
+// second: recording and instantiating costs more than the launches (4300 rows non-orthogonal, first call 5.6 ms recorded, 3.8 ms launched,
+// 3.6 ms replayed; 67 rows 0.73, 0.43 and 0.39 ms), and a caller whose row counts vary may never come back to one.
 int sample_on_lane(gelo_ctx* ctx, const Layout& L, int lane, int m, int kind, uint64_t seed, int dtype, cudaStream_t ls,
-                   bool deferred = true)
+                   bool deferred, bool single)
 {
     if (sample_small_supports(ctx, m, kind))                 // one launch: nothing to record
         return sample_attempt(ctx, L, m, kind, seed, 0u, dtype, L.A, L.Ainv, L.ldi, nullptr, ls, deferred, nullptr);
-    uint64_t* slot = ctx->lane_seed_dev + lane * 8;
-    set_seed_kernel<<<1, 1, 0, ls>>>(slot, seed);
-    GELO_TRY(after_launch(ctx));
     if (ctx->prof_on)      // per-launch timing needs real launches
-        return sample_attempt(ctx, L, m, kind, seed, 0u, dtype, L.A, L.Ainv, L.ldi, nullptr, ls, deferred, slot);
+        return sample_attempt(ctx, L, m, kind, seed, 0u, dtype, L.A, L.Ainv, L.ldi, nullptr, ls, deferred, nullptr);
+    uint64_t* slot = ctx->lane_seed_dev + lane * 8;
     const gelo_ctx::SampleKey key = { L.G, L.A, L.Ainv, L.cond_val, slot, L.m, m, kind, dtype, ctx->level3, ctx->tc_update_ctas, deferred };
     for (auto& g : ctx->graphs) {
         if (g.key == key) {
+            set_seed_kernel<<<1, 1, 0, ls>>>(slot, seed);
+            GELO_TRY(after_launch(ctx));
             GELO_CUDA_OK(cudaGraphLaunch(g.exec, ls));
             ctx->launches += g.launches;
+            g.used = ++ctx->graph_clock;
             return GELO_OK;
         }
     }
+    if (single && std::find(ctx->met, ctx->met + kMetKeys, key) == ctx->met + kMetKeys) {
+        ctx->met[ctx->met_next] = key;
+        ctx->met_next = (ctx->met_next + 1) % kMetKeys;
+        return sample_attempt(ctx, L, m, kind, seed, 0u, dtype, L.A, L.Ainv, L.ldi, nullptr, ls, deferred, nullptr);
+    }
+    set_seed_kernel<<<1, 1, 0, ls>>>(slot, seed);
+    GELO_TRY(after_launch(ctx));
     const long long before = ctx->launches;
     GELO_CUDA_OK(cudaStreamBeginCapture(ls, cudaStreamCaptureModeRelaxed));
     ctx->recording = true;
@@ -298,7 +308,15 @@ int sample_on_lane(gelo_ctx* ctx, const Layout& L, int lane, int m, int kind, ui
     const cudaError_t ie = cudaGraphInstantiate(&g.exec, graph, 0);
     cudaGraphDestroy(graph);
     if (ie != cudaSuccess) return GELO_ERR_CUDA;
-    ctx->graphs.push_back(g);
+    g.used = ++ctx->graph_clock;
+    if (ctx->graphs.size() < (size_t)kMaxGraphs) {
+        ctx->graphs.push_back(g);
+    } else {
+        auto oldest = std::min_element(ctx->graphs.begin(), ctx->graphs.end(),
+                                       [](const gelo_ctx::SampleGraph& a, const gelo_ctx::SampleGraph& b) { return a.used < b.used; });
+        cudaGraphExecDestroy(oldest->exec);                   // (one that is still running is freed when it ends)
+        *oldest = g;
+    }
     GELO_CUDA_OK(cudaGraphLaunch(g.exec, ls));
     return GELO_OK;
 }
@@ -461,7 +479,7 @@ int offload_impl(gelo_ctx* ctx, const Layout& L, const void* H, const void* W, i
         GELO_CUDA_OK(cudaEventRecord(ctx->batch_start, st));
         GELO_CUDA_OK(cudaStreamWaitEvent(ls, ctx->batch_start, 0));
         LaneJoin join(ctx, st, 1);
-        if (attempt == 0) GELO_TRY(sample_on_lane(ctx, L, 0, m, kind, seed, dtype, ls, false));
+        if (attempt == 0) GELO_TRY(sample_on_lane(ctx, L, 0, m, kind, seed, dtype, ls, false, true));
         else GELO_TRY(sample_attempt(ctx, L, m, kind, seed, (uint32_t)attempt, dtype, L.A, L.Ainv, L.ldi, nullptr, ls));
         GELO_CUDA_OK(cudaMemcpyAsync(ctx->status_host, ctx->status_dev, kStatusWords * sizeof(int), cudaMemcpyDeviceToHost, ls));
         GELO_CUDA_OK(cudaEventRecord(ctx->lane_ready[0], ls));
@@ -563,7 +581,7 @@ int offload_batch_impl(gelo_ctx* ctx, int calls, const void* const* H, const voi
         for (int i = 0; i < calls; ++i) {
             const int l = i % D;
             cudaStream_t ls = ctx->lane_stream[l];
-            GELO_TRY(sample_on_lane(ctx, L[l], l, m, kinds[i], seeds[i], dtype, ls));
+            GELO_TRY(sample_on_lane(ctx, L[l], l, m, kinds[i], seeds[i], dtype, ls, true, calls == 1));
             if (chained && i < D) GELO_CUDA_OK(cudaStreamWaitEvent(ls, ctx->batch_start, 0));
             GELO_TRY(run_shield_rows(ctx, H[i], n, d, k, shield_scale, seeds[i], dtype, L[l].S, L[l].sh, ls, ctx->shield_nu));
             GELO_TRY(mix_impl(ctx, L[l].A, L[l].ldi, H[i], k > 0 ? L[l].S : nullptr, n, k, d, dtype, L[l].U, ls, nullptr));
@@ -581,7 +599,7 @@ int offload_batch_impl(gelo_ctx* ctx, int calls, const void* const* H, const voi
         const int l = i % D;
         cudaStream_t ls = ctx->lane_stream[l];
         if (i >= D || chained) GELO_CUDA_OK(cudaStreamWaitEvent(ls, ctx->lane_free[l], 0));
-        GELO_TRY(sample_on_lane(ctx, L[l], l, m, kinds[i], seeds[i], dtype, ls));
+        GELO_TRY(sample_on_lane(ctx, L[l], l, m, kinds[i], seeds[i], dtype, ls, true, calls == 1));
         GELO_CUDA_OK(cudaEventRecord(ctx->lane_ready[l], ls));
         return GELO_OK;
     };
@@ -726,7 +744,7 @@ int offload_blockdiag_impl(gelo_ctx* ctx, int calls, const void* const* H, const
         cudaStream_t ls = ctx->lane_stream[l];
         if (v >= D) GELO_CUDA_OK(cudaStreamWaitEvent(ls, ctx->lane_free[l], 0));
         const uint64_t seed = seeds[c] ^ (0x9E3779B97F4A7C15ull * (uint64_t)(j + 1));     // a fresh A_j per group and call
-        return sample_on_lane(ctx, L[l], l, P.nd[j] + P.ns[j], GELO_ORTHOGONAL, seed, dtype, ls);
+        return sample_on_lane(ctx, L[l], l, P.nd[j] + P.ns[j], GELO_ORTHOGONAL, seed, dtype, ls, true, false);
     };
     for (long long v = 0; v < total && v < D; ++v) GELO_TRY(enqueue_sample(v));
     for (int c = 0; c < calls; ++c) {

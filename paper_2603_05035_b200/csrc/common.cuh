@@ -21,6 +21,9 @@ constexpr int kPanel = 32;
 // [1]: verdict of the last condition-number check (1 = accepted).  [2]: detail word.
 constexpr int kStatusWords = 8;
 constexpr int kMaxLanes = 32;
+// Recorded sampling graphs of a context: two kinds on every lane, for two shapes.  One takes 0.3 to 4 MB of the driver's memory.
+constexpr int kMaxGraphs = 4 * kMaxLanes;
+constexpr int kMetKeys = 16;
 
 // Kernel classes that the optional per-launch timing distinguishes.
 enum ProfClass { PROF_RANK_UPDATE = 0, PROF_VTC = 1, PROF_GEMM_TC = 2, PROF_QR_PANEL = 3, PROF_LU_PANEL = 4,
@@ -92,8 +95,11 @@ struct gelo_ctx {
                    dtype == o.dtype && level3 == o.level3 && tc_ctas == o.tc_ctas && deferred == o.deferred;
         }
     };
-    struct SampleGraph { SampleKey key; cudaGraphExec_t exec; long long launches; };
-    std::vector<SampleGraph> graphs;
+    struct SampleGraph { SampleKey key; cudaGraphExec_t exec; long long launches; unsigned long long used; };
+    std::vector<SampleGraph> graphs;                // kMaxGraphs at most; the one not used for longest makes room
+    unsigned long long graph_clock = 0;
+    SampleKey met[gelo::kMetKeys] = {};             // single calls that have run once and would record on the next
+    int met_next = 0;
     bool recording = false;                         // the launches go into such a graph
     uint64_t* lane_seed_dev = nullptr;              // one seed slot per lane
     // the batched host variant moves activations in and results out on streams of their own, through two staging pairs
