@@ -4,7 +4,7 @@
 // The B operand may be the vertical stack of two matrices (Eq. 8: H_full = [H; S])
 // and the output may be split into column thirds (Q | K | V).
 //
-// Two kernels: gemm_f32_kernel for fp32 matrices with 16-byte rows, gemm_simt_kernel for everything else.
+// Two kernels: gemm_f32_kernel for fp32 matrices with 16-byte rows where the tiles are few, gemm_simt_kernel for everything else.
 #include "common.cuh"
 
 namespace gelo {
@@ -338,10 +338,22 @@ int launch_gemm_simt(gelo_ctx* ctx, const GemmArgs& g, cudaStream_t st)
     p.kper = ceil_div(ceil_div(g.K, g.ksplit), BK) * BK;      // (the caller's slices: whole steps, none of them empty)
     p.plane = g.plane;
     const int slices = g.ksplit;
-    if (g.dtype == GELO_F32 && !g.transB && !g.B2 && aligned_rows(g.A, g.lda) && aligned_rows(g.B, g.ldb) && aligned_rows(g.C[0], g.ldc) &&
+    // gemm_f32_kernel is made for products that leave SMs idle: up to one of its 64 x 64 tiles per SM it takes 0.3 to 0.9 of the time of
+    // the tiles below (4096 x 4096 by 64 rows 268 -> 109 us, 127 rows 269 -> 187 us).  Beyond, a plain product runs faster on those, which
+    // hold four CTAs per SM instead of one: 4096 x 12288 by 127 rows 496 us there, 586 us here; 1000 x 1000 by 4096 columns
+    // 281 and 320 us.  In a second round of tiles it depends: this kernel loses what its last stage of 64 k leaves empty (200 x 200 by 4096 columns
+    // 24.8 us there, 26.9 here) and cannot hide the latency of a B that comes from DRAM (64 rows, 4096 x 12288: 371 and 384 us; 512 x 12288
+    // 51.5 and 49.4), except that it does not load rows past M (17 rows, 4096 x 16384: 365 and 340 us; a third round, by 24576
+    // columns, 490 and 516 us).  The sampler's products (transposed, in slices, or adding to C) stay here: 3000 rows orthogonal 9.7 ms
+    // like this, 9.5 ms on the tiles below, but 1075 rows 1.14 and 1.18 ms.
+    const long tiles64 = (long)ceil_div(g.N, 64) * ceil_div(g.M, kF32M) * slices;
+    const bool plain = !g.transA && g.beta == 0.0f && g.diag == 0.0f && slices == 1;
+    const bool two_rounds = ceil_div(g.K, kF32K) * kF32K - g.K <= g.K / 16 && (g.M <= 32 || (size_t)g.K * g.N * sizeof(float) <= (72u << 20));
+    const bool few_tiles = !plain || tiles64 <= (two_rounds ? 2L : 1L) * ctx->sm_count;
+    if (few_tiles && g.dtype == GELO_F32 && !g.transB && !g.B2 && aligned_rows(g.A, g.lda) && aligned_rows(g.B, g.ldb) && aligned_rows(g.C[0], g.ldc) &&
         (g.nsplit == 1 || (p.csplit % 4 == 0 && aligned_rows(p.C1, g.ldc) && aligned_rows(p.C2, g.ldc))) && g.plane % 4 == 0) {
         // rows of A and B are read in whole quads: the last one of a row may reach past its end, but not past its stride
-        const bool wide = (long)ceil_div(g.N, 64) * ceil_div(g.M, kF32M) * slices >= ctx->sm_count;
+        const bool wide = tiles64 >= ctx->sm_count;
         if (g.transA) return wide ? launch_f32<true, 64>(ctx, p, slices, st) : launch_f32<true, 32>(ctx, p, slices, st);
         return wide ? launch_f32<false, 64>(ctx, p, slices, st) : launch_f32<false, 32>(ctx, p, slices, st);
     }

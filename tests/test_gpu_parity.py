@@ -1214,6 +1214,19 @@ def test_fp32_products_of_any_depth(ctx, oracle, n, k, kind):
     assert ((Q.double() - ref).norm() / ref.norm()).item() <= TOL["f32"]
 
 
+# fp32 products on either side of the lines between the two FMA kernels: 148 tiles of 64 x 64 and one more where the last stage of k is short,
+# 296 and one more where it is full, with a last tile of eight columns and a K that ends a quad after two
+@pytest.mark.parametrize("m,d,p", [(33, 72, 9472), (33, 72, 9480), (32, 64, 18944), (32, 64, 18952), (65, 64, 9472), (1, 8, 8)])
+def test_fp32_products_on_both_fma_kernels(ctx, m, d, p):
+    g = torch.Generator(device="cuda"); g.manual_seed(m + p)
+    U = torch.randn((m, d), generator=g, device="cuda"); W = torch.randn((d, p), generator=g, device="cuda")
+    Y = torch.full((m, p), float("nan"), device="cuda")
+    ctx.project(U, W, m, d, p, "f32", Y)
+    ref = U.double() @ W.double()
+    # sums of 72 products in fp32
+    assert ((Y.double() - ref).norm() / ref.norm()).item() <= 2e-6
+
+
 # whole calls on the lanes: one over the small path, the last size that takes it and the first that does not; fewer calls than
 # lanes, a second round per lane, results in one buffer that every call overwrites (call order is promised)
 @pytest.mark.parametrize("n,k,calls,shared", [(120, 9, 6, False), (2200, 104, 5, False), (2201, 104, 5, False), (300, 15, 13, False), (300, 15, 7, True)])
