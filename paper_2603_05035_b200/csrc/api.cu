@@ -16,12 +16,34 @@ inline cudaStream_t as_stream(void* s) { return static_cast<cudaStream_t>(s); }
 inline int round_up(int x, int to) { return (x + to - 1) / to * to; }
 constexpr int kTcMinRows = 256;   // below this the factorisations are latency-bound anyway, and stay in fp32
 // Up to here fp32 samples (and 16-bit ones of less than kTcMinRows rows) take the block QR in fp32 multiply-adds instead of
-// 32-column Householder panels: orthogonal sample at 512 rows 1.52 -> 0.45 ms, 1075 rows 3.59 -> 1.19 ms, 3000 rows 12.4 -> 9.4 ms.
+// 32-column Householder panels: orthogonal sample at 512 rows 1.52 -> 0.45 ms, 1075 rows 3.59 -> 1.14 ms, 3000 rows 12.4 -> 9.7 ms.
+// That is a sample alone; see panels_hide() for the batches in which the panels are the better route.
 constexpr int kExactBlockRows = 3072;
 // And up to here Newton's iteration in fp32 multiply-adds instead of the LU, whose latency its ten products undercut:
 // non-orthogonal sample at 512 rows 3.61 -> 0.70 ms; |A^-1 A - I| / sqrt(m) there 1.1e-5 -> 4e-7.  At 1075 rows alone it is 8.09 -> 2.16 ms,
 // but 32 calls on 16 lanes lose 6%: that much arithmetic on the FMA pipes is no longer hidden.
 constexpr int kExactNewtonRows = 768;
+
+// Whether the fp32 samples of a batch go back to register panels and the LU (its lanes carry `orth` and `non` samples of either kind at a
+// time).  A sample in blocks keeps the whole GPU busy, a chain of panels 8 SMs, so enough chains side by side take less
+// time than the same samples in blocks, one after the other, however much longer each takes.  What either takes, in microseconds, measured at
+// 300 to 2900 rows:
+//   a sample in blocks, the GPU full of them     s = m^2 (2.3e-4 + 2.0e-7 m)       512 rows 87 (94), 1075 514 (507), 2900 6810 (6900)
+//   with Newton's iteration behind it            m^2 (3.45e-4 + 6.55e-7 m)         512 rows 178 (178), 768 500 (500)
+//   a chain of panels alone                      m (2.95 + 1.6e-7 m^2)             512 rows 1530 (1510), 2900 12460 (12640)
+//   with the LU behind it                        m (7.0 + 2.2e-7 m^2)              400 rows 2810 (2850), 768 5480 (5530)
+//   and what it slows the others down by         0.28 s (0.08 s below four lanes, where nothing is cut into shares of the SMs)
+// Above kExactNewtonRows the LU follows either way, and a non-orthogonal sample's QR, which is not polished, counts as 0.45 of one.
+// 32 calls on 32 lanes, d = p = 256: 768 rows orthogonal 6.7 ms in blocks, 3.9 in panels, non-orthogonal 16.0 and 7.9; 1075 rows 16.2 and 7.5; sixteen of 2900
+// rows 111 and 42; eight of 1075 rows 4.1 and 4.4.
+bool panels_hide(int m, double orth, double non, bool shares)
+{
+    const double x = m, s = x * x * (2.3e-4 + 2.0e-7 * x);
+    const bool newton = m <= kExactNewtonRows;
+    const double sn = newton ? x * x * (3.45e-4 + 6.55e-7 * x) : 0.45 * s;
+    const double chain = newton && non > 0 ? x * (7.0 + 2.2e-7 * x * x) : x * (2.95 + 1.6e-7 * x * x);
+    return orth * s + non * sn > chain + (shares ? 0.28 : 0.08) * (orth * s + non * (newton ? s : sn));
+}
 
 // How a factorisation of an m x m sample stored as `dtype` runs its level-3 updates: 0 = fp32 FMA kernels,
 // 2 = tensor cores with three bf16 products of split operands, 3 = tensor cores with one tf32 product.
@@ -184,7 +206,7 @@ int sample_attempt(gelo_ctx* ctx, const Layout& L, int m, int kind, uint64_t see
     const int l3 = level3_kind(ctx, m, dtype, true);
     // the block route signs its columns itself; the others leave that to the copy (by the diagonal of R, in L.G)
     // (fp32 storage and small matrices, l3 = 0: the same in fp32 multiply-adds)
-    const bool exact = ctx->level3 == 0 && l3 == 0 && m <= kExactBlockRows;
+    const bool exact = ctx->level3 == 0 && l3 == 0 && m <= kExactBlockRows && !(ctx->panel_samples && dtype == GELO_F32);
     const bool blocks = (l3 == 3 || exact) && gaussian_qr_supports(m);
     const float* sign = blocks ? nullptr : L.G;
     if (blocks) GELO_TRY(run_gaussian_qr(ctx, m, L.G, ldi, L.Qraw, L.tc, exact, st));
@@ -272,7 +294,8 @@ int sample_on_lane(gelo_ctx* ctx, const Layout& L, int lane, int m, int kind, ui
     if (ctx->prof_on)      // per-launch timing needs real launches
         return sample_attempt(ctx, L, m, kind, seed, 0u, dtype, L.A, L.Ainv, L.ldi, nullptr, ls, deferred, nullptr);
     uint64_t* slot = ctx->lane_seed_dev + lane * 8;
-    const gelo_ctx::SampleKey key = { L.G, L.A, L.Ainv, L.cond_val, slot, L.m, m, kind, dtype, ctx->level3, ctx->tc_update_ctas, deferred };
+    const gelo_ctx::SampleKey key = { L.G, L.A, L.Ainv, L.cond_val, slot, L.m, m, kind, dtype, ctx->level3, ctx->tc_update_ctas, ctx->panel_samples,
+                                     deferred };
     for (auto& g : ctx->graphs) {
         if (g.key == key) {
             set_seed_kernel<<<1, 1, 0, ls>>>(slot, seed);
@@ -448,6 +471,20 @@ struct LaneJoin {
     }
 };
 
+// How the lanes of a batch plan and factorise, for as long as it is being enqueued: with several lanes in flight each level-3 update takes a
+// share of the SMs (ctx->lane_tc_share-th of them).
+struct LanePlan {
+    gelo_ctx* ctx;
+    LanePlan(gelo_ctx* c, int lanes, int m, double orth, double non) : ctx(c)
+    {
+        const bool shares = lanes >= c->lane_tc_share && c->lane_tc_share > 1;
+        c->tc_update_ctas = shares ? c->sm_count / c->lane_tc_share : 0;
+        c->panel_samples = panels_hide(m, orth, non, shares);
+    }
+    LanePlan(const LanePlan&) = delete;
+    ~LanePlan() { ctx->tc_update_ctas = 0; ctx->panel_samples = false; }
+};
+
 // One whole call on the caller's stream.  A non-orthogonal pair is verified: the first attempt replays the recorded sampling
 // graph on a lane's stream beside the shield rows, and what needs the pair but only writes to the workspace (mixing, and the
 // projection where it is a launch of its own) is enqueued behind it.  The host waits for the verdict, which comes in while
@@ -552,8 +589,9 @@ int offload_batch_impl(gelo_ctx* ctx, int calls, const void* const* H, const voi
                                            project_unmix_supports(ctx, n, k, d, p, dtype, L[0].ldi, split ? 3 : 1)));
     for (int i = 0; i < calls && small; ++i) small = !misaligned(H[i]);
     if (small && calls > 1) small = !calls_depend(calls, H, (size_t)n * d * es, W, (size_t)d * p * es, Q, K, V, split ? third : (size_t)n * p * es);
-    // with several lanes in flight each level-3 update takes a share of the SMs (ctx->lane_tc_share-th of them)
-    ctx->tc_update_ctas = (D >= ctx->lane_tc_share && ctx->lane_tc_share > 1) ? ctx->sm_count / ctx->lane_tc_share : 0;
+    const int orth_calls = (int)std::count(kinds, kinds + calls, (int)GELO_ORTHOGONAL);
+    const LanePlan plan(ctx, D, m, (double)D * orth_calls / calls, (double)D * (calls - orth_calls) / calls);
+    LaneJoin join(ctx, st, D);
 
     // Back-to-back batches of the same shape on the same stream keep the lanes running across the seam: each
     // lane only waits until the products that read its previous pair are done.  Otherwise the lanes start after
@@ -653,7 +691,7 @@ int offload_batch_impl(gelo_ctx* ctx, int calls, const void* const* H, const voi
         GELO_CUDA_OK(cudaStreamWaitEvent(st, ctx->y_free[0], 0));
         GELO_CUDA_OK(cudaStreamWaitEvent(st, ctx->y_free[1], 0));
     }
-    ctx->tc_update_ctas = 0;
+    join.done();                                              // (every lane's last work has been waited for above)
     ctx->chain_valid = calls >= D && !ctx->prof_on;
     ctx->chain_stream = st;
     ctx->chain_key = L[D - 1].G;
@@ -734,11 +772,12 @@ int offload_blockdiag_impl(gelo_ctx* ctx, int calls, const void* const* H, const
     const bool split = K[0] != nullptr;
     const int qcols = split ? p / 3 : p;
     ctx->chain_valid = false;                                 // this layout is not the one a later plain batch chains onto
-    ctx->tc_update_ctas = (D >= ctx->lane_tc_share && ctx->lane_tc_share > 1) ? ctx->sm_count / ctx->lane_tc_share : 0;
+    const long long total = (long long)calls * P.nb;
+    const LanePlan plan(ctx, D, P.bmax, (double)std::min<long long>(D, total), 0.0);
+    LaneJoin join(ctx, st, D);
     GELO_CUDA_OK(cudaEventRecord(ctx->batch_start, st));
     for (int l = 0; l < D; ++l) GELO_CUDA_OK(cudaStreamWaitEvent(ctx->lane_stream[l], ctx->batch_start, 0));
 
-    const long long total = (long long)calls * P.nb;
     auto enqueue_sample = [&](long long v) -> int {
         const int l = (int)(v % D), c = (int)(v / P.nb), j = (int)(v % P.nb);
         cudaStream_t ls = ctx->lane_stream[l];
@@ -785,7 +824,7 @@ int offload_blockdiag_impl(gelo_ctx* ctx, int calls, const void* const* H, const
             if (v < total) GELO_TRY(enqueue_sample(v));
         }
     }
-    ctx->tc_update_ctas = 0;
+    join.done();
     return GELO_OK;
 }
 

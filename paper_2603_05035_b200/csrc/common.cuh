@@ -58,6 +58,7 @@ struct gelo_ctx {
     int lane_tc_share = 4;        // batches with at least this many lanes plan each level-3 update for 1/share of the SMs
     int tc_update_ctas = 0;       // CTAs that a level-3 tensor-core launch is planned for (0: one per SM): with many lanes fewer K slices
                                   // do, because the updates of several lanes run side by side
+    bool panel_samples = false;   // fp32 samples of the running batch take 32-column panels (panels_hide in api.cu)
     int level3 = 0;               // 0: tf32 tensor-core updates for bf16 calls with m >= 256; 1: always fp32 FMA;
                                   // 2: always tensor cores, three bf16 products of split operands; 3: always tensor cores, tf32
     long long launches = 0;
@@ -88,11 +89,11 @@ struct gelo_ctx {
     // the estimate: they stand behind the row norms of the data rows, so they move with n at equal m.
     struct SampleKey {
         const void *G, *A, *Ainv, *cond, *seed;
-        int rows, m, kind, dtype, level3, tc_ctas, deferred;
+        int rows, m, kind, dtype, level3, tc_ctas, panels, deferred;
         bool operator==(const SampleKey& o) const
         {
             return G == o.G && A == o.A && Ainv == o.Ainv && cond == o.cond && seed == o.seed && rows == o.rows && m == o.m && kind == o.kind &&
-                   dtype == o.dtype && level3 == o.level3 && tc_ctas == o.tc_ctas && deferred == o.deferred;
+                   dtype == o.dtype && level3 == o.level3 && tc_ctas == o.tc_ctas && panels == o.panels && deferred == o.deferred;
         }
     };
     struct SampleGraph { SampleKey key; cudaGraphExec_t exec; long long launches; unsigned long long used; };

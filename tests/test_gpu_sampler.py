@@ -156,3 +156,29 @@ def test_sampling_graphs_are_bounded(kind):
     # 128 recordings are reached at 258 rows; one of them takes 0.36 MB (62 MB for the 179 sizes that follow, if all were kept)
     assert free[300] - free[479] <= 48 << 20
     c.close()
+
+
+# fp32 batches: the samples of few lanes run in blocks, those of many in panels beside each other (768 rows: from sixteen orthogonal or
+# non-orthogonal ones on, alternating kinds from more); either way H W comes out
+@pytest.mark.parametrize("n,lanes,kinds,panels", [(768, 8, (0,), False), (768, 16, (0,), True), (768, 16, (1,), True), (768, 16, (0, 1), False),
+                                                  (1000, 16, (0, 1), True), (129, 32, (0,), False)])
+def test_fp32_batches_choose_the_route_by_what_is_in_flight(n, lanes, kinds, panels):
+    d, p = 64, 64
+    c = binding.Context(0)
+    c.set_lanes(lanes)
+    c.ensure_batch_workspace(n, 0, d, p, "f32", lanes)
+    H = [inputs.make_hidden(n, d, "f32", 40 + i, True, "cuda") for i in range(lanes)]
+    W = [inputs.make_weight(d, p, "f32", 90, "cuda")] * lanes
+    Y = torch.zeros((lanes, n, p), device="cuda")
+    call = lambda: c.qkv_offload_batch(H, W, n, 0, d, p, [kinds[i % len(kinds)] for i in range(lanes)], list(range(lanes)), 10.0, "f32", list(Y))
+    c.profile_start()
+    call()
+    assert (c.profile_stop()["qr_panel"]["launches"] > 0) == panels
+    Y.zero_()
+    call()
+    torch.cuda.synchronize()
+    assert c.last_status() == binding.OK
+    for i in range(lanes):
+        ref = H[i].double() @ W[i].double()
+        assert ((Y[i].double() - ref).norm() / ref.norm()).item() <= 1e-4           # the fp32 path's tolerance
+    c.close()
