@@ -482,7 +482,7 @@ struct LanePlan {
         c->panel_samples = panels_hide(m, orth, non, shares);
     }
     LanePlan(const LanePlan&) = delete;
-    ~LanePlan() { ctx->tc_update_ctas = 0; ctx->panel_samples = false; }
+    ~LanePlan() { ctx->tc_update_ctas = 0; ctx->panel_samples = ctx->lone_launches = false; }
 };
 
 // One whole call on the caller's stream.  A non-orthogonal pair is verified: the first attempt replays the recorded sampling
@@ -592,6 +592,11 @@ int offload_batch_impl(gelo_ctx* ctx, int calls, const void* const* H, const voi
     const int orth_calls = (int)std::count(kinds, kinds + calls, (int)GELO_ORTHOGONAL);
     const LanePlan plan(ctx, D, m, (double)D * orth_calls / calls, (double)D * (calls - orth_calls) / calls);
     LaneJoin join(ctx, st, D);
+    // Whole calls on two or three lanes: a projection that is set up early keeps its SMs while its lane's sample runs, and where the projections of
+    // all lanes take most of the GPU another lane's sample has to wait for them.  Three calls of 128 rows on three lanes, alone, d = 4096,
+    // p = 12288, 465 us chained, 303 not; 64 + 4 rows 205 and 162 us; but p = 3072 on two lanes, eight calls, 272 and 304 us, and p = 768 on
+    // three 117 and 119 us, and a sample of up to 32 rows (19 us) is over soon enough: 32 rows, p = 3072, nine calls on three lanes 123 and 140 us.
+    ctx->lone_launches = small && m > 32 && (m > 128 || 3 * D * project_unmix_ctas(ctx, p) > 2 * ctx->sm_count);
 
     // Back-to-back batches of the same shape on the same stream keep the lanes running across the seam: each
     // lane only waits until the products that read its previous pair are done.  Otherwise the lanes start after

@@ -58,6 +58,7 @@ struct gelo_ctx {
     int lane_tc_share = 4;        // batches with at least this many lanes plan each level-3 update for 1/share of the SMs
     int tc_update_ctas = 0;       // CTAs that a level-3 tensor-core launch is planned for (0: one per SM): with many lanes fewer K slices
                                   // do, because the updates of several lanes run side by side
+    bool lone_launches = false;   // whole calls run on lanes beside each other and must not hold SMs while they wait (chain_launches)
     bool panel_samples = false;   // fp32 samples of the running batch take 32-column panels (panels_hide in api.cu)
     int level3 = 0;               // 0: tf32 tensor-core updates for bf16 calls with m >= 256; 1: always fp32 FMA;
                                   // 2: always tensor cores, three bf16 products of split operands; 3: always tensor cores, tf32
@@ -135,12 +136,12 @@ static inline int after_launch(gelo_ctx* ctx) {
 // lets its successor be set up as soon as all of its own CTAs run (chain_next) and itself touches memory only after
 // chain_wait, which returns when its predecessor has finished and its results are visible.  A kernel that is launched this way always
 // waits, so the order is that of the stream.  For launches into a stream: 4300 rows non-orthogonal 5.55 -> 5.08 ms, 350 rows staged
-// 629 -> 540 us.  Not in recorded graphs, which have that already (no difference), and not with many lanes, where CTAs that only wait
-// would keep SMs from other lanes' work.
+// 629 -> 540 us.  Not in recorded graphs, which have that already (no difference), and not where CTAs that only wait would keep SMs from other
+// lanes' work: with many lanes, and with two or three whose projections do not fit beside each other (offload_batch_impl).
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-static inline bool chain_launches(const gelo_ctx* ctx) { return ctx->tc_update_ctas == 0 && !ctx->prof_on && !ctx->recording; }
+static inline bool chain_launches(const gelo_ctx* ctx) { return ctx->tc_update_ctas == 0 && !ctx->prof_on && !ctx->recording && !ctx->lone_launches; }
 
 template <typename... P, typename... A>
 int launch_chained(gelo_ctx* ctx, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
@@ -278,6 +279,7 @@ struct Tf32x3Scratch {
 // true when launch_project_unmix can serve the call: 16-bit storage, m = n + k <= 128, p a multiple of 64 whose
 // 64-column boxes leave every CTA a slab of at most 128 columns
 bool project_unmix_supports(const gelo_ctx*, int n, int k, int d, int p, int dtype, int lda, int nsplit);
+int project_unmix_ctas(const gelo_ctx*, int p);             // its CTAs, each of which has an SM to itself
 // Q | K | V (or one n x p result in Q when K = V = nullptr) = (Ainv[0:n, 0:n+k] (U W)); U: (n+k) x d, W: d x p
 int launch_project_unmix(gelo_ctx*, const void* U, const void* W, const void* Ainv, int lda, int n, int k, int d, int p,
                          int dtype, void* Q, void* K, void* V, cudaStream_t);

@@ -475,6 +475,14 @@ bool project_unmix_supports(const gelo_ctx* ctx, int n, int k, int d, int p, int
     return (boxes + ncta - 1) / ncta <= kDecMaxBoxes;
 }
 
+// As few CTAs as keep the widest slab no wider than it must be (p = 12288 on 148 SMs: 96 CTAs of two boxes each), which
+// evens the slabs out and leaves the other SMs to kernels of other streams
+int project_unmix_ctas(const gelo_ctx* ctx, int p)
+{
+    const int boxes = p / kDecBoxCols;
+    return ceil_div(boxes, ceil_div(boxes, ctx->sm_count));
+}
+
 // Q | K | V (or one n x p result when K = V = nullptr) = (Ainv[0:n, 0:m] (U W)) for m = n + k <= 128.  With
 // Ainv == nullptr the kernel stops after the first product: the result is U W itself (n + k rows).
 int launch_project_unmix(gelo_ctx* ctx, const void* U, const void* W, const void* Ainv, int lda, int n, int k, int d, int p,
@@ -490,10 +498,7 @@ int launch_project_unmix(gelo_ctx* ctx, const void* U, const void* W, const void
     prm.kpad = (m + 15) & ~15;
     prm.npad = (n + 15) & ~15;
     prm.boxes = p / kDecBoxCols;
-    // as few CTAs as keep the widest slab no wider than it must be (p = 12288 on 148 SMs: 128 CTAs of 3 boxes each), which
-    // evens the slabs out and leaves the other SMs to kernels of other streams
-    const int widest = (prm.boxes + ctx->sm_count - 1) / ctx->sm_count;
-    const int ncta = (prm.boxes + widest - 1) / widest;
+    const int ncta = project_unmix_ctas(ctx, p);
     prm.base = prm.boxes / ncta; prm.rem = prm.boxes % ncta;
     prm.nbmax = prm.base + (prm.rem > 0 ? 1 : 0);
     const uint32_t a_bytes = (uint32_t)prm.kpad * kDecRowBytes;

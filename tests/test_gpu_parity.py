@@ -676,6 +676,27 @@ def test_small_batch_with_shared_outputs_keeps_call_order():
     c.close()
 
 
+# two and three lanes: projections that fit beside each other are set up under their predecessors, others are not (12, 48 and 64 CTAs per
+# projection); the same bytes as call by call
+@pytest.mark.parametrize("lanes,p", [(3, 768), (2, 3072), (3, 3072), (2, 4096)])
+def test_small_batches_on_few_lanes_match_single_calls(lanes, p):
+    n, k, d, dt, calls = 100, 5, 512, "bf16", 7
+    c = binding.Context(0)
+    c.set_lanes(lanes)
+    c.ensure_batch_workspace(n, k, d, p, dt, lanes)
+    H = [inputs.make_hidden(n, d, dt, 40 + i, True, "cuda") for i in range(calls)]
+    W = [inputs.make_weight(d, p, dt, 90 + i, "cuda") for i in range(calls)]
+    kinds = [(ORTHOGONAL, NONORTHOGONAL)[i % 2] for i in range(calls)]
+    Y = torch.zeros((2, calls, n, p), dtype=torch.bfloat16, device="cuda")
+    for _ in range(2):
+        c.qkv_offload_batch(H, W, n, k, d, p, kinds, list(range(calls)), 10.0, dt, list(Y[0]))
+    for i in range(calls):
+        c.qkv_offload(H[i], W[i], n, k, d, p, kinds[i], i, 10.0, dt, Y[1, i])
+    torch.cuda.synchronize()
+    assert c.last_status() == binding.OK and torch.equal(Y[0], Y[1])
+    c.close()
+
+
 # a call that reads the result of the one before it, on the sizes whose calls run on their lanes (fused, and with products of their own)
 # and on one that never does
 @pytest.mark.parametrize("n,k", [(64, 4), (300, 15), (2300, 20)])
