@@ -182,3 +182,14 @@ def test_fp32_batches_choose_the_route_by_what_is_in_flight(n, lanes, kinds, pan
         ref = H[i].double() @ W[i].double()
         assert ((Y[i].double() - ref).norm() / ref.norm()).item() <= 1e-4           # the fp32 path's tolerance
     c.close()
+
+
+# the one-launch samples hold their rows in steps of eight: both sides of a few steps, the first and the last size
+@pytest.mark.parametrize("m", [7, 32, 33, 40, 41, 73, 80, 81, 104, 105, 121, 128])
+def test_one_launch_samples(oracle, m):
+    a, x = _sample(m, ORTHOGONAL, 60 + m, "f32")
+    assert np.array_equal(x, a.T)
+    assert np.linalg.norm(a.T @ a - np.eye(m)) / np.sqrt(m) <= 1e-6           # m reflections, 2^-24 each
+    q_ref, _ = oracle.householder_qr(oracle.gaussian(60 + m, 0, 0, m, m).astype(np.float32).astype(np.float64))
+    h = (m + 1) // 2
+    assert np.linalg.norm(a[:, :h] - q_ref[:, :h]) / np.sqrt(h) <= 2e-5       # columns conditioned below 6 times what R loses
