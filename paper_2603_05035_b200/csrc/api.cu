@@ -140,18 +140,19 @@ Layout carve(Arena& a, int n, int k, int d, int p, int dtype, bool host_staging)
 }
 
 // Lanes other than the first hold only what sampling needs, except where whole calls run on the lanes: small batches
-// (m <= 128, S and U of d columns) and 16-bit calls of up to kLaneCallRows rows (S, U and Y').
+// (m <= 128, S and U of d columns) and, with more than kSampleOnlyLanes lanes, 16-bit calls of up to kLaneCallRows rows (S, U and Y').
 // kLaneCallRows: up to here a product leaves SMs idle in its first and last tiles and the shield rows are three short launches,
 // so one call after the other on the caller's stream is a chain of its own: 32 layers of 315 rows on 16 lanes 3.50 -> 2.62 ms, 2150
 // rows on 32 lanes 22.0 -> 20.2 ms, eight of 1050 rows 1.95 -> 1.78 ms.  Beyond, the products fill the GPU by themselves, and Y' alone is
 // 106 MB per lane at 4300 rows.  With four lanes or less the lanes are the bound and only sample (2150 rows 27.6 ms like that,
 // 28.0 ms with whole calls).
 constexpr int kLaneCallRows = 2304;
-inline bool lane_calls(int m, int dtype) { return dtype != GELO_F32 && m > 128 && m <= kLaneCallRows; }
-inline Layout carve_lane(Arena& a, int n, int k, int d, int p, int dtype)
+constexpr int kSampleOnlyLanes = 4;
+inline bool lane_calls(int m, int dtype, int lanes) { return dtype != GELO_F32 && m > 128 && m <= kLaneCallRows && lanes > kSampleOnlyLanes; }
+inline Layout carve_lane(Arena& a, int n, int k, int d, int p, int dtype, int lanes)
 {
     const int m = n + k;
-    const bool whole = lane_calls(m, dtype);
+    const bool whole = lane_calls(m, dtype, lanes);
     return carve(a, n, k, (whole || m <= 128) ? d : 0, whole ? p : 0, dtype, false);
 }
 
@@ -575,7 +576,7 @@ int offload_batch_impl(gelo_ctx* ctx, int calls, const void* const* H, const voi
     a.cap = ctx->ws_bytes;
     Layout L[kMaxLanes];
     L[0] = carve(a, n, k, d, p, dtype, host);
-    for (int i = 1; i < D; ++i) L[i] = carve_lane(a, n, k, d, p, dtype);
+    for (int i = 1; i < D; ++i) L[i] = carve_lane(a, n, k, d, p, dtype, D);
     if (!a.ok) return GELO_ERR_WORKSPACE;
     const size_t es = elem_size(dtype);
     const bool split = K[0] != nullptr;
@@ -585,7 +586,7 @@ int offload_batch_impl(gelo_ctx* ctx, int calls, const void* const* H, const voi
     // on the lane's own S and U): the weight streams of different calls overlap at their seams and the caller's stream
     // only joins the lanes at the end of the batch.  So do 16-bit calls of a medium size (see kLaneCallRows).
     bool small = !host && D > 1 &&
-                 ((D > 4 && lane_calls(m, dtype)) || (ctx->fuse_small && m <= 128 && mix_small_supports(n, k, d, dtype) &&
+                 (lane_calls(m, dtype, D) || (ctx->fuse_small && m <= 128 && mix_small_supports(n, k, d, dtype) &&
                                            project_unmix_supports(ctx, n, k, d, p, dtype, L[0].ldi, split ? 3 : 1)));
     for (int i = 0; i < calls && small; ++i) small = !misaligned(H[i]);
     if (small && calls > 1) small = !calls_depend(calls, H, (size_t)n * d * es, W, (size_t)d * p * es, Q, K, V, split ? third : (size_t)n * p * es);
@@ -858,7 +859,7 @@ size_t batch_workspace(int n, int k, int d, int p, int dtype, int lanes)
     Arena a;
     a.cap = ~size_t(0) >> 1;
     carve(a, n, k, d, p, dtype, true);
-    for (int i = 1; i < lanes; ++i) carve_lane(a, n, k, d, p, dtype);
+    for (int i = 1; i < lanes; ++i) carve_lane(a, n, k, d, p, dtype, lanes);
     return a.off + 256;
 }
 

@@ -63,3 +63,18 @@ def test_block_diagonal_grouping_is_checked_on_the_host(lib):
     assert ws(4, 0, 64, 192, 0, 64, 8) > 0 and ws(0, 0, 64, 192, 0, 64, 8) == 0
     assert ws(4096, 204, 4096, 12288, 7, 512, 32) == 0                  # unknown element type
     assert ws(4096, 204, 4096, 12288, 2, 512, 32) == base               # half and bfloat16 have the same footprint
+
+
+def test_lanes_that_only_sample_hold_no_call_buffers(lib):
+    """Up to four lanes sample only, whatever p is; with more, 16-bit calls of up to 2304 rows run on their lanes and each has a U and a Y'."""
+    from paper_2603_05035_b200 import binding
+    L = binding.load_library()
+    per_lane = lambda n, p, dtype, lanes: L.gelo_batch_workspace_bytes(n, 0, 4096, p, dtype, lanes) - L.gelo_batch_workspace_bytes(n, 0, 4096, p, dtype, lanes - 1)
+    BF16, F32 = 1, 0
+    assert per_lane(2304, 12288, BF16, 4) == per_lane(2304, 8, BF16, 4)
+    assert per_lane(2304, 12288, BF16, 6) >= per_lane(2304, 12288, BF16, 4) + 2 * 2304 * (4096 + 12288)
+    for n, dtype in ((2305, BF16), (1000, F32)):
+        assert per_lane(n, 12288, dtype, 6) == per_lane(n, 8, dtype, 6)
+    # the need grows with every lane
+    need = [L.gelo_batch_workspace_bytes(1050, 0, 4096, 12288, BF16, lanes) for lanes in range(1, 33)]
+    assert all(a < b for a, b in zip(need, need[1:]))
