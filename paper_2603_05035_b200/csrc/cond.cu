@@ -14,6 +14,8 @@
 // slab sums spread over sixteen threads per column, the eigenvalues searched by 32 lanes at a time.  Against 32-row
 // slabs with scalar loads of x, a thread per column in the sums, a launch of its own for the recurrence and bisection by
 // a single thread: 630 -> 250 us per estimate at 4300 rows (the pass over both operators 63 -> 23 us).
+#include <cfloat>
+
 #include "common.cuh"
 #include "philox.cuh"
 
@@ -154,7 +156,9 @@ __device__ double tridiagonal_lambda_max(const float* alpha, const float* beta)
         a[i] = alpha[i];
         const double bl = i > 0 ? fabs((double)beta[i - 1]) : 0.0, br = i + 1 < k ? fabs((double)beta[i]) : 0.0;
         b2[i] = bl * bl;
-        hi = fmax(hi, fabs(a[i]) + bl + br);
+        const double reach = fabs(a[i]) + bl + br;
+        if (!(reach <= DBL_MAX)) return reach;               // matrices with NaN or infinite entries have no bound: fmax would drop a NaN
+        hi = fmax(hi, reach);
     }
     const int lane = threadIdx.x & 31;
     double lo = 0.0;

@@ -136,6 +136,20 @@ def test_cond_estimate(ctx, oracle, m, gamma):
     assert 0.88 * ref <= est <= 1.001 * ref               # a Ritz value of a few Lanczos steps: a lower estimate within ~10%
 
 
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_cond_estimate_of_broken_matrices_is_no_number(ctx, bad):
+    """The verdict is `estimate * 1.2 <= bound`: an entry that is not finite must not come out as a small estimate."""
+    m, ld = 200, 256
+    A = torch.zeros((m, ld), device="cuda"); A[:, :m] = torch.eye(m, device="cuda")
+    B = A.clone(); B[100, 50] = bad
+    c = torch.zeros(1, device="cuda")
+    for pair in ((A, B), (B, A), (B, B)):
+        ctx.cond_estimate(m, *pair, ld, c)
+        assert not c.item() <= 1e30
+    ctx.cond_estimate(m, A, A, ld, c)
+    assert abs(c.item() - 1) <= 1e-4
+
+
 # ------------------------------------------------------------------------- sample_mixing
 
 def _sample(ctx, m, kind, seed, dt):
