@@ -280,7 +280,8 @@ int gelo_qkv_offload_host(gelo_ctx* ctx, const void* H_host, const void* W_dev, 
  * never uses one twice).  Sampling A needs only the seed, so up to `lanes` calls sample
  * their mixing pairs concurrently on streams owned by the context while `stream` runs the
  * shield rows and the three products of earlier calls; results are those of gelo_qkv_offload
- * with the same (kind, seed) per call.
+ * with the same (kind, seed) per call, up to the order of the sampler's sums (from some 300 rows on, lanes cut
+ * them into other slices, and fp32 samples may be factorised in panels: see gelo_set_lane_share).
  *   H_dev[i] n x d, W_dev[i] d x p, kinds[i], seeds[i]: inputs of call i (host arrays of
  *   device pointers / values, read before the function returns).
  *   Q_dev[i], K_dev[i], V_dev[i]: outputs of call i, as in gelo_unmix (K_dev[i] == V_dev[i] ==
@@ -324,7 +325,8 @@ int gelo_qkv_offload_batch_host_async(gelo_ctx* ctx, int calls, const void* cons
  * they need.  0 bytes if an argument is invalid. */
 int gelo_set_lanes(gelo_ctx* ctx, int lanes);
 /* In batches with at least `share` lanes every tensor-core update of the factorisations is cut into work for 1/share of
- * the SMs (default 4; 1 = always all SMs): the updates of different lanes fill the rest. */
+ * the SMs (default 4; 1 = always all SMs): the updates of different lanes fill the rest.  fp32 samples are drawn
+ * in blocks or, with enough of them in flight to hide the longer chains, in 32-column panels that occupy 8 SMs each. */
 int gelo_set_lane_share(gelo_ctx* ctx, int share);
 size_t gelo_batch_workspace_bytes(int n, int k, int d, int p, int dtype, int lanes);
 

@@ -66,8 +66,45 @@ def test_inverse_of_the_nonorthogonal_sample(m, gamma, dt):
     assert np.linalg.norm(x - ref) / np.linalg.norm(ref) <= bound
 
 
-# the fp32 route: 129: its first size, one block of 64; 250: an odd split; 700: two groups of blocks; half at 200 rows takes it too
-@pytest.mark.parametrize("m,dt", [(129, "f32"), (250, "f32"), (700, "f32"), (200, "f16")])
+# bfloat16 at the last size with all corrections and the first two with one product less, against A^-1 in 64 bits.  Rounding alone is 1.66e-3 (2^-9 / sqrt(3)
+# over a binade); the shorter iteration leaves gamma^10 = 9.8e-4 beside it, 1.93e-3 together, which is what the pivoted LU came to
+# at 4096 rows (1.94e-3; 1.95e-3 at 4300, 2.17e-3 at 6000)
+@pytest.mark.parametrize("m,bound", [(4095, 1.75e-3), (4096, 2.0e-3), (4300, 2.0e-3)])
+def test_inverse_of_large_samples(m, bound):
+    c = binding.Context(0)
+    c.ensure_workspace(m, 0, 8, 24, "bf16")
+    ld = c.mixing_ld(m)
+    A = padded(m, ld, torch.bfloat16); X = padded(m, ld, torch.bfloat16)
+    c.sample_mixing(m, NONORTHOGONAL, 70 + m, "bf16", A, X, ld)
+    assert c.last_status() == binding.OK
+    c.close()
+    ref = torch.linalg.inv(A[:, :m].double())
+    assert ((X[:, :m].double() - ref).norm() / ref.norm()).item() <= bound
+
+
+# fp32 above the sizes of the iteration: the block QR, its polish and the LU of what follows, up to the last size of the route and one past it
+@pytest.mark.parametrize("m", [769, 1075, 3072, 3073])
+def test_large_fp32_samples(m):
+    c = binding.Context(0)
+    c.ensure_workspace(m, 0, 8, 24, "f32")
+    ld = c.mixing_ld(m)
+    A = padded(m, ld, torch.float32); X = padded(m, ld, torch.float32)
+    eye = torch.eye(m, device="cuda", dtype=torch.float64)
+    c.sample_mixing(m, ORTHOGONAL, 300 + m, "f32", A, X, ld)
+    a = A[:, :m].double()
+    assert torch.equal(X[:, :m], A[:, :m].T)
+    # sums of m products: sqrt(m) 2^-24 = 3.3e-6 at 3072 rows (1.4e-6 measured with the panels)
+    assert ((a.T @ a - eye).norm() / m ** 0.5).item() <= m ** 0.5 * 2.0 ** -24
+    c.sample_mixing(m, NONORTHOGONAL, 300 + m, "f32", A, X, ld)
+    # the eliminations of m columns amplify 2^-24 by a growth that goes with m: 2.3e-5 at 900 rows, 6.6e-5 at 2000
+    assert ((X[:, :m].double() @ A[:, :m].double() - eye).norm() / m ** 0.5).item() <= m * 2.0 ** -24
+    assert c.last_status() == binding.OK
+    c.close()
+
+
+# the fp32 route: 129: its first size, one block of 64; 250: an odd split; 700: two groups of blocks; 768: the last size of the iteration; half at
+# 200 rows takes it too
+@pytest.mark.parametrize("m,dt", [(129, "f32"), (250, "f32"), (700, "f32"), (768, "f32"), (200, "f16")])
 def test_exact_block_route(oracle, m, dt):
     a, x = _sample(m, ORTHOGONAL, 300 + m, dt)
     assert np.array_equal(x, a.T)
