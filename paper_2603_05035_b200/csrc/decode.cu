@@ -287,8 +287,8 @@ project_unmix_kernel(const __grid_constant__ CUtensorMap map_u, const __grid_con
 
     tc_fence_before();
     __syncthreads();
-    settle(abort_flag, prm.wait_ns);
     if (warp == 1) {
+        if (*abort_flag) settle(prm.wait_ns);                 // (the CTA's memory is its own until its last warp returns)
         __syncwarp();
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kDecTmemCols) : "memory");

@@ -593,8 +593,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     tc_fence_before();
     __syncwarp();
     if (kPair) cluster_sync(); else __syncthreads();
-    settle(abort_flag, prm.wait_ns);
     if (warp == 1) {
+        if (*abort_flag) settle(prm.wait_ns);                 // (the CTA's memory is its own until its last warp returns)
         __syncwarp();
         tc_fence_after();
         if (kPair) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");

@@ -62,9 +62,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 // What a CTA does before it returns once a wait has run out and nobody issues any more: copies, matrix instructions and arrivals
 // that are still on their way into its shared or tensor memory get a millisecond, hundreds of times what one of them
 // takes, to get there.  (Nothing is on its way with a limit of zero.)
-__device__ __forceinline__ void settle(const volatile int* abort_flag, unsigned long long limit_ns)
+static __device__ __noinline__ void settle(unsigned long long limit_ns)
 {
-    if (*abort_flag == 0 || limit_ns == 0) return;
+    if (limit_ns == 0) return;
     const unsigned long long t0 = global_ns();
     while (global_ns() - t0 < 1000000ull) {
     }
