@@ -424,25 +424,24 @@ def run_ours(args):
         proj_tflops = 2.0 * m * d * p / (stage_ms["project"] * 1e-3) / 1e12
         projection = {"kernel": "gemm_tc_kernel, Y' = U W", "bound": "tensor", "achieved": proj_tflops,
                       "peak": peaks["bf16_tflops"], "unit": "TFLOP/s", "frac": proj_tflops / peaks["bf16_tflops"],
-                      # ncu: dram read 162.6 MB + write 85.5 MB per launch (algorithmic 241.6 MB)
-                      "traffic": 248.0e6}
+                      # ncu: dram read 155.9 MB + write 87.7 MB per launch (algorithmic 241.6 MB)
+                      "traffic": 243.6e6}
         f8_tflops = 2.0 * m * d * p / (stage_ms["project_e4m3"] * 1e-3) / 1e12
         projection_e4m3 = {"kernel": "gemm_tc_kernel (kind::f8f6f4), Y' = (s_U s_W) U8 W8", "bound": "tensor", "achieved": f8_tflops,
                            "peak": 2.0 * peaks["bf16_tflops"], "unit": "TFLOP/s", "frac": f8_tflops / (2.0 * peaks["bf16_tflops"]),
                            "peak_source": peaks["source"] + " bf16 GEMM x nominal fp8/bf16 ratio 2",
-                           # ncu: dram read 69.9 MB + write 61.2 MB (algorithmic 173.6 MB; operands quantised just before were partly in L2)
-                           "traffic": 131.1e6,
-                           "note": "same product as roofline_projection_gemm on E4M3 operands; FP8-grade accuracy (see DESIGN)"}
+                           # ncu: dram read 68.2 MB + write 68.0 MB (algorithmic 173.6 MB; the end of the result was still in L2)
+                           "traffic": 136.2e6,
+                           "note": "same product as roofline_projection_gemm on E4M3 operands; FP8-grade accuracy (about 12% after unmixing)"}
         upd_tflops = 2.0 * um * un * uk / (stage_ms["tf32_update"] * 1e-3) / 1e12
         tf32_peak = 0.5 * peaks["bf16_tflops"]          # nominal dense tf32 : bf16 = 1.125 : 2.25
         update_roof = {"kernel": "gemm_tc_kernel (tf32, reduce-add epilogue), C -= V W, M=4300 N=3788 K=512",
                        "bound": "tensor", "achieved": upd_tflops, "peak": tf32_peak, "unit": "TFLOP/s",
                        "frac": upd_tflops / tf32_peak,
                        "peak_source": peaks["source"] + " bf16 GEMM x nominal tf32/bf16 ratio 0.5",
-                       # ncu: dram read 82.1 MB + write 9.0 MB per launch (algorithmic 147 MB, half of C stays in L2)
-                       "traffic": 91.1e6,
-                       "note": "the subtracting update reads and writes C at the L2 (8 bytes per entry for 1024 flop); "
-                               "710 TFLOP/s at large K"}
+                       # ncu: dram read 81.9 MB + write 12.6 MB per launch (algorithmic 147 MB, half of C stays in L2)
+                       "traffic": 94.5e6,
+                       "note": "the subtracting update reads and writes C at the L2 (8 bytes per entry for 1024 flop)"}
         per_call_ms = ms_max / args.steps / calls
         chain_tflops = chain_flops / (chain_ms * 1e-3) / 1e12
         # all arithmetic of a sweep against the time the sweep takes with every lane busy: the Householder QR of every

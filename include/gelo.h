@@ -87,12 +87,15 @@ int gelo_set_workspace(gelo_ctx* ctx, void* dev_ws, size_t bytes);
  * each with the next attempt number in the Philox counter). */
 int gelo_set_nonorthogonal(gelo_ctx* ctx, float gamma, float cond_bound, int max_attempts);
 
-/* How the level-3 updates of the blocked QR / LU are computed.
- *   0 (default): fp32 FMA kernels for fp32 calls and for m < 256; for bf16 calls with m >= 256 the QR runs single
- *      tf32 tensor-core products straight from the fp32 matrices (followed, for an orthogonal A, by one
- *      Newton-Schulz step that squares the orthogonality defect tf32 leaves) and the LU runs three bf16 products of
- *      operands held as (high, low) pairs;
- *   1: always fp32 FMA;  2: always the split-precision products;  3: always tf32.
+/* How A and its inverse are computed.
+ *   0 (default): 16-bit calls with m >= 256 factorise the Gaussian in 128-column blocks from their Gram matrices, on
+ *      single tf32 tensor-core products straight from the fp32 matrices (followed, for an orthogonal A, by one
+ *      Newton-Schulz step that squares the orthogonality defect tf32 leaves), and invert a non-orthogonal A with
+ *      gamma <= 0.55 by Newton's iteration on 16-bit products; fp32 calls of up to 3072 rows and 16-bit ones of 129 to 255
+ *      take the same blocks in fp32 FMA (and up to 768 rows the iteration).  What is left, and gelo_qr_orthogonal and
+ *      gelo_lu_inverse, take 32-column panels and the pivoted LU, in fp32 FMA or, in 16-bit calls with m >= 256, on bf16
+ *      products of operands held as (high, low) pairs;
+ *   1: panels and LU, always fp32 FMA;  2: panels and LU, always the split-precision products;  3: always tf32.
  * The split-precision products are good to about 1e-5 relative and tf32 to about 1e-3, neither of which the fp32
  * path's 1e-4 budget leaves room for, hence the default. */
 int gelo_set_level3(gelo_ctx* ctx, int mode);
@@ -165,8 +168,8 @@ int gelo_update_f32(gelo_ctx* ctx, int M, int N, int K, const float* A_dev, int 
  *   GELO_NONORTHOGONAL: A = Q0 + gamma * G1 / sqrt(m) (G1 from stream 1), rounded to the
  *                       element type, then A^-1 of that stored A; accepted when the
  *                       kappa_2 estimate * 1.2 <= bound, else resampled with the next
- *                       attempt number.  The bound is enforced on an ESTIMATE (power
- *                       iteration, a lower estimate that tests put at 0.85 .. 1.0 of the
+ *                       attempt number.  The bound is enforced on an ESTIMATE (Lanczos
+ *                       steps, a lower estimate that tests put at 0.85 .. 1.0 of the
  *                       true value, hence the factor 1 / 0.85 rounded up).  This kind WAITS for `stream` once per attempt
  *                       to read the verdict; GELO_ERR_COND after the last attempt.
  * A_dev, Ainv_dev: m x m in `dtype`, stride lda.  cond_dev (optional, device float)

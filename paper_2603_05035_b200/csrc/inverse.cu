@@ -11,9 +11,9 @@
 //     R = I - A X,   A^-1 = X + X R                   (two products, ends at gamma^10),
 //     R = I - A X,   Z = R^2 + R,   A^-1 = X + X Z    (three, gamma^15),
 // with R or Z kept small instead of added to the identity before it is rounded, and A^-1 rounded once.  The second leaves
-// 3e-5 at gamma = 1/2, nothing beside the rounding of A^-1 (bfloat16 1.66e-3, half 2.1e-4).  The first leaves 2^-10, a total of 1.93e-3 in
-// bfloat16; it serves bfloat16 from 4096 rows up, where that is what the pivoted LU had (1.96e-3 at 4300 rows, growing
-// with m) and a product costs 0.11 ms.
+// 3e-5 at gamma = 1/2, nothing beside the rounding of A^-1 (bfloat16 1.66e-3, half 2.1e-4).  The first leaves 2^-10, with the rounding 1.93e-3 in
+// bfloat16 at every m.  It serves bfloat16 from 4096 rows up, where a product costs 0.11 ms: that is where the pivoted LU's error, which
+// grows with m, reached the same (1.83e-3 at 3000 rows, 1.94e-3 at 4096, 1.95e-3 at 4300, 2.17e-3 at 6000), so that no size lost precision.
 //
 // Six or seven products at the 16-bit rate of the tensor cores replace the pivoted LU and its two triangular solves, which were
 // bound by some 1000 dependent launches: 4300 rows, one call alone 30.4 -> 8.6 ms (with eight products, four Newton steps from
