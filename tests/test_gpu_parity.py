@@ -734,6 +734,24 @@ def test_batched_calls_that_read_earlier_results_run_in_call_order(n, k):
     c.close()
 
 
+def test_batched_calls_in_place_stay_independent():
+    """A result that replaces the call's own H concerns no other call: the same bytes as with buffers of their own."""
+    for n, k in ((64, 4), (300, 15)):
+        d, dt, calls = 256, "bf16", 7
+        c = binding.Context(0)
+        c.set_lanes(6)
+        c.ensure_batch_workspace(n, k, d, d, dt, 6)
+        H = torch.stack([inputs.make_hidden(n, d, dt, 40 + i, True, "cuda") for i in range(calls)])
+        W = [inputs.make_weight(d, d, dt, 90 + i, "cuda") for i in range(calls)]
+        kinds = [(ORTHOGONAL, NONORTHOGONAL)[i % 2] for i in range(calls)]
+        Y = torch.zeros_like(H)
+        for out in (Y, H):
+            c.qkv_offload_batch(list(H), W, n, k, d, d, kinds, [500 + i for i in range(calls)], 10.0, dt, list(out))
+        torch.cuda.synchronize()
+        assert c.last_status() == binding.OK and torch.equal(H, Y) and Y.abs().sum() > 0
+        c.close()
+
+
 
 def test_batched_offload_full_size(oracle):
     w = inputs.WORKLOADS["prefill_bf16"]
