@@ -35,7 +35,7 @@
  *   - Scratch memory comes from the caller through gelo_set_workspace; no entry point
  *     except gelo_create / gelo_destroy allocates or frees device memory of its own.  The driver
  *     keeps what it needs for recorded launch graphs (the whole-call entry points replay their
- *     sampling; 0.3 to 4 MB each, 128 per context at most, from the second call of a size on).
+ *     sampling; 0.3 to 4 MB each, 512 per context at most, from the second call of a size on).
  */
 #ifndef GELO_H
 #define GELO_H

@@ -21,8 +21,9 @@ constexpr int kPanel = 32;
 // [1]: verdict of the last condition-number check (1 = accepted).  [2]: detail word.
 constexpr int kStatusWords = 8;
 constexpr int kMaxLanes = 32;
-// Recorded sampling graphs of a context: two kinds on every lane, for two shapes.  One takes 0.3 to 4 MB of the driver's memory.
-constexpr int kMaxGraphs = 4 * kMaxLanes;
+// Recorded sampling graphs of a context: two kinds on every lane, for eight shapes that a program may go round.  One takes 0.3 to 4 MB of
+// the driver's memory, and recording it 0.3 to 1.7 ms, five times its replay on the host.
+constexpr int kMaxGraphs = 16 * kMaxLanes;
 constexpr int kMetKeys = 16;
 
 // Kernel classes that the optional per-launch timing distinguishes.
