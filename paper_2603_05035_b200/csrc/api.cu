@@ -210,7 +210,9 @@ int sample_attempt(gelo_ctx* ctx, const Layout& L, int m, int kind, uint64_t see
     const bool exact = ctx->level3 == 0 && l3 == 0 && m <= kExactBlockRows && !(ctx->panel_samples && dtype == GELO_F32);
     const bool blocks = (l3 == 3 || exact) && gaussian_qr_supports(m);
     const float* sign = blocks ? nullptr : L.G;
-    if (blocks) GELO_TRY(run_gaussian_qr(ctx, m, L.G, ldi, L.Qraw, L.tc, exact, st));
+    const bool newton = ctx->level3 == 0 && newton_inverse_supports(m, dtype, ctx->gamma);
+    bool turned = false;                                     // Qraw holds Q^T
+    if (blocks) GELO_TRY(run_gaussian_qr(ctx, m, L.G, ldi, L.Qraw, L.tc, exact, st, kind == GELO_ORTHOGONAL || newton ? &turned : nullptr));
     else if (l3 == 3) GELO_TRY(run_householder_qr_tf32(ctx, m, L.G, ldi, L.Qraw, L.qr, L.tc, st));
     else if (l3) GELO_TRY(run_householder_qr_tc(ctx, m, L.G, ldi, L.Qraw, L.qr, L.tc, st));
     else GELO_TRY(run_householder_qr(ctx, m, L.G, ldi, L.Qraw, L.qr, st));
@@ -230,6 +232,7 @@ int sample_attempt(gelo_ctx* ctx, const Layout& L, int m, int kind, uint64_t see
             GELO_TRY(launch_gemm_simt(ctx, g, st));
             Q = L.A32;
         }
+        if (turned) std::swap(A_out, Ainv_out);              // (one is the other's transpose, and the polish of Q^T that of Q)
         GELO_TRY(launch_finish_mixing(ctx, m, Q, ldi, sign, ldi, dtype, A_out, Ainv_out, lda, st));
         if (cond_dev) {
             set_scalar_kernel<<<1, 1, 0, st>>>(cond_dev, 1.0f);
@@ -241,12 +244,17 @@ int sample_attempt(gelo_ctx* ctx, const Layout& L, int m, int kind, uint64_t see
     if (sign) GELO_TRY(launch_finish_mixing(ctx, m, L.Qraw, ldi, sign, ldi, GELO_F32, L.A32, nullptr, ldi, st));
     const float* Q0 = sign ? L.A32 : L.Qraw;
     const float s = ctx->gamma / sqrtf((float)m);
-    if (ctx->level3 == 0 && newton_inverse_supports(m, dtype, ctx->gamma)) {
+    if (newton) {
         // X0 = Q0^T in the stored type; the fp32 matrices that are dead by now hold two 16-bit ones each
         const size_t half = (size_t)m * ldi;
         uint16_t* g16 = reinterpret_cast<uint16_t*>(L.G);
         uint16_t* x16 = reinterpret_cast<uint16_t*>(L.X32);
-        GELO_TRY(launch_finish_mixing(ctx, m, Q0, ldi, nullptr, ldi, dtype, nullptr, g16, ldi, st));
+        if (turned) {
+            GELO_TRY(launch_turn_back(ctx, m, L.Qraw, ldi, dtype, g16, L.A32, st));
+            Q0 = L.A32;
+        } else {
+            GELO_TRY(launch_finish_mixing(ctx, m, Q0, ldi, nullptr, ldi, dtype, nullptr, g16, ldi, st));
+        }
         GELO_TRY(launch_gaussian_to(ctx, dtype, m, m, seed, GELO_STREAM_G1, attempt, s, Q0, ldi, A_out, lda, st, seed_dev));
         GELO_TRY(run_newton_inverse(ctx, m, dtype, ctx->gamma, A_out, lda, g16, g16 + half, x16, x16 + half, ldi, Ainv_out, lda, st));
     } else if (blocks && exact && m <= kExactNewtonRows && ctx->gamma <= 0.55f) {
@@ -898,7 +906,10 @@ int gelo_create(gelo_ctx** out, int device)
     lanes_ok = lanes_ok && cudaMalloc(&ctx->lane_seed_dev, kMaxLanes * 8 * sizeof(uint64_t)) == cudaSuccess;
     lanes_ok = lanes_ok && cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking) == cudaSuccess &&
                cudaEventCreateWithFlags(&ctx->side_from, cudaEventDisableTiming) == cudaSuccess &&
-               cudaEventCreateWithFlags(&ctx->side_done, cudaEventDisableTiming) == cudaSuccess;
+               cudaEventCreateWithFlags(&ctx->side_done, cudaEventDisableTiming) == cudaSuccess &&
+               cudaStreamCreateWithFlags(&ctx->form, cudaStreamNonBlocking) == cudaSuccess &&
+               cudaEventCreateWithFlags(&ctx->form_from, cudaEventDisableTiming) == cudaSuccess &&
+               cudaEventCreateWithFlags(&ctx->form_done, cudaEventDisableTiming) == cudaSuccess;
     lanes_ok = lanes_ok && cudaStreamCreateWithFlags(&ctx->copy_in, cudaStreamNonBlocking) == cudaSuccess &&
                cudaStreamCreateWithFlags(&ctx->copy_out, cudaStreamNonBlocking) == cudaSuccess;
     for (int b = 0; b < 2 && lanes_ok; ++b)
@@ -929,6 +940,9 @@ int gelo_destroy(gelo_ctx* ctx)
     if (ctx->side) cudaStreamDestroy(ctx->side);
     if (ctx->side_from) cudaEventDestroy(ctx->side_from);
     if (ctx->side_done) cudaEventDestroy(ctx->side_done);
+    if (ctx->form) { cudaStreamSynchronize(ctx->form); cudaStreamDestroy(ctx->form); }
+    if (ctx->form_from) cudaEventDestroy(ctx->form_from);
+    if (ctx->form_done) cudaEventDestroy(ctx->form_done);
     if (ctx->copy_in) { cudaStreamSynchronize(ctx->copy_in); cudaStreamDestroy(ctx->copy_in); }
     if (ctx->copy_out) { cudaStreamSynchronize(ctx->copy_out); cudaStreamDestroy(ctx->copy_out); }
     for (int b = 0; b < 2; ++b) {

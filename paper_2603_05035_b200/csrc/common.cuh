@@ -59,6 +59,7 @@ struct gelo_ctx {
     int lane_tc_share = 4;        // batches with at least this many lanes plan each level-3 update for 1/share of the SMs
     int tc_update_ctas = 0;       // CTAs that a level-3 tensor-core launch is planned for (0: one per SM): with many lanes fewer K slices
                                   // do, because the updates of several lanes run side by side
+    bool tc_cap = false;          // ... and does not get more than that many either
     bool lone_launches = false;   // whole calls run on lanes beside each other and must not hold SMs while they wait (chain_launches)
     bool panel_samples = false;   // fp32 samples of the running batch take 32-column panels (panels_hide in api.cu)
     int level3 = 0;               // 0: tf32 tensor-core updates for bf16 calls with m >= 256; 1: always fp32 FMA;
@@ -78,6 +79,8 @@ struct gelo_ctx {
     cudaEvent_t batch_start = nullptr;
     cudaStream_t side = nullptr;                    // branches of recorded sampling graphs
     cudaEvent_t side_from = nullptr, side_done = nullptr;
+    cudaStream_t form = nullptr;                    // where a QR that runs alone forms Q while it factorises
+    cudaEvent_t form_from = nullptr, form_done = nullptr;
     // a batched call may chain onto the previous one (lanes wait for their own lane_free events only) when
     // nothing else has touched the workspace in between
     bool chain_valid = false;
@@ -332,9 +335,9 @@ int run_householder_qr_tc(gelo_ctx*, int m, float* R, int ld, float* Q, const Qr
 int run_householder_qr_tf32(gelo_ctx*, int m, float* R, int ld, float* Q, const QrScratch&, const TcScratch&, cudaStream_t);
 // The orthogonal factor of a GAUSSIAN matrix, blocks factorised through their Gram matrices (qr_block.cu; relies on the
 // blocks being well conditioned), on tf32 products or (exact) on fp32 multiply-adds.  G is overwritten with the reflectors; Q
-// receives the factor whose R has a positive diagonal.
+// receives the factor whose R has a positive diagonal, or its transpose (*transposed; only where the caller gives the pointer).
 bool gaussian_qr_supports(int m);
-int run_gaussian_qr(gelo_ctx*, int m, float* G, int ld, float* Q, const TcScratch&, bool exact, cudaStream_t);
+int run_gaussian_qr(gelo_ctx*, int m, float* G, int ld, float* Q, const TcScratch&, bool exact, cudaStream_t, bool* transposed);
 // One Newton-Schulz step Q <- Q - Q (Q^T Q - I) / 2 on the tensor cores in tf32: squares the orthogonality defect
 // that tf32 updates leave in Q.  D and Qold are m x ld scratch matrices.
 int polish_orthogonal_tf32(gelo_ctx*, int m, float* Q, int ld, float* D, float* Qold, cudaStream_t);
@@ -377,6 +380,8 @@ int run_cond_estimate(gelo_ctx*, int m, const void* A, const void* Ainv, int ld,
 // sign_diag (optional, fp32 matrix with stride lds): column j is multiplied by sign(sign_diag[j*lds + j]).
 int launch_finish_mixing(gelo_ctx*, int m, const float* src, int lds_src, const float* sign_diag,
                          int lds_diag, int dtype, void* dst, void* dstT, int ldd, cudaStream_t);
+// rounded (16-bit dtype) = Qt, Q = Qt^T; m x m, all of stride ld (a multiple of 64)
+int launch_turn_back(gelo_ctx*, int m, const float* Qt, int ld, int dtype, void* rounded, float* Q, cudaStream_t);
 // dst (dtype) = round(src fp32), m x m; back (optional, fp32, stride ldb, may alias src) = the stored values widened again
 int launch_narrow(gelo_ctx*, int m, const float* src, int lds, int dtype, void* dst, int ldd, cudaStream_t,
                   float* back = nullptr, int ldb = 0);

@@ -105,6 +105,40 @@ __global__ void __launch_bounds__(256) finish_mixing16_kernel(int m, const float
     }
 }
 
+// From Q^T in fp32: the same rounded to a 16-bit type, and Q in fp32.  All three of stride ld; 64 x 64 tiles as above.
+// Bound by memory (185 MB at 4300 rows, 30 us).
+template <typename T>
+__global__ void __launch_bounds__(256) turn_back_kernel(int m, const float* __restrict__ Qt, int ld, T* __restrict__ rounded, float* __restrict__ Q)
+{
+    chain_next();
+    chain_wait();
+    __shared__ float tile[64][65];
+    const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
+    const int x = 4 * (threadIdx.x & 15), y = threadIdx.x >> 4;
+    float4 v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {                             // (ld is a multiple of 64: a tile's columns lie within the stride)
+        const int r = r0 + 16 * i + y;
+        v[i] = r < m ? *reinterpret_cast<const float4*>(Qt + (size_t)r * ld + c0 + x) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int rl = 16 * i + y;
+        __align__(8) T t[4];
+        put(t, v[i].x); put(t + 1, v[i].y); put(t + 2, v[i].z); put(t + 3, v[i].w);
+        if (r0 + rl < m) *reinterpret_cast<uint2*>(rounded + (size_t)(r0 + rl) * ld + c0 + x) = *reinterpret_cast<const uint2*>(t);
+        tile[rl][x] = v[i].x; tile[rl][x + 1] = v[i].y; tile[rl][x + 2] = v[i].z; tile[rl][x + 3] = v[i].w;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int r = c0 + 16 * i + y;
+        if (r < m)
+            *reinterpret_cast<float4*>(Q + (size_t)r * ld + r0 + x) =
+                make_float4(tile[x][16 * i + y], tile[x + 1][16 * i + y], tile[x + 2][16 * i + y], tile[x + 3][16 * i + y]);
+    }
+}
+
 // dst = convert(src) for an m x m matrix, four consecutive columns per thread (rows start 16-byte aligned for the
 // wider of the two types, which every row stride of this library guarantees); `back`, if given, receives the stored
 // values widened again (what a later fp32 computation on the stored matrix must start from).
@@ -470,6 +504,18 @@ int launch_finish_mixing(gelo_ctx* ctx, int m, const float* src, int lds, const 
     else
         GELO_TRY(launch_chained(ctx, finish_mixing_kernel<float>, grid, 256, 0, st, m, src, lds, sign_diag, ldg,
                                static_cast<float*>(dst), static_cast<float*>(dstT), ldd));
+    return after_launch(ctx);
+}
+
+int launch_turn_back(gelo_ctx* ctx, int m, const float* Qt, int ld, int dtype, void* rounded, float* Q, cudaStream_t st)
+{
+    if (ld % 64) return GELO_ERR_INVALID;
+    const dim3 tiles(ceil_div(m, 64), ceil_div(m, 64));
+    if (dtype == GELO_BF16)
+        GELO_TRY(launch_chained(ctx, turn_back_kernel<__nv_bfloat16>, tiles, 256, 0, st, m, Qt, ld, static_cast<__nv_bfloat16*>(rounded), Q));
+    else if (dtype == GELO_F16)
+        GELO_TRY(launch_chained(ctx, turn_back_kernel<__half>, tiles, 256, 0, st, m, Qt, ld, static_cast<__half*>(rounded), Q));
+    else return GELO_ERR_UNSUPPORTED;
     return after_launch(ctx);
 }
 

@@ -654,11 +654,30 @@ start_q_kernel(float* __restrict__ Q, int ld, int m, int bf, const float* __rest
     *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
 }
 
+// For the last f rows of -Q^T: a copy of the f x m block (stride ld), and Qf (f x f) with the columns flipped where its R (diagonal of Rf) is
+// positive, so that Qf^T times the copy is what these rows have to be.
+__global__ void __launch_bounds__(256)
+last_rows_kernel(const float* __restrict__ rows, float* __restrict__ copy, int f, int m, float* __restrict__ Qf, const float* __restrict__ Rf, int ld)
+{
+    chain_next();
+    chain_wait();
+    const int r = blockIdx.y, c = blockIdx.x * 256 + threadIdx.x;
+    if (c < m) copy[(size_t)r * ld + c] = rows[(size_t)r * ld + c];
+    if (c < f && !(Rf[(size_t)c * ld + c] < 0.0f)) Qf[(size_t)r * ld + c] = -Qf[(size_t)r * ld + c];
+}
+
 }  // namespace
+
+// Rows from which a QR that has the GPU to itself forms Q^T while it factorises (see run_gaussian_qr), and the SMs that it does that on.
+// From three superblocks on there is something to form beside the next one, and one spare matrix has room for the products' scratch: one call
+// alone at 1600 rows 1173 -> 1125 us, 2150 rows 1578 -> 1460, 4300 rows orthogonal 3837 -> 3512, non-orthogonal 4485 -> 4026 us.
+// On all SMs the chain's launches would wait for tiles of 20 to 30 us (4304 us); on 48, 64, 96 and 128 of them 4089, 4099, 4112 and 4148 us.
+constexpr int kFormRows = 3 * kSuper;
+constexpr int kFormSms = 80;
 
 bool gaussian_qr_supports(int m) { return m > FB; }
 
-int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcScratch& tc, bool exact, cudaStream_t st)
+int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcScratch& tc, bool exact, cudaStream_t st, bool* transposed)
 {
     static bool attr_done[64] = {};
     if (ctx->device >= 0 && ctx->device < 64 && !attr_done[ctx->device]) {
@@ -666,7 +685,6 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
         attr_done[ctx->device] = true;
     }
     const float loss1 = exact ? 1.0f : 1.0f + kTf32TruncLoss, loss2 = loss1 * loss1;
-    const int width = ctx->tc_update_ctas > 0 ? ctx->tc_update_ctas : ctx->sm_count;   // CTAs one launch may use
     const int round = exact ? 0 : 1;
     // In a recorded graph of a call that runs alone, what nobody waits for yet goes into branches of the graph (on the context's side
     // stream): the merges, which are needed at the end of a superblock, and the last square with its columns of Q.
@@ -684,9 +702,35 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
         GELO_CUDA_OK(cudaStreamWaitEvent(st, ctx->side_done, 0));
         return GELO_OK;
     };
+    // A QR that has the GPU to itself spends most of its time in launches that leave SMs idle, half of it in block factors on three SMs.
+    // Beside them it forms Q^T: the reflectors of a superblock are applied to the identity as they are to the columns on the right, on a stream
+    // of its own, while the next superblock is factorised, on kFormSms of the SMs so that the chain finds others free.  That
+    // takes half as many operations again as accumulating Q backwards, which needs the last reflector first, so it is not
+    // for lanes, where SM time counts.
+    const bool forming = transposed && !exact && ctx->tc_update_ctas == 0 && m >= kFormRows && tc.big[0];
+    struct FormGuard {                                       // however it ends, the caller's stream comes after all launches
+        gelo_ctx* ctx; cudaStream_t st; bool on;
+        ~FormGuard()
+        {
+            if (on && cudaEventRecord(ctx->form_done, ctx->form) == cudaSuccess) cudaStreamWaitEvent(st, ctx->form_done, 0);
+        }
+    } form_guard = { ctx, st, false };
+    auto form_after = [&]() -> int {                         // what goes to the stream that forms Q^T next waits for what st has by now
+        GELO_CUDA_OK(cudaEventRecord(ctx->form_from, st));
+        GELO_CUDA_OK(cudaStreamWaitEvent(ctx->form, ctx->form_from, 0));
+        form_guard.on = true;
+        return GELO_OK;
+    };
+    struct FormLaunches {                                    // launches that are planned for kFormSms and get no more
+        gelo_ctx* ctx;
+        explicit FormLaunches(gelo_ctx* c) : ctx(c) { c->tc_update_ctas = kFormSms; c->tc_cap = true; }
+        FormLaunches(const FormLaunches&) = delete;
+        ~FormLaunches() { ctx->tc_update_ctas = 0; ctx->tc_cap = false; }
+    };
 
     // V^T C with few output tiles: the rows are cut into slices whose partial products are summed in a fixed order
     auto slices = [&](int M, int N, int K, int most) {
+        const int width = ctx->tc_update_ctas > 0 ? ctx->tc_update_ctas : ctx->sm_count;       // CTAs one launch may use
         int want;
         if (!exact && gemm_tile_cols(ctx, M, N, K, 1, 4, true, 64) == 64) {
             want = width / (ceil_div(M, 128) * ceil_div(N, 64));      // one round of narrow tiles
@@ -714,24 +758,25 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
         if (used) *used = g.ksplit;
         return launch_gemm_simt(ctx, g, cur);
     };
-    // C (rows from c0) <- (I - V op(T^T) V^T) C for the merged reflectors of a superblock (kv columns from c0); scratch from column
-    // `at` on
-    auto apply = [&](int c0, int kv, const float* Tt, float* C, int nc, bool transpose, int at = 0) -> int {
+    // C (rows from c0) <- (I - V op(T^T) V^T) C for the merged reflectors of a superblock (kv columns from c0)
+    struct ApplyScratch { float *w, *tw, *planes; int most; };       // V^T C, its product with T, `most` K slices of the former
+    const ApplyScratch scratch = { tc.w32[0], tc.w32[1], tc.wf32, kSuperKSplit };
+    auto apply = [&](int c0, int kv, const float* Tt, float* C, int nc, bool transpose, const ApplyScratch& s) -> int {
         const int nr = m - c0;
         const int nc8 = (nc + 7) & ~7;
         const float* V = G + (size_t)c0 * ld + c0;
-        const int want = slices(kv, nc8, nr, kSuperKSplit);
+        const int want = slices(kv, nc8, nr, s.most);
         if (want <= 1) {
-            GELO_TRY(gemm(kv, nc8, nr, V, ld, true, C, ld, false, tc.w32[0] + at, ld, true, loss2, 1, 0, nullptr));
+            GELO_TRY(gemm(kv, nc8, nr, V, ld, true, C, ld, false, s.w, ld, true, loss2, 1, 0, nullptr));
         } else {
             int used = 0;
             const size_t plane = (size_t)kv * ld;
-            GELO_TRY(gemm(kv, nc8, nr, V, ld, true, C, ld, false, tc.wf32 + at, ld, false, 1.0f, want, plane, &used));
-            GELO_TRY(launch_sum_planes(ctx, tc.wf32 + at, plane, used, ld, kv, nc8, loss2, tc.w32[0] + at, ld, cur, !exact));
+            GELO_TRY(gemm(kv, nc8, nr, V, ld, true, C, ld, false, s.planes, ld, false, 1.0f, want, plane, &used));
+            GELO_TRY(launch_sum_planes(ctx, s.planes, plane, used, ld, kv, nc8, loss2, s.w, ld, cur, !exact));
         }
         // (the factor loss1 makes up for the truncation of V in the last product)
-        GELO_TRY(gemm(kv, nc8, kv, Tt, kSuper, transpose, tc.w32[0] + at, ld, false, tc.w32[1] + at, ld, true, loss1, 1, 0, nullptr));
-        return gemm(nr, nc, kv, V, ld, false, tc.w32[1] + at, ld, true, C, ld, false, 1.0f, 1, 0, nullptr);
+        GELO_TRY(gemm(kv, nc8, kv, Tt, kSuper, transpose, s.w, ld, false, s.tw, ld, true, loss1, 1, 0, nullptr));
+        return gemm(nr, nc, kv, V, ld, false, s.tw, ld, true, C, ld, false, 1.0f, 1, 0, nullptr);
     };
 
     // Block columns: 128 wide while at least twice as many rows are left, then narrower ones (half of the rows, a multiple of eight) down to a
@@ -747,6 +792,15 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
     start.push_back(bf);
     const int nblocks = (int)start.size() - 1;
     const int per = kSuper / FB;
+    // the spare matrix (m x ld): two block rows, the rest for K slices
+    float* spare = static_cast<float*>(tc.big[0]);
+    const ApplyScratch form_scratch = { spare, spare + (size_t)kSuper * ld, spare + (size_t)2 * kSuper * ld, (m - 2 * kSuper) / kSuper };
+    if (forming) {
+        *transposed = true;
+        GELO_TRY(form_after());
+        GELO_TRY(launch_chained(ctx, start_q_kernel, dim3(ceil_div(ld, 1024), m), 256, 0, ctx->form, Q, ld, m, m, G, 0, ld));   // -I
+        GELO_TRY(after_launch(ctx));
+    }
     // ---- factorisation ----
     GELO_CUDA_OK(cudaMemsetAsync(tc.tsuper, 0, (size_t)ceil_div(nblocks, per) * kSuper * kSuper * sizeof(float), st));
     for (int s = 0; s < nblocks; s += per) {
@@ -796,7 +850,31 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
                 GELO_TRY(gemm(nr, send - bend, ob, P, ld, false, Wb + (bend - s0), ld, true, P + ob, ld, false, 1.0f, 1, 0, nullptr));
         }
         if (fork && e - s > 1) GELO_TRY(join());
-        GELO_TRY(apply(s0, send - s0, Ts, G + (size_t)s0 * ld + send, m - send, false));
+        GELO_TRY(apply(s0, send - s0, Ts, G + (size_t)s0 * ld + send, m - send, false, scratch));
+        if (forming) {                                       // (after that update, which fills the GPU)
+            GELO_TRY(form_after());
+            const FormLaunches on_few(ctx);
+            cur = ctx->form;
+            GELO_TRY(apply(s0, send - s0, Ts, Q + (size_t)s0 * ld, m, false, form_scratch));
+            cur = st;
+        }
+    }
+    if (forming) {
+        // Q^T = diag(-I, (Qf S)^T) H^T, of which the other stream has formed -H^T; S flips where R of the last square is negative
+        const int f = m - bf;
+        float *Qf = tc.w32[0], *rows = Q + (size_t)bf * ld;
+        GELO_TRY(launch_qr_small(ctx, f, G + (size_t)bf * ld + bf, ld, Qf, st));
+        GELO_CUDA_OK(cudaEventRecord(ctx->form_done, ctx->form));
+        GELO_CUDA_OK(cudaStreamWaitEvent(st, ctx->form_done, 0));
+        form_guard.on = false;
+        GELO_TRY(launch_chained(ctx, last_rows_kernel, dim3(ceil_div(m, 256), f), 256, 0, st, rows, tc.w32[1], f, m, Qf,
+                                G + (size_t)bf * ld + bf, ld));
+        GELO_TRY(after_launch(ctx));
+        GemmArgs g;
+        g.M = f; g.N = m; g.K = f;
+        g.A = Qf; g.lda = ld; g.transA = true; g.B = tc.w32[1]; g.ldb = ld;
+        g.C[0] = rows; g.ldc = ld;
+        return launch_gemm_simt(ctx, g, st);
     }
     // ---- the square that is left, and Q accumulated backwards, one superblock at a time ----
     auto form_q = [&](int c0, int c1) -> int {               // columns c0 .. c1 - 1
@@ -807,7 +885,7 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
             const int e = (s + per < nblocks) ? s + per : nblocks;
             const int s0 = start[s], from = c0 > s0 ? c0 : s0;
             GELO_TRY(apply(s0, start[e] - s0, tc.tsuper + (size_t)(s / per) * kSuper * kSuper, Q + (size_t)s0 * ld + from, c1 - from, true,
-                           c0));
+                           { tc.w32[0] + c0, tc.w32[1] + c0, tc.wf32 + c0, kSuperKSplit }));
         }
         return GELO_OK;
     };

@@ -45,6 +45,28 @@ def test_block_qr_of_a_gaussian(oracle, m):
     assert np.median(np.sum(a * q_ref, axis=0)) > 1 - 1e-4
 
 
+# A sample alone forms Q^T while it factorises from 1536 rows on: the last size of the other route and the first of this one, an odd one, a
+# last superblock of few columns
+@pytest.mark.parametrize("m", [1535, 1536, 1547, 2131, 2560])
+def test_factor_formed_beside_the_factorisation(oracle, m):
+    a, x = _sample(m, ORTHOGONAL, 900 + m, "f16")
+    assert np.array_equal(x, a.T)
+    d = a.T @ a - np.eye(m)
+    assert np.linalg.norm(d) / np.sqrt(m) <= 6e-4             # as in the test above
+    q_ref, r = np.linalg.qr(oracle.gaussian(900 + m, 0, 0, m, m).astype(np.float32).astype(np.float64))
+    q_ref *= np.sign(np.diag(r))
+    h = m // 2
+    assert np.linalg.norm(a[:, :h] - q_ref[:, :h]) / np.sqrt(h) <= 4e-4 * (2 + m / 128)
+    # a wrong sign or a row of the last square that has not been turned shows in single columns
+    along = np.sum(a * q_ref, axis=0)
+    assert along[: m - 128].min() > 0.9 and np.median(along[-64:]) > 0.9
+    # non-orthogonal: b = Q + G1 / (2 sqrt(m)), Q without the polish, which took the noise of the tf32 products out of a
+    b, y = _sample(m, NONORTHOGONAL, 900 + m, "f16")
+    assert np.linalg.norm(b @ y - np.eye(m)) / np.sqrt(m) <= 1.2e-3       # rounding of A^-1, 2.1e-4 relative, times |A| <= 1.5 and |A^-1| <= 3.3
+    q = b - 0.5 / np.sqrt(m) * oracle.gaussian(900 + m, 1, 0, m, m)
+    assert np.linalg.norm(q[:, :h] - q_ref[:, :h]) / np.sqrt(h) <= 2 * 4e-4 * (2 + m / 128)
+
+
 # 256: the first size of the iteration, a single pair of tile rows; 257 and 300: ragged tiles; gamma 0.55 is the last it takes,
 # 0.6 goes to the LU
 @pytest.mark.parametrize("m,gamma,dt", [(256, 0.5, "f16"), (257, 0.5, "bf16"), (300, 0.55, "f16"), (700, 0.5, "f16"), (300, 0.6, "f16")])
