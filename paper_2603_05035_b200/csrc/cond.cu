@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kCondChunkCols * kCondParts) cond_reduce_kerne
 }
 
 // Largest eigenvalue of the symmetric tridiagonal matrix (alpha[0..k-1]; beta[0..k-2]), found by one warp that cuts the
-// interval from 0 to the Gershgorin bound into 33 at a time (twelve rounds: 2^-60 of the bound) by the number of
+// interval from 0 to the Gershgorin bound into 33 at a time (seven rounds: 2^-35 of the bound, which a float rounds to) by the number of
 // eigenvalues below each point (Sturm sequence).  A breakdown (beta = 0) only decouples the matrix: the count stays valid.
 __device__ double tridiagonal_lambda_max(const float* alpha, const float* beta)
 {
@@ -162,7 +162,7 @@ __device__ double tridiagonal_lambda_max(const float* alpha, const float* beta)
     }
     const int lane = threadIdx.x & 31;
     double lo = 0.0;
-    for (int round = 0; round < 12; ++round) {
+    for (int round = 0; round < 7; ++round) {
         const double step = (hi - lo) * (1.0 / 33.0), x = lo + (lane + 1) * step;
         bool all_below = true;                               // all k eigenvalues lie below x
         double q = 1.0;

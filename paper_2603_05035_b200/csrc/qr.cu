@@ -495,82 +495,135 @@ t_merge_kernel(const float* __restrict__ part, int slabs, int ldp, const float* 
 // A decode-shaped call mixes a few dozen rows, and for such a matrix the blocked path above is some thirty dependent
 // launches of a few microseconds each.  Here one CTA does everything with the matrix in registers: eight consecutive
 // lanes share COLUMN c (lane h of the group holds rows h, h + 8, ...), so applying a reflector to a column is a dozen
-// private FMAs plus a three-step shuffle inside the group, and the only block-wide communication is the reflector
-// itself, which the owners of column j write to shared memory once per column (one barrier per column).  The
-// reflectors stay in shared memory; afterwards each group builds its column of Q = H_0 ... H_(m-1) by applying them
-// backwards to e_c (only H_j with j <= c touch it), with no barrier at all.
+// private FMAs plus a three-step shuffle inside the group.  What bounds it is the chain of the m columns.  A link is: the owners of column j
+// publish it as it stands, one barrier, and every group sums, below row j, both its product with its own column and its
+// square; the reflector (its scalars, worked out by everybody, times that column) needs no second round.  v_j . x_c is x_c[j] + scale_j * (that
+// product), v_j being 1 in row j and scale_j times the column below.  The columns stay in shared memory and are scaled at the end;
+// then each group builds its column of Q = H_0 ... H_(m-1) by applying the reflectors backwards to e_c, two per shuffle: with
+// g = v_(j+1) . v_j known, w_j after H_(j+1) is w_j - g tau_(j+1) w_(j+1).  Only H_j with j <= c touch e_c.
+// Against owners that normalise their column before they publish it, shuffles of single groups and one reflector at a time, a whole sample in
+// fp32: 32 rows 21 -> 18 us, 64 rows 46 -> 36, 72 rows 50 -> 40, 96 rows 87 -> 65; a link of the chain 1090 -> 780 cycles at 64 columns,
+// 660 -> 520 at the last ones.
 // Same conventions as the blocked path: R (upper triangle, diagonal of either sign) overwrites G, Q is unsigned.
 template <int RM>
 struct QrSmall {
     static constexpr int RPT = RM / 8;
     float* Vs;                                // RM x RM: row j = reflector j over the rows
-    float* tau_s;
-    int m, c, h;
-    unsigned gmask;                           // the eight lanes of this column
+    float *tau_s, *scale_s, *beta_s, *g_s;   // g_s[q]: v_(2q+1) . v_(2q)
+    int m, c, h, c_max;                       // c_max: the last column of this warp.  Whole warps take every step, which a shuffle needs to be cheap
 
     __device__ __forceinline__ QrSmall(float* smem, int rows)
-        : Vs(smem), tau_s(smem + RM * RM), m(rows), c(threadIdx.x >> 3), h(threadIdx.x & 7), gmask(0xFFu << (threadIdx.x & 24))
+        : Vs(smem), tau_s(smem + RM * RM), scale_s(tau_s + RM), beta_s(scale_s + RM), g_s(beta_s + RM), m(rows), c(threadIdx.x >> 3),
+          h(threadIdx.x & 7), c_max(c | 3)
     {
     }
     __device__ __forceinline__ float group_sum(float v) const
     {
-        v += __shfl_xor_sync(gmask, v, 1);
-        v += __shfl_xor_sync(gmask, v, 2);
-        v += __shfl_xor_sync(gmask, v, 4);
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        v += __shfl_xor_sync(0xffffffffu, v, 4);
         return v;
     }
-    // x: column c of the matrix -> column c of R; the reflectors stay in Vs
+    // x: column c of the matrix -> column c of R; the reflectors go to Vs, zero past m.  All threads of the CTA.
     __device__ __forceinline__ void factorise(float (&x)[RPT]) const
     {
-        for (int j = 0; j < m; ++j) {
-            if (c == j) {
-                float s = 0.0f, a = 0.0f;
+        if (c == 0) {
 #pragma unroll
-                for (int i = 0; i < RPT; ++i) {
-                    const int r = h + 8 * i;
-                    s = fmaf((r > j) ? x[i] : 0.0f, x[i], s);
-                    a += (r == j) ? x[i] : 0.0f;
+            for (int k = 0; k < RPT; ++k) Vs[h + 8 * k] = x[k];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {                      // (so that rows above the current eight cost nothing)
+#pragma unroll 1
+            for (int hh = 0; hh < 8; ++hh) {
+                const int j = 8 * i + hh;
+                if (j >= m) break;
+                if (c_max >= j) {
+                    float v[RPT], p = 0.0f, p1 = 0.0f, s = 0.0f, s1 = 0.0f;
+#pragma unroll
+                    for (int k = i; k < RPT; ++k) v[k] = Vs[j * RM + h + 8 * k];
+                    const float alpha = __shfl_sync(0xffffffffu, v[i], hh, 8), xj = __shfl_sync(0xffffffffu, x[i], hh, 8);
+                    v[i] = h > hh ? v[i] : 0.0f;
+#pragma unroll
+                    for (int k = i; k < RPT; ++k) {
+                        float& pk = ((k - i) & 1) ? p1 : p;
+                        float& sk = ((k - i) & 1) ? s1 : s;
+                        pk = fmaf(v[k], x[k], pk);
+                        sk = fmaf(v[k], v[k], sk);
+                    }
+                    const float sigma = group_sum(s + s1), dot = group_sum(p + p1);
+                    float beta = alpha, tau = 0.0f, scale = 0.0f;
+                    if (sigma > 0.0f) {
+                        // every thread works these out, so they have to be short: hardware approximations and a Newton step each
+                        const float n2 = fmaf(alpha, alpha, sigma);
+                        float r = rsqrtf(n2);
+                        float norm = n2 * r;
+                        norm = fmaf(0.5f * r, fmaf(-norm, norm, n2), norm);
+                        r = fmaf(r, fmaf(-norm, r, 1.0f), r);                    // 1 / norm
+                        const float far = fabsf(alpha) + norm;
+                        float inv = __fdividef(1.0f, far);
+                        inv = fmaf(inv, fmaf(-far, inv, 1.0f), inv);
+                        beta = -copysignf(norm, alpha);
+                        tau = far * r;
+                        scale = copysignf(inv, alpha);
+                    }
+                    const float tw = c > j ? tau * fmaf(scale, dot, xj) : 0.0f, f = tw * scale;
+                    if (h == hh) x[i] -= tw;
+#pragma unroll
+                    for (int k = i; k < RPT; ++k) x[k] = fmaf(-f, v[k], x[k]);   // (v is zero down to row j)
+                    if (c == j + 1) {
+#pragma unroll
+                        for (int k = i; k < RPT; ++k) Vs[(j + 1) * RM + h + 8 * k] = x[k];
+                    }
+                    if (threadIdx.x == 8 * RM - 1) { tau_s[j] = tau; scale_s[j] = scale; beta_s[j] = beta; }
                 }
-                const float sigma = group_sum(s), alpha = group_sum(a);
-                float beta = alpha, tau = 0.0f, scale = 0.0f;
-                if (sigma > 0.0f) {
-                    beta = -copysignf(sqrtf(fmaf(alpha, alpha, sigma)), alpha);
-                    tau = (beta - alpha) / beta;
-                    scale = 1.0f / (alpha - beta);
-                }
-#pragma unroll
-                for (int i = 0; i < RPT; ++i) {
-                    const int r = h + 8 * i;
-                    Vs[j * RM + r] = (r < j) ? 0.0f : ((r == j) ? 1.0f : x[i] * scale);
-                    x[i] = (r < j) ? x[i] : ((r == j) ? beta : 0.0f);
-                }
-                if (h == 0) tau_s[j] = tau;
-            }
-            __syncthreads();
-            if (c > j && c < m) {
-                const float* v = Vs + j * RM + h;
-                float w = 0.0f;
-#pragma unroll
-                for (int i = 0; i < RPT; ++i) w = fmaf(v[8 * i], x[i], w);        // v is zero above row j
-                const float tw = tau_s[j] * group_sum(w);
-#pragma unroll
-                for (int i = 0; i < RPT; ++i) x[i] = fmaf(-tw, v[8 * i], x[i]);
+                __syncthreads();
             }
         }
+#pragma unroll
+        for (int k = 0; k < RPT; ++k) {
+            const int r = h + 8 * k;
+            if (r >= c && c < m) x[k] = r == c ? beta_s[c] : 0.0f;
+        }
+        for (int e = threadIdx.x; e < RM * RM; e += 8 * RM) {
+            const int j = e / RM, r = e - j * RM;
+            Vs[e] = j >= m || r < j ? 0.0f : (r == j ? 1.0f : Vs[e] * scale_s[j]);
+        }
+        if (threadIdx.x >= m && threadIdx.x < RM) tau_s[threadIdx.x] = 0.0f;
+        __syncthreads();
+        if (c_max < RM / 2) {
+            const float* v = Vs + 2 * c * RM + h;
+            float g = 0.0f;
+#pragma unroll
+            for (int k = 0; k < RPT; ++k) g = fmaf(v[8 * k], v[RM + 8 * k], g);
+            g = group_sum(g);
+            if (h == 0) g_s[c] = g;
+        }
+        __syncthreads();
     }
     // column c of Q
     __device__ __forceinline__ void form_q(float (&x)[RPT]) const
     {
 #pragma unroll
         for (int i = 0; i < RPT; ++i) x[i] = (h + 8 * i == c) ? 1.0f : 0.0f;
-        for (int j = c; j >= 0; --j) {
-            const float* v = Vs + j * RM + h;
-            float w = 0.0f;
 #pragma unroll
-            for (int i = 0; i < RPT; ++i) w = fmaf(v[8 * i], x[i], w);
-            const float tw = tau_s[j] * group_sum(w);
+        for (int i = RPT - 1; i >= 0; --i) {                 // the four pairs whose reflectors begin in rows 8 i .. 8 i + 7
+#pragma unroll 1
+            for (int q = min(c_max >> 1, 4 * i + 3); q >= 4 * i; --q) {   // (reflectors past c leave e_c as it is)
+                const float* v = Vs + 2 * q * RM + h;
+                float a[RPT], b[RPT], w0 = 0.0f, w1 = 0.0f;
 #pragma unroll
-            for (int i = 0; i < RPT; ++i) x[i] = fmaf(-tw, v[8 * i], x[i]);
+                for (int k = i; k < RPT; ++k) {
+                    a[k] = v[8 * k]; b[k] = v[RM + 8 * k];
+                    w0 = fmaf(a[k], x[k], w0);
+                    w1 = fmaf(b[k], x[k], w1);
+                }
+                w0 = group_sum(w0);
+                w1 = group_sum(w1);
+                const float t1 = tau_s[2 * q + 1] * w1, t0 = tau_s[2 * q] * fmaf(-g_s[q], t1, w0);
+#pragma unroll
+                for (int k = i; k < RPT; ++k) x[k] = fmaf(-t0, a[k], fmaf(-t1, b[k], x[k]));
+            }
         }
     }
 };
@@ -591,17 +644,16 @@ qr_small_kernel(float* __restrict__ G, int ld, int m, float* __restrict__ Q)
         x[i] = (r < m && c < m) ? G[(size_t)r * ld + c] : 0.0f;
     }
     q.factorise(x);
-    if (c >= m) return;
 #pragma unroll
     for (int i = 0; i < QrSmall<RM>::RPT; ++i) {
         const int r = q.h + 8 * i;
-        if (r < m) G[(size_t)r * ld + c] = x[i];
+        if (r < m && c < m) G[(size_t)r * ld + c] = x[i];
     }
     q.form_q(x);
 #pragma unroll
     for (int i = 0; i < QrSmall<RM>::RPT; ++i) {
         const int r = q.h + 8 * i;
-        if (r < m) Q[(size_t)r * ld + c] = x[i];
+        if (r < m && c < m) Q[(size_t)r * ld + c] = x[i];
     }
 }
 
@@ -646,7 +698,7 @@ sample_small_kernel(int m, uint64_t seed, uint32_t attempt, T* __restrict__ A, T
 #pragma unroll
     for (int i = 0; i < QrSmall<RM>::RPT; ++i) d += (q.h + 8 * i == c) ? x[i] : 0.0f;
     const float sign = q.group_sum(d) < 0.0f ? -1.0f : 1.0f;
-    if (c < m) q.form_q(x);
+    q.form_q(x);
     __syncthreads();                          // the reflectors have been read
     float* out = qs_smem;                     // row stride RM + 1: read by rows and by columns
     if (c < m) {
@@ -661,7 +713,7 @@ sample_small_kernel(int m, uint64_t seed, uint32_t attempt, T* __restrict__ A, T
     }
 }
 
-constexpr int qr_small_smem(int RM) { return (RM * (RM + 1) + RM) * (int)sizeof(float); }
+constexpr int qr_small_smem(int RM) { return (RM * RM + 4 * RM) * (int)sizeof(float); }       // (reflectors, then the result in rows of RM + 1)
 
 template <typename F>
 int qr_small_attr(gelo_ctx* ctx, F* kernel, int smem, bool (&done)[64])
@@ -695,7 +747,7 @@ int launch_sample_small_rm(gelo_ctx* ctx, int m, uint64_t seed, uint32_t attempt
 constexpr int kSmallQrRows = 128;
 
 // f(RM) for the smallest instance that holds m rows, in steps of eight: the time grows with the instance (the rows a thread holds, and the
-// columns of the reflectors), 20 us for 32 rows, 53 for 72, 98 for 96 and 186 for 128.
+// columns of the reflectors), 18 us for 32 rows, 36 for 64 and 65 for 96.
 template <int RM = 32, typename F>
 int with_small_rows(int m, F&& f)
 {
