@@ -82,7 +82,7 @@ struct Layout {
     void* Yd = nullptr;       // n x p
     void* Hd2 = nullptr;      // second pair: the batched host variant alternates between the two
     void* Yd2 = nullptr;
-    Tf32x3Scratch t3;         // fp32 path: tf32 (hi, lo) copies of the operands of the three products
+    Tf32x3Scratch t3;         // fp32 path: partial products of the three products
 };
 
 Layout carve(Arena& a, int n, int k, int d, int p, int dtype, bool host_staging)
@@ -120,13 +120,6 @@ Layout carve(Arena& a, int n, int k, int d, int p, int dtype, bool host_staging)
     L.U = a.take((size_t)L.m * d * es);
     L.Yp = a.take((size_t)L.m * p * es);
     if (dtype == GELO_F32 && d > 0 && p > 0) {
-        const size_t wide = (size_t)(L.m > d ? L.m : d);
-        L.t3.a_elems = (size_t)L.m * round_up((int)wide, 4);
-        L.t3.b_elems = wide * round_up(p > d ? p : d, 32);
-        for (int h = 0; h < 2; ++h) {
-            L.t3.a[h] = static_cast<float*>(a.take(L.t3.a_elems * 4));
-            L.t3.b[h] = static_cast<float*>(a.take(L.t3.b_elems * 4));
-        }
         L.t3.c_elems = (size_t)L.m * (p > d ? p : d);
         L.t3.planes = static_cast<float*>(a.take(L.t3.c_elems * kTf32x3Slices * 4));
     }
@@ -368,28 +361,19 @@ int sample_mixing_impl(gelo_ctx* ctx, const Layout& L, int m, int kind, uint64_t
     return GELO_ERR_COND;
 }
 
-// A product of the offload.  Large fp32 products run on the tensor cores as three tf32 products of (hi, lo) operand
-// pairs when the call has scratch for the pairs (error about 1e-6, inside the fp32 path's 1e-4); everything else goes
-// to the bf16 / half tensor-core kernel or the FFMA kernel.  Any K and stacked operands: 1024 + 51 rows, d = 4096, p = 12288, mixing
-// and unmixing, which the FFMA kernel took for their K of 1075, 1.45 -> 0.55 ms; 32 such calls 114 -> 99 ms.
+// A product of the offload.  Large fp32 products of the calls run on the tensor cores as three tf32 products of operand
+// pairs (error about 1e-6, inside the fp32 path's 1e-4); everything else goes to the bf16 / half tensor-core kernel or the FFMA
+// kernel.  Any K and stacked operands.
 int product(gelo_ctx* ctx, const GemmArgs& g, const Tf32x3Scratch* t3, cudaStream_t st)
 {
-    const int lda3 = round_up(g.K, 4), ldb3 = round_up(g.N, 32);
-    // (rows of A are read in whole quads: the last one may reach past K, but not past the stride)
-    if (g.dtype == GELO_F32 && t3 && t3->a[0] && !g.transA && !g.transB && g.M >= 128 && 2.0 * g.M * (double)g.N * g.K >= 1e9 &&
-        (g.lda % 4) == 0 && g.lda >= lda3 && (g.ldb % 4) == 0 && (g.ldc % 4) == 0 && !misaligned(g.B2) &&
-        (g.N % 4) == 0 && (g.N % g.nsplit) == 0 && ((g.N / g.nsplit) % 8) == 0 && !misaligned(g.A) && !misaligned(g.B) &&
-        (size_t)g.M * lda3 <= t3->a_elems && (size_t)g.K * ldb3 <= t3->b_elems) {
-        const int k1 = g.B2 ? g.b_split : g.K;               // the rows of a stacked operand go below each other
-        const size_t below = (size_t)k1 * ldb3;
-        GELO_TRY(launch_split_tf32(ctx, static_cast<const float*>(g.A), g.lda, g.M, lda3, t3->a[0], t3->a[1], lda3, st));
-        GELO_TRY(launch_split_tf32(ctx, static_cast<const float*>(g.B), g.ldb, k1, g.N, t3->b[0], t3->b[1], ldb3, st));
-        if (k1 < g.K)
-            GELO_TRY(launch_split_tf32(ctx, static_cast<const float*>(g.B2), g.ldb, g.K - k1, g.N, t3->b[0] + below, t3->b[1] + below, ldb3, st));
+    // (rows of A are whole quads: the last one may reach past K, but not past the stride)
+    if (g.dtype == GELO_F32 && t3 && t3->planes && !g.transA && !g.transB && g.M >= 128 && 2.0 * g.M * (double)g.N * g.K >= 1e9 &&
+        (g.lda % 4) == 0 && g.lda >= round_up(g.K, 4) && (g.ldb % 4) == 0 && (g.ldc % 4) == 0 && !misaligned(g.B2) &&
+        (g.N % 4) == 0 && (g.N % g.nsplit) == 0 && ((g.N / g.nsplit) % 8) == 0 && !misaligned(g.A) && !misaligned(g.B)) {
         float* const C[3] = { static_cast<float*>(g.C[0]), static_cast<float*>(g.C[1]), static_cast<float*>(g.C[2]) };
         float* planes = (size_t)g.M * g.N <= t3->c_elems ? t3->planes : nullptr;
-        return launch_gemm_tf32x3(ctx, g.M, g.N, g.K, t3->a[0], t3->a[1], lda3, t3->b[0], t3->b[1], ldb3, C, g.ldc, g.nsplit,
-                                  planes, st);
+        return launch_gemm_tf32x3(ctx, g.M, g.N, g.K, static_cast<const float*>(g.A), g.lda, static_cast<const float*>(g.B),
+                                  static_cast<const float*>(g.B2), g.b_split, g.ldb, C, g.ldc, g.nsplit, planes, st);
     }
     return gemm_dispatch(ctx, g, st);
 }

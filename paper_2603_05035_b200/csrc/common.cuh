@@ -174,7 +174,7 @@ struct ProfScope {
     ~ProfScope() { if (e1) cudaEventRecord(e1, st); }
 };
 
-static inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
+__host__ __device__ static inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 static inline size_t elem_size(int dtype) { return dtype == GELO_F32 ? 4 : 2; }
 
 // ---- sampling ---------------------------------------------------------------------
@@ -254,28 +254,19 @@ int launch_gemm_e4m3(gelo_ctx*, int M, int N, int K, const void* A8, int lda, co
 // when it stored them pass through the tensor core unchanged and need no correction.
 constexpr float kTf32TruncLoss = 3.5224e-4f;
 
-// fp32 products on the tensor cores with fp32-grade accuracy: every operand is held as a pair of tf32 values
-// (hi = x rounded to tf32, lo = the remainder rounded to tf32) and the product is accumulated as
-// hi*hi + hi*lo + lo*hi in fp32 (the dropped lo*lo term is 2^-22 of the product).  C_q (q = 0 .. nsplit-1) receives
-// the q-th column block of the M x N result; strides in elements, all multiples of 4, N / nsplit a multiple of 8.
-// The tensor core adds into its fp32 accumulator with truncation, which costs about 2^-25 of the running sum per
-// instruction, coherently: 5e-5 after the 1536 instructions of a K = 4096 product.  With `planes` (room for
-// kTf32x3Slices * M * N floats) the K range is cut into that many slices with an accumulator each, summed afterwards in
-// round-to-nearest fp32 in a fixed order, which brings the product back to a few 1e-6.
+// fp32 products on the tensor cores with fp32-grade accuracy (gemm_x3_kernel in gemm_tc.cu): C_q (q = 0 .. nsplit-1) receives the q-th
+// column block of A B, A M x K, B K x N; the rows of B from b_split on come from B2 if that is given.  Strides in elements,
+// all multiples of 4, N / nsplit a multiple of 8.  planes: room for kTf32x3Slices * M * N floats, or null.
 constexpr int kTf32x3Slices = 8;
-int launch_gemm_tf32x3(gelo_ctx*, int M, int N, int K, const float* Ahi, const float* Alo, int lda, const float* Bhi,
-                       const float* Blo, int ldb, float* const C[3], int ldc, int nsplit, float* planes, cudaStream_t);
+int launch_gemm_tf32x3(gelo_ctx*, int M, int N, int K, const float* A, int lda, const float* B, const float* B2, int b_split, int ldb,
+                       float* const C[3], int ldc, int nsplit, float* planes, cudaStream_t);
 // C_q[r, c] = sum over `parts` planes (M x N, dense) of the entry (r, q * csplit + c), planes added in order
 int launch_sum_planes_routed(gelo_ctx*, const float* planes, size_t plane, int parts, int rows, int cols, float* const C[3],
                              int ldc, int csplit, cudaStream_t);
-// hi / lo tf32 pair of a rows x cols fp32 block (cols a multiple of 4, 16-byte aligned rows)
-int launch_split_tf32(gelo_ctx*, const float* src, int lds, int rows, int cols, float* hi, float* lo, int ldo, cudaStream_t);
-// scratch of the tf32-pair products of the fp32 path: operand copies of at most a_elems / b_elems floats each
+// scratch of the fp32 path's tensor-core products: kTf32x3Slices partial products of at most c_elems floats each
 struct Tf32x3Scratch {
-    float* a[2] = {nullptr, nullptr};
-    float* b[2] = {nullptr, nullptr};
-    float* planes = nullptr;              // kTf32x3Slices partial products of at most c_elems floats each
-    size_t a_elems = 0, b_elems = 0, c_elems = 0;
+    float* planes = nullptr;
+    size_t c_elems = 0;
 };
 
 // ---- projection and unmixing of a small batch in one kernel (decode.cu) ---------------------------------

@@ -607,6 +607,199 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
     }
 }
 
+// ---- fp32 products: three tf32 products of operand pairs that are made on the way ------------------------------------
+//
+// C = A B in fp32 with fp32-grade accuracy: x = hi + lo, hi = x as the tensor core reads it (its 13 low bits dropped), lo = x - hi rounded to
+// tf32; lo hi + hi lo + hi hi in fp32 (lo lo, 2^-22 of a term, is dropped).  A stage holds the fp32 tiles as TMA brings them, which ARE the hi operands, and
+// beside them their lo parts, which four warps work out in shared memory (element by element at the same place, so the swizzle does not
+// matter).  The tensor core adds into its accumulator with truncation, 2^-25 of the running sum per instruction and coherent, so an
+// accumulator only takes kX3Slice k-blocks (24 instructions); the epilogue warps add it to sums in registers, rounded to nearest,
+// while the other accumulator fills.  Relative error against 64 bits, at 512 rows: K = 504 7.0e-7 -> 4.5e-7, K = 4096 5.3e-6 -> 4.8e-7 (before: pairs
+// written to memory, K in eight slices); with 48 instructions 9.3e-7.
+//
+// Tiles of 256 x 192 on a pair of CTAs, one tile (or K slice of one) per pair.  Bound by shared memory: per k-block and SM 28 KB come in, are read and
+// written by the converters and read three times by the matrix instructions, 1310 cycles at 128 bytes each, against 1180 cycles of
+// tf32 arithmetic.  192 columns instead of 256 for the registers that the sums take and for the rounds: 512 x 12288 makes
+// 128 tiles for 74 pairs.  A pair of tiles per SM pair takes 1.14 us per k-block, 86% of the 0.71 PFLOP/s that the library's plain tf32 products reach.
+// Against a pass that splits each operand into pairs, a product that reads them from memory and a sum over eight planes:
+// 512 x 12288 x 4096 351 -> 310 us, x 512 123 -> 51 us; eight calls of 512 rows 5.04 -> 3.90 ms, 32 of 1075 rows on 16 lanes 52.1 -> 49.4 ms.
+constexpr int kX3N = 192, kX3Cols = kX3N / 2, kX3Stages = 4, kX3Slice = 2;
+constexpr int kX3ConvWarps = 4;
+constexpr int kX3Threads = kThreads + 32 * kX3ConvWarps;
+constexpr uint32_t kX3BBytes = kX3Cols / 32 * 4096u;
+constexpr uint32_t kX3Raw = kABytes + kX3BBytes;              // one stage of fp32 tiles; as much again for their lo parts
+constexpr uint32_t kX3Smem = kX3Stages * 2 * kX3Raw + 1024 + 256;    // (the results leave through the first stage, when nothing reads it any more)
+static_assert(kX3Smem <= 227 * 1024, "shared memory budget");
+static_assert(kX3Raw % 1024 == 0, "tiles start on swizzle atoms");
+constexpr uint32_t kX3Idesc = (1u << 4) | (2u << 7) | (2u << 10) | (1u << 16) | ((uint32_t)(kX3N >> 3) << 17) | ((uint32_t)(2 * BM >> 4) << 24);
+
+struct X3Params {
+    TcParams out;                   // M, N, C0..C2, ldc, csplit, plane; wait_ns, status
+    int kb, kb0, per;               // k-blocks of 32 in all, of the first B, per K slice
+    int a_k1, b_row1;               // where the blocks of the second B start in A's columns and in its rows
+    int b3d;
+};
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kX3Threads, 1)
+gemm_x3_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b0, const __grid_constant__ CUtensorMap map_b1,
+               const X3Params prm)
+{
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    const uint32_t bars = base + kX3Stages * 2 * kX3Raw;
+    uint8_t* bars_gen = smem_raw + (bars - raw);
+    auto full_bar = [&](int s) { return bars + 8u * s; };                        // this CTA's tiles are there
+    auto conv_bar = [&](int s) { return bars + 8u * (kX3Stages + s); };          // leader: so are the lo parts in both CTAs
+    auto empty_bar = [&](int s) { return bars + 8u * (2 * kX3Stages + s); };
+    auto acc_full_bar = [&](int a) { return bars + 8u * (3 * kX3Stages + a); };
+    auto acc_empty_bar = [&](int a) { return bars + 8u * (3 * kX3Stages + 2 + a); };
+    constexpr uint32_t kMisc = 8 * (3 * kX3Stages + 4);
+    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bars_gen + kMisc);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(bars_gen + kMisc + 8);
+    static_assert(kMisc + 16 <= 256, "barriers fit");
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = (int)cluster_rank();
+    const TcParams& out = prm.out;
+    const int m_tiles = ceil_div(out.M, 2 * BM), mn_tiles = m_tiles * ceil_div(out.N, kX3N);
+    const int tile = blockIdx.x >> 1, mn = tile % mn_tiles, slice = tile / mn_tiles;
+    const int m0 = mn % m_tiles * 2 * BM + rank * BM, n_tile = mn / m_tiles * kX3N;
+    const int kb_lo = slice * prm.per, blocks = min(prm.kb - kb_lo, prm.per);
+
+    chain_next();
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kX3Stages; ++s) { mbar_init(full_bar(s), 1); mbar_init(conv_bar(s), 2 * kX3ConvWarps); mbar_init(empty_bar(s), 1); }
+        for (int a = 0; a < 2; ++a) { mbar_init(acc_full_bar(a), 1); mbar_init(acc_empty_bar(a), 2 * kEpiWarps); }
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncwarp();
+    cluster_sync();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    chain_wait();
+    bool ok = true;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            const int n0 = n_tile + rank * kX3Cols;
+            for (int it = 0; it < blocks; ++it) {
+                const int s = it % kX3Stages;
+                if (!mbar_wait(empty_bar(s), ((it / kX3Stages) & 1u) ^ 1u, abort_flag, out.wait_ns)) { ok = false; break; }
+                const uint32_t sa = base + s * 2 * kX3Raw, sb = sa + kABytes;
+                const int kb = kb_lo + it;
+                const bool second = kb >= prm.kb0;
+                const CUtensorMap* mb = second ? &map_b1 : &map_b0;
+                const int k = second ? prm.a_k1 + 32 * (kb - prm.kb0) : 32 * kb, row = second ? prm.b_row1 + 32 * (kb - prm.kb0) : 32 * kb;
+                mbar_expect_tx(full_bar(s), kX3Raw);
+                tma_load_2d(sa, &map_a, k, m0, full_bar(s));
+                if (prm.b3d) {
+                    tma_load_3d(sb, mb, 0, row, n0 / 32, full_bar(s));
+                } else {
+#pragma unroll
+                    for (int j = 0; j < kX3Cols / 32; ++j) tma_load_2d(sb + j * 4096u, mb, n0 + 32 * j, row, full_bar(s));
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0 && rank == 0) {
+            for (int it = 0; it < blocks; ++it) {
+                const int s = it % kX3Stages, sl = it / kX3Slice, a = sl & 1;
+                if (it % kX3Slice == 0) {
+                    if (!mbar_wait_cluster(acc_empty_bar(a), ((sl >> 1) & 1u) ^ 1u, abort_flag, out.wait_ns)) { ok = false; break; }
+                    tc_fence_after();
+                }
+                if (!mbar_wait_cluster(conv_bar(s), (it / kX3Stages) & 1u, abort_flag, out.wait_ns)) { ok = false; break; }
+                const uint32_t sa = base + s * 2 * kX3Raw, sb = sa + kABytes, d = tmem_base + 256u * a;
+                const uint64_t a_hi = smem_desc(sa, 16, 1024), a_lo = smem_desc(sa + kX3Raw, 16, 1024);
+                const uint64_t b_hi = smem_desc(sb, 4096, 512, 1), b_lo = smem_desc(sb + kX3Raw, 4096, 512, 1);
+                tc_mma4_tf32_pair(d, a_lo, b_hi, 2, 64, kX3Idesc, it % kX3Slice != 0);
+                tc_mma4_tf32_pair(d, a_hi, b_lo, 2, 64, kX3Idesc, 1);
+                tc_mma4_tf32_pair(d, a_hi, b_hi, 2, 64, kX3Idesc, 1);
+                tc_commit_pair(empty_bar(s));
+                if (it % kX3Slice == kX3Slice - 1 || it == blocks - 1) tc_commit_pair(acc_full_bar(a));
+            }
+        }
+    } else if (warp < 2 + kEpiWarps) {
+        const int quarter = warp & 3, half = (warp - 2) >> 2;
+        const uint32_t buf = base + (uint32_t)(warp - 2) * 4096u;
+        float sum[kX3Cols];
+#pragma unroll
+        for (int j = 0; j < kX3Cols; ++j) sum[j] = 0.0f;
+        const int slices = ceil_div(blocks, kX3Slice);
+#pragma unroll 1
+        for (int sl = 0; sl < slices; ++sl) {
+            const int a = sl & 1;
+            if (!mbar_wait(acc_full_bar(a), (sl >> 1) & 1u, abort_flag, out.wait_ns)) { ok = false; break; }
+            tc_fence_after();
+            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + 256u * a + (uint32_t)(half * kX3Cols);
+#pragma unroll
+            for (int c = 0; c < kX3Cols; c += 32) {
+                uint32_t v[32];
+                tc_ld_32cols(taddr + c, v);
+                tc_ld_wait();
+#pragma unroll
+                for (int j = 0; j < 32; ++j) sum[c + j] += __uint_as_float(v[j]);
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(map_rank(acc_empty_bar(a), 0));
+        }
+        if (ok) {
+#pragma unroll
+            for (int c = 0; c < kX3Cols; c += 32) {
+                uint32_t v[32];
+#pragma unroll
+                for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(sum[c + j]);
+                if (n_tile + half * kX3Cols + c < out.N)
+                    store_tile32(out, v, buf, m0 + quarter * 32, n_tile + half * kX3Cols + c, lane, slice);
+            }
+        }
+    } else {
+        const int t = threadIdx.x - kThreads;
+        for (int it = 0; it < blocks; ++it) {
+            const int s = it % kX3Stages;
+            if (!mbar_wait(full_bar(s), (it / kX3Stages) & 1u, abort_flag, out.wait_ns)) { ok = false; break; }
+            const uint32_t src = base + s * 2 * kX3Raw;
+            constexpr int kEach = kX3Raw / (16 * 32 * kX3ConvWarps);
+            static_assert(kX3Raw % (16 * 32 * kX3ConvWarps) == 0, "whole rounds");
+            float x[kEach][4];
+#pragma unroll
+            for (int i = 0; i < kEach; ++i)                   // all loads before the first store
+                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[i][0]), "=f"(x[i][1]), "=f"(x[i][2]), "=f"(x[i][3])
+                             : "r"(src + 16u * (t + 32 * kX3ConvWarps * i)) : "memory");
+#pragma unroll
+            for (int i = 0; i < kEach; ++i) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) x[i][j] = round_tf32(x[i][j] - __uint_as_float(__float_as_uint(x[i][j]) & 0xffffe000u));
+                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"
+                             ::"r"(src + kX3Raw + 16u * (t + 32 * kX3ConvWarps * i)), "f"(x[i][0]), "f"(x[i][1]), "f"(x[i][2]), "f"(x[i][3]) : "memory");
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(map_rank(conv_bar(s), 0));
+        }
+    }
+    if (!ok) { *abort_flag = 1; atomicCAS(out.status, 0, (int)GELO_ERR_TIMEOUT); }
+
+    tc_fence_before();
+    __syncwarp();
+    cluster_sync();
+    if (warp == 1) {
+        if (*abort_flag) settle(out.wait_ns);
+        __syncwarp();
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
+    }
+}
+
 // ---- host side ----------------------------------------------------------------------------------
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -1172,50 +1365,64 @@ int launch_gemm_e4m3(gelo_ctx* ctx, int M, int N, int K, const void* A8, int lda
     return launch_tiles<256, false, false, false, true>(ctx, pair, ma, ma, mb, mb, ma, p, 2.0 * M * (double)N * K, st);
 }
 
-int launch_gemm_tf32x3(gelo_ctx* ctx, int M, int N, int K, const float* Ahi, const float* Alo, int lda, const float* Bhi,
-                       const float* Blo, int ldb, float* const C[3], int ldc, int nsplit, float* planes, cudaStream_t st)
+int launch_gemm_tf32x3(gelo_ctx* ctx, int M, int N, int K, const float* A, int lda, const float* B, const float* B2, int b_split, int ldb,
+                       float* const C[3], int ldc, int nsplit, float* planes, cudaStream_t st)
 {
     if (M <= 0 || N <= 0 || K <= 0) return GELO_OK;
     if (!ctx->tmap_encode) return GELO_ERR_CUDA;
-    if (nsplit < 1 || nsplit > 3 || (N % nsplit) || ((N / nsplit) % 8) || (lda % 4) || (ldb % 4) || (ldc % 4) ||
-        !aligned16(Ahi) || !aligned16(Alo) || !aligned16(Bhi) || !aligned16(Blo))
+    if (nsplit < 1 || nsplit > 3 || (N % nsplit) || ((N / nsplit) % 8) || (lda % 4) || (ldb % 4) || (ldc % 4) || !aligned16(A) || !aligned16(B) ||
+        (B2 && (!aligned16(B2) || b_split <= 0 || b_split >= K)))
         return GELO_ERR_INVALID;
     for (int q = 0; q < nsplit; ++q)
         if (!C[q] || !aligned16(C[q])) return GELO_ERR_INVALID;
-    const int kb = ceil_div(K, 32);
-    // (N a multiple of 8, so the planes' rows are whole chunks)
-    const bool sliced = planes && kb >= 2 * kTf32x3Slices && aligned16(planes);
-    const int per = sliced ? ceil_div(kb, kTf32x3Slices) : kb;
-    const bool pair = use_pair(ctx, M, N, ceil_div(kb, per), false, TC_STORE_F32);
-    const uint32_t cols = pair ? 128 : 256;
-    CUtensorMap a0, a1, b0, b1;
+    const int rows = B2 ? b_split : K;
+    CUtensorMap ma, b0, b1;
     bool b3d = false, b3d1 = false;
-    if (!make_map_f32_box(ctx, &a0, Ahi, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BM) ||
-        !make_map_f32_box(ctx, &a1, Alo, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BM) ||
-        !make_map_nmajor(ctx, &b0, Bhi, 4, true, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, 32, cols, &b3d) ||
-        !make_map_nmajor(ctx, &b1, Blo, 4, true, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, 32, cols, &b3d1) || b3d != b3d1)
+    if (!make_map_f32_box(ctx, &ma, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BM) ||
+        !make_map_nmajor(ctx, &b0, B, 4, true, (uint64_t)N, (uint64_t)rows, (uint64_t)ldb, 32, kX3Cols, &b3d))
         return GELO_ERR_CUDA;
-    TcParams p = {};
-    p.M = M; p.N = N;
-    p.nseg = 3;
-    p.seg[0] = TcSegment{0, 0, 0, 0, kb};
-    p.seg[1] = TcSegment{0, 1, 0, 0, kb};
-    p.seg[2] = TcSegment{1, 0, 0, 0, kb};
-    p.status = ctx->status_dev;
-    p.b3d = b3d ? 1 : 0;
-    p.ksplit = 1; p.kb_per_split = 1 << 30; p.plane = 0;
-    p.mode = TC_STORE_F32;
-    p.out_scale = 1.0f; p.post_scale = 1.0f;
-    float* const Cq[3] = { C[0], C[nsplit > 1 ? 1 : 0], C[nsplit > 2 ? 2 : 0] };
-    if (sliced) {
-        p.ksplit = ceil_div(kb, per); p.kb_per_split = per; p.plane = (long long)M * N;
-        p.C0 = planes; p.C1 = planes; p.C2 = planes; p.ldc = N; p.csplit = N;
-        GELO_TRY((launch_tiles<256, false, true, false>(ctx, pair, a0, a1, b0, b1, a0, p, 6.0 * M * (double)N * K, st)));
-        return launch_sum_planes_routed(ctx, planes, (size_t)M * N, p.ksplit, M, N, Cq, ldc, N / nsplit, st);
+    b1 = b0;
+    X3Params p = {};
+    p.kb0 = p.kb = ceil_div(rows, 32);
+    if (B2) {
+        if (!make_map_nmajor(ctx, &b1, B2, 4, true, (uint64_t)N, (uint64_t)(K - b_split), (uint64_t)ldb, 32, kX3Cols, &b3d1) || b3d1 != b3d)
+            return GELO_ERR_CUDA;
+        p.a_k1 = b_split & ~3;                                // (16-byte aligned; the rows of B2 above its first read as zero)
+        p.b_row1 = p.a_k1 - b_split;
+        p.kb += ceil_div(K - p.a_k1, 32);
     }
-    p.C0 = Cq[0]; p.C1 = Cq[1]; p.C2 = Cq[2];
-    p.ldc = ldc; p.csplit = N / nsplit;
-    return launch_tiles<256, false, true, false>(ctx, pair, a0, a1, b0, b1, a0, p, 6.0 * M * (double)N * K, st);
+    p.b3d = b3d ? 1 : 0;
+    const int tiles = ceil_div(M, 2 * BM) * ceil_div(N, kX3N);
+    // K slices where they fill the rounds better than whole tiles and that is worth their planes, which are written and read: microseconds,
+    // with 1.14 per k-block, 6 per tile for its first copies and its stores, 6 TB/s for the planes and 5 for the launch that sums them.  1075 x 12288
+    // x 4096 in three slices 741 -> 730; 512 rows stay whole (310).
+    int slices = 1;
+    double best = 0.0;
+    for (int t = 1; t <= kTf32x3Slices && (t == 1 || (planes && aligned16(planes) && p.kb >= 8 * t)); ++t) {
+        const double us = ceil_div(tiles * t, ctx->sm_count / 2) * (1.14 * ceil_div(p.kb, t) + 6.0) + (t > 1 ? 5.0 + 8e-6 * t * (double)M * N / 6.0 : 0.0);
+        if (t == 1 || us < best) { best = us; slices = t; }
+    }
+    p.per = ceil_div(p.kb, slices);
+    slices = ceil_div(p.kb, p.per);                           // no empty slice
+    TcParams& o = p.out;
+    o.M = M; o.N = N;
+    o.status = ctx->status_dev; o.wait_ns = ctx->wait_limit_ns;
+    float* const Cq[3] = { C[0], C[nsplit > 1 ? 1 : 0], C[nsplit > 2 ? 2 : 0] };
+    o.C0 = Cq[0]; o.C1 = Cq[1]; o.C2 = Cq[2]; o.ldc = ldc; o.csplit = N / nsplit;
+    if (slices > 1) {                                         // (N is a multiple of 8, so the planes' rows are whole chunks)
+        o.C0 = o.C1 = o.C2 = planes; o.ldc = N; o.csplit = N; o.plane = (long long)M * N;
+    }
+    static bool attr_done[64] = {};
+    if (ctx->device >= 0 && ctx->device < 64 && !attr_done[ctx->device]) {
+        GELO_CUDA_OK(cudaFuncSetAttribute(gemm_x3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kX3Smem));
+        attr_done[ctx->device] = true;
+    }
+    {
+        ProfScope ps(ctx, PROF_GEMM_TC, 6.0 * M * (double)N * K, st);
+        GELO_TRY(launch_chained(ctx, gemm_x3_kernel, 2 * tiles * slices, kX3Threads, kX3Smem, st, ma, b0, b1, p));
+    }
+    GELO_TRY(after_launch(ctx));
+    return slices > 1 ? launch_sum_planes_routed(ctx, planes, (size_t)M * N, slices, M, N, Cq, ldc, N / nsplit, st) : GELO_OK;
 }
 
 }  // namespace gelo

@@ -241,6 +241,21 @@ __device__ __forceinline__ bool tc_mma4_try(uint32_t tmem_d, uint64_t da, uint64
 }
 #undef GELO_TC_MMA4_TRY
 
+// The four instructions of one stage of a CTA pair in tf32, without a barrier test
+__device__ __forceinline__ void tc_mma4_tf32_pair(uint32_t tmem_d, uint64_t da, uint64_t db, uint64_t astep, uint64_t bstep, uint32_t idesc,
+                                                  uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %5, p;\n\t"
+        "tcgen05.mma.cta_group::2.kind::tf32 [%0], %3, %4, %5, 1;\n\t"
+        "tcgen05.mma.cta_group::2.kind::tf32 [%0], %7, %8, %5, 1;\n\t"
+        "tcgen05.mma.cta_group::2.kind::tf32 [%0], %9, %10, %5, 1;\n\t}"
+        ::"r"(tmem_d), "l"(da), "l"(db), "l"(da + astep), "l"(db + bstep), "r"(idesc), "r"(accumulate), "l"(da + 2 * astep),
+          "l"(db + 2 * bstep), "l"(da + 3 * astep), "l"(db + 3 * bstep) : "memory");
+}
+
 __device__ __forceinline__ float round_tf32(float x)
 {
     uint32_t r;

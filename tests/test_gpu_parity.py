@@ -1266,6 +1266,26 @@ def test_fp32_products_of_any_depth(ctx, oracle, n, k, kind):
     assert ((Q.double() - ref).norm() / ref.norm()).item() <= TOL["f32"]
 
 
+# The tensor-core kernel of the large ones by itself: tiles of 256 x 192 with one row, a few columns (not whole boxes of 32) or a few k over, K from two
+# k-blocks to many, whole tiles and K slices
+@pytest.mark.parametrize("m,d,p", [(129, 4104, 1000), (257, 2056, 1992), (512, 40, 24600), (300, 504, 4096), (1075, 4096, 1536)])
+def test_fp32_products_on_the_tensor_cores(m, d, p):
+    c = binding.Context(0)
+    c.ensure_workspace(m, 0, d, p, "f32")
+    g = torch.Generator(device="cuda")
+    g.manual_seed(m)
+    U = torch.randn((m, d), generator=g, device="cuda")
+    W = torch.randn((d, p), generator=g, device="cuda")
+    Y = torch.full((m, p), float("nan"), device="cuda")
+    c.project(U, W, m, d, p, "f32", Y)
+    assert c.last_status() == binding.OK
+    ref = U.double() @ W.double()
+    # 24 truncated additions of 2^-25 each, half of that on the average, the dropped lo lo of 2^-23 and the sums' own rounding
+    assert ((Y.double() - ref).norm() / ref.norm()).item() <= 8e-7
+    assert (Y.double() - ref).abs().max().item() <= 1e-5 * d ** 0.5
+    c.close()
+
+
 # fp32 products on either side of the lines between the two FMA kernels: 148 tiles of 64 x 64 and one more where the last stage of k is short,
 # 296 and one more where it is full, with a last tile of eight columns and a K that ends a quad after two
 @pytest.mark.parametrize("m,d,p", [(33, 72, 9472), (33, 72, 9480), (32, 64, 18944), (32, 64, 18952), (65, 64, 9472), (1, 8, 8)])
