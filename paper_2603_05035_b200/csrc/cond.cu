@@ -18,6 +18,7 @@
 
 #include "common.cuh"
 #include "philox.cuh"
+#include "tc_ptx.cuh"
 
 namespace gelo {
 
@@ -309,6 +310,143 @@ __global__ void __launch_bounds__(256) cond_step_kernel(CondViews v)
     }
 }
 
+// All steps in one launch for a matrix whose rows fit the shared memory of eight CTAs (16 bits: up to 920 rows, fp32: 656).  A cluster per
+// operator; each CTA keeps its rows on chip, forms its part of Op^T (Op v), and after one barrier of the cluster every CTA adds the eight
+// parts up in the same order and does the recurrence for itself, so the vector never travels.  Bound by latency, 2 us a step; as
+// launches of their own the steps take 8 us each.  With the verdict,
+// fp32: 64 rows 56 -> 19 us, 350 rows 63 -> 33, 512 rows 64 -> 44, 650 rows 75 -> 62.
+constexpr int kSmallCtas = 8, kSmallThreads = 1024;
+struct CondSmallPlan { int rows, lds; size_t slab, bytes; };
+CondSmallPlan cond_small_plan(int m, int es)
+{
+    CondSmallPlan p;
+    p.rows = ceil_div(m, kSmallCtas);
+    p.lds = (m + 7) & ~7;
+    p.slab = (3 * (size_t)p.lds + 2 * kSmallThreads + ((p.rows + 3) & ~3) + 32) * sizeof(float);     // what stands before the rows
+    p.slab = (p.slab + 15) & ~size_t(15);
+    p.bytes = p.slab + (size_t)p.rows * p.lds * es;
+    return p;
+}
+bool cond_small_supports(int m, int es) { return m <= kSmallThreads && cond_small_plan(m, es).bytes <= 227 * 1024; }
+
+template <typename T>
+__global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThreads, 1)
+cond_small_kernel(CondViews v, uint64_t seed, uint32_t attempt, int rows_per, int lds, int slab_offset)
+{
+    chain_next();
+    chain_wait();
+    extern __shared__ __align__(16) uint8_t cs_smem[];
+    float* vs = reinterpret_cast<float*>(cs_smem);           // the Lanczos vector
+    float* part = vs + lds;                                  // [2][lds] this CTA's part of w, in turn
+    float* sums = part + 2 * lds;                            // [2 kSmallThreads]
+    float* ys = sums + 2 * kSmallThreads;
+    float* red = ys + ((rows_per + 3) & ~3);
+    T* slab = reinterpret_cast<T*>(cs_smem + slab_offset);
+    const int z = blockIdx.y, rank = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, m = v.m;
+    const int r0 = rank * rows_per, rows = max(0, min(rows_per, m - r0)), groups = lds >> 3;
+    const T* op = static_cast<const T*>(v.op[z]);
+    constexpr int kVec = 16 / (int)sizeof(T);
+    for (int e = tid; e < rows * (lds / kVec); e += kSmallThreads) {             // (rows of the operator are whole groups of eight)
+        const int r = e / (lds / kVec), c = (e - r * (lds / kVec)) * kVec;
+        __align__(16) T t[kVec];
+        *reinterpret_cast<uint4*>(t) = *reinterpret_cast<const uint4*>(op + (size_t)(r0 + r) * v.ld + c);
+#pragma unroll
+        for (int j = 0; j < kVec; ++j)
+            if (c + j >= m) t[j] = T(0.0f);                   // (what stands past the last column is no data)
+        *reinterpret_cast<uint4*>(slab + (size_t)r * lds + c) = *reinterpret_cast<const uint4*>(t);
+    }
+    float vi = 0.0f, vp = 0.0f, bprev = 0.0f;                // entry tid of the vector and of the one before; every CTA has them all
+    if (4 * tid < lds) {
+        float g[4];
+        gaussian_block(seed, ((uint64_t)z * v.mpad + 4 * tid) >> 2, GELO_STREAM_POWER, attempt, g);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) vs[4 * tid + j] = 4 * tid + j < m ? g[j] : 0.0f;
+    }
+    __syncthreads();
+    if (tid < m) vi = vs[tid];
+    {
+        const float nrm = sqrtf(cond_block_sum(vi * vi, red)), inv = nrm > 0.0f ? 1.0f / nrm : 0.0f;
+        vi *= inv;
+        if (tid < m) vs[tid] = vi;
+    }
+    const int pairs = lds >> 1, parts = min(8, kSmallThreads / pairs), my_q = tid / pairs, my_c = 2 * (tid - my_q * pairs);
+    for (int step = 0; step < kLanczosSteps; ++step) {
+        __syncthreads();                                     // vs
+        for (int r = warp; r < rows; r += kSmallThreads / 32) {
+            float s = 0.0f;
+#pragma unroll 4
+            for (int g = lane; g < groups; g += 32) {
+                float e[8], x[8];
+                load8(slab + (size_t)r * lds + 8 * g, e);
+                load8(vs + 8 * g, x);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) s = fmaf(e[j], x[j], s);
+            }
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+            if (lane == 0) ys[r] = s;
+        }
+        __syncthreads();
+        if (my_q < parts) {                                  // rows q, q + parts, ... of two columns
+            const int q = my_q, c = my_c;
+            float a = 0.0f, b = 0.0f;
+#pragma unroll 8
+            for (int r = q; r < rows; r += parts) {
+                const T* t = slab + (size_t)r * lds + c;
+                a = fmaf((float)t[0], ys[r], a);
+                b = fmaf((float)t[1], ys[r], b);
+            }
+            sums[q * lds + c] = a;
+            sums[q * lds + c + 1] = b;
+        }
+        __syncthreads();
+        float* mine = part + (step & 1) * lds;
+        if (tid < lds) {
+            float s = sums[tid];
+            for (int q = 1; q < parts; ++q) s += sums[q * lds + tid];
+            mine[tid] = s;
+        }
+        // (a part is written again two steps later, after the barrier at which everybody has read it)
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        float w = 0.0f;
+        if (tid < m) {
+            float t[kSmallCtas];
+#pragma unroll
+            for (int k = 0; k < kSmallCtas; ++k)             // all on their way before the first is added
+                asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(t[k]) : "r"(tcx::map_rank(tcx::smem_u32(mine + tid), k)));
+#pragma unroll
+            for (int k = 0; k < kSmallCtas; ++k) w += t[k];
+        }
+        const float a = cond_block_sum(vi * w, red);
+        w = w - a * vi - bprev * vp;
+        const float b = sqrtf(cond_block_sum(w * w, red)), inv = b > 0.0f ? 1.0f / b : 0.0f;
+        vp = vi;
+        vi = w * inv;
+        bprev = b;
+        if (tid < m) vs[tid] = vi;
+        if (rank == 0 && tid == 0) {
+            v.tri[z * 2 * kLanczosSteps + step] = a;
+            v.tri[z * 2 * kLanczosSteps + kLanczosSteps + step] = b;
+        }
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");        // nobody's shared memory goes while others read it
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+template <typename T>
+int launch_cond_small(gelo_ctx* ctx, const CondViews& v, cudaStream_t st)
+{
+    static bool done[64] = {};
+    if (ctx->device >= 0 && ctx->device < 64 && !done[ctx->device]) {
+        GELO_CUDA_OK(cudaFuncSetAttribute(cond_small_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        done[ctx->device] = true;
+    }
+    const CondSmallPlan p = cond_small_plan(v.m, (int)sizeof(T));
+    GELO_TRY(launch_chained(ctx, cond_small_kernel<T>, dim3(kSmallCtas, 2), kSmallThreads, p.bytes, st, v, 0x5eedull, 0u, p.rows, p.lds, (int)p.slab));
+    return after_launch(ctx);
+}
+
 int cond_slabs(int m) { return ceil_div(m, kCondRows) < kCondSlabsMax ? ceil_div(m, kCondRows) : kCondSlabsMax; }
 
 }  // namespace
@@ -338,6 +476,13 @@ int run_cond_estimate(gelo_ctx* ctx, int m, const void* A, const void* Ainv, int
     v.done = reinterpret_cast<unsigned*>(s.scal);
     const size_t ys_bytes = (size_t)v.rows_per * sizeof(float);
     if (ys_bytes > 48 * 1024) return GELO_ERR_UNSUPPORTED;
+    if (cond_small_supports(m, (int)elem_size(dtype))) {
+        if (dtype == GELO_BF16) GELO_TRY(launch_cond_small<__nv_bfloat16>(ctx, v, st));
+        else if (dtype == GELO_F16) GELO_TRY(launch_cond_small<__half>(ctx, v, st));
+        else GELO_TRY(launch_cond_small<float>(ctx, v, st));
+        GELO_TRY(launch_chained(ctx, cond_verdict_kernel, 1, 64, 0, st, v, bound, cond_out, ctx->status_dev, deferred ? 1 : 0));
+        return after_launch(ctx);
+    }
     dim3 gi(ceil_div(v.mpad, 4 * 256), 2);
     GELO_TRY(launch_chained(ctx, cond_init_kernel, gi, 256, 0, st, v, 0x5eedull, 0u));
     GELO_TRY(after_launch(ctx));

@@ -252,3 +252,27 @@ def test_one_launch_samples(oracle, m):
     q_ref, _ = oracle.householder_qr(oracle.gaussian(60 + m, 0, 0, m, m).astype(np.float32).astype(np.float64))
     h = (m + 1) // 2
     assert np.linalg.norm(a[:, :h] - q_ref[:, :h]) / np.sqrt(h) <= 2e-5       # columns conditioned below 6 times what R loses
+
+
+# The estimate of kappa_2 in one launch: one row per CTA and less, ragged rows and columns, its last fp32 size and the first of the general route; in
+# bfloat16 its last size and the next through a sample
+@pytest.mark.parametrize("m,dt", [(2, "f32"), (9, "f32"), (135, "f32"), (656, "f32"), (657, "f32"), (920, "bf16"), (921, "bf16")])
+def test_condition_estimate_on_both_routes(m, dt):
+    c = binding.Context(0)
+    c.ensure_workspace(m, 0, 8, 24, dt)
+    ld = c.mixing_ld(m)
+    A = padded(m, ld, TDT[dt]); X = padded(m, ld, TDT[dt])
+    est = torch.zeros(1, device="cuda")
+    if dt == "f32":
+        g = torch.Generator().manual_seed(m)
+        a = torch.eye(m, dtype=torch.float64) + 0.5 * torch.randn((m, m), generator=g, dtype=torch.float64) / m ** 0.5
+        A[:, :m] = a.float(); X[:, :m] = torch.linalg.inv(A[:, :m].double()).float()
+        A[:, m:] = float("inf"); X[:, m:] = float("nan")          # the padding is never read as data
+        c.cond_estimate(m, A, X, ld, est)
+    else:
+        c.sample_mixing(m, NONORTHOGONAL, 3, dt, A, X, ld, est)
+    assert c.last_status() == binding.OK
+    s = torch.linalg.svdvals(A[:, :m].double())
+    ref = (s[0] / s[-1]).item()
+    assert 0.85 * ref <= est.item() <= 1.01 * ref                # a lower estimate; of A and of A^-1 as stored
+    c.close()
