@@ -617,12 +617,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
 // while the other accumulator fills.  Relative error against 64 bits, at 512 rows: K = 504 7.0e-7 -> 4.5e-7, K = 4096 5.3e-6 -> 4.8e-7 (before: pairs
 // written to memory, K in eight slices); with 48 instructions 9.3e-7.
 //
-// Tiles of 256 x 192 on a pair of CTAs, one tile (or K slice of one) per pair.  Bound by shared memory: per k-block and SM 28 KB come in, are read and
-// written by the converters and read three times by the matrix instructions, 1310 cycles at 128 bytes each, against 1180 cycles of
-// tf32 arithmetic.  192 columns instead of 256 for the registers that the sums take and for the rounds: 512 x 12288 makes
-// 128 tiles for 74 pairs.  A pair of tiles per SM pair takes 1.14 us per k-block, 86% of the 0.71 PFLOP/s that the library's plain tf32 products reach.
+// Tiles of 256 x 192 on a pair of CTAs, one tile (or K slice of one) per pair.  Per k-block and SM 28 KB come in, are read and
+// written by the converters and read three times by the matrix instructions: 1310 cycles of shared memory at 128 bytes each, and 1180 cycles of
+// tf32 arithmetic.  It takes 2100: what bounds it is the latency from one role to the next (tensor pipe 54% busy).  192 columns instead of 256 for the registers that the sums take and for the rounds: 512 x 12288 makes
+// 128 tiles for 74 pairs.  A tile takes 1.1 us per k-block, 86% of the 0.71 PFLOP/s that the library's plain tf32 products reach.
 // Against a pass that splits each operand into pairs, a product that reads them from memory and a sum over eight planes:
-// 512 x 12288 x 4096 351 -> 310 us, x 512 123 -> 51 us; eight calls of 512 rows 5.04 -> 3.90 ms, 32 of 1075 rows on 16 lanes 52.1 -> 49.4 ms.
+// 512 x 12288 x 4096 351 -> 304 us, x 512 123 -> 50 us; eight calls of 512 rows 5.04 -> 3.90 ms, 32 of 1075 rows on 16 lanes 52.1 -> 49.4 ms.
 constexpr int kX3N = 192, kX3Cols = kX3N / 2, kX3Stages = 4, kX3Slice = 2;
 constexpr int kX3ConvWarps = 4;
 constexpr int kX3Threads = kThreads + 32 * kX3ConvWarps;
@@ -778,7 +778,8 @@ gemm_x3_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 #pragma unroll
             for (int i = 0; i < kEach; ++i) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) x[i][j] = round_tf32(x[i][j] - __uint_as_float(__float_as_uint(x[i][j]) & 0xffffe000u));
+                for (int j = 0; j < 4; ++j)                   // (half a unit of tf32 added to the magnitude, the rest dropped when it is read: rounded to nearest)
+                    x[i][j] = __uint_as_float(__float_as_uint(x[i][j] - __uint_as_float(__float_as_uint(x[i][j]) & 0xffffe000u)) + 0x1000u);
                 asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"
                              ::"r"(src + kX3Raw + 16u * (t + 32 * kX3ConvWarps * i)), "f"(x[i][0]), "f"(x[i][1]), "f"(x[i][2]), "f"(x[i][3]) : "memory");
             }
@@ -1395,7 +1396,7 @@ int launch_gemm_tf32x3(gelo_ctx* ctx, int M, int N, int K, const float* A, int l
     const int tiles = ceil_div(M, 2 * BM) * ceil_div(N, kX3N);
     // K slices where they fill the rounds better than whole tiles and that is worth their planes, which are written and read: microseconds,
     // with 1.14 per k-block, 6 per tile for its first copies and its stores, 6 TB/s for the planes and 5 for the launch that sums them.  1075 x 12288
-    // x 4096 in three slices 741 -> 730; 512 rows stay whole (310).
+    // x 4096 in three slices 741 -> 730 (709 since); 512 rows stay whole (304).
     int slices = 1;
     double best = 0.0;
     for (int t = 1; t <= kTf32x3Slices && (t == 1 || (planes && aligned16(planes) && p.kb >= 8 * t)); ++t) {
