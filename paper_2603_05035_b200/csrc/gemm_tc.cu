@@ -72,7 +72,8 @@ struct TcParams {
     const void* add; int ldadd;     // TC_AFFINE16: out = out_scale * acc + diag_sub on the diagonal + post_scale * the entry of `add` (optional)
     int tri, tri_tiles;             // TC_STORE_SYM16: the result is symmetric; only the tri_tiles tiles that reach the diagonal or lie
                                     // above it are computed, and what lies below them is filled in by mirroring
-    int tiles, stride;              // stride > 0: all tiles, and how many CTAs (pairs) share them in turn instead of taking from the queue
+    int tiles, stride;              // tf32 products, stride > 0: all tiles, and how many CTAs (pairs) share them in turn instead of taking from the
+                                    // queue.  (Looked at by the 16-bit and 8-bit instances too, E4M3 at 2150 x 12288 x 4096 took 92.6 instead of 90.9 us)
     uint32_t idesc;                 // instruction descriptor (filled in by the launcher)
     unsigned long long wait_ns;     // limit of every mbarrier wait, nanoseconds (filled in by the launcher from the context)
     int* status;
@@ -435,7 +436,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
                             for (int j = 0; j < Cfg::kCols / Cfg::kBoxCols; ++j)
                                 load_2d(sb + j * Cfg::kBoxBytes, mb, n0 + j * Cfg::kBoxCols, seg.b_row0 + kb * Cfg::kBKE);
                         }
-                        if (rank == 0 && !asked && prm.stride == 0) {     // the next tile, while this one's operands come in
+                        if (rank == 0 && !asked && (!kTf32 || prm.stride == 0)) {     // the next tile, while this one's operands come in
                             mbar_expect_tx(clc_bar, 16);
                             clc_try_cancel(clc_slot, clc_bar);
                             asked = true;
@@ -446,7 +447,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
                     if (asked && !mbar_wait(clc_bar, tile_it & 1u, abort_flag, prm.wait_ns)) ok = false;
                     if (!ok) break;
                     asked = false;
-                    if (prm.stride > 0) {
+                    if (kTf32 && prm.stride > 0) {
                         tile = tile + prm.stride < prm.tiles ? tile + prm.stride : -1;
                     } else {
                         const int x = clc_answer(clc_slot);
@@ -919,7 +920,7 @@ int launch_tiles_as(gelo_ctx* ctx, const CUtensorMap& a0, const CUtensorMap& a1,
     {
         ProfScope ps(ctx, PROF_GEMM_TC, flops, st);
         cudaLaunchConfig_t cfg = {};
-        const int most = ctx->tc_cap ? ctx->tc_update_ctas / (kPair ? 2 : 1) : tiles;
+        const int most = kTf32 && ctx->tc_cap ? ctx->tc_update_ctas / (kPair ? 2 : 1) : tiles;
         q.tiles = tiles;
         q.stride = most < tiles ? most : 0;
         cfg.gridDim = dim3((most < tiles ? most : tiles) * (kPair ? 2 : 1));
