@@ -29,6 +29,8 @@
 //   context's status word, stops issuing work, lets what is in flight arrive, releases tensor memory and returns.
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -72,8 +74,7 @@ struct TcParams {
     const void* add; int ldadd;     // TC_AFFINE16: out = out_scale * acc + diag_sub on the diagonal + post_scale * the entry of `add` (optional)
     int tri, tri_tiles;             // TC_STORE_SYM16: the result is symmetric; only the tri_tiles tiles that reach the diagonal or lie
                                     // above it are computed, and what lies below them is filled in by mirroring
-    int tiles, stride;              // tf32 products, stride > 0: all tiles, and how many CTAs (pairs) share them in turn instead of taking from the
-                                    // queue.  (Looked at by the 16-bit and 8-bit instances too, E4M3 at 2150 x 12288 x 4096 took 92.6 instead of 90.9 us)
+    int tiles, stride;              // kShare: all tiles, and how many CTAs (pairs) share them
     uint32_t idesc;                 // instruction descriptor (filled in by the launcher)
     unsigned long long wait_ns;     // limit of every mbarrier wait, nanoseconds (filled in by the launcher from the context)
     int* status;
@@ -305,7 +306,9 @@ __device__ __forceinline__ void store_symmetric(const TcParams& prm, int gm, int
     }
 }
 
-template <int BN, bool kStaging, bool kTf32, bool kAMn, bool kF8, bool kPair>
+// kShare: prm.stride CTAs (pairs) share the tiles in turn instead of taking them from the queue.  Instances of their own: looked at by every one of
+// them, the stride cost E4M3 at 2150 x 12288 x 4096 92.6 instead of 90.9 us and a tf32 update of 512 x 4096 x 512 12.5 instead of 12.2.
+template <int BN, bool kStaging, bool kTf32, bool kAMn, bool kF8, bool kPair, bool kShare>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_a1,
                const __grid_constant__ CUtensorMap map_b0, const __grid_constant__ CUtensorMap map_b1,
@@ -436,7 +439,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
                             for (int j = 0; j < Cfg::kCols / Cfg::kBoxCols; ++j)
                                 load_2d(sb + j * Cfg::kBoxBytes, mb, n0 + j * Cfg::kBoxCols, seg.b_row0 + kb * Cfg::kBKE);
                         }
-                        if (rank == 0 && !asked && (!kTf32 || prm.stride == 0)) {     // the next tile, while this one's operands come in
+                        if (!kShare && rank == 0 && !asked) {     // the next tile, while this one's operands come in
                             mbar_expect_tx(clc_bar, 16);
                             clc_try_cancel(clc_slot, clc_bar);
                             asked = true;
@@ -447,7 +450,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
                     if (asked && !mbar_wait(clc_bar, tile_it & 1u, abort_flag, prm.wait_ns)) ok = false;
                     if (!ok) break;
                     asked = false;
-                    if (kTf32 && prm.stride > 0) {
+                    if (kShare) {
                         tile = tile + prm.stride < prm.tiles ? tile + prm.stride : -1;
                     } else {
                         const int x = clc_answer(clc_slot);
@@ -899,13 +902,13 @@ bool use_pair(const gelo_ctx* ctx, int M, int N, int slices, bool tri, int mode)
     return ceil_div(tile_count(M, N, slices, tri, true), width / 2) <= ceil_div(tile_count(M, N, slices, tri, false), width);
 }
 
-template <int BN, bool kStaging, bool kTf32, bool kAMn, bool kF8, bool kPair>
+template <int BN, bool kStaging, bool kTf32, bool kAMn, bool kF8, bool kPair, bool kShare = false>
 int launch_tiles_as(gelo_ctx* ctx, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0, const CUtensorMap& b1,
                     const CUtensorMap& c, const TcParams& p, double flops, cudaStream_t st)
 {
     using Cfg = TcCfg<BN, kStaging, kTf32, kAMn, kF8, kPair>;
     static_assert(Cfg::kSmemBytes <= 227 * 1024, "shared memory budget");
-    auto kernel = gemm_tc_kernel<BN, kStaging, kTf32, kAMn, kF8, kPair>;
+    auto kernel = gemm_tc_kernel<BN, kStaging, kTf32, kAMn, kF8, kPair, kShare>;
     static bool attr_done[64] = {};
     if (ctx->device >= 0 && ctx->device < 64 && !attr_done[ctx->device]) {
         GELO_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmemBytes));
@@ -920,10 +923,9 @@ int launch_tiles_as(gelo_ctx* ctx, const CUtensorMap& a0, const CUtensorMap& a1,
     {
         ProfScope ps(ctx, PROF_GEMM_TC, flops, st);
         cudaLaunchConfig_t cfg = {};
-        const int most = kTf32 && ctx->tc_cap ? ctx->tc_update_ctas / (kPair ? 2 : 1) : tiles;
         q.tiles = tiles;
-        q.stride = most < tiles ? most : 0;
-        cfg.gridDim = dim3((most < tiles ? most : tiles) * (kPair ? 2 : 1));
+        q.stride = kShare ? std::min(tiles, ctx->tc_update_ctas / (kPair ? 2 : 1)) : tiles;
+        cfg.gridDim = dim3(q.stride * (kPair ? 2 : 1));
         cfg.blockDim = dim3(kThreads);
         cfg.dynamicSmemBytes = Cfg::kSmemBytes;
         cfg.stream = st;
@@ -943,6 +945,11 @@ template <int BN, bool kStaging, bool kTf32 = false, bool kAMn = false, bool kF8
 int launch_tiles(gelo_ctx* ctx, bool pair, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0, const CUtensorMap& b1,
                  const CUtensorMap& c, const TcParams& p, double flops, cudaStream_t st)
 {
+    if constexpr (BN == 256 && kTf32) {                       // (launches that may not have the whole GPU are planned with 256 columns)
+        if (ctx->tc_cap)
+            return pair ? launch_tiles_as<BN, kStaging, kTf32, kAMn, kF8, true, true>(ctx, a0, a1, b0, b1, c, p, flops, st)
+                        : launch_tiles_as<BN, kStaging, kTf32, kAMn, kF8, false, true>(ctx, a0, a1, b0, b1, c, p, flops, st);
+    }
     if constexpr (BN == 256) {
         if (pair) return launch_tiles_as<BN, kStaging, kTf32, kAMn, kF8, true>(ctx, a0, a1, b0, b1, c, p, flops, st);
     }
