@@ -146,54 +146,74 @@ __global__ void __launch_bounds__(kCondChunkCols * kCondParts) cond_reduce_kerne
 }
 
 // Largest eigenvalue of the symmetric tridiagonal matrix (alpha[0..k-1]; beta[0..k-2]), found by one warp that cuts the
-// interval from 0 to the Gershgorin bound into 33 at a time (seven rounds: 2^-35 of the bound, which a float rounds to) by the number of
+// interval from 0 to the Gershgorin bound into 33 at a time by the number of
 // eigenvalues below each point (Sturm sequence).  A breakdown (beta = 0) only decouples the matrix: the count stays valid.
-__device__ double tridiagonal_lambda_max(const float* alpha, const float* beta)
-{
-    constexpr int k = kLanczosSteps;
-    double a[k], b2[k], hi = 0.0;
-#pragma unroll
-    for (int i = 0; i < k; ++i) {
-        a[i] = alpha[i];
-        const double bl = i > 0 ? fabs((double)beta[i - 1]) : 0.0, br = i + 1 < k ? fabs((double)beta[i]) : 0.0;
-        b2[i] = bl * bl;
-        const double reach = fabs(a[i]) + bl + br;
-        if (!(reach <= DBL_MAX)) return reach;               // matrices with NaN or infinite entries have no bound: fmax would drop a NaN
-        hi = fmax(hi, reach);
-    }
-    const int lane = threadIdx.x & 31;
-    double lo = 0.0;
-    for (int round = 0; round < 7; ++round) {
-        const double step = (hi - lo) * (1.0 / 33.0), x = lo + (lane + 1) * step;
-        bool all_below = true;                               // all k eigenvalues lie below x
-        double q = 1.0;
+struct TopEigenvalue {
+    static constexpr int k = kLanczosSteps;
+    double a[k], b2[k], lo, hi;                              // it lies between lo and hi
+    bool bounded;
+
+    __device__ __forceinline__ TopEigenvalue(const float* alpha, const float* beta) : lo(0.0), hi(0.0), bounded(true)
+    {
 #pragma unroll
         for (int i = 0; i < k; ++i) {
-            q = a[i] - x - (i > 0 ? b2[i] / q : 0.0);
-            if (q == 0.0) q = -1e-300;
-            all_below = all_below && q < 0.0;
+            a[i] = alpha[i];
+            const double bl = i > 0 ? fabs((double)beta[i - 1]) : 0.0, br = i + 1 < k ? fabs((double)beta[i]) : 0.0;
+            b2[i] = bl * bl;
+            const double reach = fabs(a[i]) + bl + br;
+            // (matrices with NaN or infinite entries have no bound: fmax would drop a NaN)
+            if (bounded && !(reach <= DBL_MAX)) { bounded = false; lo = hi = reach; }
+            if (bounded) hi = fmax(hi, reach);
         }
-        const uint32_t mask = __ballot_sync(0xffffffffu, all_below);
-        const int first = mask ? __ffs(mask) - 1 : 32;       // the first point with everything below it
-        const double h = first < 32 ? lo + (first + 1) * step : hi;
-        lo = lo + first * step;
-        hi = h;
     }
-    return 0.5 * (lo + hi);
-}
+    __device__ __forceinline__ void narrow(int rounds)
+    {
+        if (!bounded) return;
+        const int lane = threadIdx.x & 31;
+#pragma unroll 1
+        for (int round = 0; round < rounds; ++round) {
+            const double step = (hi - lo) * (1.0 / 33.0), x = lo + (lane + 1) * step;
+            bool all_below = true;                           // all k eigenvalues lie below x
+            double q = 1.0;
+#pragma unroll
+            for (int i = 0; i < k; ++i) {
+                q = a[i] - x - (i > 0 ? b2[i] / q : 0.0);
+                if (q == 0.0) q = -1e-300;
+                all_below = all_below && q < 0.0;
+            }
+            const uint32_t mask = __ballot_sync(0xffffffffu, all_below);
+            const int first = mask ? __ffs(mask) - 1 : 32;   // the first point with everything below it
+            const double h = first < 32 ? lo + (first + 1) * step : hi;
+            lo = lo + first * step;
+            hi = h;
+        }
+    }
+};
 
-// One warp per operator.
+// One warp per operator.  Twelve rounds leave 2^-60 of the bound.  After seven (2^-35) both ends of the intervals nearly always give
+// the same float, which then is that of twelve; only where they do not are the other five done.
 __global__ void __launch_bounds__(64) cond_verdict_kernel(CondViews v, float bound, float* cond_out, int* status, int deferred)
 {
     chain_next();
     chain_wait();
-    __shared__ double lam[2];
+    __shared__ double lo[2], hi[2];
     const int z = threadIdx.x >> 5;
-    const double l = tridiagonal_lambda_max(v.tri + z * 2 * kLanczosSteps, v.tri + z * 2 * kLanczosSteps + kLanczosSteps);
-    if ((threadIdx.x & 31) == 0) lam[z] = l;
+    TopEigenvalue top(v.tri + z * 2 * kLanczosSteps, v.tri + z * 2 * kLanczosSteps + kLanczosSteps);
+    auto publish = [&]() {
+        if ((threadIdx.x & 31) == 0) { lo[z] = top.lo; hi[z] = top.hi; }
+        __syncthreads();
+    };
+    top.narrow(7);
+    publish();
+    const bool settled = (float)(sqrt(lo[0]) * sqrt(lo[1])) == (float)(sqrt(hi[0]) * sqrt(hi[1]));
     __syncthreads();
+    if (!settled) {
+        top.narrow(5);
+        publish();
+    }
     if (threadIdx.x != 0) return;
-    const float c = (float)(sqrt(lam[0]) * sqrt(lam[1]));    // lambda_max(Op^T Op) = sigma_max^2
+    // lambda_max(Op^T Op) = sigma_max^2
+    const float c = (float)(sqrt(0.5 * (lo[0] + hi[0])) * sqrt(0.5 * (lo[1] + hi[1])));
     if (cond_out) cond_out[0] = c;
     const int ok = (c * 1.2f <= bound && c == c) ? 1 : 0;   // the estimate is a lower one (tests: >= 0.85 of the true value)
     status[1] = ok;

@@ -276,3 +276,26 @@ def test_condition_estimate_on_both_routes(m, dt):
     ref = (s[0] / s[-1]).item()
     assert 0.85 * ref <= est.item() <= 1.01 * ref                # a lower estimate; of A and of A^-1 as stored
     c.close()
+
+
+# The eigenvalue search is carried to the last bit of the float it returns.  1 x 1 operators have the square of their entry, rounded once, as the only
+# entry of their Lanczos matrix; these are pairs whose result lies so close to the middle of two floats that the bracket of the first seven rounds,
+# 33^-7 wide and with its upper end on the eigenvalue, has its own middle on the other side
+def test_condition_estimate_to_the_last_bit():
+    rng = np.random.default_rng(7)
+    a = rng.uniform(0.5, 2.0, 1 << 20).astype(np.float32)
+    x = rng.uniform(0.5, 2.0, 1 << 20).astype(np.float32)
+    lam = [(t * t).astype(np.float64) for t in (a, x)]
+    est = (np.sqrt(lam[0]) * np.sqrt(lam[1])).astype(np.float32)
+    short = (np.sqrt(lam[0] * (1 - 0.5 * 33.0 ** -7)) * np.sqrt(lam[1] * (1 - 0.5 * 33.0 ** -7))).astype(np.float32)
+    pick = np.flatnonzero(est != short)[:16]
+    assert len(pick) == 16
+    c = binding.Context(0)
+    c.ensure_workspace(1, 0, 8, 24, "f32")
+    A = torch.zeros((1, 8), device="cuda"); X = torch.zeros((1, 8), device="cuda"); out = torch.zeros(16, device="cuda")
+    for i, j in enumerate(pick):
+        A[0, 0] = float(a[j]); X[0, 0] = float(x[j])
+        c.cond_estimate(1, A, X, 8, out[i:])
+    assert c.last_status() == binding.OK
+    assert np.array_equal(out.cpu().numpy(), est[pick])
+    c.close()
