@@ -299,3 +299,31 @@ def test_condition_estimate_to_the_last_bit():
     assert c.last_status() == binding.OK
     assert np.array_equal(out.cpu().numpy(), est[pick])
     c.close()
+
+
+# The scalars of a reflector are as good as the rounded square root and divisions: Q of a 2 x 2 matrix is one reflector, whose few operations are repeated here in
+# binary32.  An approximation that is off by a unit now and then shows in one of its four entries
+def test_reflector_scalars_of_the_one_launch_sample():
+    c = binding.Context(0)
+    c.ensure_workspace(2, 0, 8, 24, "f32")
+    A = torch.zeros((400, 2, 64), device="cuda"); X = torch.zeros((2, 64), device="cuda"); G = torch.zeros((400, 2, 2), device="cuda")
+    for s in range(400):
+        c.sample_gaussian(2, 2, 2, 4000 + s, 0, 0, 1.0, G[s])
+        c.sample_mixing(2, ORTHOGONAL, 4000 + s, "f32", A[s], X, 64)
+    assert c.last_status() == binding.OK
+    f = lambda v: np.asarray(v, dtype=np.float32)
+    g = G.cpu().numpy()
+    a, b = g[:, 0, 0], g[:, 1, 0]
+    fma = lambda x, y, z: f(x.astype(np.float64) * y + z)          # (48 bits of product and a term of like size: rounded once, but for rare ties)
+    beta = -np.copysign(np.sqrt(fma(a, a, b * b)), a)
+    tau, v = (beta - a) / beta, b * (f(1) / (a - beta))
+    t = tau * v
+    q = np.stack([np.stack([f(1) - tau, -t], 1), np.stack([-t, fma(-t, v, f(1))], 1)], 1)          # q[:, row, column]
+    # columns signed by the diagonal of R
+    x0, x1 = g[:, 0, 1], g[:, 1, 1]
+    tw = tau * fma(f(1) / (a - beta), b * x1, x0)
+    r = np.stack([beta, fma(-tw, v, x1)], 1)
+    q *= np.where(r < 0, f(-1), f(1))[:, None, :]
+    same = (A[:, :, :2].cpu().numpy() == q).all(axis=(1, 2))
+    assert same.mean() >= 0.98
+    c.close()
