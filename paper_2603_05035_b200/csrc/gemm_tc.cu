@@ -613,13 +613,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
 
 // ---- fp32 products: three tf32 products of operand pairs that are made on the way ------------------------------------
 //
-// C = A B in fp32 with fp32-grade accuracy: x = hi + lo, hi = x as the tensor core reads it (its 13 low bits dropped), lo = x - hi rounded to
-// tf32; lo hi + hi lo + hi hi in fp32 (lo lo, 2^-22 of a term, is dropped).  A stage holds the fp32 tiles as TMA brings them, which ARE the hi operands, and
-// beside them their lo parts, which four warps work out in shared memory (element by element at the same place, so the swizzle does not
-// matter).  The tensor core adds into its accumulator with truncation, 2^-25 of the running sum per instruction and coherent, so an
-// accumulator only takes kX3Slice k-blocks (24 instructions); the epilogue warps add it to sums in registers, rounded to nearest,
-// while the other accumulator fills.  Relative error against 64 bits, at 512 rows: K = 504 7.0e-7 -> 4.5e-7, K = 4096 5.3e-6 -> 4.8e-7 (before: pairs
-// written to memory, K in eight slices); with 48 instructions 9.3e-7.
+// C = A B in fp32 with fp32-grade accuracy: x = hi + lo, both parts rounded to tf32; lo hi + hi lo + hi hi in fp32.  lo is 2^-11 of x at
+// most and of either sign, so lo lo, which is dropped, is 2^-22 of a term at most and cancels (with hi = x as the tensor core reads it, its 13 low
+// bits cut off, it is up to 2^-20 and always of the term's sign: products of positive entries came out 8.2e-7 low instead of 4.2e-7).
+// A stage holds the fp32 tiles as TMA brings them, which four warps round in place, and beside them their lo parts (element by element at the
+// same place, so the swizzle does not matter).  The tensor core adds into its accumulator with truncation, 2^-25 of the running sum per
+// instruction and coherent, so an accumulator only takes kX3Slice k-blocks (24 instructions); the epilogue warps add it to sums in
+// registers, rounded to nearest, while the other accumulator fills.  Relative error against 64 bits: K = 504 3.7e-7 (hi cut off 4.5e-7; pairs
+// written to memory, K in eight slices 7.0e-7), K = 4096 4.0e-7 (4.8e-7, 5.3e-6); with 48 instructions twice that.
 //
 // Tiles of 256 x 192 on a pair of CTAs, one tile (or K slice of one) per pair.  Per k-block and SM 28 KB come in, are read and
 // written by the converters and read three times by the matrix instructions: 1310 cycles of shared memory at 128 bytes each, and 1180 cycles of
@@ -643,6 +644,14 @@ struct X3Params {
     int a_k1, b_row1;               // where the blocks of the second B start in A's columns and in its rows
     int b3d;
 };
+
+// The pair of an fp32 value as bits: hi rounded to tf32 (half a unit added to the magnitude, what is below dropped), lo the rest, which the
+// tensor core rounds the same way by dropping what is below half a unit more.
+__device__ __forceinline__ void x3_pair(float x, uint32_t& hi, uint32_t& lo)
+{
+    hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+    lo = __float_as_uint(x - __uint_as_float(hi)) + 0x1000u;
+}
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kX3Threads, 1)
 gemm_x3_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b0, const __grid_constant__ CUtensorMap map_b1,
@@ -775,17 +784,21 @@ gemm_x3_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             constexpr int kEach = kX3Raw / (16 * 32 * kX3ConvWarps);
             static_assert(kX3Raw % (16 * 32 * kX3ConvWarps) == 0, "whole rounds");
             float x[kEach][4];
+            auto put = [&](int i, const uint32_t (&h)[4], const uint32_t (&l)[4]) {
+                const uint32_t at = src + 16u * (t + 32 * kX3ConvWarps * i);
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]) : "memory");
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at + kX3Raw), "r"(l[0]), "r"(l[1]), "r"(l[2]), "r"(l[3]) : "memory");
+            };
 #pragma unroll
             for (int i = 0; i < kEach; ++i)                   // all loads before the first store
                 asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[i][0]), "=f"(x[i][1]), "=f"(x[i][2]), "=f"(x[i][3])
                              : "r"(src + 16u * (t + 32 * kX3ConvWarps * i)) : "memory");
 #pragma unroll
             for (int i = 0; i < kEach; ++i) {
+                uint32_t h[4], l[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j)                   // (half a unit of tf32 added to the magnitude, the rest dropped when it is read: rounded to nearest)
-                    x[i][j] = __uint_as_float(__float_as_uint(x[i][j] - __uint_as_float(__float_as_uint(x[i][j]) & 0xffffe000u)) + 0x1000u);
-                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"
-                             ::"r"(src + kX3Raw + 16u * (t + 32 * kX3ConvWarps * i)), "f"(x[i][0]), "f"(x[i][1]), "f"(x[i][2]), "f"(x[i][3]) : "memory");
+                for (int j = 0; j < 4; ++j) x3_pair(x[i][j], h[j], l[j]);
+                put(i, h, l);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();

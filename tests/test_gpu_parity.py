@@ -1280,9 +1280,32 @@ def test_fp32_products_on_the_tensor_cores(m, d, p):
     c.project(U, W, m, d, p, "f32", Y)
     assert c.last_status() == binding.OK
     ref = U.double() @ W.double()
-    # 24 truncated additions of 2^-25 each, half of that on the average, the dropped lo lo of 2^-23 and the sums' own rounding
+    # 24 truncated additions of 2^-25 each, half of that on the average, beside which the dropped lo lo (2^-22 of a term at most, of either sign) and the
+    # sums' own rounding are small
     assert ((Y.double() - ref).norm() / ref.norm()).item() <= 8e-7
     assert (Y.double() - ref).abs().max().item() <= 1e-5 * d ** 0.5
+    c.close()
+
+
+# The operand pairs by themselves: U is diagonal, so every result is one product of two entries and there is nothing to add up.  With both parts rounded to
+# nearest lo is half a unit of tf32 at most, 2^-11 of the entry, its own rounding 2^-23, the dropped lo lo 2^-22, and three truncated additions take up to
+# 2^-23 each: 3.5 x 2^-22 in all.  Entries of 1 + 2^-10 - 2^-23 have parts of 1 + 2^-10 and -2^-23, of which only the additions lose anything; cut off
+# instead of rounded, lo would be nearly 2^-10 and the dropped lo lo nearly 2^-20
+@pytest.mark.parametrize("dist,bound", [("uniform", 3.5 * 2.0 ** -22), ("adverse", 1.5 * 2.0 ** -22)])
+def test_fp32_operand_pairs(dist, bound):
+    n, p = 512, 2048
+    c = binding.Context(0)
+    c.ensure_workspace(n, 0, n, p, "f32")
+    g = torch.Generator(device="cuda"); g.manual_seed(5)
+    W = torch.rand((n, p), generator=g, device="cuda") + 1
+    u = torch.rand(n, generator=g, device="cuda") + 1
+    if dist == "adverse":
+        W.fill_(1 + 2.0 ** -10 - 2.0 ** -23); u.fill_(1 + 2.0 ** -10 - 2.0 ** -23)
+    Y = torch.empty((n, p), device="cuda")
+    c.project(torch.diag(u).contiguous(), W, n, n, p, "f32", Y)
+    assert c.last_status() == binding.OK
+    ref = u.double()[:, None] * W.double()
+    assert ((Y.double() - ref).abs() / ref).max().item() <= bound
     c.close()
 
 
