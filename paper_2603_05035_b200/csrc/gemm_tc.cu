@@ -646,10 +646,24 @@ struct X3Params {
 };
 
 // The pair of an fp32 value as bits: hi rounded to tf32 (half a unit added to the magnitude, what is below dropped), lo the rest, which the
-// tensor core rounds the same way by dropping what is below half a unit more.
-__device__ __forceinline__ void x3_pair(float x, uint32_t& hi, uint32_t& lo)
+// tensor core rounds the same way by dropping what is below half a unit more.  `bad` becomes NaN where that cannot be: the value or its hi is not finite.
+__device__ __forceinline__ void x3_pair(float x, uint32_t& hi, uint32_t& lo, float& bad)
 {
     hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+    const float rest = x - __uint_as_float(hi);
+    bad = fmaf(rest, 0.0f, bad);
+    lo = __float_as_uint(rest) + 0x1000u;
+}
+// ... for those: a NaN stays one, infinities give NaN, and what would round up to infinity is cut off instead
+__device__ __forceinline__ void x3_pair_any(float x, uint32_t& hi, uint32_t& lo)
+{
+    const uint32_t u = __float_as_uint(x);
+    if (!(fabsf(x) <= 3.402823466e38f)) {
+        hi = lo = 0x7fc00000u;
+        return;
+    }
+    hi = (u + 0x1000u) & 0xffffe000u;
+    if ((hi & 0x7f800000u) == 0x7f800000u) hi = u & 0xffffe000u;
     lo = __float_as_uint(x - __uint_as_float(hi)) + 0x1000u;
 }
 
@@ -783,7 +797,7 @@ gemm_x3_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             const uint32_t src = base + s * 2 * kX3Raw;
             constexpr int kEach = kX3Raw / (16 * 32 * kX3ConvWarps);
             static_assert(kX3Raw % (16 * 32 * kX3ConvWarps) == 0, "whole rounds");
-            float x[kEach][4];
+            float x[kEach][4], bad = 0.0f;
             auto put = [&](int i, const uint32_t (&h)[4], const uint32_t (&l)[4]) {
                 const uint32_t at = src + 16u * (t + 32 * kX3ConvWarps * i);
                 asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]) : "memory");
@@ -797,8 +811,17 @@ gemm_x3_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             for (int i = 0; i < kEach; ++i) {
                 uint32_t h[4], l[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) x3_pair(x[i][j], h[j], l[j]);
+                for (int j = 0; j < 4; ++j) x3_pair(x[i][j], h[j], l[j], bad);
                 put(i, h, l);
+            }
+            if (bad != 0.0f) {
+#pragma unroll
+                for (int i = 0; i < kEach; ++i) {
+                    uint32_t h[4], l[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) x3_pair_any(x[i][j], h[j], l[j]);
+                    put(i, h, l);
+                }
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();

@@ -1309,6 +1309,33 @@ def test_fp32_operand_pairs(dist, bound):
     c.close()
 
 
+# A NaN, whatever its bits, and an infinity reach every result that their row of U or column of W takes part in, as something that is not finite, and no other;
+# the largest finite values are not taken for infinities
+@pytest.mark.parametrize("bits", [0x7f800001, 0xff801fff, 0x7fc00000, 0x7fffffff, 0x7f800000, 0xff800000])
+def test_fp32_products_carry_what_is_not_finite(bits):
+    m, d, p = 300, 512, 4096
+    c = binding.Context(0)
+    c.ensure_workspace(m, 0, d, p, "f32")
+    g = torch.Generator(device="cuda"); g.manual_seed(9)
+    U = torch.randn((m, d), generator=g, device="cuda"); W = torch.randn((d, p), generator=g, device="cuda")
+    U[290, :] = 0; U[290, 7] = 3.4028e38                      # rounds up to infinity in tf32
+    W[7, :] = W[7, :].clamp(-0.9, 0.9)
+    ref = U.double() @ W.double()
+    signed = bits - (1 << 32) if bits >= 1 << 31 else bits
+    U.view(torch.int32)[17, 33] = signed
+    W.view(torch.int32)[400, 1234] = signed
+    Y = torch.empty((m, p), device="cuda")
+    c.project(U, W, m, d, p, "f32", Y)
+    assert c.last_status() == binding.OK
+    hit = torch.zeros((m, p), dtype=torch.bool, device="cuda"); hit[17, :] = True; hit[:, 1234] = True
+    assert not torch.isfinite(Y[hit]).any()
+    if bits & 0x7fffff:
+        assert torch.isnan(Y[hit]).all()
+    assert torch.isfinite(Y[~hit]).all()
+    assert ((Y.double() - ref)[~hit].abs() <= 1e-5 * (U.double().nan_to_num().abs() @ W.double().nan_to_num().abs())[~hit]).all()
+    c.close()
+
+
 # fp32 products on either side of the lines between the two FMA kernels: 148 tiles of 64 x 64 and one more where the last stage of k is short,
 # 296 and one more where it is full, with a last tile of eight columns and a K that ends a quad after two
 @pytest.mark.parametrize("m,d,p", [(33, 72, 9472), (33, 72, 9480), (32, 64, 18944), (32, 64, 18952), (65, 64, 9472), (1, 8, 8)])
