@@ -268,6 +268,30 @@ __device__ __forceinline__ void store_tile32(const TcParams& prm, const uint32_t
     __syncwarp();
 }
 
+// 16 fp32 columns of 32 rows (a lane holds one row) from column gn on, through 2 KiB of shared memory: four lanes per row.
+__device__ __forceinline__ void store_cols16(const TcParams& prm, const float* f, uint32_t buf, int m0, int gn, int lane, long long offset)
+{
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"
+                     ::"r"(buf + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4)), "f"(f[4 * q]), "f"(f[4 * q + 1]), "f"(f[4 * q + 2]), "f"(f[4 * q + 3]) : "memory");
+    __syncwarp();
+    const int c = lane & 3, n = gn + 4 * c;
+    const int part = n / prm.csplit;
+    float* base = static_cast<float*>(part == 0 ? prm.C0 : (part == 1 ? prm.C1 : prm.C2));
+    float* dst = base + offset + (long long)(m0 + (lane >> 2)) * prm.ldc + (n - part * prm.csplit);
+    if (n < prm.N) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = 8 * i + (lane >> 2);
+            float4 v;
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(buf + r * 64 + ((c ^ ((r >> 1) & 3)) << 4)) : "memory");
+            if (m0 + r < prm.M) *reinterpret_cast<float4*>(dst + (size_t)(8 * i) * prm.ldc) = v;
+        }
+    }
+    __syncwarp();
+}
+
 // The product as a (hi, lo) bf16 pair, eight columns from gn on.
 template <int G>
 __device__ __forceinline__ void emit_split(const TcParams& prm, int gm, int gn, const uint32_t (&w)[32])
@@ -622,20 +646,28 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
 // registers, rounded to nearest, while the other accumulator fills.  Relative error against 64 bits: K = 504 3.7e-7 (hi cut off 4.5e-7; pairs
 // written to memory, K in eight slices 7.0e-7), K = 4096 4.0e-7 (4.8e-7, 5.3e-6); with 48 instructions twice that.
 //
-// Tiles of 256 x 192 on a pair of CTAs, one tile (or K slice of one) per pair.  Per k-block and SM 28 KB come in, are read and
-// written by the converters and read three times by the matrix instructions: 1310 cycles of shared memory at 128 bytes each, and 1180 cycles of
-// tf32 arithmetic.  It takes 2100: what bounds it is the latency from one role to the next (tensor pipe 54% busy).  192 columns instead of 256 for the registers that the sums take and for the rounds: 512 x 12288 makes
-// 128 tiles for 74 pairs.  A tile takes 1.1 us per k-block, 86% of the 0.71 PFLOP/s that the library's plain tf32 products reach.
-// Against a pass that splits each operand into pairs, a product that reads them from memory and a sum over eight planes:
-// 512 x 12288 x 4096 351 -> 304 us, x 512 123 -> 50 us; eight calls of 512 rows 5.04 -> 3.90 ms, 32 of 1075 rows on 16 lanes 52.1 -> 49.4 ms.
-constexpr int kX3N = 192, kX3Cols = kX3N / 2, kX3Stages = 4, kX3Slice = 2;
-constexpr int kX3ConvWarps = 4;
+// Tiles of 256 x 192 on a pair of CTAs; a pair takes one unit (a tile, or a K slice of one) after the other from the hardware's queue, and the epilogue warps
+// store one unit's sums while the next one's products run.  192 columns instead of 256 for the registers that the sums take.
+// Bound by shared memory: per k-block and SM 28 KB come in, are read and written twice by the converters and read by twelve matrix instructions (84 KB, or
+// 120 with the half of B that comes from the other SM), 1530 to 1810 cycles at 128 bytes each, against 1180 cycles of tf32 arithmetic; a k-block
+// takes 1960.  Two groups of two warps work on a stage each, so that one's waits and fence pass beside the other's arithmetic (one group of four
+// with one unit per pair of CTAs took 2250), and the low parts have three places of their own beside four for the tiles.
+// Microseconds, one unit per pair -> this; in brackets the route before either, pairs written to memory, a product that reads them and a sum over eight planes:
+//   512 x 12288 x 4096  303 -> 277 (350)    1075 x 12288 x 4096  710 -> 642 (670)    800 x 4096 x 4096  223 -> 193 (187)
+//   257 x 12288 x 256  32.6 -> 27.9 (21.7)  768 x 12288 x 256   49.3 -> 38.9 (33.9)  512 x 12288 x 512  49.6 -> 44.0 (124)
+// What is left of the last route's lead lies where K is at most some 450 and 256 x 192 tiles fill a round badly; its error was larger everywhere.
+constexpr int kX3N = 192, kX3Cols = kX3N / 2, kX3Slice = 2;
+constexpr int kX3Stages = 4, kX3LoStages = 3;                 // fp32 tiles on their way, being worked on or read; their low parts
+constexpr int kX3ConvWarps = 4, kX3Groups = 2;
 constexpr int kX3Threads = kThreads + 32 * kX3ConvWarps;
 constexpr uint32_t kX3BBytes = kX3Cols / 32 * 4096u;
-constexpr uint32_t kX3Raw = kABytes + kX3BBytes;              // one stage of fp32 tiles; as much again for their lo parts
-constexpr uint32_t kX3Smem = kX3Stages * 2 * kX3Raw + 1024 + 256;    // (the results leave through the first stage, when nothing reads it any more)
+constexpr uint32_t kX3Raw = kABytes + kX3BBytes;              // one stage of fp32 tiles; as much again for their low parts
+constexpr uint32_t kX3StoreBytes = kEpiWarps * 32 * 64;       // 32 rows of 64 bytes per epilogue warp
+constexpr uint32_t kX3BarBytes = 384;
+constexpr uint32_t kX3Smem = (kX3Stages + kX3LoStages) * kX3Raw + kX3StoreBytes + 1024 + kX3BarBytes;
 static_assert(kX3Smem <= 227 * 1024, "shared memory budget");
 static_assert(kX3Raw % 1024 == 0, "tiles start on swizzle atoms");
+static_assert(kX3LoStages < kX3Stages, "see the converters' wait for a free place");
 constexpr uint32_t kX3Idesc = (1u << 4) | (2u << 7) | (2u << 10) | (1u << 16) | ((uint32_t)(kX3N >> 3) << 17) | ((uint32_t)(2 * BM >> 4) << 24);
 
 struct X3Params {
@@ -674,30 +706,35 @@ gemm_x3_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
-    const uint32_t bars = base + kX3Stages * 2 * kX3Raw;
+    const uint32_t lo_base = base + kX3Stages * kX3Raw, staging = lo_base + kX3LoStages * kX3Raw;
+    const uint32_t bars = staging + kX3StoreBytes;
     uint8_t* bars_gen = smem_raw + (bars - raw);
     auto full_bar = [&](int s) { return bars + 8u * s; };                        // this CTA's tiles are there
-    auto conv_bar = [&](int s) { return bars + 8u * (kX3Stages + s); };          // leader: so are the lo parts in both CTAs
+    auto conv_bar = [&](int s) { return bars + 8u * (kX3Stages + s); };          // leader: so are the pairs in both CTAs
     auto empty_bar = [&](int s) { return bars + 8u * (2 * kX3Stages + s); };
     auto acc_full_bar = [&](int a) { return bars + 8u * (3 * kX3Stages + a); };
     auto acc_empty_bar = [&](int a) { return bars + 8u * (3 * kX3Stages + 2 + a); };
     constexpr uint32_t kMisc = 8 * (3 * kX3Stages + 4);
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bars_gen + kMisc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(bars_gen + kMisc + 8);
-    static_assert(kMisc + 16 <= 256, "barriers fit");
+    constexpr uint32_t kClc = (kMisc + 24 + 15) & ~15u;
+    const uint32_t clc_bar = bars + kMisc + 16, clc_slot = bars + kClc;
+    auto tile_bar = [&](int i) { return bars + kClc + 16u + 8u * i; };
+    const uint32_t ring_base = bars + kClc + 16u + 8u * kRing;
+    static_assert(kClc + 16 + 12 * kRing <= kX3BarBytes, "barriers and ring fit");
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = (int)cluster_rank();
     const TcParams& out = prm.out;
     const int m_tiles = ceil_div(out.M, 2 * BM), mn_tiles = m_tiles * ceil_div(out.N, kX3N);
-    const int tile = blockIdx.x >> 1, mn = tile % mn_tiles, slice = tile / mn_tiles;
-    const int m0 = mn % m_tiles * 2 * BM + rank * BM, n_tile = mn / m_tiles * kX3N;
-    const int kb_lo = slice * prm.per, blocks = min(prm.kb - kb_lo, prm.per);
+    const int first_tile = blockIdx.x >> 1;
 
     chain_next();
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kX3Stages; ++s) { mbar_init(full_bar(s), 1); mbar_init(conv_bar(s), 2 * kX3ConvWarps); mbar_init(empty_bar(s), 1); }
+        for (int s = 0; s < kX3Stages; ++s) { mbar_init(full_bar(s), 1); mbar_init(conv_bar(s), 2 * kX3ConvWarps / kX3Groups); mbar_init(empty_bar(s), 1); }
         for (int a = 0; a < 2; ++a) { mbar_init(acc_full_bar(a), 1); mbar_init(acc_empty_bar(a), 2 * kEpiWarps); }
+        mbar_init(clc_bar, 1);
+        for (int i = 0; i < kRing; ++i) mbar_init(tile_bar(i), 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -714,118 +751,176 @@ gemm_x3_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     chain_wait();
     bool ok = true;
 
+    // The units of a pair (a tile, or a K slice of one): the one that it was launched for, then what the leader's producer gets from the hardware's queue,
+    // handed on through a ring as in gemm_tc_kernel.  The roles are at most kX3Stages + 3 units apart.
+    auto next_tile = [&](uint32_t it) -> int {
+        const int i = it % kRing;
+        if (!mbar_wait_cluster(tile_bar(i), (it / kRing) & 1u, abort_flag, out.wait_ns)) { ok = false; return -1; }
+        int t;
+        asm volatile("ld.shared.s32 %0, [%1];" : "=r"(t) : "r"(ring_base + 4u * i) : "memory");
+        return t;
+    };
+    auto blocks_of = [&](int tile) { return min(prm.kb - tile / mn_tiles * prm.per, prm.per); };
+
     if (warp == 0) {
         if (lane == 0) {
-            const int n0 = n_tile + rank * kX3Cols;
-            for (int it = 0; it < blocks; ++it) {
-                const int s = it % kX3Stages;
-                if (!mbar_wait(empty_bar(s), ((it / kX3Stages) & 1u) ^ 1u, abort_flag, out.wait_ns)) { ok = false; break; }
-                const uint32_t sa = base + s * 2 * kX3Raw, sb = sa + kABytes;
-                const int kb = kb_lo + it;
-                const bool second = kb >= prm.kb0;
-                const CUtensorMap* mb = second ? &map_b1 : &map_b0;
-                const int k = second ? prm.a_k1 + 32 * (kb - prm.kb0) : 32 * kb, row = second ? prm.b_row1 + 32 * (kb - prm.kb0) : 32 * kb;
-                mbar_expect_tx(full_bar(s), kX3Raw);
-                tma_load_2d(sa, &map_a, k, m0, full_bar(s));
-                if (prm.b3d) {
-                    tma_load_3d(sb, mb, 0, row, n0 / 32, full_bar(s));
-                } else {
+            uint32_t it = 0;
+            bool asked = false;
+            int tile = first_tile;
+            for (uint32_t unit = 0; tile >= 0; ++unit) {
+                const int mn = tile % mn_tiles, kb_lo = tile / mn_tiles * prm.per, blocks = blocks_of(tile);
+                const int m0 = mn % m_tiles * 2 * BM + rank * BM, n0 = mn / m_tiles * kX3N + rank * kX3Cols;
+                for (int b = 0; b < blocks; ++b, ++it) {
+                    const int s = it % kX3Stages;
+                    if (!mbar_wait(empty_bar(s), ((it / kX3Stages) & 1u) ^ 1u, abort_flag, out.wait_ns)) { ok = false; break; }
+                    const uint32_t sa = base + s * kX3Raw, sb = sa + kABytes;
+                    const int kb = kb_lo + b;
+                    const bool second = kb >= prm.kb0;
+                    const CUtensorMap* mb = second ? &map_b1 : &map_b0;
+                    const int k = second ? prm.a_k1 + 32 * (kb - prm.kb0) : 32 * kb, row = second ? prm.b_row1 + 32 * (kb - prm.kb0) : 32 * kb;
+                    mbar_expect_tx(full_bar(s), kX3Raw);
+                    tma_load_2d(sa, &map_a, k, m0, full_bar(s));
+                    if (prm.b3d) {
+                        tma_load_3d(sb, mb, 0, row, n0 / 32, full_bar(s));
+                    } else {
 #pragma unroll
-                    for (int j = 0; j < kX3Cols / 32; ++j) tma_load_2d(sb + j * 4096u, mb, n0 + 32 * j, row, full_bar(s));
+                        for (int j = 0; j < kX3Cols / 32; ++j) tma_load_2d(sb + j * 4096u, mb, n0 + 32 * j, row, full_bar(s));
+                    }
+                    // The next unit, while the last of this one's operands come in.  Asked for at once, it would be taken from a pair of SMs
+                    // that is about to be free: 300 x 4096 x 504 25.9 -> 27.4 us, 32 calls of 512 rows on 32 lanes 3.74 -> 3.98 ms
+                    if (rank == 0 && b == blocks - 1) {
+                        mbar_expect_tx(clc_bar, 16);
+                        clc_try_cancel(clc_slot, clc_bar);
+                        asked = true;
+                    }
+                }
+                if (rank == 0) {
+                    if (asked && !mbar_wait(clc_bar, unit & 1u, abort_flag, out.wait_ns)) ok = false;
+                    if (!ok) break;
+                    asked = false;
+                    const int x = clc_answer(clc_slot);
+                    tile = x >= 0 ? x >> 1 : -1;
+                    const uint32_t slot = ring_base + 4u * (unit % kRing), bar = tile_bar(unit % kRing);
+                    asm volatile("st.shared.s32 [%0], %1;" ::"r"(slot), "r"(tile) : "memory");
+                    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(map_rank(slot, 1)), "r"(tile) : "memory");
+                    mbar_arrive_cluster(map_rank(bar, 1));
+                    mbar_arrive(bar);
+                } else {
+                    if (!ok) break;
+                    tile = next_tile(unit);
                 }
             }
         }
     } else if (warp == 1) {
         if (lane == 0 && rank == 0) {
-            for (int it = 0; it < blocks; ++it) {
-                const int s = it % kX3Stages, sl = it / kX3Slice, a = sl & 1;
-                if (it % kX3Slice == 0) {
-                    if (!mbar_wait_cluster(acc_empty_bar(a), ((sl >> 1) & 1u) ^ 1u, abort_flag, out.wait_ns)) { ok = false; break; }
-                    tc_fence_after();
+            uint32_t it = 0, run = 0;                         // stages, and runs of kX3Slice of them
+            for (int tile = first_tile, unit = 0; tile >= 0 && ok; tile = ok ? next_tile(unit) : -1, ++unit) {
+                const int blocks = blocks_of(tile);
+                for (int b = 0; b < blocks; ++b, ++it) {
+                    const int s = it % kX3Stages, a = run & 1;
+                    if (b % kX3Slice == 0) {
+                        if (!mbar_wait_cluster(acc_empty_bar(a), ((run >> 1) & 1u) ^ 1u, abort_flag, out.wait_ns)) { ok = false; break; }
+                        tc_fence_after();
+                    }
+                    if (!mbar_wait_cluster(conv_bar(s), (it / kX3Stages) & 1u, abort_flag, out.wait_ns)) { ok = false; break; }
+                    const uint32_t sa = base + s * kX3Raw, sl = lo_base + it % kX3LoStages * kX3Raw, d = tmem_base + 256u * a;
+                    const uint64_t a_hi = smem_desc(sa, 16, 1024), a_lo = smem_desc(sl, 16, 1024);
+                    const uint64_t b_hi = smem_desc(sa + kABytes, 4096, 512, 1), b_lo = smem_desc(sl + kABytes, 4096, 512, 1);
+                    tc_mma4_tf32_pair(d, a_lo, b_hi, 2, 64, kX3Idesc, b % kX3Slice != 0);
+                    tc_mma4_tf32_pair(d, a_hi, b_lo, 2, 64, kX3Idesc, 1);
+                    tc_mma4_tf32_pair(d, a_hi, b_hi, 2, 64, kX3Idesc, 1);
+                    tc_commit_pair(empty_bar(s));
+                    if (b % kX3Slice == kX3Slice - 1 || b == blocks - 1) { tc_commit_pair(acc_full_bar(a)); ++run; }
                 }
-                if (!mbar_wait_cluster(conv_bar(s), (it / kX3Stages) & 1u, abort_flag, out.wait_ns)) { ok = false; break; }
-                const uint32_t sa = base + s * 2 * kX3Raw, sb = sa + kABytes, d = tmem_base + 256u * a;
-                const uint64_t a_hi = smem_desc(sa, 16, 1024), a_lo = smem_desc(sa + kX3Raw, 16, 1024);
-                const uint64_t b_hi = smem_desc(sb, 4096, 512, 1), b_lo = smem_desc(sb + kX3Raw, 4096, 512, 1);
-                tc_mma4_tf32_pair(d, a_lo, b_hi, 2, 64, kX3Idesc, it % kX3Slice != 0);
-                tc_mma4_tf32_pair(d, a_hi, b_lo, 2, 64, kX3Idesc, 1);
-                tc_mma4_tf32_pair(d, a_hi, b_hi, 2, 64, kX3Idesc, 1);
-                tc_commit_pair(empty_bar(s));
-                if (it % kX3Slice == kX3Slice - 1 || it == blocks - 1) tc_commit_pair(acc_full_bar(a));
             }
         }
     } else if (warp < 2 + kEpiWarps) {
         const int quarter = warp & 3, half = (warp - 2) >> 2;
-        const uint32_t buf = base + (uint32_t)(warp - 2) * 4096u;
-        float sum[kX3Cols];
+        const uint32_t buf = staging + (uint32_t)(warp - 2) * 2048u;
+        uint32_t run = 0;
+        for (int tile = first_tile, unit = 0; tile >= 0 && ok; tile = ok ? next_tile(unit) : -1, ++unit) {
+            float sum[kX3Cols];
 #pragma unroll
-        for (int j = 0; j < kX3Cols; ++j) sum[j] = 0.0f;
-        const int slices = ceil_div(blocks, kX3Slice);
+            for (int j = 0; j < kX3Cols; ++j) sum[j] = 0.0f;
+            const int runs = ceil_div(blocks_of(tile), kX3Slice);
 #pragma unroll 1
-        for (int sl = 0; sl < slices; ++sl) {
-            const int a = sl & 1;
-            if (!mbar_wait(acc_full_bar(a), (sl >> 1) & 1u, abort_flag, out.wait_ns)) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + 256u * a + (uint32_t)(half * kX3Cols);
+            for (int r = 0; r < runs; ++r, ++run) {
+                const int a = run & 1;
+                if (!mbar_wait(acc_full_bar(a), (run >> 1) & 1u, abort_flag, out.wait_ns)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + 256u * a + (uint32_t)(half * kX3Cols);
 #pragma unroll
-            for (int c = 0; c < kX3Cols; c += 32) {
-                uint32_t v[32];
-                tc_ld_32cols(taddr + c, v);
-                tc_ld_wait();
+                for (int c = 0; c < kX3Cols; c += 16) {
+                    uint32_t v[16];
+                    tc_ld_16cols(taddr + c, v);
+                    tc_ld_wait();
 #pragma unroll
-                for (int j = 0; j < 32; ++j) sum[c + j] += __uint_as_float(v[j]);
+                    for (int j = 0; j < 16; ++j) sum[c + j] += __uint_as_float(v[j]);
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(map_rank(acc_empty_bar(a), 0));
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(map_rank(acc_empty_bar(a), 0));
-        }
-        if (ok) {
+            if (ok) {
+                const int mn = tile % mn_tiles;
+                const int m0 = mn % m_tiles * 2 * BM + rank * BM + quarter * 32, n0 = mn / m_tiles * kX3N + half * kX3Cols;
 #pragma unroll
-            for (int c = 0; c < kX3Cols; c += 32) {
-                uint32_t v[32];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(sum[c + j]);
-                if (n_tile + half * kX3Cols + c < out.N)
-                    store_tile32(out, v, buf, m0 + quarter * 32, n_tile + half * kX3Cols + c, lane, slice);
+                for (int c = 0; c < kX3Cols; c += 16)
+                    if (n0 + c < out.N) store_cols16(out, sum + c, buf, m0, n0 + c, lane, (long long)(tile / mn_tiles) * out.plane);
             }
         }
     } else {
-        const int t = threadIdx.x - kThreads;
-        for (int it = 0; it < blocks; ++it) {
-            const int s = it % kX3Stages;
-            if (!mbar_wait(full_bar(s), (it / kX3Stages) & 1u, abort_flag, out.wait_ns)) { ok = false; break; }
-            const uint32_t src = base + s * 2 * kX3Raw;
-            constexpr int kEach = kX3Raw / (16 * 32 * kX3ConvWarps);
-            static_assert(kX3Raw % (16 * 32 * kX3ConvWarps) == 0, "whole rounds");
-            float x[kEach][4], bad = 0.0f;
-            auto put = [&](int i, const uint32_t (&h)[4], const uint32_t (&l)[4]) {
-                const uint32_t at = src + 16u * (t + 32 * kX3ConvWarps * i);
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]) : "memory");
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at + kX3Raw), "r"(l[0]), "r"(l[1]), "r"(l[2]), "r"(l[3]) : "memory");
-            };
-#pragma unroll
-            for (int i = 0; i < kEach; ++i)                   // all loads before the first store
-                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[i][0]), "=f"(x[i][1]), "=f"(x[i][2]), "=f"(x[i][3])
-                             : "r"(src + 16u * (t + 32 * kX3ConvWarps * i)) : "memory");
-#pragma unroll
-            for (int i = 0; i < kEach; ++i) {
-                uint32_t h[4], l[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) x3_pair(x[i][j], h[j], l[j], bad);
-                put(i, h, l);
-            }
-            if (bad != 0.0f) {
-#pragma unroll
-                for (int i = 0; i < kEach; ++i) {
-                    uint32_t h[4], l[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) x3_pair_any(x[i][j], h[j], l[j]);
-                    put(i, h, l);
+        // converters: two warps per stage, two stages at a time, so that one's waits and fence pass beside the other's arithmetic
+        const int group = (warp - 2 - kEpiWarps) / (kX3ConvWarps / kX3Groups);
+        constexpr int kGroupThreads = 32 * kX3ConvWarps / kX3Groups, kEach = 14;
+        constexpr int kRounds = kX3Raw / (16 * kGroupThreads * kEach);
+        static_assert(kX3Raw % (16 * kGroupThreads * kEach) == 0, "whole rounds");
+        const uint32_t t = 16u * ((threadIdx.x - kThreads) % kGroupThreads);
+        uint32_t it = 0;
+        for (int tile = first_tile, unit = 0; tile >= 0 && ok; tile = ok ? next_tile(unit) : -1, ++unit) {
+            const int blocks = blocks_of(tile);
+            for (int b = 0; b < blocks; ++b, ++it) {
+                if (it % kX3Groups != group) continue;
+                const int s = it % kX3Stages;
+                if (!mbar_wait(full_bar(s), (it / kX3Stages) & 1u, abort_flag, out.wait_ns)) { ok = false; break; }
+                if (it >= kX3LoStages) {
+                    // the place of the low parts was last that of stage it - kX3LoStages; its barrier is at most one phase further, since the
+                    // next one that it counts comes after this stage
+                    const uint32_t old = it - kX3LoStages;
+                    if (!mbar_wait(empty_bar(old % kX3Stages), (old / kX3Stages) & 1u, abort_flag, out.wait_ns)) { ok = false; break; }
                 }
+                const uint32_t hi_at = base + s * kX3Raw + t, lo_at = lo_base + it % kX3LoStages * kX3Raw + t;
+#pragma unroll 1
+                for (int r = 0; r < kRounds; ++r) {
+                    const uint32_t off = r * (16u * kGroupThreads * kEach);
+                    float x[kEach][4], bad = 0.0f;
+#pragma unroll
+                    for (int i = 0; i < kEach; ++i)           // all loads before the first store
+                        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[i][0]), "=f"(x[i][1]), "=f"(x[i][2]), "=f"(x[i][3])
+                                     : "r"(hi_at + off + 16u * kGroupThreads * i) : "memory");
+#pragma unroll
+                    for (int i = 0; i < kEach; ++i) {
+                        uint32_t h[4], l[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) x3_pair(x[i][j], h[j], l[j], bad);
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(hi_at + off + 16u * kGroupThreads * i), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]) : "memory");
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(lo_at + off + 16u * kGroupThreads * i), "r"(l[0]), "r"(l[1]), "r"(l[2]), "r"(l[3]) : "memory");
+                    }
+                    if (bad != 0.0f) {
+#pragma unroll
+                        for (int i = 0; i < kEach; ++i) {
+                            uint32_t h[4], l[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) x3_pair_any(x[i][j], h[j], l[j]);
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(hi_at + off + 16u * kGroupThreads * i), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]) : "memory");
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(lo_at + off + 16u * kGroupThreads * i), "r"(l[0]), "r"(l[1]), "r"(l[2]), "r"(l[3]) : "memory");
+                        }
+                    }
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(map_rank(conv_bar(s), 0));
             }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(map_rank(conv_bar(s), 0));
         }
     }
     if (!ok) { *abort_flag = 1; atomicCAS(out.status, 0, (int)GELO_ERR_TIMEOUT); }
@@ -1439,12 +1534,12 @@ int launch_gemm_tf32x3(gelo_ctx* ctx, int M, int N, int K, const float* A, int l
     p.b3d = b3d ? 1 : 0;
     const int tiles = ceil_div(M, 2 * BM) * ceil_div(N, kX3N);
     // K slices where they fill the rounds better than whole tiles and that is worth their planes, which are written and read: microseconds,
-    // with 1.14 per k-block, 6 per tile for its first copies and its stores, 6 TB/s for the planes and 5 for the launch that sums them.  1075 x 12288
-    // x 4096 in three slices 741 -> 730 (709 since); 512 rows stay whole (304).
+    // with 1.06 per k-block, 2 per unit for what is not hidden of its seams, 6 TB/s for the planes and 5 for the launch that sums them.  1075 x 3072
+    // x 1024 76 -> 67, 257 x 12288 x 4096 276 -> 264; 512 x 12288 x 4096 stays whole (277).
     int slices = 1;
     double best = 0.0;
     for (int t = 1; t <= kTf32x3Slices && (t == 1 || (planes && aligned16(planes) && p.kb >= 8 * t)); ++t) {
-        const double us = ceil_div(tiles * t, ctx->sm_count / 2) * (1.14 * ceil_div(p.kb, t) + 6.0) + (t > 1 ? 5.0 + 8e-6 * t * (double)M * N / 6.0 : 0.0);
+        const double us = ceil_div(tiles * t, ctx->sm_count / 2) * (1.06 * ceil_div(p.kb, t) + 2.0) + (t > 1 ? 5.0 + 8e-6 * t * (double)M * N / 6.0 : 0.0);
         if (t == 1 || us < best) { best = us; slices = t; }
     }
     p.per = ceil_div(p.kb, slices);

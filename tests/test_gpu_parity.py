@@ -1287,6 +1287,25 @@ def test_fp32_products_on_the_tensor_cores(m, d, p):
     c.close()
 
 
+# Many units per pair of CTAs, so that copies, converters, products and stores are in different ones: of a single k-block, of three (an accumulator run cut
+# short), and K slices of several tiles that are not all of one length (1075 x 3072 x 1032: 33 k-blocks in slices of 9 and less)
+@pytest.mark.parametrize("m,d,p", [(512, 32, 33000), (300, 96, 24600), (1075, 1032, 3072), (641, 72, 12288)])
+def test_fp32_products_of_many_units(m, d, p):
+    c = binding.Context(0)
+    c.ensure_workspace(m, 0, d, p, "f32")
+    g = torch.Generator(device="cuda"); g.manual_seed(m)
+    W = torch.randn((d, p), generator=g, device="cuda")
+    for i in range(3):
+        U = torch.randn((m, d), generator=g, device="cuda")
+        Y = torch.full((m, p), float("nan"), device="cuda")
+        c.project(U, W, m, d, p, "f32", Y)
+        ref = U.double() @ W.double()
+        assert ((Y.double() - ref).norm() / ref.norm()).item() <= 8e-7
+        assert (Y.double() - ref).abs().max().item() <= 1e-5 * d ** 0.5      # (as above)
+    assert c.last_status() == binding.OK
+    c.close()
+
+
 # The operand pairs by themselves: U is diagonal, so every result is one product of two entries and there is nothing to add up.  With both parts rounded to
 # nearest lo is half a unit of tf32 at most, 2^-11 of the entry, its own rounding 2^-23, the dropped lo lo 2^-22, and three truncated additions take up to
 # 2^-23 each: 3.5 x 2^-22 in all.  Entries of 1 + 2^-10 - 2^-23 have parts of 1 + 2^-10 and -2^-23, of which only the additions lose anything; cut off
