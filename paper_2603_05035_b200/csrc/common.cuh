@@ -79,7 +79,7 @@ struct gelo_ctx {
     cudaEvent_t batch_start = nullptr;
     cudaStream_t side = nullptr;                    // branches of recorded sampling graphs
     cudaEvent_t side_from = nullptr, side_done = nullptr;
-    cudaStream_t form = nullptr;                    // where a QR that runs alone forms Q while it factorises
+    cudaStream_t form = nullptr;                    // where a QR with at most two others beside it forms Q while it factorises
     cudaEvent_t form_from = nullptr, form_done = nullptr;
     // a batched call may chain onto the previous one (lanes wait for their own lane_free events only) when
     // nothing else has touched the workspace in between

@@ -668,12 +668,19 @@ last_rows_kernel(const float* __restrict__ rows, float* __restrict__ copy, int f
 
 }  // namespace
 
-// Rows from which a QR that has the GPU to itself forms Q^T while it factorises (see run_gaussian_qr), and the SMs that it does that on.
-// From three superblocks on there is something to form beside the next one, and one spare matrix has room for the products' scratch: one call
-// alone at 1600 rows 1173 -> 1125 us, 2150 rows 1578 -> 1460, 4300 rows orthogonal 3837 -> 3512, non-orthogonal 4485 -> 4026 us.
-// On all SMs the chain's launches would wait for tiles of 20 to 30 us (4304 us); on 48, 64, 96 and 128 of them 4089, 4099, 4112 and 4148 us.
+// Rows from which a QR with at most two others beside it forms Q^T while it factorises (see run_gaussian_qr), and the SMs that it does that on.
+// From three superblocks on there is something to form beside the next one, and one spare matrix has room for the products' scratch.  Whole
+// calls, d = 4096, p = 12288, us, Q accumulated backwards -> this:
+//                              1536 rows      1600 rows      2150 rows      4300 rows      4300 rows non-orthogonal
+//   one call                   1018 ->  976   1142 -> 1036   1509 -> 1415   3794 -> 3461   4403 -> 4056
+//   two at once, two lanes     1315 -> 1217   1431 -> 1304   2008 -> 1856   5430 -> 5046   6633 -> 6261
+//   three at once, three lanes 1530 -> 1432   1667 -> 1552   2458 -> 2282   7161 -> 6784   9016 -> 8725
+// Fewer SMs leave more of them to the chains: 64 are as good for one call and up to 1% slower for two or three, 80 and 96 0.3% and 1 to 2%,
+// 112 0.5% and 2%; on all of them the chain's launches wait for tiles of 20 to 30 us (4304 us where 80 gave 4026).
+// The factor is as good: 2150 rows in half, orthogonal, columns 3.19e-3 -> 3.20e-3 off (the first half of them 7.5e-4 -> 8.0e-4), unpolished
+// 3.35e-3 -> 3.36e-3 (1.12e-3 -> 1.11e-3) with Q^T Q - I 2.07e-3 -> 2.06e-3; at 4300 rows 1.92e-3 -> 1.85e-3.
 constexpr int kFormRows = 3 * kSuper;
-constexpr int kFormSms = 80;
+constexpr int kFormSms = 48;
 
 bool gaussian_qr_supports(int m) { return m > FB; }
 
@@ -687,8 +694,9 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
     const float loss1 = exact ? 1.0f : 1.0f + kTf32TruncLoss, loss2 = loss1 * loss1;
     const int round = exact ? 0 : 1;
     // In a recorded graph of a call that runs alone, what nobody waits for yet goes into branches of the graph (on the context's side
-    // stream): the merges, which are needed at the end of a superblock, and the last square with its columns of Q.
-    // 2150 rows orthogonal, one call 1.61 -> 1.56 ms; 4300 non-orthogonal 4.51 -> 4.41 ms.
+    // stream): the merges, which are needed at the end of a superblock (with them 2150 rows orthogonal, one call 1.61 -> 1.56 ms; 4300 non-orthogonal
+    // 4.51 -> 4.41), and, where Q is accumulated backwards, the last square with its columns of Q (1400 + 70 rows 914 -> 912 us, 1000 + 50 and
+    // below no difference).
     const bool fork = ctx->recording && ctx->tc_update_ctas == 0;
     cudaStream_t cur = st;                                   // where the products go
     auto branch = [&]() -> int {
@@ -702,11 +710,12 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
         GELO_CUDA_OK(cudaStreamWaitEvent(st, ctx->side_done, 0));
         return GELO_OK;
     };
-    // A QR that has the GPU to itself spends most of its time in launches that leave SMs idle, half of it in block factors on three SMs.
+    // A QR alone, or one of two or three, spends most of its time in launches that leave SMs idle, half of it in block factors on three SMs.
     // Beside them it forms Q^T: the reflectors of a superblock are applied to the identity as they are to the columns on the right, on a stream
     // of its own, while the next superblock is factorised, on kFormSms of the SMs so that the chain finds others free.  That
     // takes half as many operations again as accumulating Q backwards, which needs the last reflector first, so it is not
-    // for lanes, where SM time counts.
+    // for four lanes and more (tc_update_ctas), which fill the GPU.  Samples side by side share the stream while they are recorded, one
+    // after the other; replayed, each has a branch of its own.
     const bool forming = transposed && !exact && ctx->tc_update_ctas == 0 && m >= kFormRows && tc.big[0];
     struct FormGuard {                                       // however it ends, the caller's stream comes after all launches
         gelo_ctx* ctx; cudaStream_t st; bool on;
