@@ -1355,6 +1355,26 @@ def test_fp32_products_carry_what_is_not_finite(bits):
     c.close()
 
 
+# The kernel of the large fp32 products with a wait limit of zero: every role gives up before the first copy, nothing is written
+def test_zero_wait_limit_reaches_the_fp32_products():
+    m, d, p = 256, 256, 8192                                  # (too short for K slices, whose sum is a launch of its own)
+    c = binding.Context(0)
+    c.ensure_workspace(m, 0, d, p, "f32")
+    g = torch.Generator(device="cuda"); g.manual_seed(2)
+    U = torch.randn((m, d), generator=g, device="cuda"); W = torch.randn((d, p), generator=g, device="cuda")
+    Y = torch.full((m, p), float("nan"), device="cuda")
+    c.set_wait_limit_ns(0)
+    c.project(U, W, m, d, p, "f32", Y)
+    assert c.last_status() == binding.ERR_TIMEOUT
+    assert torch.isnan(Y).all()
+    c.set_wait_limit_ns(2_000_000_000)
+    c.project(U, W, m, d, p, "f32", Y)
+    assert c.last_status() == binding.OK
+    ref = U.double() @ W.double()
+    assert ((Y.double() - ref).norm() / ref.norm()).item() <= 8e-7
+    c.close()
+
+
 # fp32 products on either side of the lines between the two FMA kernels: 148 tiles of 64 x 64 and one more where the last stage of k is short,
 # 296 and one more where it is full, with a last tile of eight columns and a K that ends a quad after two
 @pytest.mark.parametrize("m,d,p", [(33, 72, 9472), (33, 72, 9480), (32, 64, 18944), (32, 64, 18952), (65, 64, 9472), (1, 8, 8)])
