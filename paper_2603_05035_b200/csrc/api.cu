@@ -297,7 +297,7 @@ int sample_on_lane(gelo_ctx* ctx, const Layout& L, int lane, int m, int kind, ui
         return sample_attempt(ctx, L, m, kind, seed, 0u, dtype, L.A, L.Ainv, L.ldi, nullptr, ls, deferred, nullptr);
     uint64_t* slot = ctx->lane_seed_dev + lane * 8;
     const gelo_ctx::SampleKey key = { L.G, L.A, L.Ainv, L.cond_val, slot, L.m, m, kind, dtype, ctx->level3, ctx->tc_update_ctas, ctx->panel_samples,
-                                     deferred };
+                                     forms_beside(ctx, m), deferred };
     for (auto& g : ctx->graphs) {
         if (g.key == key) {
             set_seed_kernel<<<1, 1, 0, ls>>>(slot, seed);
@@ -472,10 +472,11 @@ struct LanePlan {
     {
         const bool shares = lanes >= c->lane_tc_share && c->lane_tc_share > 1;
         c->tc_update_ctas = shares ? c->sm_count / c->lane_tc_share : 0;
+        c->in_flight = lanes;
         c->panel_samples = panels_hide(m, orth, non, shares);
     }
     LanePlan(const LanePlan&) = delete;
-    ~LanePlan() { ctx->tc_update_ctas = 0; ctx->panel_samples = ctx->lone_launches = false; }
+    ~LanePlan() { ctx->tc_update_ctas = 0; ctx->in_flight = 1; ctx->panel_samples = ctx->lone_launches = false; }
 };
 
 // One whole call on the caller's stream.  A non-orthogonal pair is verified: the first attempt replays the recorded sampling

@@ -60,6 +60,7 @@ struct gelo_ctx {
     int tc_update_ctas = 0;       // CTAs that a level-3 tensor-core launch is planned for (0: one per SM): with many lanes fewer K slices
                                   // do, because the updates of several lanes run side by side
     bool tc_cap = false;          // ... and does not get more than that many either
+    int in_flight = 1;            // samples that are drawn beside each other (the lanes of the running batch)
     bool lone_launches = false;   // whole calls run on lanes beside each other and must not hold SMs while they wait (chain_launches)
     bool panel_samples = false;   // fp32 samples of the running batch take 32-column panels (panels_hide in api.cu)
     int level3 = 0;               // 0: tf32 tensor-core updates for bf16 calls with m >= 256; 1: always fp32 FMA;
@@ -79,7 +80,7 @@ struct gelo_ctx {
     cudaEvent_t batch_start = nullptr;
     cudaStream_t side = nullptr;                    // branches of recorded sampling graphs
     cudaEvent_t side_from = nullptr, side_done = nullptr;
-    cudaStream_t form = nullptr;                    // where a QR with at most two others beside it forms Q while it factorises
+    cudaStream_t form = nullptr;                    // where a QR with few others beside it forms Q while it factorises
     cudaEvent_t form_from = nullptr, form_done = nullptr;
     // a batched call may chain onto the previous one (lanes wait for their own lane_free events only) when
     // nothing else has touched the workspace in between
@@ -94,11 +95,11 @@ struct gelo_ctx {
     // the estimate: they stand behind the row norms of the data rows, so they move with n at equal m.
     struct SampleKey {
         const void *G, *A, *Ainv, *cond, *seed;
-        int rows, m, kind, dtype, level3, tc_ctas, panels, deferred;
+        int rows, m, kind, dtype, level3, tc_ctas, panels, beside, deferred;
         bool operator==(const SampleKey& o) const
         {
             return G == o.G && A == o.A && Ainv == o.Ainv && cond == o.cond && seed == o.seed && rows == o.rows && m == o.m && kind == o.kind &&
-                   dtype == o.dtype && level3 == o.level3 && tc_ctas == o.tc_ctas && panels == o.panels && deferred == o.deferred;
+                   dtype == o.dtype && level3 == o.level3 && tc_ctas == o.tc_ctas && panels == o.panels && beside == o.beside && deferred == o.deferred;
         }
     };
     struct SampleGraph { SampleKey key; cudaGraphExec_t exec; long long launches; unsigned long long used; };
@@ -328,6 +329,7 @@ int run_householder_qr_tf32(gelo_ctx*, int m, float* R, int ld, float* Q, const 
 // blocks being well conditioned), on tf32 products or (exact) on fp32 multiply-adds.  G is overwritten with the reflectors; Q
 // receives the factor whose R has a positive diagonal, or its transpose (*transposed; only where the caller gives the pointer).
 bool gaussian_qr_supports(int m);
+bool forms_beside(const gelo_ctx*, int m);       // what decides that (beside the precision)
 int run_gaussian_qr(gelo_ctx*, int m, float* G, int ld, float* Q, const TcScratch&, bool exact, cudaStream_t, bool* transposed);
 // One Newton-Schulz step Q <- Q - Q (Q^T Q - I) / 2 on the tensor cores in tf32: squares the orthogonality defect
 // that tf32 updates leave in Q.  D and Qold are m x ld scratch matrices.

@@ -668,7 +668,7 @@ last_rows_kernel(const float* __restrict__ rows, float* __restrict__ copy, int f
 
 }  // namespace
 
-// Rows from which a QR with at most two others beside it forms Q^T while it factorises (see run_gaussian_qr), and the SMs that it does that on.
+// Rows from which a QR with few others beside it forms Q^T while it factorises (see run_gaussian_qr), and the SMs that it does that on.
 // From three superblocks on there is something to form beside the next one, and one spare matrix has room for the products' scratch.  Whole
 // calls, d = 4096, p = 12288, us, Q accumulated backwards -> this:
 //                              1536 rows      1600 rows      2150 rows      4300 rows      4300 rows non-orthogonal
@@ -681,6 +681,14 @@ last_rows_kernel(const float* __restrict__ rows, float* __restrict__ copy, int f
 // 3.35e-3 -> 3.36e-3 (1.12e-3 -> 1.11e-3) with Q^T Q - I 2.07e-3 -> 2.06e-3; at 4300 rows 1.92e-3 -> 1.85e-3.
 constexpr int kFormRows = 3 * kSuper;
 constexpr int kFormSms = 48;
+// Lanes that share the SMs out fill the GPU with four samples.  Where they do not (gelo_set_lane_share), forming Q beside them gains as long as the samples in
+// flight have some 32000 rows in all: 4 x 2150 rows 3005 -> 2848 us, 16 x 1600 6295 -> 6081, but 16 x 2150 9992 -> 10056, 16 x 4300 34919 -> 35821.
+constexpr int kFormRowsInFlight = 32000;
+
+bool forms_beside(const gelo_ctx* ctx, int m)
+{
+    return ctx->tc_update_ctas == 0 && m >= kFormRows && (long long)ctx->in_flight * m <= kFormRowsInFlight;
+}
 
 bool gaussian_qr_supports(int m) { return m > FB; }
 
@@ -710,13 +718,13 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
         GELO_CUDA_OK(cudaStreamWaitEvent(st, ctx->side_done, 0));
         return GELO_OK;
     };
-    // A QR alone, or one of two or three, spends most of its time in launches that leave SMs idle, half of it in block factors on three SMs.
+    // A QR alone, or one of a few, spends most of its time in launches that leave SMs idle, half of it in block factors on three SMs.
     // Beside them it forms Q^T: the reflectors of a superblock are applied to the identity as they are to the columns on the right, on a stream
     // of its own, while the next superblock is factorised, on kFormSms of the SMs so that the chain finds others free.  That
     // takes half as many operations again as accumulating Q backwards, which needs the last reflector first, so it is not
-    // for four lanes and more (tc_update_ctas), which fill the GPU.  Samples side by side share the stream while they are recorded, one
+    // for a GPU that is full (forms_beside).  Samples side by side share the stream while they are recorded, one
     // after the other; replayed, each has a branch of its own.
-    const bool forming = transposed && !exact && ctx->tc_update_ctas == 0 && m >= kFormRows && tc.big[0];
+    const bool forming = transposed && !exact && forms_beside(ctx, m) && tc.big[0];
     struct FormGuard {                                       // however it ends, the caller's stream comes after all launches
         gelo_ctx* ctx; cudaStream_t st; bool on;
         ~FormGuard()

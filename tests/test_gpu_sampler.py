@@ -95,6 +95,30 @@ def test_factors_formed_in_small_batches(calls, n, k):
     c.close()
 
 
+# Factors are formed beside their factorisations only while the samples in flight do not fill the GPU (32000 rows in all), also where lanes do not share
+# the SMs out (share 1): beyond, another number of launches per call
+def test_factors_are_formed_for_few_samples_only():
+    n, d, p, dt = 1536, 64, 64, "bf16"
+    W = inputs.make_weight(d, p, dt, 1, "cuda")
+    H = [inputs.make_hidden(n, d, dt, 1, True, "cuda")] * 24
+    launches = {}
+    for calls in (1, 4, 24):
+        c = binding.Context(0)
+        c.set_lanes(calls)
+        c.set_lane_share(1)
+        c.ensure_batch_workspace(n, 0, d, p, dt, calls)
+        Y = torch.zeros((calls, n, p), dtype=TDT[dt], device="cuda")
+        for run in range(2):
+            c.launch_count(reset=True)
+            c.qkv_offload_batch(H[:calls], [W] * calls, n, 0, d, p, [ORTHOGONAL] * calls, list(range(calls)), 10.0, dt, list(Y))
+            launches[calls] = c.launch_count() / calls
+        assert c.last_status() == binding.OK
+        ref = H[0].double() @ W.double()
+        assert all(((y.double() - ref).norm() / ref.norm()).item() <= 2e-2 for y in Y)       # the bf16 path's tolerance
+        c.close()
+    assert launches[4] == launches[1] and launches[24] != launches[1]
+
+
 # 256: the first size of the iteration, a single pair of tile rows; 257 and 300: ragged tiles; gamma 0.55 is the last it takes,
 # 0.6 goes to the LU
 @pytest.mark.parametrize("m,gamma,dt", [(256, 0.5, "f16"), (257, 0.5, "bf16"), (300, 0.55, "f16"), (700, 0.5, "f16"), (300, 0.6, "f16")])
