@@ -591,7 +591,7 @@ def measure_workload(name, lanes, steps, warmup, calls=0, latency_steps=0):
     # the plain, unprotected projection through the same entry point, hence on the same kernel as the chain's products
     timed("plain_project", lambda r: ctx.project(Hs[r % calls], Ws[r % calls], n, d, p, w.dtype, Yp), 32)
     if w.dtype == "f32":
-        # a context without workspace has no room for operand pairs: the same product on the FP32 FMA pipes
+        # a context without workspace runs the same product on the FP32 FMA pipes
         bare = gelo.Context(dev.index)
         timed("plain_project_fma", lambda r: bare.project(Hs[r % calls], Ws[r % calls], n, d, p, w.dtype, Yp), 8)
         bare.close()

@@ -417,9 +417,10 @@ int unmix_impl(gelo_ctx* ctx, const void* Ainv, int lda, const void* Yp, int n, 
     return product(ctx, g, t3, st);
 }
 
-// The single-stage entry points have no scratch of their own; when the context holds a workspace, the large fp32 products of
-// projection and unmixing run on the tensor cores exactly as inside the whole call (so that a plain
-// H W through gelo_project is timed on the same kernel as the obfuscated chain).  Without one they stay on the FMA kernel.
+// The single-stage entry points have no scratch of their own; when the context holds a workspace with room for a call of these sizes, the large fp32
+// products of projection and unmixing run on the tensor cores exactly as inside the whole call (so that a plain
+// H W through gelo_project is timed on the same kernel as the obfuscated chain).  Without one they stay on the FMA kernel, as gelo_mix does: the
+// tensor-core kernel needs scratch only to cut K into slices, but a caller without workspace has always had the FMA kernel's sums.
 const Tf32x3Scratch* stage_pairs(gelo_ctx* ctx, int rows, int k, int d, int p, int dtype, Layout* L)
 {
     if (dtype != GELO_F32 || !ctx->ws) return nullptr;

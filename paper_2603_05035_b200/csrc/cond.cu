@@ -8,7 +8,8 @@
 // The operators are the matrices as stored (bf16 or fp32), i.e. exactly what the mixing and unmixing products
 // read.  All sums have a fixed order, so the estimate is bit-reproducible.
 //
-// A step is two launches: cond_step_kernel, bound by reading both operators (74 MB at 4300 rows in bf16, which stay in
+// Where the rows of a matrix fit the shared memory of eight CTAs (16 bits: up to 920 rows, fp32: 656) all steps are one launch, cond_small_kernel.
+// Beyond, a step is two: cond_step_kernel, bound by reading both operators (74 MB at 4300 rows in bf16, which stay in
 // L2 from step to step), and cond_reduce_kernel, whose last CTA also does the Lanczos recurrence.  What counts is
 // loads in flight: slabs of 16 rows (538 CTAs at 4300 rows) with two rows per warp and whole-vector loads of x, the
 // slab sums spread over sixteen threads per column, the eigenvalues searched by 32 lanes at a time.  Against 32-row
@@ -334,7 +335,10 @@ __global__ void __launch_bounds__(256) cond_step_kernel(CondViews v)
 // operator; each CTA keeps its rows on chip, forms its part of Op^T (Op v), and after one barrier of the cluster every CTA adds the eight
 // parts up in the same order and does the recurrence for itself, so the vector never travels.  Bound by latency, 2 us a step; as
 // launches of their own the steps take 8 us each.  With the verdict,
-// fp32: 64 rows 56 -> 19 us, 350 rows 63 -> 33, 512 rows 64 -> 44, 650 rows 75 -> 62.
+// fp32: 64 rows 56 -> 19 us, 350 rows 63 -> 33, 512 rows 64 -> 44, 650 rows 75 -> 62.  Batches gain too, though the two clusters need sixteen
+// SMs of their own: calls with d = 1024 and a non-orthogonal A, the general route -> this, us: bf16, 8 x 315 rows on 8 lanes 589 -> 539, 32 x 350 on
+// 32 lanes 1156 -> 1090, 32 x 900 on 32 lanes 3570 -> 3348; fp32, 8 x 64 on 8 lanes 414 -> 409, 32 x 300 on 32 lanes 3760 -> 3744, 32 x 512 5594 -> 5559;
+// only 32 x 130 in fp32 on 16 or 32 lanes lose, 2590 -> 2610 (waited for 2795 -> 2771).
 constexpr int kSmallCtas = 8, kSmallThreads = 1024;
 struct CondSmallPlan { int rows, lds; size_t slab, bytes; };
 CondSmallPlan cond_small_plan(int m, int es)
