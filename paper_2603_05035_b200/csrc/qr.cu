@@ -502,8 +502,7 @@ t_merge_kernel(const float* __restrict__ part, int slabs, int ldp, const float* 
 // then each group builds its column of Q = H_0 ... H_(m-1) by applying the reflectors backwards to e_c, two per shuffle: with
 // g = v_(j+1) . v_j known, w_j after H_(j+1) is w_j - g tau_(j+1) w_(j+1).  Only H_j with j <= c touch e_c.
 // Against owners that normalise their column before they publish it, shuffles of single groups and one reflector at a time, a whole sample in
-// fp32: 32 rows 21 -> 18 us, 64 rows 46 -> 36, 72 rows 50 -> 40, 96 rows 87 -> 65; a link of the chain 1090 -> 780 cycles at 64 columns,
-// 660 -> 520 at the last ones.
+// fp32, back to back: 32 rows 18.6 -> 11.6 us, 64 rows 45.7 -> 28.9, 68 rows 49.3 -> 34.3, 96 rows 98.3 -> 57.9.
 // Same conventions as the blocked path: R (upper triangle, diagonal of either sign) overwrites G, Q is unsigned.
 template <int RM>
 struct QrSmall {
@@ -751,7 +750,7 @@ int launch_sample_small_rm(gelo_ctx* ctx, int m, uint64_t seed, uint32_t attempt
 constexpr int kSmallQrRows = 128;
 
 // f(RM) for the smallest instance that holds m rows, in steps of eight: the time grows with the instance (the rows a thread holds, and the
-// columns of the reflectors), 18 us for 32 rows, 36 for 64 and 65 for 96.
+// columns of the reflectors), 12 us for 32 rows, 29 for 64 and 58 for 96.
 template <int RM = 32, typename F>
 int with_small_rows(int m, F&& f)
 {

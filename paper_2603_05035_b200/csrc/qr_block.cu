@@ -797,7 +797,7 @@ int run_gaussian_qr(gelo_ctx* ctx, int m, float* G, int ld, float* Q, const TcSc
     };
 
     // Block columns: 128 wide while at least twice as many rows are left, then narrower ones (half of the rows, a multiple of eight) down to a
-    // square of at most 96 rows for the Householder kernel, which takes 36 us for 64 rows and 65 for 96, against about
+    // square of at most 96 rows for the Householder kernel, which takes 29 us for 64 rows and 58 for 96, against about
     // 50 us for a block.
     std::vector<int> start;
     int bf = 0;                                              // first column of the square that is left for Householder
